@@ -22,44 +22,131 @@
 // The minimum can be attained at several scales; the smallest is reported.
 // FP8-quantised optimum: the better of floor_E4M3(s*) and ceil_E4M3(s*) (ties
 // to the floor), each scored with the sweep's arithmetic contract.
+//
+// One thread per block, in two passes over the 7n segments.  The first screens:
+// the value of a segment's quadratic at its minimum is A - B^2/C (A = sum w a^2),
+// so B and C alone rank it, to a few fp32 roundings of A.  The seven segments of
+// one element run together, two to a packed f32x2 operation, over magnitudes and
+// weights kept in shared memory (a column per thread, no bank conflicts); a
+// segment that could still be the minimum is noted in a short list.  The second
+// pass scores the list's remaining segments (about one per block) exactly, in
+// element order and in fp32 sums of w e^2, and takes the smallest.  See screen_ok
+// and screen_limit for why the first pass cannot lose the second one's answer.
+// Bound by instruction issue: about 33 (MSE) or 37 (WMSE) instructions for each pair of
+// elements (i, j) of a block, against about 15 times that when every segment was
+// scored in full with the rounding done by selects.
 #include "nvfp4_device.cuh"
 #include "nvfp4_kernels.h"
 
 namespace nvfp4 {
 
-__constant__ float kMid[7] = {0.25f, 0.75f, 1.25f, 1.75f, 2.5f, 3.5f, 5.0f};
+constexpr int kOptThreads = 128;
+constexpr int kOptList = 24;          // segments noted by the screen; more: every segment is scored
+
+__constant__ float kMid[8] = {0.25f, 0.75f, 1.25f, 1.75f, 2.5f, 3.5f, 5.0f, 5.0f};
 __constant__ float kGrid[8] = {0.0f, 0.5f, 1.0f, 1.5f, 2.0f, 3.0f, 4.0f, 6.0f};
 
-// Nearest E2M1 magnitude of t >= 0 (ties to even), as a float.
+// Nearest E2M1 magnitudes of a pair of t >= 0 (ties to even), as f16x2.
+__device__ __forceinline__ void rn_grid2(float tl, float th, float& gl, float& gh) {
+    uint32_t h2;
+    asm("{\n\t.reg .b8 q;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 q, %1, %2;\n\t"
+        "cvt.rn.f16x2.e2m1x2 %0, q;\n\t}"
+        : "=r"(h2) : "f"(th), "f"(tl));
+    gl = f16bits_to_f32((uint16_t)(h2 & 0xFFFFu));
+    gh = f16bits_to_f32((uint16_t)(h2 >> 16));
+}
 __device__ __forceinline__ float rn_grid(float t) {
-    const uint32_t code = e2m1x2(t, 0.0f) & 0x7u;
-    const float g[8] = {0.0f, 0.5f, 1.0f, 1.5f, 2.0f, 3.0f, 4.0f, 6.0f};
-    float r = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 8; k++) r = (code == (uint32_t)k) ? g[k] : r;
-    return r;
+    float g, unused;
+    rn_grid2(t, 0.0f, g, unused);
+    return g;
 }
 
+// A thread's block in shared memory: element j at [j * kOptThreads].
+template <int OBJ>
+struct Column {
+    const float* a;
+    const float* w;
+    __device__ __forceinline__ float mag(int j) const { return a[j * kOptThreads]; }
+    __device__ __forceinline__ float wt(int j) const { return OBJ ? w[j * kOptThreads] : 1.0f; }
+};
+
 // Loss of E4M3 scale code c under the sweep's contract (t = fl(y*fl(1/v)),
-// q = RNE_E2M1(t), e = fl(y - q*v), fp32 accumulation in element order).
+// q = RNE_E2M1(t), e = fl(y - q*v), fp32 accumulation in element order); the
+// loss of a magnitude is that of either sign.
 template <int BLOCK, int OBJ>
-__device__ float contract_loss(const float (&y)[BLOCK], const float (&w)[BLOCK], int c) {
-    const uint16_t vh = e4m3_to_f16bits((uint32_t)c);
-    const float v = f16bits_to_f32(vh);
+__device__ __noinline__ float contract_loss(Column<OBJ> col, int c) {
+    const float v = f16bits_to_f32(e4m3_to_f16bits((uint32_t)c));
     const float r = __frcp_rn(v);
     float L = 0.0f;
-#pragma unroll
+#pragma unroll 8
     for (int i = 0; i < BLOCK; i++) {
-        const float t = __fmul_rn(y[i], r);
-        const float q = copysignf(rn_grid(fabsf(t)), t);
-        const float e = __fmaf_rn(-q, v, y[i]);
-        L = __fmaf_rn(OBJ ? __fmul_rn(w[i], e) : e, e, L);
+        const float a = col.mag(i);
+        const float e = __fmaf_rn(-rn_grid(__fmul_rn(a, r)), v, a);
+        L = __fmaf_rn(OBJ ? __fmul_rn(col.wt(i), e) : e, e, L);
     }
     return L;
 }
 
+// ~ 1/b for b = a_i / mu_k, shrunk by 2^-20 so that quotients at (or within
+// ~1e-6 of) a midpoint take the lower neighbour: the assignment just above b
+// even when breakpoints coincide (equal magnitudes are common in bf16 blocks).
+__device__ __forceinline__ float segment_rcp(float mid, float ra) {
+    return __fmul_rn(__fmul_rn(mid, ra), 1.0f - 9.5367431640625e-07f);
+}
+
+// One segment in full: its least-squares scale and loss, and the running best.
+// The optimum can be attained on several segments (e.g. one dominant element
+// that can sit on 6, 4, 3, ... grid points while the rest round to 0): the
+// smallest such scale is kept, within fp32 ties.
+template <int BLOCK, int OBJ>
+__device__ __noinline__ void score_segment(Column<OBJ> col, int i, int k, float& best, float& best_s) {
+    const float ai = col.mag(i);
+    if (!(ai > 0.0f)) return;
+    const float r = segment_rcp(kMid[k], __frcp_rn(ai));
+    float B = 0.0f, C = 0.0f;
+#pragma unroll 8
+    for (int j = 0; j < BLOCK; j++) {
+        const float a = col.mag(j), w = col.wt(j);
+        const float g = (j == i) ? kGrid[k] : rn_grid(__fmul_rn(a, r));
+        B = __fmaf_rn(__fmul_rn(w, a), g, B);
+        C = __fmaf_rn(__fmul_rn(w, g), g, C);
+    }
+    if (!(C > 0.0f)) return;
+    const float s = __fdiv_rn(B, C);
+    float L = 0.0f;
+#pragma unroll 8
+    for (int j = 0; j < BLOCK; j++) {
+        const float a = col.mag(j);
+        const float g = (j == i) ? kGrid[k] : rn_grid(__fmul_rn(a, r));
+        const float e = __fmaf_rn(-s, g, a);
+        L = __fmaf_rn(__fmul_rn(col.wt(j), e), e, L);
+    }
+    if (L < best * (1.0f - 1e-6f) || (L <= best * (1.0f + 1e-6f) && s < best_s)) {
+        best = fminf(best, L);
+        best_s = s;
+    }
+}
+
+// How far the screen's A - B^2/C can lie from the scored loss, relative to A:
+// B and C carry at most n + 1 roundings each and B^2/C <= A (Cauchy-Schwarz), so
+// 3(n + 1) + 4 roundings of A, and the list entry drops 2^-14 of its own value
+// (covered by the factor 1 + 2^-9 beside it).  n 2^-20 is over four times that.
+// The scored pass compares losses within 1e-6, so anything farther than that
+// from the least loss leaves no trace in its result: a better segment replaces
+// it whichever comes first.
+template <int BLOCK>
+__device__ __forceinline__ float screen_limit(float least, float A) {
+    return __fmaf_rn(A, BLOCK * 9.5367431640625e-07f, least * 1.001953125f);
+}
+
 template <int DT, int OBJ, int BLOCK>
-__global__ void __launch_bounds__(128) optimal_scale_kernel(OptParams p) {
+__global__ void __launch_bounds__(kOptThreads) optimal_scale_kernel(OptParams p) {
+    extern __shared__ float smem[];
+    float* sa = smem + threadIdx.x;
+    float* sw = sa + BLOCK * kOptThreads;
+    uint32_t* list = reinterpret_cast<uint32_t*>(sa + (OBJ ? 2 : 1) * BLOCK * kOptThreads);
+    const Column<OBJ> col{sa, sw};
     const float S = __ldg(p.S);
     const float E = __frcp_rn(S);
     const bool usable = (S > 0.0f) && isfinite(S) && isfinite(E);
@@ -67,75 +154,97 @@ __global__ void __launch_bounds__(128) optimal_scale_kernel(OptParams p) {
     for (int64_t blk = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; blk < p.nblocks; blk += stride) {
         const int64_t row = blk / p.kb, kbi = blk - row * p.kb;
         const int64_t off = row * p.cols + kbi * BLOCK;
-        float y[BLOCK], a[BLOCK], w[BLOCK];
-#pragma unroll
+        const float* wp = p.w + row * p.w_row_stride + kbi * BLOCK;
+        // s -> infinity: everything rounds to 0;  s -> 0+: every non-zero element saturates at 6
+        float best = 0.0f, B0 = 0.0f, C0 = 0.0f;
+        bool sane = true;
+#pragma unroll 16
         for (int i = 0; i < BLOCK; i++) {
             const float xv = DT == 0 ? __uint_as_float((uint32_t)(static_cast<const uint16_t*>(p.x)[off + i]) << 16)
                                      : static_cast<const float*>(p.x)[off + i];
-            y[i] = usable ? __fmul_rn(xv, E) : 0.0f;
-            a[i] = fabsf(y[i]);
-            w[i] = OBJ ? __ldg(p.w + row * p.w_row_stride + kbi * BLOCK + i) : 1.0f;
+            const float a = fabsf(usable ? __fmul_rn(xv, E) : 0.0f);
+            const float w = OBJ ? __ldg(wp + i) : 1.0f;
+            sa[i * kOptThreads] = a;
+            if (OBJ) sw[i * kOptThreads] = w;
+            const float wa = __fmul_rn(w, a), g = a > 0.0f ? 6.0f : 0.0f;
+            best = __fmaf_rn(wa, a, best);
+            B0 = __fmaf_rn(wa, g, B0);
+            C0 = __fmaf_rn(__fmul_rn(w, g), g, C0);
+            sane = sane && (a == 0.0f || a > 1e-15f) && (!OBJ || w == 0.0f || (w > 1e-18f && w < 1e30f));
         }
-        // s -> infinity: everything rounds to 0
-        float best = 0.0f;
-#pragma unroll
-        for (int i = 0; i < BLOCK; i++) best = __fmaf_rn(w[i] * a[i], a[i], best);
+        const float A = best;
         float best_s = 0.0f;
-        // s -> 0+: every non-zero element saturates at 6
-        {
-            float B = 0.0f, C = 0.0f;
-#pragma unroll
+        if (C0 > 0.0f) {
+            const float s = __fdiv_rn(B0, C0);
+            float L = 0.0f;
+#pragma unroll 16
             for (int i = 0; i < BLOCK; i++) {
-                const float g = a[i] > 0.0f ? 6.0f : 0.0f;
-                B = __fmaf_rn(w[i] * a[i], g, B);
-                C = __fmaf_rn(w[i] * g, g, C);
+                const float a = col.mag(i);
+                const float e = __fmaf_rn(-s, a > 0.0f ? 6.0f : 0.0f, a);
+                L = __fmaf_rn(__fmul_rn(col.wt(i), e), e, L);
             }
-            if (C > 0.0f) {
-                const float s = __fdiv_rn(B, C);
-                float L = 0.0f;
+            if (L < best) {
+                best = L;
+                best_s = s;
+            }
+        }
+        // The screen's bound holds for non-negative weights and sums far from
+        // overflow and underflow; other blocks (NaN and inf among them) are scored in full.
+        const bool screen_ok = sane && A > 1e-25f && A < 1e30f;
+        int noted = 0;
+        float least = best;
+        if (screen_ok) {
+            for (int i = 0; i < BLOCK; i++) {
+                const float ai = col.mag(i);
+                const float ra = ai > 0.0f ? __frcp_rn(ai) : 0.0f;      // zero: every code is 0, C = 0, not noted
+                u64 r2[4], B2[4], C2[4];
 #pragma unroll
-                for (int i = 0; i < BLOCK; i++) {
-                    const float e = __fmaf_rn(-s, a[i] > 0.0f ? 6.0f : 0.0f, a[i]);
-                    L = __fmaf_rn(w[i] * e, e, L);
+                for (int q = 0; q < 4; q++) {
+                    r2[q] = pack2(segment_rcp(kMid[2 * q], ra), segment_rcp(kMid[2 * q + 1], ra));
+                    B2[q] = C2[q] = 0ull;
                 }
-                if (L < best) {
-                    best = L;
-                    best_s = s;
+#pragma unroll 4
+                for (int j = 0; j < BLOCK; j++) {
+                    const float a = col.mag(j), w = col.wt(j);
+                    const u64 a2 = pack2(a, a);
+                    const float wa = OBJ ? __fmul_rn(w, a) : a;
+                    const u64 wa2 = pack2(wa, wa), w2 = pack2(w, w);
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        float tl, th, gl, gh;
+                        unpack2(mul2(a2, r2[q]), tl, th);
+                        rn_grid2(tl, th, gl, gh);
+                        const u64 g2 = pack2(gl, gh);
+                        B2[q] = fma2(wa2, g2, B2[q]);
+                        C2[q] = fma2(OBJ ? mul2(w2, g2) : g2, g2, C2[q]);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 7; k++) {
+                    float b0, b1, c0, c1;
+                    unpack2(B2[k >> 1], b0, b1);
+                    unpack2(C2[k >> 1], c0, c1);
+                    const float B = (k & 1) ? b1 : b0, C = (k & 1) ? c1 : c0;
+                    const float est = fmaxf(__fmaf_rn(-B, __fdividef(B, C), A), 0.0f);   // NaN for C = 0: 0 by fmaxf
+                    if (C > 0.0f && est <= screen_limit<BLOCK>(least, A)) {
+                        if (noted < kOptList)
+                            list[noted * kOptThreads] = (__float_as_uint(est) & ~511u) | (uint32_t)(i * 7 + k);
+                        noted++;
+                        least = fminf(least, est);
+                    }
                 }
             }
         }
-        for (int i = 0; i < BLOCK; i++) {
-            if (!(a[i] > 0.0f)) continue;
-            const float ra = __frcp_rn(a[i]);
-            for (int k = 0; k < 7; k++) {
-                // ~ 1/b for b = a_i / mu_k, shrunk by 2^-20 so that quotients at
-                // (or within ~1e-6 of) a midpoint take the lower neighbour: the
-                // assignment just above b even when breakpoints coincide
-                // (equal magnitudes are common in bf16 blocks)
-                const float r = __fmul_rn(__fmul_rn(kMid[k], ra), 1.0f - 9.5367431640625e-07f);
-                float B = 0.0f, C = 0.0f;
-                float g[BLOCK];
-#pragma unroll
-                for (int j = 0; j < BLOCK; j++) {
-                    g[j] = (j == i) ? kGrid[k] : rn_grid(__fmul_rn(a[j], r));
-                    B = __fmaf_rn(w[j] * a[j], g[j], B);
-                    C = __fmaf_rn(w[j] * g[j], g[j], C);
-                }
-                if (!(C > 0.0f)) continue;
-                const float s = __fdiv_rn(B, C);
-                float L = 0.0f;
-#pragma unroll
-                for (int j = 0; j < BLOCK; j++) {
-                    const float e = __fmaf_rn(-s, g[j], a[j]);
-                    L = __fmaf_rn(w[j] * e, e, L);
-                }
-                // the optimum can be attained on several segments (e.g. one dominant
-                // element that can sit on 6, 4, 3, ... grid points while the rest
-                // round to 0): keep the smallest such scale, within fp32 ties
-                if (L < best * (1.0f - 1e-6f) || (L <= best * (1.0f + 1e-6f) && s < best_s)) {
-                    best = fminf(best, L);
-                    best_s = s;
-                }
+        if (!screen_ok || noted > kOptList) {
+            for (int i = 0; i < BLOCK; i++)
+                for (int k = 0; k < 7; k++) score_segment<BLOCK, OBJ>(col, i, k, best, best_s);
+        } else {
+            const float limit = screen_limit<BLOCK>(least, A);
+            for (int n = 0; n < noted; n++) {
+                const uint32_t e = list[n * kOptThreads];
+                if (__uint_as_float(e & ~511u) > limit) continue;
+                const int id = (int)(e & 511u);
+                score_segment<BLOCK, OBJ>(col, id / 7, id % 7, best, best_s);
             }
         }
         p.s_opt[blk] = best_s;
@@ -149,8 +258,8 @@ __global__ void __launch_bounds__(128) optimal_scale_kernel(OptParams p) {
                 int ce = fl;
                 const float vfl = f16bits_to_f32(e4m3_to_f16bits((uint32_t)fl));
                 if (vfl < best_s && fl < 126) ce = fl + 1;
-                const float Lfl = contract_loss<BLOCK, OBJ>(y, w, fl);
-                const float Lce = ce == fl ? Lfl : contract_loss<BLOCK, OBJ>(y, w, ce);
+                const float Lfl = contract_loss<BLOCK, OBJ>(col, fl);
+                const float Lce = ce == fl ? Lfl : contract_loss<BLOCK, OBJ>(col, ce);
                 code = (Lce < Lfl) ? ce : fl;
                 Lf = (Lce < Lfl) ? Lce : Lfl;
             }
@@ -160,17 +269,27 @@ __global__ void __launch_bounds__(128) optimal_scale_kernel(OptParams p) {
     }
 }
 
+template <int DT, int OBJ, int BLOCK>
+static cudaError_t opt_launch(const OptParams& p, int sms, cudaStream_t s) {
+    constexpr int smem = ((OBJ ? 2 : 1) * BLOCK + kOptList) * kOptThreads * (int)sizeof(float);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(optimal_scale_kernel<DT, OBJ, BLOCK>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    int64_t grid = (p.nblocks + kOptThreads - 1) / kOptThreads;
+    if (grid > (int64_t)sms * 64) grid = (int64_t)sms * 64;
+    optimal_scale_kernel<DT, OBJ, BLOCK><<<(int)grid, kOptThreads, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
 template <int DT, int OBJ>
 static cudaError_t opt_block(const OptParams& p, int block, int sms, cudaStream_t s) {
-    int64_t grid = (p.nblocks + 127) / 128;
-    if (grid > (int64_t)sms * 16) grid = (int64_t)sms * 16;
-    if (grid < 1) grid = 1;
     switch (block) {
-        case 16: optimal_scale_kernel<DT, OBJ, 16><<<(int)grid, 128, 0, s>>>(p); break;
-        case 32: optimal_scale_kernel<DT, OBJ, 32><<<(int)grid, 128, 0, s>>>(p); break;
-        default: optimal_scale_kernel<DT, OBJ, 64><<<(int)grid, 128, 0, s>>>(p); break;
+        case 16: return opt_launch<DT, OBJ, 16>(p, sms, s);
+        case 32: return opt_launch<DT, OBJ, 32>(p, sms, s);
+        default: return opt_launch<DT, OBJ, 64>(p, sms, s);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_optimal_scale(const OptParams& p, int dtype, int obj, int block, int sms, cudaStream_t s) {
