@@ -12,11 +12,11 @@
 //   H_pi = (U + I) D (U + I)^T with U_ik = L[n-1-i][n-1-k] / L[n-1-k][n-1-k]
 //   (J L J is upper triangular) and D_k = L[n-1-k][n-1-k]^2.
 // Quantize (rows independent):
-//   T = W_pi (fp32); per 64-column panel, one warp per row walks the columns in
-//   order -- What_k = Q(T_k) at the element's fixed scale, e_k = W_k - What_k,
-//   T_j += e_k U_kj for the later columns of the panel -- then the trailing
-//   columns get T += E_panel U_panel,rest (the GEMM); finally the nibbles are
-//   scattered back to the original column order.
+//   T = W_pi (fp32); per 256-column super-panel, one lane per row walks the
+//   columns in order -- What_k = Q(T_k) at the element's fixed scale, e_k = W_k -
+//   What_k, T_j += e_k U_kj for the later columns of the super-panel -- then the
+//   later columns get T += E U (the GEMM); finally the nibbles are scattered back
+//   to the original column order.
 // Q follows the sweep's float32 contract: y = fl(t*E), q = RNE_E2M1(fl(y*r_c)),
 // What = fl(fl(q*v_c)*S); a zero-scale block or an unusable S gives signed
 // zeros; an exactly zero y takes the +0 code.
@@ -450,144 +450,277 @@ __global__ void __launch_bounds__(256) gather_w_kernel(LdlqParams p) {
         }
 }
 
-// One LDLQ panel of P <= 64 columns (P % 16 == 0).  TPR threads per row
-// (adjacent lanes), thread k of a row owning columns (64/TPR)k .. (64/TPR)(k+1)-1
-// in registers: at column s the owner quantizes it at its fixed scale, writes
-// the error to EpT[s][r], and the error reaches the row's other threads by
-// shuffle; each thread then updates its targets through up[s][c] = U[k0+s][k0+c]
-// (zero for c <= s and past the panel).  Splitting the 64-wide update shortens
-// the sequential chain per column.  The CTA's rows of original weights and the
-// reciprocal and value of each element's scale code are staged in shared memory
-// first, so the owner's step depends on its target alone.  The walk is
-// latency-bound (one dependent quantize -> shuffle -> update chain per column), so
-// weights with few rows take 16 threads per row (twice the warps in flight) and
-// tall ones 8 (fewer shuffles and owner steps per warp).
-constexpr int kPanelThreads = 128;
-constexpr int64_t kPanelWideRows = 8192;            // below this many rows: 16 threads per row
-template <int TPR>
-__host__ __device__ constexpr int panel_rows() {
-    return kPanelThreads / TPR;
+// One super-panel of up to 256 columns (a multiple of 8): every column is
+// quantized in order and its error fed to the later columns of the super-panel.
+//
+// A CTA takes 32 rows, one per lane, in every one of its 8 warps, and walks the
+// super-panel in sub-panels of 64 columns, 8 to a warp.  At step o of a sub-panel
+// warp o walks its 8 columns alone -- the chain quantize -> error -> update never
+// leaves the lane -- and publishes the 8 errors of its 32 rows; after one barrier
+// the later warps apply them to their own columns, T_c += e_j U_jc with U_jc the
+// same for all lanes (broadcast reads of shared memory, fetched into registers
+// before the barrier).  A finished sub-panel updates the later ones with K = 64 on
+// mma.sync (three TF32 products per term, as the trailing GEMM): there a warp
+// holds the 32 x 8 targets of its group as two accumulator fragments, U comes
+// from global memory in fragment order (each value is used once), and a 12-word
+// row stride in shared memory turns fragments back into rows.
+//
+// Bound by the chain, about 45 cycles of dependent arithmetic per column and a
+// barrier per 8 columns.  Splitting a row's columns over lanes instead (eight or
+// sixteen threads per row, a shuffle per column, panels of 64 with a GEMM between
+// them) repeats the quantize step once per row rather than once per 32 rows and
+// was issue-bound at 520 cycles per column; updating all 256 columns through
+// broadcast reads was bound by shared-memory returns (a word per lane and
+// multiply-add) at 260.
+constexpr int kGroupCols = 8;
+constexpr int kWalkWarps = 8;
+constexpr int kWalkRows = 32;
+constexpr int kWalkThreads = 32 * kWalkWarps;
+constexpr int kSubCols = kGroupCols * kWalkWarps;                       // 64
+constexpr int kSubs = kLdlqPanel / kSubCols;                            // 4
+constexpr int kErrStride = 40;                                          // words per column of errors: conflict-free A fragments
+constexpr int kTurnStride = 12;                                         // words per row of a group's targets
+constexpr int kUTiles = kWalkWarps * (kWalkWarps + 1) / 2;              // 8 x 8 tiles of a sub-panel's upper triangle
+constexpr int kWalkSmem = (kSubs * kUTiles * 64 + 2 * kSubCols * kErrStride + kWalkWarps * kWalkRows * kTurnStride + 128) * 4;
+
+// First tile of tile row g (tiles g, g+1, .. of the columns) of a sub-panel.
+__device__ __forceinline__ int u_tile_row(int g) { return g * kWalkWarps - (g * (g - 1)) / 2; }
+
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
-template <int TPR>
-__host__ __device__ constexpr int panel_smem() {
-    return (kP * kP + 128 + 2 * panel_rows<TPR>() * (kP + 1)) * 4 + panel_rows<TPR>() * (kP + 4) * 2;
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-template <int DT, int TPR>
-__global__ void __launch_bounds__(kPanelThreads) panel_kernel(LdlqParams p, int64_t k0, int P, float* EpT) {
-    constexpr int kPanelTpr = TPR;                    // threads per row
-    constexpr int kPanelTargets = kP / TPR;           // targets per thread
-    constexpr int kPanelRows = panel_rows<TPR>();
-    static_assert(kPanelTargets % 4 == 0 && 16 % kPanelTargets == 0, "a thread's targets are whole float4s in a block");
+// x = hi + lo, hi a TF32 value (13 mantissa bits cleared), lo exact in fp32 (the MMA reads its top 11 bits).
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+    hi = __float_as_uint(x) & 0xFFFFE000u;
+    lo = __float_as_uint(__fsub_rn(x, __uint_as_float(hi)));
+}
+__device__ __forceinline__ void mma_16n8k8_tf32(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// UVEC: U is 16-byte aligned (its rows then are too: n is a multiple of 16).
+template <bool UVEC>
+__global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int64_t s0, int span, float* EpT) {
     extern __shared__ __align__(16) float dsm[];
-    float (*up)[kP] = reinterpret_cast<float (*)[kP]>(dsm);                    // [kP][kP]
-    float* rtab = dsm + kP * kP;                                               // [128]
-    float (*wsm)[kP + 1] = reinterpret_cast<float (*)[kP + 1]>(rtab + 128);    // [kPanelRows][kP + 1] weights
-    float (*rsm)[kP + 1] = wsm + kPanelRows;                                   // fl(1/v) of the element's code, or 0
-    uint16_t (*vsm)[kP + 4] = reinterpret_cast<uint16_t (*)[kP + 4]>(rsm + kPanelRows);   // f16 bits of v
-    for (int e = threadIdx.x; e < kP * kP; e += blockDim.x) {
-        const int s = e / kP, c = e % kP;
-        up[s][c] = (s < c && c < P) ? p.U[(k0 + s) * p.n + k0 + c] : 0.0f;
-    }
-    for (int c = threadIdx.x; c < 128; c += blockDim.x)
-        rtab[c] = (c >= 1 && c <= 126) ? __frcp_rn(f16bits_to_f32(e4m3_to_f16bits((uint32_t)c))) : 0.0f;
-    __syncthreads();                                  // rtab before the row blocks read it
+    float* ut = dsm;                                              // [kSubs][kUTiles][8][8]
+    float* es = dsm + kSubs * kUTiles * 64;                       // [2][kSubCols][kErrStride]
+    float* turn = es + 2 * kSubCols * kErrStride;                 // [kWalkWarps][kWalkRows][kTurnStride]
+    float* rtab = turn + kWalkWarps * kWalkRows * kTurnStride;    // [128] fl(1/v) of each code, 0 for a zero scale
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float S = __ldg(p.S);
     const float Einv = __frcp_rn(S);
     const bool usable = (S > 0.0f) && isfinite(S) && isfinite(Einv);
     const float E = usable ? Einv : 1.0f;
     const float Sq = usable ? S : 0.0f;               // an unusable S reconstructs zeros (q is a signed zero then)
-    const int lane = threadIdx.x & 31;
-    const int kq = threadIdx.x % kPanelTpr;           // this thread's share of the columns
-    const int rr = threadIdx.x / kPanelTpr;           // row within the CTA's block
-    for (int64_t rb = (int64_t)blockIdx.x * kPanelRows; rb < p.rows; rb += (int64_t)gridDim.x * kPanelRows) {
-        __syncthreads();                              // rtab written / previous row block done with the row arrays
-        {
-            float4 wv[kPanelRows * kP / 4 / kPanelThreads];
-            uint32_t cv[kPanelRows * kP / 4 / kPanelThreads];
-#pragma unroll
-            for (int u = 0; u < kPanelRows * kP / 4 / kPanelThreads; u++) {
-                const int e = threadIdx.x + kPanelThreads * u, row = e / (kP / 4), j = 4 * (e % (kP / 4));
-                const bool ok = rb + row < p.rows && j < P;
-                wv[u] = ok ? *reinterpret_cast<const float4*>(p.Wp + (rb + row) * p.n + k0 + j) : make_float4(0, 0, 0, 0);
-                cv[u] = ok ? *reinterpret_cast<const uint32_t*>(p.sfp + (rb + row) * p.n + k0 + j) : 0u;
+
+    // each sub-panel's U tiles: row i from its own tile's first column on
+#pragma unroll 1
+    for (int q = 0; q < kSubs; q++) {
+        const int i1 = min(span, (q + 1) * kSubCols);
+        for (int i = q * kSubCols + warp; i < i1; i += kWalkWarps) {
+            const int g = (i >> 3) & (kWalkWarps - 1), cb = i & ~7;
+            const float* src = p.U + (s0 + i) * p.n + s0 + cb;
+            float* dst = ut + (q * kUTiles + u_tile_row(g)) * 64 + (i & 7) * 8;
+            if (UVEC) {
+                const int c = 4 * lane;
+                if (c < i1 - cb) cp_async16(dst + (c >> 3) * 64 + (c & 7), src + c);
+            } else {
+                for (int c = lane; c < i1 - cb; c += 32) cp_async4(dst + (c >> 3) * 64 + (c & 7), src + c, true);
             }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    // an unusable S or a zero code: r = 0 turns every target into a signed zero
+    if (tid < 128)
+        rtab[tid] = (usable && tid >= 1 && tid <= 126) ? __frcp_rn(f16bits_to_f32(e4m3_to_f16bits((uint32_t)tid))) : 0.0f;
+
+    const int64_t row0 = (int64_t)blockIdx.x * kWalkRows, last = p.rows - 1;
+    const int64_t r = row0 + lane;
+    const bool active = r <= last;
+    const int64_t rbase = (active ? r : last) * p.n + s0;         // lanes past the last row repeat it and store nothing
+    const int wc = warp * kGroupCols;                             // this warp's columns within a sub-panel
+    float* tw = turn + warp * kWalkRows * kTurnStride;
+
+    // targets of this warp's group in sub-panels 1.. as accumulator fragments: rows
+    // 16 m + lane / 4 (+ 8), columns 2 (lane % 4), + 1
+    float acc[kSubs][2][4];
 #pragma unroll
-            for (int u = 0; u < kPanelRows * kP / 4 / kPanelThreads; u++) {
-                const int e = threadIdx.x + kPanelThreads * u, row = e / (kP / 4), j = 4 * (e % (kP / 4));
-                const float wq[4] = {wv[u].x, wv[u].y, wv[u].z, wv[u].w};
+    for (int q = 1; q < kSubs; q++) {
+        const int c = q * kSubCols + wc;
+        if (c < span) {
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const uint32_t cs = (cv[u] >> (8 * q)) & 0xFFu;
-                    wsm[row][j + q] = wq[q];
-                    // an unusable S or a zero code: r = 0 turns every target into a signed zero
-                    rsm[row][j + q] = usable ? rtab[cs & 127u] : 0.0f;
-                    vsm[row][j + q] = e4m3_to_f16bits(cs);
+            for (int m = 0; m < 2; m++)
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    int64_t rr = row0 + 16 * m + 8 * h + (lane >> 2);
+                    rr = rr <= last ? rr : last;
+                    const float2 v = *reinterpret_cast<const float2*>(p.T + rr * p.n + s0 + c + 2 * (lane & 3));
+                    acc[q][m][2 * h] = v.x;
+                    acc[q][m][2 * h + 1] = v.y;
+                }
+        }
+    }
+    u64 t[4];                                                     // the row's targets in the group being walked
+    if (wc < span) {
+        const float4 a = *reinterpret_cast<const float4*>(p.T + rbase + wc);
+        const float4 b = *reinterpret_cast<const float4*>(p.T + rbase + wc + 4);
+        t[0] = pack2(a.x, a.y);
+        t[1] = pack2(a.z, a.w);
+        t[2] = pack2(b.x, b.y);
+        t[3] = pack2(b.z, b.w);
+    }
+    // operands of the warp's next walk: original weights and scale codes
+    float4 wa, wb;
+    uint2 cd;
+    auto fetch = [&](int q) {
+        const int c = q * kSubCols + wc;
+        if (c < span) {
+            wa = *reinterpret_cast<const float4*>(p.Wp + rbase + c);
+            wb = *reinterpret_cast<const float4*>(p.Wp + rbase + c + 4);
+            cd = *reinterpret_cast<const uint2*>(p.sfp + rbase + c);
+        }
+    };
+    fetch(0);
+    // acc[q] (this warp's group of sub-panel q) += errors of sub-panel q0 x U
+    auto update = [&](float (&c)[2][4], int q0, int q) {
+        const float* ub = p.U + (s0 + q0 * kSubCols + (lane & 3)) * p.n + s0 + q * kSubCols + wc + (lane >> 2);
+        const float* eb = es + (q0 & 1) * (kSubCols * kErrStride) + (lane & 3) * kErrStride + (lane >> 2);
+        float u[2 * kSubCols / 8];
+#pragma unroll
+        for (int k = 0; k < kSubCols / 8; k++) {
+            u[2 * k] = __ldg(ub + (int64_t)(8 * k) * p.n);
+            u[2 * k + 1] = __ldg(ub + (int64_t)(8 * k + 4) * p.n);
+        }
+#pragma unroll
+        for (int k = 0; k < kSubCols / 8; k++) {
+            uint32_t bh[2], bl[2];
+            split_tf32(u[2 * k], bh[0], bl[0]);
+            split_tf32(u[2 * k + 1], bh[1], bl[1]);
+#pragma unroll
+            for (int m = 0; m < 2; m++) {
+                const float* e = eb + 8 * k * kErrStride + 16 * m;
+                uint32_t ah[4], al[4];
+                split_tf32(e[0], ah[0], al[0]);
+                split_tf32(e[8], ah[1], al[1]);
+                split_tf32(e[4 * kErrStride], ah[2], al[2]);
+                split_tf32(e[4 * kErrStride + 8], ah[3], al[3]);
+                mma_16n8k8_tf32(c[m], ah, bh);
+                mma_16n8k8_tf32(c[m], ah, bl);
+                mma_16n8k8_tf32(c[m], al, bh);
+            }
+        }
+    };
+
+    cp_async_wait<3>();
+    static_assert(kSubs == 4, "one commit group of U tiles per sub-panel");
+    __syncthreads();                                   // rtab and the first sub-panel's tiles
+#pragma unroll
+    for (int q = 0; q < kSubs; q++) {
+        const int ng = min(kWalkWarps, span / kGroupCols - q * kWalkWarps);      // groups of this sub-panel
+        if (ng <= 0) break;
+        const float* uq = ut + q * kUTiles * 64;
+        float* eq = es + (q & 1) * (kSubCols * kErrStride) + lane;
+        float4 un[2 * kGroupCols];                     // U tile of the last published group and this warp's
+#pragma unroll 1
+        for (int o = 0; o < ng; o++) {                 // errors up to group o - 1 are published
+            if (o > 0 && warp >= o && warp < ng) {
+                const float* e = eq + (o - 1) * kGroupCols * kErrStride;
+#pragma unroll
+                for (int j = 0; j < kGroupCols; j++) {
+                    const float ej = e[j * kErrStride];
+                    const u64 e2 = pack2(ej, ej);
+                    t[0] = fma2(e2, pack2(un[2 * j].x, un[2 * j].y), t[0]);
+                    t[1] = fma2(e2, pack2(un[2 * j].z, un[2 * j].w), t[1]);
+                    t[2] = fma2(e2, pack2(un[2 * j + 1].x, un[2 * j + 1].y), t[2]);
+                    t[3] = fma2(e2, pack2(un[2 * j + 1].z, un[2 * j + 1].w), t[3]);
                 }
             }
-        }
-        __syncthreads();
-        const int64_t r = rb + rr;
-        const bool active = r < p.rows;               // a row's threads share r
-        const int c0 = kPanelTargets * kq;
-        float t[kPanelTargets];
+            if (warp > o && warp < ng) {
+                const float4* u = reinterpret_cast<const float4*>(uq + (u_tile_row(o) + warp - o) * 64);
 #pragma unroll
-        for (int g = 0; g < kPanelTargets / 4; g++) {
-            const float4 v = (active && c0 + 4 * g < P) ? *reinterpret_cast<const float4*>(p.T + r * p.n + k0 + c0 + 4 * g)
-                                                        : make_float4(0, 0, 0, 0);
-            t[4 * g] = v.x;
-            t[4 * g + 1] = v.y;
-            t[4 * g + 2] = v.z;
-            t[4 * g + 3] = v.w;
-        }
-        uint32_t packed[kPanelTargets / 4] = {};
-#pragma unroll 1
-        for (int kb = 0; kb < P / kPanelTargets; kb++) {   // the share whose columns are walked now
-            const bool own = kq == kb && active;
-            const int src = (lane & ~(kPanelTpr - 1)) | kb;
+                for (int j = 0; j < 2 * kGroupCols; j++) un[j] = u[j];
+            }
+            if (warp == o) {
+                float tt[8];
 #pragma unroll
-            for (int j = 0; j < kPanelTargets; j++) {
-                const int s = kPanelTargets * kb + j;
-                // the column's operands do not depend on the targets: loaded ahead of the chain
-                const float rs = rsm[rr][s], ws = wsm[rr][s];
-                const uint16_t vh = vsm[rr][s];
-                float e = 0.0f;
-                if (own) {
+                for (int h = 0; h < 4; h++) unpack2(t[h], tt[2 * h], tt[2 * h + 1]);
+                const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                float rs[8];
+                uint16_t vh[8];
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const uint32_t c = ((j < 4 ? cd.x : cd.y) >> (8 * (j & 3))) & 0x7Fu;
+                    rs[j] = rtab[c];
+                    vh[j] = e4m3_to_f16bits(c);
+                }
+                const float4* u = reinterpret_cast<const float4*>(uq + u_tile_row(o) * 64);
+                float* e = eq + o * kGroupCols * kErrStride;
+                float* eg = EpT + (int64_t)(q * kSubCols + o * kGroupCols) * p.rows + r;
+                uint32_t packed[2] = {0u, 0u};
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
                     // What = fl(fl(q v) S) with q = RNE_E2M1(fl(y r)), y = fl(t E); q v is
                     // exact, formed by one mixed fma with a +0 addend (a zero q gives +0)
-                    const float y = __fmul_rn(t[j], E);
-                    uint32_t nib = e2m1x2(__fmul_rn(y, rs), 0.0f) & 0xFu;
+                    const float y = __fmul_rn(tt[j], E);
+                    uint32_t nib;
                     float qv;
                     asm("{\n\t.reg .b8 b;\n\t.reg .b32 h2;\n\t.reg .b16 ql, qh;\n\t"
-                        "cvt.u8.u32 b, %1;\n\tcvt.rn.f16x2.e2m1x2 h2, b;\n\tmov.b32 {ql, qh}, h2;\n\t"
-                        "fma.rn.f32.f16 %0, ql, %2, %3;\n\t}"
-                        : "=f"(qv) : "r"(nib), "h"(vh), "f"(0.0f));
-                    if (y == 0.0f) nib = 0;                // an exactly zero target takes the +0 code
-                    e = __fsub_rn(ws, __fmul_rn(qv, Sq));
-                    packed[j / 4] |= nib << (8 * (j % 4));
-                    EpT[(int64_t)s * p.rows + r] = e;
-                }
-                e = __shfl_sync(0xffffffffu, e, src);
-                const float* us = &up[s][c0];
+                        "cvt.rn.satfinite.e2m1x2.f32 b, %4, %2;\n\t"
+                        "cvt.rn.f16x2.e2m1x2 h2, b;\n\tmov.b32 {ql, qh}, h2;\n\t"
+                        "fma.rn.f32.f16 %0, ql, %3, %4;\n\t"
+                        "cvt.u32.u8 %1, b;\n\t}"
+                        : "=f"(qv), "=r"(nib) : "f"(__fmul_rn(y, rs[j])), "h"(vh[j]), "f"(0.0f));
+                    const float ej = __fsub_rn(w[j], __fmul_rn(qv, Sq));
+                    const float4 u0 = u[2 * j], u1 = u[2 * j + 1];
+                    const float uv[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
 #pragma unroll
-                for (int g = 0; g < kPanelTargets / 4; g++) {
-                    const float4 u = *reinterpret_cast<const float4*>(us + 4 * g);
-                    t[4 * g + 0] = __fmaf_rn(e, u.x, t[4 * g + 0]);
-                    t[4 * g + 1] = __fmaf_rn(e, u.y, t[4 * g + 1]);
-                    t[4 * g + 2] = __fmaf_rn(e, u.z, t[4 * g + 2]);
-                    t[4 * g + 3] = __fmaf_rn(e, u.w, t[4 * g + 3]);
+                    for (int c = j + 1; c < 8; c++) tt[c] = __fmaf_rn(ej, uv[c], tt[c]);
+                    e[j * kErrStride] = ej;
+                    if (active) eg[(int64_t)j * p.rows] = ej;
+                    // an exactly zero target takes the +0 code
+                    packed[j >> 2] |= (y == 0.0f ? 0u : nib & 0xFu) << (8 * (j & 3));
                 }
+                if (active) *reinterpret_cast<uint2*>(p.qb + rbase + q * kSubCols + wc) = make_uint2(packed[0], packed[1]);
+                fetch(q + 1);
             }
+            if (o == ng - 1) {                         // the next sub-panel's tiles
+                if (q == 0) cp_async_wait<2>();
+                else if (q == 1) cp_async_wait<1>();
+                else cp_async_wait<0>();
+            }
+            __syncthreads();
         }
-        if (active && c0 < P) {
-            uint8_t* q = p.qb + r * p.n + k0 + c0;    // one byte per column: kPanelTargets bytes
-            if constexpr (kPanelTargets == 16)
-                *reinterpret_cast<uint4*>(q) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-            else if constexpr (kPanelTargets == 8)
-                *reinterpret_cast<uint2*>(q) = make_uint2(packed[0], packed[1]);
-            else
-                *reinterpret_cast<uint32_t*>(q) = packed[0];
+        if (q + 1 < kSubs && (q + 1) * kSubCols + wc < span) {
+            float (&c)[2][4] = acc[q + 1];
+            update(c, q, q + 1);
+            // fragments to one row per lane
+#pragma unroll
+            for (int m = 0; m < 2; m++)
+#pragma unroll
+                for (int h = 0; h < 2; h++)
+                    *reinterpret_cast<float2*>(tw + (16 * m + 8 * h + (lane >> 2)) * kTurnStride + 2 * (lane & 3)) =
+                        make_float2(c[m][2 * h], c[m][2 * h + 1]);
+            __syncwarp();
+            const float4 a = *reinterpret_cast<const float4*>(tw + lane * kTurnStride);
+            const float4 b = *reinterpret_cast<const float4*>(tw + lane * kTurnStride + 4);
+            t[0] = pack2(a.x, a.y);
+            t[1] = pack2(a.z, a.w);
+            t[2] = pack2(b.x, b.y);
+            t[3] = pack2(b.z, b.w);
+            __syncwarp();
         }
+#pragma unroll
+        for (int q2 = q + 2; q2 < kSubs; q2++)
+            if (q2 * kSubCols + wc < span) update(acc[q2], q, q2);
     }
 }
 
@@ -710,10 +843,9 @@ size_t ldlq_quantize_workspace(int64_t rows, int64_t n) {
     return (size_t)(2 * up(rows * n * 4) + 2 * up(rows * n) + 2 * up((int64_t)kLdlqPanel * rows * 4) + up(n * 4));
 }
 
-// Columns in super-panels of kLdlqPanel (256): each 64-column panel is walked by
-// panel_kernel and its errors update the rest of the super-panel at once (K = 64);
-// after the super-panel, GEMMs with K = 256 update every later column, so the
-// targets are read and written once per 256 columns.  Look-ahead: that update
+// Columns in super-panels of kLdlqPanel (256), each walked by walk_kernel; after
+// the super-panel, GEMMs with K = 256 update every later column, so the targets
+// are read and written once per 256 columns.  Look-ahead: that update
 // is split into the next super-panel's columns, which run with its panel walks
 // on the high-priority stream, and the rest, which runs on `s` concurrently
 // with them; the super-panels' errors alternate between two EpT buffers.
@@ -740,24 +872,20 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
         gather_w_kernel<1><<<rg, 256, 0, s>>>(p);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    const bool uvec = (reinterpret_cast<uintptr_t>(p.U) & 15) == 0;
+    const auto walk = uvec ? walk_kernel<true> : walk_kernel<false>;
     static std::atomic<bool> attr_set[64];        // per device: the shared-memory opt-in is done
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(panel_kernel<0, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, panel_smem<8>());
+        e = cudaFuncSetAttribute(walk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmem);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(panel_kernel<1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, panel_smem<8>());
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(panel_kernel<0, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, panel_smem<16>());
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(panel_kernel<1, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, panel_smem<16>());
+            e = cudaFuncSetAttribute(walk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
     }
-    const bool wide = p.rows < kPanelWideRows;
-    const int prow = wide ? panel_rows<16>() : panel_rows<8>();
-    const unsigned pg = (unsigned)imin64((p.rows + prow - 1) / prow, (int64_t)sms * 16);
+    const unsigned wg = (unsigned)((p.rows + kWalkRows - 1) / kWalkRows);
     LookAhead* la = nullptr;
     std::unique_lock<std::mutex> lock;
     e = lookahead_for_current_device(&la, &lock);
@@ -770,25 +898,9 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     for (int64_t s0 = 0; s0 < p.n; s0 += kLdlqPanel, sp++) {
         const int64_t span = imin64(kLdlqPanel, p.n - s0);
         float* EpT = EpTs[sp & 1];
-        for (int64_t k0 = s0; k0 < s0 + span; k0 += kP) {
-            const int P = (int)imin64(kP, s0 + span - k0);
-            float* Ek = EpT + (k0 - s0) * p.rows;
-            if (wide) {
-                if (dtype == 0) panel_kernel<0, 16><<<pg, kPanelThreads, panel_smem<16>(), c>>>(p, k0, P, Ek);
-                else panel_kernel<1, 16><<<pg, kPanelThreads, panel_smem<16>(), c>>>(p, k0, P, Ek);
-            } else {
-                if (dtype == 0) panel_kernel<0, 8><<<pg, kPanelThreads, panel_smem<8>(), c>>>(p, k0, P, Ek);
-                else panel_kernel<1, 8><<<pg, kPanelThreads, panel_smem<8>(), c>>>(p, k0, P, Ek);
-            }
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            const int64_t rest_in = s0 + span - (k0 + P);
-            if (rest_in > 0) {
-                e = update_gemm<true, false, false>(p.T + k0 + P, p.n, Ek, p.rows, p.U + k0 * p.n + k0 + P, p.n,
-                                                    p.rows, rest_in, P, 1.0f, p.status, c);
-                if (e != cudaSuccess) return e;
-            }
-        }
+        walk<<<wg, kWalkThreads, kWalkSmem, c>>>(p, s0, (int)span, EpT);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
         const int64_t rest = p.n - (s0 + span);
         if (rest > 0) {
             const int64_t next = imin64(kLdlqPanel, rest);
