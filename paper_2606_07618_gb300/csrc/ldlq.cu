@@ -22,6 +22,7 @@
 // zeros; an exactly zero y takes the +0 code.
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -454,24 +455,33 @@ __global__ void __launch_bounds__(256) gather_w_kernel(LdlqParams p) {
 // quantized in order and its error fed to the later columns of the super-panel.
 //
 // A CTA takes 32 rows, one per lane, in every one of its 8 warps, and walks the
-// super-panel in sub-panels of 64 columns, 8 to a warp.  At step o of a sub-panel
-// warp o walks its 8 columns alone -- the chain quantize -> error -> update never
-// leaves the lane -- and publishes the 8 errors of its 32 rows; after one barrier
-// the later warps apply them to their own columns, T_c += e_j U_jc with U_jc the
-// same for all lanes (broadcast reads of shared memory, fetched into registers
-// before the barrier).  A finished sub-panel updates the later ones with K = 64 on
-// mma.sync (three TF32 products per term, as the trailing GEMM): there a warp
-// holds the 32 x 8 targets of its group as two accumulator fragments, U comes
-// from global memory in fragment order (each value is used once), and a 12-word
-// row stride in shared memory turns fragments back into rows.
+// super-panel in sub-panels of 64 columns, a group of 8 to a warp.  At step o of a
+// sub-panel warp o walks its group alone -- the chain quantize -> error -> update
+// never leaves the lane -- and publishes the 8 errors of its 32 rows; one barrier
+// ends the step.  The later warps then apply these errors to their own groups by
+// fp32 multiply-adds (U, the same for all lanes, was read into registers before
+// the barrier), so the next walk starts after 32 packed operations.  Beside the
+// walk every other warp applies published errors to its groups of the later
+// sub-panels with mma.sync (K = 8, three TF32 products per term as the trailing
+// GEMM), a group's 32 x 8 targets being two accumulator fragments: the last
+// published errors to the next sub-panel, those of the sub-panel before to the
+// ones after it.  A walking warp makes up the one step it missed when the
+// sub-panel is done, and turns its next group's fragments into rows (through
+// shared memory, 12-word rows).
 //
-// Bound by the chain, about 45 cycles of dependent arithmetic per column and a
-// barrier per 8 columns.  Splitting a row's columns over lanes instead (eight or
-// sixteen threads per row, a shuffle per column, panels of 64 with a GEMM between
-// them) repeats the quantize step once per row rather than once per 32 rows and
-// was issue-bound at 520 cycles per column; updating all 256 columns through
-// broadcast reads was bound by shared-memory returns (a word per lane and
-// multiply-add) at 260.
+// Bound by the chain: 35 cycles of dependent arithmetic per column (52 with the
+// rest of a column's instructions), and a barrier and the last group's update per
+// 8 columns.  An mma.sync takes 8.5 cycles of its quarter of the SM and about 70
+// until its result is there, so none of them is on the chain but two or three per
+// sub-panel.  Splitting a row's columns over lanes instead (eight or sixteen
+// threads per row, a shuffle per column, panels of 64 with a GEMM between them)
+// repeats the quantize step once per row rather than once per 32 rows and was
+// issue-bound at 520 cycles per column; applying all errors by multiply-adds on
+// broadcast reads of U was bound by the shared-memory returns (a word per lane
+// and multiply-add) at 260, all by mma.sync by its latency at 220.
+//
+// The upper triangle of the super-panel's U block is staged by one bulk copy per
+// row (the wait for it is bounded: status bit 16, as the trailing GEMM's waits).
 constexpr int kGroupCols = 8;
 constexpr int kWalkWarps = 8;
 constexpr int kWalkRows = 32;
@@ -479,21 +489,30 @@ constexpr int kWalkThreads = 32 * kWalkWarps;
 constexpr int kSubCols = kGroupCols * kWalkWarps;                       // 64
 constexpr int kSubs = kLdlqPanel / kSubCols;                            // 4
 constexpr int kErrStride = 40;                                          // words per column of errors: conflict-free A fragments
+constexpr int kErrSlot = kGroupCols * kErrStride;
 constexpr int kTurnStride = 12;                                         // words per row of a group's targets
-constexpr int kUTiles = kWalkWarps * (kWalkWarps + 1) / 2;              // 8 x 8 tiles of a sub-panel's upper triangle
-constexpr int kWalkSmem = (kSubs * kUTiles * 64 + 2 * kSubCols * kErrStride + kWalkWarps * kWalkRows * kTurnStride + 128) * 4;
+constexpr int kUWords = 8 * (3 * 264 + 4 * (232 + 200 + 168 + 136 + 104 + 72 + 40) + 8);   // see u_row
+constexpr int kWalkSmem = (kUWords + 2 * kWalkWarps * kErrSlot + kWalkWarps * kWalkRows * kTurnStride + 128) * 4;
 
-// First tile of tile row g (tiles g, g+1, .. of the columns) of a sub-panel.
-__device__ __forceinline__ int u_tile_row(int g) { return g * kWalkWarps - (g * (g - 1)) / 2; }
+// The staged upper triangle of U: row 8 g + j holds columns 8 g .. 255, its pitch
+// rounded up to 8 words modulo 32 (the rows of B fragments then lie in distinct
+// banks): 264 words for g < 3, then 32 fewer every four groups.
+__device__ __forceinline__ int u_pitch(int g) { return g < 3 ? 264 : 232 - 32 * ((g - 3) >> 2); }
+__device__ __forceinline__ int u_row(int g) {                           // word offset of row 8 g
+    if (g < 3) return 8 * 264 * g;
+    const int m = (g - 3) >> 2;
+    return 8 * (3 * 264 + 4 * (232 * m - 16 * m * (m - 1)) + ((g - 3) & 3) * (232 - 32 * m));
+}
 
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+// Untiled bulk copy to shared memory (16-byte aligned, a multiple of 16 bytes), completion on bar.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
 }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
+
+// Every warp arrives once per step, the walking one from its own branch.
+__device__ __forceinline__ void step_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
 
 // x = hi + lo, hi a TF32 value (13 mantissa bits cleared), lo exact in fp32 (the MMA reads its top 11 bits).
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
@@ -501,7 +520,7 @@ __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) 
     lo = __float_as_uint(__fsub_rn(x, __uint_as_float(hi)));
 }
 __device__ __forceinline__ void mma_16n8k8_tf32(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
                  "{%0, %1, %2, %3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
@@ -511,46 +530,44 @@ __device__ __forceinline__ void mma_16n8k8_tf32(float (&c)[4], const uint32_t (&
 template <bool UVEC>
 __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int64_t s0, int span, float* EpT) {
     extern __shared__ __align__(16) float dsm[];
-    float* ut = dsm;                                              // [kSubs][kUTiles][8][8]
-    float* es = dsm + kSubs * kUTiles * 64;                       // [2][kSubCols][kErrStride]
-    float* turn = es + 2 * kSubCols * kErrStride;                 // [kWalkWarps][kWalkRows][kTurnStride]
+    __shared__ __align__(8) uint64_t s_ubar;
+    float* ut = dsm;                                              // U, see u_row
+    float* es = dsm + kUWords;                                    // [2][kWalkWarps][8][kErrStride]: two sub-panels' errors
+    float* turn = es + 2 * kWalkWarps * kErrSlot;                 // [kWalkWarps][kWalkRows][kTurnStride]
     float* rtab = turn + kWalkWarps * kWalkRows * kTurnStride;    // [128] fl(1/v) of each code, 0 for a zero scale
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const float S = __ldg(p.S);
-    const float Einv = __frcp_rn(S);
-    const bool usable = (S > 0.0f) && isfinite(S) && isfinite(Einv);
-    const float E = usable ? Einv : 1.0f;
-    const float Sq = usable ? S : 0.0f;               // an unusable S reconstructs zeros (q is a signed zero then)
-
-    // each sub-panel's U tiles: row i from its own tile's first column on
-#pragma unroll 1
-    for (int q = 0; q < kSubs; q++) {
-        const int i1 = min(span, (q + 1) * kSubCols);
-        for (int i = q * kSubCols + warp; i < i1; i += kWalkWarps) {
-            const int g = (i >> 3) & (kWalkWarps - 1), cb = i & ~7;
-            const float* src = p.U + (s0 + i) * p.n + s0 + cb;
-            float* dst = ut + (q * kUTiles + u_tile_row(g)) * 64 + (i & 7) * 8;
-            if (UVEC) {
-                const int c = 4 * lane;
-                if (c < i1 - cb) cp_async16(dst + (c >> 3) * 64 + (c & 7), src + c);
-            } else {
-                for (int c = lane; c < i1 - cb; c += 32) cp_async4(dst + (c >> 3) * 64 + (c & 7), src + c, true);
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    // an unusable S or a zero code: r = 0 turns every target into a signed zero
-    if (tid < 128)
-        rtab[tid] = (usable && tid >= 1 && tid <= 126) ? __frcp_rn(f16bits_to_f32(e4m3_to_f16bits((uint32_t)tid))) : 0.0f;
+    const int ng = span / kGroupCols;
+    const int wc = warp * kGroupCols;                             // this warp's columns within a sub-panel
 
     const int64_t row0 = (int64_t)blockIdx.x * kWalkRows, last = p.rows - 1;
     const int64_t r = row0 + lane;
     const bool active = r <= last;
     const int64_t rbase = (active ? r : last) * p.n + s0;         // lanes past the last row repeat it and store nothing
-    const int wc = warp * kGroupCols;                             // this warp's columns within a sub-panel
     float* tw = turn + warp * kWalkRows * kTurnStride;
-
-    // targets of this warp's group in sub-panels 1.. as accumulator fragments: rows
+    // the row's targets in the group being walked, packed pairs
+    u64 t[4];
+    auto set_rows = [&](const float* src) {
+        const float4 a = *reinterpret_cast<const float4*>(src);
+        const float4 b = *reinterpret_cast<const float4*>(src + 4);
+        t[0] = pack2(a.x, a.y);
+        t[1] = pack2(a.z, a.w);
+        t[2] = pack2(b.x, b.y);
+        t[3] = pack2(b.z, b.w);
+    };
+    if (wc < span) set_rows(p.T + rbase + wc);
+    // operands of the warp's next walk: original weights and scale codes
+    float4 wa, wb;
+    uint2 cd;
+    auto fetch = [&](int q) {
+        const int c = q * kSubCols + wc;
+        if (c < span) {
+            wa = *reinterpret_cast<const float4*>(p.Wp + rbase + c);
+            wb = *reinterpret_cast<const float4*>(p.Wp + rbase + c + 4);
+            cd = *reinterpret_cast<const uint2*>(p.sfp + rbase + c);
+        }
+    };
+    fetch(0);
+    // targets of this warp's groups in sub-panels 1.. as accumulator fragments: rows
     // 16 m + lane / 4 (+ 8), columns 2 (lane % 4), + 1
     float acc[kSubs][2][4];
 #pragma unroll
@@ -569,74 +586,120 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
                 }
         }
     }
-    u64 t[4];                                                     // the row's targets in the group being walked
-    if (wc < span) {
-        const float4 a = *reinterpret_cast<const float4*>(p.T + rbase + wc);
-        const float4 b = *reinterpret_cast<const float4*>(p.T + rbase + wc + 4);
-        t[0] = pack2(a.x, a.y);
-        t[1] = pack2(a.z, a.w);
-        t[2] = pack2(b.x, b.y);
-        t[3] = pack2(b.z, b.w);
+    // row i of the super-panel's U from column 8 (i / 8) on: one bulk copy per row,
+    // or 4-byte copies where U is not 16-byte aligned
+    const uint32_t ubar = tc::smem_u32(&s_ubar);
+    if (UVEC) {
+        if (tid == 0) {
+            tc::mbar_init(ubar, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            tc::mbar_expect_tx(ubar, (uint32_t)(32 * kGroupCols * ng * (ng + 1) / 2));   // 8 rows of 32 (ng - g) bytes per group
+        }
+        __syncthreads();
+        if (tid < span) {
+            const int g = tid >> 3;
+            bulk_load(tc::smem_u32(ut + u_row(g) + (tid & 7) * u_pitch(g)), p.U + (s0 + tid) * p.n + s0 + 8 * g,
+                      (uint32_t)(span - 8 * g) * 4, ubar);
+        }
+    } else {
+        for (int i = warp; i < span; i += kWalkWarps) {
+            const int g = i >> 3;
+            const float* src = p.U + (s0 + i) * p.n + s0;
+            float* dst = ut + u_row(g) + (i & 7) * u_pitch(g) - 8 * g;
+            for (int c = 8 * g + lane; c < span; c += 32) cp_async4(dst + c, src + c, true);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    // operands of the warp's next walk: original weights and scale codes
-    float4 wa, wb;
-    uint2 cd;
-    auto fetch = [&](int q) {
-        const int c = q * kSubCols + wc;
-        if (c < span) {
-            wa = *reinterpret_cast<const float4*>(p.Wp + rbase + c);
-            wb = *reinterpret_cast<const float4*>(p.Wp + rbase + c + 4);
-            cd = *reinterpret_cast<const uint2*>(p.sfp + rbase + c);
+    const float S = __ldg(p.S);
+    const float Einv = __frcp_rn(S);
+    const bool usable = (S > 0.0f) && isfinite(S) && isfinite(Einv);
+    const float E = usable ? Einv : 1.0f;
+    const float Sq = usable ? S : 0.0f;               // an unusable S reconstructs zeros (q is a signed zero then)
+    // an unusable S or a zero code: r = 0 turns every target into a signed zero
+    if (tid < 128)
+        rtab[tid] = (usable && tid >= 1 && tid <= 126) ? __frcp_rn(f16bits_to_f32(e4m3_to_f16bits((uint32_t)tid))) : 0.0f;
+
+    float rs[kGroupCols];
+    uint16_t vh[kGroupCols];
+    auto scales = [&]() {
+#pragma unroll
+        for (int j = 0; j < kGroupCols; j++) {
+            const uint32_t code = ((j < 4 ? cd.x : cd.y) >> (8 * (j & 3))) & 0x7Fu;
+            rs[j] = rtab[code];
+            vh[j] = e4m3_to_f16bits(code);
         }
     };
-    fetch(0);
-    // acc[q] (this warp's group of sub-panel q) += errors of sub-panel q0 x U
-    auto update = [&](float (&c)[2][4], int q0, int q) {
-        const float* ub = p.U + (s0 + q0 * kSubCols + (lane & 3)) * p.n + s0 + q * kSubCols + wc + (lane >> 2);
-        const float* eb = es + (q0 & 1) * (kSubCols * kErrStride) + (lane & 3) * kErrStride + (lane >> 2);
-        float u[2 * kSubCols / 8];
+    // the errors of group g as A fragments (row = row of the CTA, k = column of the group)
+    auto load_errors = [&](uint32_t (&ah)[2][4], uint32_t (&al)[2][4], int g) {
+        const float* e = es + (g & (2 * kWalkWarps - 1)) * kErrSlot + (lane & 3) * kErrStride + (lane >> 2);
 #pragma unroll
-        for (int k = 0; k < kSubCols / 8; k++) {
-            u[2 * k] = __ldg(ub + (int64_t)(8 * k) * p.n);
-            u[2 * k + 1] = __ldg(ub + (int64_t)(8 * k + 4) * p.n);
+        for (int m = 0; m < 2; m++) {
+            split_tf32(e[16 * m], ah[m][0], al[m][0]);
+            split_tf32(e[16 * m + 8], ah[m][1], al[m][1]);
+            split_tf32(e[16 * m + 4 * kErrStride], ah[m][2], al[m][2]);
+            split_tf32(e[16 * m + 4 * kErrStride + 8], ah[m][3], al[m][3]);
         }
+    };
+    // the rows of group g of U as a B fragment, for the columns of this warp's group in sub-panel q
+    auto load_u = [&](uint32_t (&bh)[2], uint32_t (&bl)[2], int g, int q) {
+        const int up = u_pitch(g);
+        const float* u = ut + u_row(g) + (lane & 3) * up + (lane >> 2) + q * kSubCols + wc - 8 * g;
+        split_tf32(u[0], bh[0], bl[0]);
+        split_tf32(u[4 * up], bh[1], bl[1]);
+    };
+    auto products = [&](float (&c)[2][4], const uint32_t (&ah)[2][4], const uint32_t (&al)[2][4], const uint32_t (&bh)[2],
+                        const uint32_t (&bl)[2]) {
 #pragma unroll
-        for (int k = 0; k < kSubCols / 8; k++) {
-            uint32_t bh[2], bl[2];
-            split_tf32(u[2 * k], bh[0], bl[0]);
-            split_tf32(u[2 * k + 1], bh[1], bl[1]);
+        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(c[m], ah[m], bh);
 #pragma unroll
-            for (int m = 0; m < 2; m++) {
-                const float* e = eb + 8 * k * kErrStride + 16 * m;
-                uint32_t ah[4], al[4];
-                split_tf32(e[0], ah[0], al[0]);
-                split_tf32(e[8], ah[1], al[1]);
-                split_tf32(e[4 * kErrStride], ah[2], al[2]);
-                split_tf32(e[4 * kErrStride + 8], ah[3], al[3]);
-                mma_16n8k8_tf32(c[m], ah, bh);
-                mma_16n8k8_tf32(c[m], ah, bl);
-                mma_16n8k8_tf32(c[m], al, bh);
-            }
-        }
+        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(c[m], ah[m], bl);
+#pragma unroll
+        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(c[m], al[m], bh);
     };
 
-    cp_async_wait<3>();
-    static_assert(kSubs == 4, "one commit group of U tiles per sub-panel");
-    __syncthreads();                                   // rtab and the first sub-panel's tiles
+    bool staged = true;
+    if (UVEC) staged = tc::mbar_wait(ubar, 0);
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (__syncthreads_or(!staged)) {                   // U never arrived: report it and leave the outputs alone
+        if (tid == 0 && p.status) atomicOr(p.status, tc::kStatusTimeout);
+        return;
+    }
+    scales();
 #pragma unroll
     for (int q = 0; q < kSubs; q++) {
-        const int ng = min(kWalkWarps, span / kGroupCols - q * kWalkWarps);      // groups of this sub-panel
-        if (ng <= 0) break;
-        const float* uq = ut + q * kUTiles * 64;
-        float* eq = es + (q & 1) * (kSubCols * kErrStride) + lane;
-        float4 un[2 * kGroupCols];                     // U tile of the last published group and this warp's
+        const int nq = min(kWalkWarps, ng - q * kWalkWarps);      // groups of this sub-panel
+        if (nq <= 0) break;
+        // acc[q + 1] += errors of group g of this sub-panel
+        auto near = [&](int o) {
+            if ((q + 1) * kSubCols + wc < span) {
+                uint32_t ah[2][4], al[2][4], bh[2], bl[2];
+                load_u(bh, bl, q * kWalkWarps + o, q + 1);
+                load_errors(ah, al, q * kWalkWarps + o);
+                products(acc[q + 1 < kSubs ? q + 1 : 0], ah, al, bh, bl);
+            }
+        };
+        // acc[q + 1 ..] += errors of group o of the sub-panel before
+        auto far = [&](int o) {
+            if (q > 0 && (q + 1) * kSubCols + wc < span) {
+                uint32_t ah[2][4], al[2][4], bh[kSubs][2], bl[kSubs][2];
+#pragma unroll
+                for (int q2 = q + 1; q2 < kSubs; q2++)
+                    if (q2 * kSubCols + wc < span) load_u(bh[q2], bl[q2], (q - 1) * kWalkWarps + o, q2);
+                load_errors(ah, al, (q - 1) * kWalkWarps + o);
+#pragma unroll
+                for (int q2 = q + 1; q2 < kSubs; q2++)
+                    if (q2 * kSubCols + wc < span) products(acc[q2], ah, al, bh[q2], bl[q2]);
+            }
+        };
+        float4 un[2 * kGroupCols];                     // U: rows of the group being walked, columns of this warp's
 #pragma unroll 1
-        for (int o = 0; o < ng; o++) {                 // errors up to group o - 1 are published
-            if (o > 0 && warp >= o && warp < ng) {
-                const float* e = eq + (o - 1) * kGroupCols * kErrStride;
+        for (int o = 0; o < nq; o++) {                 // errors up to group o - 1 are published
+            const int g = q * kWalkWarps + o;
+            if (o > 0 && warp >= o && warp < nq) {
+                const float* ep = es + ((g - 1) & (2 * kWalkWarps - 1)) * kErrSlot + lane;
 #pragma unroll
                 for (int j = 0; j < kGroupCols; j++) {
-                    const float ej = e[j * kErrStride];
+                    const float ej = ep[j * kErrStride];
                     const u64 e2 = pack2(ej, ej);
                     t[0] = fma2(e2, pack2(un[2 * j].x, un[2 * j].y), t[0]);
                     t[1] = fma2(e2, pack2(un[2 * j].z, un[2 * j].w), t[1]);
@@ -644,27 +707,14 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
                     t[3] = fma2(e2, pack2(un[2 * j + 1].z, un[2 * j + 1].w), t[3]);
                 }
             }
-            if (warp > o && warp < ng) {
-                const float4* u = reinterpret_cast<const float4*>(uq + (u_tile_row(o) + warp - o) * 64);
-#pragma unroll
-                for (int j = 0; j < 2 * kGroupCols; j++) un[j] = u[j];
-            }
             if (warp == o) {
-                float tt[8];
+                float tt[8], ev[8];
 #pragma unroll
                 for (int h = 0; h < 4; h++) unpack2(t[h], tt[2 * h], tt[2 * h + 1]);
                 const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-                float rs[8];
-                uint16_t vh[8];
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const uint32_t c = ((j < 4 ? cd.x : cd.y) >> (8 * (j & 3))) & 0x7Fu;
-                    rs[j] = rtab[c];
-                    vh[j] = e4m3_to_f16bits(c);
-                }
-                const float4* u = reinterpret_cast<const float4*>(uq + u_tile_row(o) * 64);
-                float* e = eq + o * kGroupCols * kErrStride;
-                float* eg = EpT + (int64_t)(q * kSubCols + o * kGroupCols) * p.rows + r;
+                float* e = es + (g & (2 * kWalkWarps - 1)) * kErrSlot + lane;
+                const float* ud = ut + u_row(g);
+                const int dp = u_pitch(g);
                 uint32_t packed[2] = {0u, 0u};
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
@@ -679,30 +729,45 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
                         "fma.rn.f32.f16 %0, ql, %3, %4;\n\t"
                         "cvt.u32.u8 %1, b;\n\t}"
                         : "=f"(qv), "=r"(nib) : "f"(__fmul_rn(y, rs[j])), "h"(vh[j]), "f"(0.0f));
-                    const float ej = __fsub_rn(w[j], __fmul_rn(qv, Sq));
-                    const float4 u0 = u[2 * j], u1 = u[2 * j + 1];
-                    const float uv[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+                    ev[j] = __fsub_rn(w[j], __fmul_rn(qv, Sq));
+                    if (j < 7) {
+                        const float4 u0 = *reinterpret_cast<const float4*>(ud + j * dp);
+                        const float4 u1 = *reinterpret_cast<const float4*>(ud + j * dp + 4);
+                        const float uv[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
 #pragma unroll
-                    for (int c = j + 1; c < 8; c++) tt[c] = __fmaf_rn(ej, uv[c], tt[c]);
-                    e[j * kErrStride] = ej;
-                    if (active) eg[(int64_t)j * p.rows] = ej;
+                        for (int c = j + 1; c < 8; c++) tt[c] = __fmaf_rn(ev[j], uv[c], tt[c]);
+                    }
+                    e[j * kErrStride] = ev[j];
                     // an exactly zero target takes the +0 code
                     packed[j >> 2] |= (y == 0.0f ? 0u : nib & 0xFu) << (8 * (j & 3));
                 }
-                if (active) *reinterpret_cast<uint2*>(p.qb + rbase + q * kSubCols + wc) = make_uint2(packed[0], packed[1]);
+                step_barrier();                        // publish before the global stores
+                if (active) {
+                    float* eg = EpT + (int64_t)g * kGroupCols * p.rows + r;
+#pragma unroll
+                    for (int j = 0; j < 8; j++) eg[(int64_t)j * p.rows] = ev[j];
+                    *reinterpret_cast<uint2*>(p.qb + rbase + g * kGroupCols) = make_uint2(packed[0], packed[1]);
+                }
                 fetch(q + 1);
+                continue;
             }
-            if (o == ng - 1) {                         // the next sub-panel's tiles
-                if (q == 0) cp_async_wait<2>();
-                else if (q == 1) cp_async_wait<1>();
-                else cp_async_wait<0>();
+            if (warp > o && warp < nq) {
+                const float* u = ut + u_row(g) + (warp - o) * kGroupCols;
+                const int up = u_pitch(g);
+#pragma unroll
+                for (int j = 0; j < 2 * kGroupCols; j++) un[j] = *reinterpret_cast<const float4*>(u + (j >> 1) * up + 4 * (j & 1));
             }
-            __syncthreads();
+            if (o > 0) near(o - 1);
+            far(o);
+            step_barrier();
         }
+        // here sub-panel q + 1 exists only if this one is full; its rows need the last
+        // group's errors, and what this warp missed while it walked
         if (q + 1 < kSubs && (q + 1) * kSubCols + wc < span) {
-            float (&c)[2][4] = acc[q + 1];
-            update(c, q, q + 1);
-            // fragments to one row per lane
+            far(warp);
+            if (warp > 0) near(warp - 1);
+            near(kWalkWarps - 1);
+            const float (&c)[2][4] = acc[q + 1 < kSubs ? q + 1 : 0];
 #pragma unroll
             for (int m = 0; m < 2; m++)
 #pragma unroll
@@ -710,17 +775,10 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
                     *reinterpret_cast<float2*>(tw + (16 * m + 8 * h + (lane >> 2)) * kTurnStride + 2 * (lane & 3)) =
                         make_float2(c[m][2 * h], c[m][2 * h + 1]);
             __syncwarp();
-            const float4 a = *reinterpret_cast<const float4*>(tw + lane * kTurnStride);
-            const float4 b = *reinterpret_cast<const float4*>(tw + lane * kTurnStride + 4);
-            t[0] = pack2(a.x, a.y);
-            t[1] = pack2(a.z, a.w);
-            t[2] = pack2(b.x, b.y);
-            t[3] = pack2(b.z, b.w);
+            set_rows(tw + lane * kTurnStride);
             __syncwarp();
+            scales();
         }
-#pragma unroll
-        for (int q2 = q + 2; q2 < kSubs; q2++)
-            if (q2 * kSubCols + wc < span) update(acc[q2], q, q2);
     }
 }
 
