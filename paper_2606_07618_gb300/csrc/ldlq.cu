@@ -111,124 +111,338 @@ __global__ void __launch_bounds__(256) gather_h_kernel(const float* H, int64_t n
     }
 }
 
-// Cholesky of the nb x nb diagonal block at k0 (lower, in place) and its inverse
-// (lower, 64 x 64) into Linv.  The block is padded to 64 with an identity; each
-// of the 256 threads keeps a 4 x 4 tile in registers.  The pivots stay
-// unscaled, A = M diag(p) M^T with M unit lower triangular: at column j the
-// threads holding column j publish it to shared memory (double-buffered, one
-// barrier per column) and every tile subtracts a_ij a_lj / p_j (rows i > j,
-// columns l > j; the upper parts of the tiles take the same updates unread).  Then
-// L = M diag(sqrt p) and L^-1 = diag(1/sqrt p) M^-1, with M^-1 by forward
-// elimination in the same scheme (column k of M and row k of M^-1 published per
-// step).  A pivot that is not positive and finite sets bit 4 of the status word
-// and is replaced by 1 so the values stay finite.
-__global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t k0, int nb, float* Linv,
-                                                    int* status) {
-    __shared__ __align__(16) float colv[2][kP];
-    __shared__ __align__(16) float rowv[2][kP];
-    __shared__ float piv[kP];
-    const int r0 = (threadIdx.x >> 4) * 4, c0 = (threadIdx.x & 15) * 4;
-    float t[4][4];
-    float x[4][4];                                   // X = M^-1 (unit lower), built alongside
+// out[r][c] = sum_{k < K} x[r][k] y[c][k] for the rows r = r0 + RS i and columns
+// c = c0 + CS j of a thread's 4 x 4 tile; x and y in shared memory, kPad words per
+// row, K a multiple of 4.  Even and odd k are summed apart (packed fp32).
+constexpr int kPad = kP + 4;          // rows 4 banks apart: eight lanes' 16-byte reads cover all banks
+template <int RS, int CS>
+__device__ __forceinline__ void tile_dot(const float* x, int r0, const float* y, int c0, int K, float (&out)[4][4]) {
+    u64 acc[4][4];
 #pragma unroll
-    for (int di = 0; di < 4; di++)
+    for (int i = 0; i < 4; i++)
 #pragma unroll
-        for (int dl = 0; dl < 4; dl++) {
-            const int i = r0 + di, l = c0 + dl;
-            float v = (i < nb && l < nb && l <= i) ? A[(k0 + i) * n + k0 + l] : 0.0f;
-            if (i >= nb && i == l) v = 1.0f;
-            t[di][dl] = v;
-            x[di][dl] = i == l ? 1.0f : 0.0f;
+        for (int j = 0; j < 4; j++) acc[i][j] = 0ull;
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float4 a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) a[i] = *reinterpret_cast<const float4*>(x + (r0 + RS * i) * kPad + k);
+#pragma unroll
+        for (int j = 0; j < 4; j++) b[j] = *reinterpret_cast<const float4*>(y + (c0 + CS * j) * kPad + k);
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                acc[i][j] = fma2(pack2(a[i].x, a[i].y), pack2(b[j].x, b[j].y), acc[i][j]);
+                acc[i][j] = fma2(pack2(a[i].z, a[i].w), pack2(b[j].z, b[j].w), acc[i][j]);
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            float lo, hi;
+            unpack2(acc[i][j], lo, hi);
+            out[i][j] = __fadd_rn(lo, hi);
         }
-    // Step j: column j of the reduced matrix gives the pivot and the multipliers
-    // m_ij = a_ij / p_j (= M's column j); the trailing update and the inverse's
-    // row operation X_i -= m_ij X_j (row j of X is final at step j) share one
-    // barrier.  Per entry the inverse sees its updates in the order k = 0, 1, ...
+}
+
+// 1/p to an ulp without the branches of the rounded form: the hardware's
+// approximation and one Newton step (tiny and huge p, where that step would leave
+// the normal range, take the rounded form).
+__device__ __forceinline__ float rcp_fast(float p) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(p));
+    r = __fmaf_rn(r, __fmaf_rn(-p, r, 1.0f), r);
+    if (!(p > 1e-36f && p < 1e36f)) r = __frcp_rn(p);
+    return r;
+}
+
+// One panel's sequential part, in one CTA: the Cholesky factor of the nb x nb
+// diagonal block at k0 (lower, in place), its inverse Linv (64 x 64, lower), and the
+// solved panel of the next 64 rows, Xtop = A[k0 + nb .., k0 ..] Linv^T.
+//
+// The block is padded to 64 with an identity and held as 4 x 4 tiles in registers:
+// thread (I, J) holds tile (I, J) of the block for J <= I and, for J > I, tile
+// (J, I) of X = M^-1 (threads on the diagonal hold that one too).  The pivots stay
+// unscaled, A = M diag(p) M^T with M unit lower triangular.  Block step b: thread
+// (b, b) factors its tile and publishes M_bb and 1/p; after a barrier the tiles
+// below it become W = A M_bb^-T and the multipliers W / p, and the tiles of X's row
+// b are eliminated; after another, every remaining tile takes its rank-4 update,
+// tile -= m_I W_J^T or X tile -= m_I X_b (X_b is kept transposed, so the two are
+// the same code).  Then L = M diag(sqrt p) and Linv = diag(1/sqrt p) X.  A pivot
+// that is not positive and finite sets bit 4 of the status word and is replaced by
+// 1 so the values stay finite.
+//
+// Bound by latency: 16 steps of a 4-pivot chain (a reciprocal and two dependent
+// multiply-adds per pivot), two barriers and a rank-4 update.  One column per step
+// (64 barriers, every thread updating a tile of both matrices) took 17.8 us.
+__global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t k0, int nb, float* Linv, float* Xtop,
+                                                    int* status) {
+    extern __shared__ __align__(16) float psm[];
+    float* sl = psm;                                 // [64][kPad] Linv
+    float* st = psm + kP * kPad;                     // [64][kPad] the next 64 rows of the panel
+    __shared__ __align__(16) float sw[kP][4], smul[kP][4], sx[kP][4];   // W, W / p, X_b^T
+    __shared__ float sm[6], sip[4], piv[kP];
+    const int I = threadIdx.x >> 4, J = threadIdx.x & 15;
+    const bool low = J <= I, diag = I == J;
+    const int R = low ? I : J, C = low ? J : I;      // the thread's tile: (R, C) of A (low) or of X
+    const int nt = (int)(n - k0 - nb < kP ? n - k0 - nb : kP);          // rows of Xtop
+    // the previous panel's kernel updated this block column
+    grid_dependency_wait();
+    // every load before the first store to shared memory: one trip to L2
+    float v[kP * kP / 256], w[kP * kP / 256];
+#pragma unroll
+    for (int e = 0; e < kP * kP / 256; e++) {
+        const int r = e * 4 + (threadIdx.x >> 6), c = threadIdx.x & 63;
+        v[e] = r < nb && c <= r ? A[(k0 + r) * n + k0 + c] : r == c ? 1.0f : 0.0f;
+        w[e] = r < nt ? A[(k0 + nb + r) * n + k0 + c] : 0.0f;
+    }
+#pragma unroll
+    for (int e = 0; e < kP * kP / 256; e++) {
+        const int r = e * 4 + (threadIdx.x >> 6), c = threadIdx.x & 63;
+        sl[r * kPad + c] = v[e];
+        st[r * kPad + c] = w[e];
+    }
+    __syncthreads();
+    float t[4][4], xd[4][4];                         // xd: the diagonal tile of X
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (low) q = *reinterpret_cast<const float4*>(sl + (4 * R + i) * kPad + 4 * C);
+        t[i][0] = q.x;
+        t[i][1] = q.y;
+        t[i][2] = q.z;
+        t[i][3] = q.w;
+#pragma unroll
+        for (int j = 0; j < 4; j++) xd[i][j] = i == j ? 1.0f : 0.0f;
+    }
     int bad = 0;
-    // columns in groups of four, so that a tile's column j - c0 (and row j - r0)
-    // is a compile-time index: the owners publish without selects
-    for (int jb = 0; jb < kP; jb += 4) {
+#pragma unroll 1
+    for (int b = 0; b < kP / 4; b++) {
+        if (diag && I == b) {
+            float p[4], ip[4], m[4][4];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int j = jb + q, b = q & 1;
-            if (c0 == jb)
+            for (int j = 0; j < 4; j++) {
+                const bool ok = t[j][j] > 0.0f && t[j][j] <= 3.402823466e38f;
+                bad |= !ok;
+                p[j] = ok ? t[j][j] : 1.0f;
+                ip[j] = rcp_fast(p[j]);
 #pragma unroll
-                for (int di = 0; di < 4; di++) colv[b][r0 + di] = t[di][q];
-            if (r0 == jb)                            // row j of X
+                for (int i = j + 1; i < 4; i++) m[i][j] = __fmul_rn(t[i][j], ip[j]);
 #pragma unroll
-                for (int dc = 0; dc < 4; dc++) rowv[b][c0 + dc] = x[q][dc];
-            __syncthreads();
-            float p = colv[b][j];
-            if (!(p > 0.0f) || !isfinite(p)) {
-                bad = 1;
-                p = 1.0f;
-            }
-            if (threadIdx.x == 0) piv[j] = p;
-            const float ip = __frcp_rn(p);
-            const float4 ci = *reinterpret_cast<const float4*>(&colv[b][r0]);
-            const float4 cl = *reinterpret_cast<const float4*>(&colv[b][c0]);
-            const float4 xj = *reinterpret_cast<const float4*>(&rowv[b][c0]);
-            const float civ[4] = {ci.x, ci.y, ci.z, ci.w}, clv[4] = {cl.x, cl.y, cl.z, cl.w};
-            const float xjv[4] = {xj.x, xj.y, xj.z, xj.w};
-            // rows i <= j and columns l <= j take a zero multiplier instead of a
-            // predicate: the skipped terms are exact zeros (the tiles' upper parts
-            // are never read back and stay finite; row j of M^-1 is zero beyond
-            // column j), so all 32 updates run unconditionally
-            float am[4], cm[4];
+                for (int i = j + 1; i < 4; i++)
 #pragma unroll
-            for (int d = 0; d < 4; d++) {
-                am[d] = r0 + d > j ? __fmul_rn(civ[d], ip) : 0.0f;
-                cm[d] = c0 + d > j ? clv[d] : 0.0f;
+                    for (int l = j + 1; l <= i; l++) t[i][l] = __fmaf_rn(-m[i][j], t[l][j], t[i][l]);
             }
 #pragma unroll
-            for (int di = 0; di < 4; di++)
+            for (int j = 0; j < 4; j++) {
+                sip[j] = ip[j];
+                piv[4 * b + j] = p[j];
+            }
+            sm[0] = m[1][0];
+            sm[1] = m[2][0];
+            sm[2] = m[2][1];
+            sm[3] = m[3][0];
+            sm[4] = m[3][1];
+            sm[5] = m[3][2];
 #pragma unroll
-                for (int dl = 0; dl < 4; dl++) {
-                    t[di][dl] = __fmaf_rn(-am[di], cm[dl], t[di][dl]);
-                    x[di][dl] = __fmaf_rn(-am[di], xjv[dl], x[di][dl]);
+            for (int i = 1; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < i; j++) t[i][j] = m[i][j];     // M_bb stays in the tile
+        }
+        __syncthreads();
+        const float m10 = sm[0], m20 = sm[1], m21 = sm[2], m30 = sm[3], m31 = sm[4], m32 = sm[5];
+        if (low && J == b && I > b) {                 // W = A M_bb^-T
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                t[i][1] = __fmaf_rn(-t[i][0], m10, t[i][1]);
+                t[i][2] = __fmaf_rn(-t[i][0], m20, t[i][2]);
+                t[i][3] = __fmaf_rn(-t[i][0], m30, t[i][3]);
+                t[i][2] = __fmaf_rn(-t[i][1], m21, t[i][2]);
+                t[i][3] = __fmaf_rn(-t[i][1], m31, t[i][3]);
+                t[i][3] = __fmaf_rn(-t[i][2], m32, t[i][3]);
+                *reinterpret_cast<float4*>(sw[4 * I + i]) = make_float4(t[i][0], t[i][1], t[i][2], t[i][3]);
+                *reinterpret_cast<float4*>(smul[4 * I + i]) =
+                    make_float4(__fmul_rn(t[i][0], sip[0]), __fmul_rn(t[i][1], sip[1]), __fmul_rn(t[i][2], sip[2]),
+                                __fmul_rn(t[i][3], sip[3]));
+            }
+        }
+        if (R == b && (!low || diag)) {               // row b of X: forward elimination by M_bb
+            float x[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) x[i][j] = diag ? xd[i][j] : t[i][j];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                x[1][j] = __fmaf_rn(-m10, x[0][j], x[1][j]);
+                x[2][j] = __fmaf_rn(-m20, x[0][j], x[2][j]);
+                x[3][j] = __fmaf_rn(-m30, x[0][j], x[3][j]);
+                x[2][j] = __fmaf_rn(-m21, x[1][j], x[2][j]);
+                x[3][j] = __fmaf_rn(-m31, x[1][j], x[3][j]);
+                x[3][j] = __fmaf_rn(-m32, x[2][j], x[3][j]);
+                *reinterpret_cast<float4*>(sx[4 * C + j]) = make_float4(x[0][j], x[1][j], x[2][j], x[3][j]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    if (diag) xd[i][j] = x[i][j];
+                    else t[i][j] = x[i][j];
+                }
+        }
+        __syncthreads();
+        if (R > b && (low ? C > b : C <= b)) {
+            const float(*y)[4] = low ? &sw[4 * C] : &sx[4 * C];
+            float4 mr[4], yc[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                mr[i] = *reinterpret_cast<const float4*>(smul[4 * R + i]);
+                yc[i] = *reinterpret_cast<const float4*>(y[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    t[i][j] = __fmaf_rn(-mr[i].x, yc[j].x, t[i][j]);
+                    t[i][j] = __fmaf_rn(-mr[i].y, yc[j].y, t[i][j]);
+                    t[i][j] = __fmaf_rn(-mr[i].z, yc[j].z, t[i][j]);
+                    t[i][j] = __fmaf_rn(-mr[i].w, yc[j].w, t[i][j]);
                 }
         }
     }
+    // L into the block, Linv = diag(1 / sqrt p) X into shared and global memory
     __syncthreads();
-    // M (strictly lower part) in the tiles: m_il = a_il / p_l
+    float* sq = &sw[0][0];                           // sqrt p, then 1 / sqrt p
+    if (threadIdx.x < kP) {
+        sq[threadIdx.x] = __fsqrt_rn(piv[threadIdx.x]);
+        sq[kP + threadIdx.x] = __frsqrt_rn(piv[threadIdx.x]);
+    }
+    __syncthreads();
 #pragma unroll
-    for (int di = 0; di < 4; di++)
+    for (int i = 0; i < 4; i++) {
+        const int r = 4 * R + i;
+        if (low) {
 #pragma unroll
-        for (int dl = 0; dl < 4; dl++)
-            if (c0 + dl < r0 + di) t[di][dl] = __fmul_rn(t[di][dl], __frcp_rn(piv[c0 + dl]));
-#pragma unroll
-    for (int di = 0; di < 4; di++)
-#pragma unroll
-        for (int dl = 0; dl < 4; dl++) {
-            const int i = r0 + di, l = c0 + dl;
-            const float sl = __fsqrt_rn(piv[l]);
-            if (i < nb && l <= i) A[(k0 + i) * n + k0 + l] = i == l ? sl : __fmul_rn(t[di][dl], sl);
-            Linv[i * kP + l] = l <= i ? __fmul_rn(x[di][dl], __frsqrt_rn(piv[i])) : 0.0f;
+            for (int j = 0; j < 4; j++) {
+                const int c = 4 * C + j;
+                // W = M p, so below the diagonal tile L = M sqrt p = W / sqrt p
+                const float o = !diag ? __fmul_rn(t[i][j], sq[kP + c]) : r == c ? sq[c] : __fmul_rn(t[i][j], sq[c]);
+                if (r < nb && c <= r) A[(k0 + r) * n + k0 + c] = o;
+            }
         }
-    if (threadIdx.x == 0 && bad && status) atomicOr(status, 4);
+        if (!low || diag) {
+            const float q = sq[kP + r];
+            float o[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) o[j] = 4 * C + j <= r ? __fmul_rn(diag ? xd[i][j] : t[i][j], q) : 0.0f;
+            const float4 x = make_float4(o[0], o[1], o[2], o[3]), z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            *reinterpret_cast<float4*>(sl + r * kPad + 4 * C) = x;
+            *reinterpret_cast<float4*>(Linv + r * kP + 4 * C) = x;
+            if (!diag) {                              // the upper part: zero
+                *reinterpret_cast<float4*>(sl + (4 * C + i) * kPad + 4 * R) = z;
+                *reinterpret_cast<float4*>(Linv + (4 * C + i) * kP + 4 * R) = z;
+            }
+        }
+    }
+    if (bad && status) atomicOr(status, 4);
+    __syncthreads();
+    // Xtop: rows I + 16 i, columns J + 16 j of the solved panel
+    if (nt > 0) {
+        float o[4][4];
+        tile_dot<16, 16>(st, I, sl, J, kP, o);
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) Xtop[(I + 16 * i) * kP + J + 16 * j] = o[i][j];
+    }
 }
 
-// Panel below the diagonal block: rows i >= k0+nb, X = A_panel * Linv^T (one warp per row).
-__global__ void __launch_bounds__(256) trsm_kernel(float* A, int64_t n, int64_t k0, int nb, const float* Linv) {
-    __shared__ float li[kP][kP + 1];
-    __shared__ float row[8][kP];
-    for (int e = threadIdx.x; e < kP * kP; e += blockDim.x) li[e / kP][e % kP] = Linv[e];
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int64_t i = k0 + nb + (int64_t)blockIdx.x * 8 + warp; i < n; i += (int64_t)gridDim.x * 8) {
-        float* ai = A + i * n + k0;
-        row[warp][lane] = lane < nb ? ai[lane] : 0.0f;
-        row[warp][lane + 32] = lane + 32 < nb ? ai[lane + 32] : 0.0f;
-        __syncwarp();
-        float x0 = 0.0f, x1 = 0.0f;
-        for (int l = 0; l < nb; l++) {
-            const float al = row[warp][l];
-            x0 = __fmaf_rn(al, li[lane][l], x0);
-            x1 = __fmaf_rn(al, li[lane + 32][l], x1);
+// The rows i >= k0 + 64 of one panel, 32 per CTA: the solved panel X = A Linv^T
+// (in place), then the next panel's block column, A[i][k0 + 64 ..] -= X Xtop^T, up
+// to column i.  Everything in fp32 from shared memory; a separate panel solve and a
+// tensor-core update of a 64-wide column spent 14 us here on launches, tile fills
+// and half-empty tiles.
+constexpr int kPanelRows = 32;
+constexpr int kPanelSmem = (2 * kP + 2 * kPanelRows) * kPad * 4;
+template <bool VEC>
+__global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t k0, const float* Linv, const float* Xtop) {
+    extern __shared__ __align__(16) float psm[];
+    float* sl = psm;                                 // [64][kPad] Linv
+    float* st = sl + kP * kPad;                      // [64][kPad] Xtop
+    float* sa = st + kP * kPad;                      // [32][kPad] the rows
+    float* sx = sa + kPanelRows * kPad;              // [32][kPad] the solved rows
+    const int64_t i0 = k0 + kP + (int64_t)blockIdx.x * kPanelRows;
+    const int rows = (int)(n - i0 < kPanelRows ? n - i0 : kPanelRows);
+    // every load before the first store to shared memory: one trip to L2
+    constexpr int kQ = kP / 4;
+    float4 vl[kP * kQ / 128], vt[kP * kQ / 128], va[kPanelRows * kQ / 128];
+#pragma unroll
+    for (int u = 0; u < kPanelRows * kQ / 128; u++) {
+        const int e = threadIdx.x + 128 * u, r = e / kQ, c = 4 * (e % kQ);
+        va[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (r < rows) {
+            const float* a = A + (i0 + r) * n + k0 + c;
+            if (VEC) va[u] = *reinterpret_cast<const float4*>(a);
+            else va[u] = make_float4(a[0], a[1], a[2], a[3]);
         }
-        __syncwarp();
-        if (lane < nb) ai[lane] = x0;
-        if (lane + 32 < nb) ai[lane + 32] = x1;
+    }
+#pragma unroll
+    for (int u = 0; u < kP * kQ / 128; u++) {
+        vl[u] = reinterpret_cast<const float4*>(Linv)[threadIdx.x + 128 * u];
+        vt[u] = reinterpret_cast<const float4*>(Xtop)[threadIdx.x + 128 * u];
+    }
+#pragma unroll
+    for (int u = 0; u < kPanelRows * kQ / 128; u++) {
+        const int e = threadIdx.x + 128 * u;
+        *reinterpret_cast<float4*>(sa + (e / kQ) * kPad + 4 * (e % kQ)) = va[u];
+    }
+#pragma unroll
+    for (int u = 0; u < kP * kQ / 128; u++) {
+        const int e = threadIdx.x + 128 * u;
+        *reinterpret_cast<float4*>(sl + (e / kQ) * kPad + 4 * (e % kQ)) = vl[u];
+        *reinterpret_cast<float4*>(st + (e / kQ) * kPad + 4 * (e % kQ)) = vt[u];
+    }
+    __syncthreads();
+    // thread: rows ty + 8 i, columns 4 tx .. (phase 1: Linv's row c ends at column c) or tx + 16 j
+    const int ty = threadIdx.x & 7, tx = threadIdx.x >> 3;
+    float o[4][4];
+    tile_dot<8, 1>(sa, ty, sl, 4 * tx, 4 * tx + 4, o);
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+        *reinterpret_cast<float4*>(sx + (ty + 8 * i) * kPad + 4 * tx) = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+    __syncthreads();
+    // the solved rows, and the block column's values, which the products below come off
+    float4 vc[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int64_t r = i0 + ty + 8 * i, c0 = k0 + kP + 4 * tx;
+        vc[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (r >= n) continue;
+        float* a = A + r * n + k0 + 4 * tx;
+        if (VEC) {
+            *reinterpret_cast<float4*>(a) = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+            if (c0 + 3 <= r) vc[i] = *reinterpret_cast<const float4*>(A + r * n + c0);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++) a[j] = o[i][j];
+        }
+    }
+    tile_dot<8, 1>(sx, ty, st, 4 * tx, kP, o);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int64_t r = i0 + ty + 8 * i, c0 = k0 + kP + 4 * tx;
+        if (r >= n) continue;
+        float* c = A + r * n + c0;
+        if (VEC && c0 + 3 <= r) {
+            *reinterpret_cast<float4*>(c) = make_float4(__fsub_rn(vc[i].x, o[i][0]), __fsub_rn(vc[i].y, o[i][1]),
+                                                        __fsub_rn(vc[i].z, o[i][2]), __fsub_rn(vc[i].w, o[i][3]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (c0 + j <= r) c[j] = __fsub_rn(c[j], o[i][j]);
+        }
     }
 }
 
@@ -797,7 +1011,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* qb, const int3
 }  // namespace
 
 size_t ldlq_prepare_workspace(int64_t n) {
-    return (size_t)((n * 4 + 255) / 256 * 256) + 256 + (size_t)kP * kP * 4;
+    return (size_t)((n * 4 + 255) / 256 * 256) + 256 + (size_t)2 * kP * kP * 4;
 }
 
 // Stream and events of the factorization's look-ahead, one set per device,
@@ -840,6 +1054,7 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     float* d = reinterpret_cast<float*>(w);
     float* lam = reinterpret_cast<float*>(w + (n * 4 + 255) / 256 * 256);
     float* Linv = lam + 64;
+    float* Xtop = Linv + kP * kP;
     diag_kernel<<<1, 1024, 0, s>>>(H, n, damp, d, lam, status);
     rank_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d, n, perm);
     const unsigned rg = (unsigned)imin64(n, (int64_t)sms * 8);
@@ -847,9 +1062,9 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // Look-ahead: the trailing update of panel k is split into the next panel's
-    // block column (on the high-priority stream, with the next diagonal factor
-    // and panel solve) and the rest (on `s`, overlapping them).  The two
-    // updates of one block column from different panels are ordered by events.
+    // block column (on the high-priority stream, in the kernel that solves the
+    // panel, with the diagonal factors) and the rest (on `s`, overlapping them).
+    // The two updates of one block column from different panels are ordered by events.
     LookAhead* la = nullptr;
     std::unique_lock<std::mutex> lock;
     e = lookahead_for_current_device(&la, &lock);
@@ -857,26 +1072,27 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     cudaStream_t c = la->crit;
     if ((e = cudaEventRecord(la->fork, s)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(c, la->fork, 0)) != cudaSuccess) return e;
+    constexpr int kPotrfSmem = 2 * kP * kPad * 4;
+    static_assert(kPotrfSmem <= 48 * 1024, "no shared-memory opt-in");
+    const bool vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
+    const auto panel = vec ? panel_kernel<true> : panel_kernel<false>;
+    if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPanelSmem)) != cudaSuccess) return e;
     bool have_rest = false;              // rest_done recorded by this call (waits stay inside a capture)
     for (int64_t k0 = 0; k0 < n; k0 += kP) {
         const int nb = (int)imin64(kP, n - k0);
-        potrf_kernel<<<1, 256, 0, c>>>(U, n, k0, nb, Linv, status);
+        potrf_kernel<<<1, 256, kPotrfSmem, c>>>(U, n, k0, nb, Linv, Xtop, status);
         const int64_t rest = n - k0 - nb;
         if (rest > 0) {
-            const unsigned tg = (unsigned)imin64((rest + 7) / 8, (int64_t)sms * 8);
-            trsm_kernel<<<tg, 256, 0, c>>>(U, n, k0, nb, Linv);
-            float* P = U + (k0 + nb) * n + k0;         // the solved panel, rows k0+nb..n-1
             const int64_t nb2 = imin64(kP, rest);      // width of the next panel
-            float* C = U + (k0 + nb) * n + k0 + nb;
-            if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
             // the next block column also took the previous panel's rest update
             if (have_rest && (e = cudaStreamWaitEvent(c, la->rest_done, 0)) != cudaSuccess) return e;
-            e = update_gemm<false, true, true>(C, n, P, n, P, n, rest, nb2, nb, -1.0f, status, c);
-            if (e != cudaSuccess) return e;
+            panel<<<(unsigned)((rest + kPanelRows - 1) / kPanelRows), 128, kPanelSmem, c>>>(U, n, k0, Linv, Xtop);
             if (rest > nb2) {
+                float* P = U + (k0 + nb + nb2) * n + k0;      // the solved panel's rows past the next block column
+                float* C = P + nb + nb2;
+                if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(s, la->panel_done, 0)) != cudaSuccess) return e;
-                e = update_gemm<false, true, true>(C + nb2 * n + nb2, n, P + nb2 * n, n, P + nb2 * n, n, rest - nb2,
-                                                   rest - nb2, nb, -1.0f, status, s);
+                e = update_gemm<false, true, true>(C, n, P, n, P, n, rest - nb2, rest - nb2, nb, -1.0f, status, s);
                 if (e != cudaSuccess) return e;
                 if ((e = cudaEventRecord(la->rest_done, s)) != cudaSuccess) return e;
                 have_rest = true;
