@@ -75,35 +75,33 @@ __global__ void __launch_bounds__(1024) diag_kernel(const float* H, int64_t n, f
 }
 
 // perm[rank(i)] = i, rank by (key desc, index asc): a total order, so perm is a
-// permutation of 0..n-1 whatever the keys.
+// permutation of 0..n-1 whatever the keys.  A warp per channel, its lanes over the
+// others (one thread per channel left 16 CTAs walking 4096 keys each: 85 us at n =
+// 4096).
 __global__ void __launch_bounds__(256) rank_kernel(const float* d, int64_t n, int32_t* perm) {
-    __shared__ float sd[1024];
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const float di = i < n ? sort_key(d[i]) : 0.0f;
-    int64_t rank = 0;
-    for (int64_t base = 0; base < n; base += 1024) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < 1024; t += blockDim.x) sd[t] = base + t < n ? sort_key(d[base + t]) : 0.0f;
-        __syncthreads();
-        if (i < n) {
-            const int lim = (int)min((int64_t)1024, n - base);
-            for (int t = 0; t < lim; t++) {
-                const float dj = sd[t];
-                rank += (dj > di) || (dj == di && base + t < i);
-            }
-        }
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (i >= n) return;
+    const float di = sort_key(d[i]);
+    unsigned rank = 0;
+#pragma unroll 4
+    for (int64_t j = lane; j < n; j += 32) {
+        const float dj = sort_key(__ldg(d + j));
+        rank += (dj > di) || (dj == di && j < i);
     }
-    if (i < n) perm[rank] = (int32_t)i;
+    rank = __reduce_add_sync(0xffffffffu, rank);
+    if (lane == 0) perm[rank] = (int32_t)i;
 }
 
-// A[a][b] = H[p(a)][p(b)] (+ lambda on the diagonal), p(a) = perm[n-1-a].
+// A[a][b] = H[p(a)][p(b)] (+ lambda on the diagonal) for b <= a, p(a) = perm[n-1-a];
+// nothing reads the upper part.
 __global__ void __launch_bounds__(256) gather_h_kernel(const float* H, int64_t n, const int32_t* perm,
                                                        const float* lam, float* A) {
     const float l = lam[0];
     for (int64_t a = blockIdx.x; a < n; a += gridDim.x) {
         const float* hrow = H + (int64_t)perm[n - 1 - a] * n;
         float* arow = A + a * n;
-        for (int64_t b = threadIdx.x; b < n; b += blockDim.x) {
+        for (int64_t b = threadIdx.x; b <= a; b += blockDim.x) {
             float v = hrow[perm[n - 1 - b]];
             if (a == b) v = __fadd_rn(v, l);
             arow[b] = v;
@@ -148,14 +146,11 @@ __device__ __forceinline__ void tile_dot(const float* x, int r0, const float* y,
 }
 
 // 1/p to an ulp without the branches of the rounded form: the hardware's
-// approximation and one Newton step (tiny and huge p, where that step would leave
-// the normal range, take the rounded form).
+// approximation and, where its residual is a normal number, one Newton step.
 __device__ __forceinline__ float rcp_fast(float p) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(p));
-    r = __fmaf_rn(r, __fmaf_rn(-p, r, 1.0f), r);
-    if (!(p > 1e-36f && p < 1e36f)) r = __frcp_rn(p);
-    return r;
+    return p > 1e-37f ? __fmaf_rn(r, __fmaf_rn(-p, r, 1.0f), r) : r;
 }
 
 // One panel's sequential part, in one CTA: the Cholesky factor of the nb x nb
@@ -164,19 +159,21 @@ __device__ __forceinline__ float rcp_fast(float p) {
 //
 // The block is padded to 64 with an identity and held as 4 x 4 tiles in registers:
 // thread (I, J) holds tile (I, J) of the block for J <= I and, for J > I, tile
-// (J, I) of X = M^-1 (threads on the diagonal hold that one too).  The pivots stay
+// (J, I) of X = M^-1, transposed (threads on the diagonal hold that one too).  The pivots stay
 // unscaled, A = M diag(p) M^T with M unit lower triangular.  Block step b: thread
 // (b, b) factors its tile and publishes M_bb and 1/p; after a barrier the tiles
 // below it become W = A M_bb^-T and the multipliers W / p, and the tiles of X's row
-// b are eliminated; after another, every remaining tile takes its rank-4 update,
-// tile -= m_I W_J^T or X tile -= m_I X_b (X_b is kept transposed, so the two are
-// the same code).  Then L = M diag(sqrt p) and Linv = diag(1/sqrt p) X.  A pivot
-// that is not positive and finite sets bit 4 of the status word and is replaced by
-// 1 so the values stay finite.
+// b take the same steps; after another, every remaining tile takes its rank-4
+// update, tile -= m_I W_J^T or X^T tile -= X_b^T m_I^T (the same code).  Then
+// L = M diag(sqrt p) and Linv = diag(1/sqrt p) X.  A pivot that is not positive and
+// finite sets bit 4 of the status word and is replaced by 1 so the values stay finite.
 //
-// Bound by latency: 16 steps of a 4-pivot chain (a reciprocal and two dependent
-// multiply-adds per pivot), two barriers and a rank-4 update.  One column per step
-// (64 barriers, every thread updating a tile of both matrices) took 17.8 us.
+// Bound by latency: 16 steps of a 4-pivot chain (620 cycles: a reciprocal and two
+// dependent multiply-adds per pivot), two barriers and a rank-4 update (660), about
+// 13 us with the loads and stores, and 1.7 us for Xtop.  One column per step (64
+// barriers, every thread updating a tile of both matrices) took 17.8 us without
+// Xtop; one warp factoring 16 x 16 blocks, the column going round by shuffles or
+// through shared memory, 480-560 cycles per column.
 __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t k0, int nb, float* Linv, float* Xtop,
                                                     int* status) {
     extern __shared__ __align__(16) float psm[];
@@ -246,14 +243,26 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
             sm[3] = m[3][0];
             sm[4] = m[3][1];
             sm[5] = m[3][2];
+            // X's diagonal tile M_bb^-1 (unit lower), transposed for the update
+            xd[1][0] = -m[1][0];
+            xd[2][1] = -m[2][1];
+            xd[3][2] = -m[3][2];
+            xd[2][0] = __fmaf_rn(m[2][1], m[1][0], -m[2][0]);
+            xd[3][1] = __fmaf_rn(m[3][2], m[2][1], -m[3][1]);
+            xd[3][0] = __fmaf_rn(-m[3][2], xd[2][0], __fmaf_rn(-m[3][1], xd[1][0], -m[3][0]));
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                *reinterpret_cast<float4*>(sx[4 * b + j]) = make_float4(xd[0][j], xd[1][j], xd[2][j], xd[3][j]);
 #pragma unroll
             for (int i = 1; i < 4; i++)
 #pragma unroll
                 for (int j = 0; j < i; j++) t[i][j] = m[i][j];     // M_bb stays in the tile
         }
         __syncthreads();
-        const float m10 = sm[0], m20 = sm[1], m21 = sm[2], m30 = sm[3], m31 = sm[4], m32 = sm[5];
-        if (low && J == b && I > b) {                 // W = A M_bb^-T
+        // W = A M_bb^-T below the block; X's row b, held transposed, takes the same steps
+        if (J == b && !diag) {
+            const float m10 = sm[0], m20 = sm[1], m21 = sm[2], m30 = sm[3], m31 = sm[4], m32 = sm[5];
+            float* dst = low ? &sw[4 * R][0] : &sx[4 * C][0];
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 t[i][1] = __fmaf_rn(-t[i][0], m10, t[i][1]);
@@ -262,43 +271,22 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
                 t[i][2] = __fmaf_rn(-t[i][1], m21, t[i][2]);
                 t[i][3] = __fmaf_rn(-t[i][1], m31, t[i][3]);
                 t[i][3] = __fmaf_rn(-t[i][2], m32, t[i][3]);
-                *reinterpret_cast<float4*>(sw[4 * I + i]) = make_float4(t[i][0], t[i][1], t[i][2], t[i][3]);
-                *reinterpret_cast<float4*>(smul[4 * I + i]) =
-                    make_float4(__fmul_rn(t[i][0], sip[0]), __fmul_rn(t[i][1], sip[1]), __fmul_rn(t[i][2], sip[2]),
-                                __fmul_rn(t[i][3], sip[3]));
+                *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(t[i][0], t[i][1], t[i][2], t[i][3]);
+                if (low)
+                    *reinterpret_cast<float4*>(smul[4 * R + i]) =
+                        make_float4(__fmul_rn(t[i][0], sip[0]), __fmul_rn(t[i][1], sip[1]), __fmul_rn(t[i][2], sip[2]),
+                                    __fmul_rn(t[i][3], sip[3]));
             }
-        }
-        if (R == b && (!low || diag)) {               // row b of X: forward elimination by M_bb
-            float x[4][4];
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) x[i][j] = diag ? xd[i][j] : t[i][j];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                x[1][j] = __fmaf_rn(-m10, x[0][j], x[1][j]);
-                x[2][j] = __fmaf_rn(-m20, x[0][j], x[2][j]);
-                x[3][j] = __fmaf_rn(-m30, x[0][j], x[3][j]);
-                x[2][j] = __fmaf_rn(-m21, x[1][j], x[2][j]);
-                x[3][j] = __fmaf_rn(-m31, x[1][j], x[3][j]);
-                x[3][j] = __fmaf_rn(-m32, x[2][j], x[3][j]);
-                *reinterpret_cast<float4*>(sx[4 * C + j]) = make_float4(x[0][j], x[1][j], x[2][j], x[3][j]);
-            }
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    if (diag) xd[i][j] = x[i][j];
-                    else t[i][j] = x[i][j];
-                }
         }
         __syncthreads();
         if (R > b && (low ? C > b : C <= b)) {
-            const float(*y)[4] = low ? &sw[4 * C] : &sx[4 * C];
+            // A: t[i][j] -= m_(R i) . W_(C j);  X^T: t[i][j] -= X_b^T_(C i) . m_(R j)
+            const float(*u)[4] = low ? &smul[4 * R] : &sx[4 * C];
+            const float(*y)[4] = low ? &sw[4 * C] : &smul[4 * R];
             float4 mr[4], yc[4];
 #pragma unroll
             for (int i = 0; i < 4; i++) {
-                mr[i] = *reinterpret_cast<const float4*>(smul[4 * R + i]);
+                mr[i] = *reinterpret_cast<const float4*>(u[i]);
                 yc[i] = *reinterpret_cast<const float4*>(y[i]);
             }
 #pragma unroll
@@ -336,7 +324,7 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
             const float q = sq[kP + r];
             float o[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) o[j] = 4 * C + j <= r ? __fmul_rn(diag ? xd[i][j] : t[i][j], q) : 0.0f;
+            for (int j = 0; j < 4; j++) o[j] = 4 * C + j <= r ? __fmul_rn(diag ? xd[i][j] : t[j][i], q) : 0.0f;
             const float4 x = make_float4(o[0], o[1], o[2], o[3]), z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             *reinterpret_cast<float4*>(sl + r * kPad + 4 * C) = x;
             *reinterpret_cast<float4*>(Linv + r * kP + 4 * C) = x;
@@ -1056,7 +1044,7 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     float* Linv = lam + 64;
     float* Xtop = Linv + kP * kP;
     diag_kernel<<<1, 1024, 0, s>>>(H, n, damp, d, lam, status);
-    rank_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(d, n, perm);
+    rank_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(d, n, perm);
     const unsigned rg = (unsigned)imin64(n, (int64_t)sms * 8);
     gather_h_kernel<<<rg, 256, 0, s>>>(H, n, perm, lam, U);
     cudaError_t e = cudaGetLastError();
