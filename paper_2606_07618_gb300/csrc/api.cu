@@ -366,7 +366,6 @@ nvfp4_status group_common(int method, const nvfp4_group_tensor* tensors, int cou
         }
     GroupParams p;
     std::memset(&p, 0, sizeof(p));
-    int64_t rows[NVFP4_GROUP_MAX];
     int64_t seg = 0;
     for (int k = 0; k < count; k++) {
         const int i = order[k];
@@ -386,7 +385,7 @@ nvfp4_status group_common(int method, const nvfp4_group_tensor* tensors, int cou
         g.narrow = sh[i].narrow;
         if (g.narrow && g.kb > 0) g.kb_div = make_fast_div((uint32_t)g.kb);
         g.s_index = i;
-        rows[k] = t.rows;
+        g.rows = t.rows;
         const int64_t unit = kGroupCtaSegments;          // a CTA's segments never straddle two tensors
         if (g.nseg > INT64_MAX - seg - unit) return NVFP4_ERR_RANGE;
         seg += (g.nseg + unit - 1) / unit * unit;
@@ -404,7 +403,7 @@ nvfp4_status group_common(int method, const nvfp4_group_tensor* tensors, int cou
     p.amax_bits = dyn ? static_cast<unsigned*>(workspace) : nullptr;
     p.arrived = dyn ? static_cast<unsigned*>(workspace) + kGroupMax : nullptr;
     p.wait_extra = wait_extra;
-    const cudaError_t e = launch_quantize_group(p, rows, dt == NVFP4_IN_BF16 ? 0 : 1, method,
+    const cudaError_t e = launch_quantize_group(p, dt == NVFP4_IN_BF16 ? 0 : 1, method,
                                                 obj == NVFP4_OBJ_WMSE ? 1 : 0, block, sms,
                                                 static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;

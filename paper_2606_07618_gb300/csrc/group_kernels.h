@@ -19,7 +19,7 @@ struct GroupTensor {
     uint8_t* codes;
     uint8_t* sf_linear;
     uint8_t* sf_swizzled;
-    int64_t kb, kpad4;
+    int64_t rows, kb, kpad4;
     int64_t nseg;              // 16-element segments
     int64_t seg_begin;         // first index in the concatenated segment space (multiple of 32)
     int64_t nvec;              // 16-byte input vectors (global-scale reduction)
@@ -57,8 +57,8 @@ constexpr int kGroupCtaSegments = 256;
 // (ScaleSweep only); block 16/32/64.  Zeroes the workspace counters (dyn),
 // launches the grouped kernel (cooperative when dyn; with p.pipelined, a
 // ScaleSweep and at least two tensors, the four launches of the pipelined
-// schedule instead) and the swizzle pad kernels for shapes that need them.
-cudaError_t launch_quantize_group(const GroupParams& p, const int64_t* rows, int dtype, int method, int obj,
-                                  int block, int sms, cudaStream_t s);
+// schedule instead).
+cudaError_t launch_quantize_group(const GroupParams& p, int dtype, int method, int obj, int block, int sms,
+                                  cudaStream_t s);
 
 }  // namespace nvfp4

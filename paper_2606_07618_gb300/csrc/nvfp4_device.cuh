@@ -46,29 +46,43 @@ __device__ __forceinline__ uint32_t e2m1x2(float lo, float hi) {
     return r;
 }
 
-// One candidate step on an element pair: t = fl(y*r) (packed), q = RNE_E2M1(t),
+// Eight fp32 (four packed pairs) -> a word of eight E2M1 codes, the first in the
+// lowest nibble: the converts' bytes are assembled by the conversions themselves.
+__device__ __forceinline__ uint32_t e2m1x8(u64 t0, u64 t1, u64 t2, u64 t3) {
+    uint32_t r;
+    asm("{\n\t.reg .b8 a, b, c, d;\n\t.reg .b32 l0, h0, l1, h1, l2, h2, l3, h3;\n\t"
+        "mov.b64 {l0, h0}, %1;\n\tmov.b64 {l1, h1}, %2;\n\tmov.b64 {l2, h2}, %3;\n\tmov.b64 {l3, h3}, %4;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 a, h0, l0;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 b, h1, l1;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 c, h2, l2;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 d, h3, l3;\n\t"
+        "mov.b32 %0, {a, b, c, d};\n\t}"
+        : "=r"(r) : "l"(t0), "l"(t1), "l"(t2), "l"(t3));
+    return r;
+}
+
+// One candidate step on an element pair: from t = fl(y*r), q = RNE_E2M1(t),
 // e = fl(y - q*v) computed as fma(q, -v, y) with q and -v as exact f16
 // operands, returned packed {e_lo, e_hi}.  nv = f16 bit pattern of -v_c.
-__device__ __forceinline__ u64 cand_err2(u64 y2, u64 r2, uint16_t nv) {
+__device__ __forceinline__ u64 err2_of_t(u64 t2, u64 y2, uint16_t nv) {
     u64 e2;
     asm("{\n\t"
-        ".reg .b64 t2;\n\t"
         ".reg .b32 tl, th, yl, yh, h2, el, eh;\n\t"
         ".reg .b16 ql, qh;\n\t"
         ".reg .b8 q;\n\t"
-        "mul.rn.f32x2 t2, %1, %2;\n\t"
-        "mov.b64 {tl, th}, t2;\n\t"
+        "mov.b64 {tl, th}, %1;\n\t"
         "cvt.rn.satfinite.e2m1x2.f32 q, th, tl;\n\t"
         "cvt.rn.f16x2.e2m1x2 h2, q;\n\t"
         "mov.b32 {ql, qh}, h2;\n\t"
-        "mov.b64 {yl, yh}, %1;\n\t"
+        "mov.b64 {yl, yh}, %2;\n\t"
         "fma.rn.f32.f16 el, ql, %3, yl;\n\t"
         "fma.rn.f32.f16 eh, qh, %3, yh;\n\t"
         "mov.b64 %0, {el, eh};\n\t"
         "}"
-        : "=l"(e2) : "l"(y2), "l"(r2), "h"(nv));
+        : "=l"(e2) : "l"(t2), "l"(y2), "h"(nv));
     return e2;
 }
+__device__ __forceinline__ u64 cand_err2(u64 y2, u64 r2, uint16_t nv) { return err2_of_t(mul2(y2, r2), y2, nv); }
 
 // E4M3 code -> f16 bit pattern of its value (exact), via the native decode.
 __device__ __forceinline__ uint16_t e4m3_to_f16bits(uint32_t code) {
@@ -103,10 +117,35 @@ __device__ __forceinline__ int e4m3_floor_code(float s) {
     return (int)__fmul_rn(s, 512.0f);                // 1..7, exact scaling then truncation
 }
 
+// fl(m / 6) for m >= 0 without the division: a correctly rounded quotient by one
+// residual step (compared with the division over every mantissa; below the normal
+// range it may differ, where every caller's result is the smallest scale anyway).
+__device__ __forceinline__ float sixth(float m) {
+    const float q = __fmul_rn(m, 0.16666667163372039794921875f);
+    return __fmaf_rn(__fmaf_rn(-6.0f, q, m), 0.16666667163372039794921875f, q);
+}
+
+// e4m3_floor_code(fl(m / 6)) for m >= 0 (NaN and inf give 126): m >= 6 v_c exactly
+// when the product of m and fl(1/6), which is a third of an ulp above 1/6, rounded
+// towards zero reaches v_c -- compared with the division for every fp32 m that
+// reaches a code below the largest.  Normal codes are the top bits of that
+// product, those below 2^-5 its integer part in units of 2^-9.
+__device__ __forceinline__ int e4m3_floor_code_of_sixth(float m) {
+    const float s = __fmul_rz(m, 0.16666667163372039794921875f);
+    const int sub = (int)(__float_as_uint(__fmaf_rz(s, 512.0f, 8388608.0f)) & 0xFFu);
+    const int top = (int)(__float_as_uint(s) >> 20) - 960;
+    return min(s < 0.03125f ? sub : top, 126);
+}
+
 // Byte offset of scale (row r, scale column k) in the 128x4-atom swizzled
 // layout read by block-scaled MMA (kpad4 = ceil(kblocks/4)).
 __device__ __forceinline__ int64_t swizzle_offset(int64_t r, int64_t k, int64_t kpad4) {
     return ((r >> 7) * kpad4 + (k >> 2)) * 512 + (r & 31) * 16 + ((r >> 5) & 3) * 4 + (k & 3);
+}
+
+// The same with 32-bit row, column and atom index (rows * scale columns < 2^32).
+__device__ __forceinline__ int64_t swizzle_offset32(uint32_t r, uint32_t k, uint32_t kpad4) {
+    return (int64_t)((r >> 7) * kpad4 + (k >> 2)) * 512 + (int)((r & 31) * 16 + ((r >> 5) & 3) * 4 + (k & 3));
 }
 
 // Streaming 16-byte load that bypasses L1 allocation (each byte is read once).
@@ -115,6 +154,12 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
+}
+// 32 bytes at once (32-byte aligned).  A lane that reads its 32-byte sector in two
+// 16-byte halves makes two requests per line and, past L1, fetches the sector twice.
+__device__ __forceinline__ void ld_stream32(const void* p, uint4& a, uint4& b) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
 }
 __device__ __forceinline__ uint4 ld_ro16(const void* p) {
     uint4 v;

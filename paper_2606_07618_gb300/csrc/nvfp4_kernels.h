@@ -45,8 +45,6 @@ cudaError_t launch_quantize(const QuantParams& p, int dtype, int method, int obj
 // p.S_out/part_max/part_bad/barrier in the caller's workspace).
 cudaError_t launch_quantize_dynamic(const QuantParams& p, int dtype, int method, int obj, int block, int sms,
                                     cudaStream_t s);
-// Zero the pads of a swizzled scale buffer when rows % 128 or kb % 4 != 0.
-cudaError_t launch_swizzle_pad(const QuantParams& p, int sms, cudaStream_t s);
 // Fill the derived fields of p (window mode, row/column need, fast divider).
 void prepare_quant_params(QuantParams& p, int method, int obj, int block, bool* fix);
 

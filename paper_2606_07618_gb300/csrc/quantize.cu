@@ -4,16 +4,6 @@
 
 namespace nvfp4 {
 
-// Zero the padding bytes of the swizzled layout (rows past `rows`, scale
-// columns past `kb`); only launched when the shape is not 128x4-aligned.
-__global__ void swizzle_pad_kernel(uint8_t* sf, int64_t rows, int64_t kb, int64_t kpad4, int64_t rows_pad) {
-    const int64_t total = rows_pad * kpad4 * 4;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / (kpad4 * 4), k = i - r * (kpad4 * 4);
-        if (r >= rows || k >= kb) sf[swizzle_offset(r, k, kpad4)] = 0;
-    }
-}
-
 template <int DT, int METHOD, int OBJ, int BLOCK, int FIX>
 static cudaError_t launch_one(const QuantParams& p, int sms, cudaStream_t s) {
     static std::atomic<int> occ_cache[kOccDevices];
@@ -21,7 +11,17 @@ static cudaError_t launch_one(const QuantParams& p, int sms, cudaStream_t s) {
     const int64_t threads_needed = (p.nseg + 31) & ~(int64_t)31;
     int64_t grid = (threads_needed + 255) / 256;
     const int64_t cap = (int64_t)sms * occ;
-    if (grid > cap) grid = cap;
+    if (grid > cap) {
+        grid = cap;
+        // 4/6 with one weight vector: up to 1/32 fewer CTAs so that a lane keeps its columns
+        const int64_t row = p.kb * (BLOCK / 16);
+        if (METHOD == 2 && OBJ == 1 && p.w_row_stride == 0)
+            for (int64_t g = cap; g >= cap - cap / 32; g--)
+                if (g * 256 % row == 0) {
+                    grid = g;
+                    break;
+                }
+    }
     quantize_kernel<DT, METHOD, OBJ, BLOCK, FIX, 0><<<(int)grid, 256, 0, s>>>(p);
     return cudaGetLastError();
 }
@@ -64,18 +64,6 @@ void prepare_quant_params(QuantParams& p, int method, int obj, int block, bool* 
     if (p.narrow) p.kb_div = make_fast_div((uint32_t)p.kb);
 }
 
-cudaError_t launch_swizzle_pad(const QuantParams& p, int sms, cudaStream_t s) {
-    if (p.sf_swizzled && (p.rows % 128 != 0 || p.kb % 4 != 0) && p.rows > 0 && p.kb > 0) {
-        const int64_t rows_pad = (p.rows + 127) / 128 * 128;
-        const int64_t total = rows_pad * p.kpad4 * 4;
-        int64_t grid = (total + 255) / 256;
-        if (grid > (int64_t)sms * 8) grid = (int64_t)sms * 8;
-        swizzle_pad_kernel<<<(int)grid, 256, 0, s>>>(p.sf_swizzled, p.rows, p.kb, p.kpad4, rows_pad);
-        return cudaGetLastError();
-    }
-    return cudaSuccess;
-}
-
 cudaError_t launch_quantize(const QuantParams& p_in, int dtype, int method, int obj, int block, int sms,
                             cudaStream_t s) {
     QuantParams p = p_in;
@@ -94,7 +82,7 @@ cudaError_t launch_quantize(const QuantParams& p_in, int dtype, int method, int 
         }
         if (e != cudaSuccess) return e;
     }
-    return launch_swizzle_pad(p, sms, s);
+    return cudaSuccess;
 }
 
 }  // namespace nvfp4

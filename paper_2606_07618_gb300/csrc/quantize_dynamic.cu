@@ -53,8 +53,7 @@ cudaError_t launch_quantize_dynamic(const QuantParams& p_in, int dtype, int meth
         else if (obj == 1) e = dyn_block<1, 0, 1>(p, fix, block, sms, s);
         else e = dyn_block<1, 0, 0>(p, fix, block, sms, s);
     }
-    if (e != cudaSuccess) return e;
-    return launch_swizzle_pad(p, sms, s);
+    return e;
 }
 
 }  // namespace nvfp4

@@ -279,11 +279,12 @@ __device__ __forceinline__ void sweep_segments(const GroupTensor& d, const Cand*
     int bestc;
     if (METHOD == 0) {
         float best;
-        const int I0 = e4m3_floor_code(__fdiv_rn(m, 6.0f));
+        const int I0 = e4m3_floor_code_of_sixth(m);
         const Cand* tb = tab + (I0 + FIX_LO + kTabOff);
-        bestc = I0 + FIX_LO + default_window_argmin<OBJ, BLOCK, true>(y2, w2, ma, mb, tb, best, wok);
+        bestc = I0 + FIX_LO + default_window_argmin<OBJ, BLOCK, true>(y2, w2, ma, mb, tb, best, wok,
+                                                                           octave_window<OBJ, BLOCK, true>(zero, I0));
     } else {
-        bestc = max((int)e4m3_rn_code(__fdiv_rn(m, 6.0f)), 1);
+        bestc = max((int)e4m3_rn_code(sixth(m)), 1);
     }
     uint32_t packed[2];
     if (zero) {
@@ -303,25 +304,25 @@ __device__ __forceinline__ void sweep_segments(const GroupTensor& d, const Cand*
         const float r = tab[bestc + kTabOff].r;
         const u64 r2 = pack2(r, r);
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            uint32_t b[4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                float lo, hi;
-                unpack2(mul2(y2[4 * h + j], r2), lo, hi);
-                b[j] = e2m1x2(lo, hi);
-            }
-            packed[h] = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
-        }
+        for (int h = 0; h < 2; h++)
+            packed[h] = e2m1x8(mul2(y2[4 * h], r2), mul2(y2[4 * h + 1], r2), mul2(y2[4 * h + 2], r2),
+                               mul2(y2[4 * h + 3], r2));
     }
     if (valid) {
         *reinterpret_cast<uint2*>(d.codes + g * 8) = make_uint2(packed[0], packed[1]);
         if ((g % SEGS) == 0) {
             if (d.sf_linear) d.sf_linear[blk] = (uint8_t)bestc;
             if (BLOCK == 16 && d.sf_swizzled) {
-                int64_t row, kbi;                               // recomputed here: not live across the sweep
-                row_col(row, kbi);
-                d.sf_swizzled[swizzle_offset(row, kbi, d.kpad4)] = (uint8_t)bestc;
+                // recomputed here: not live across the sweep
+                if (d.narrow) {
+                    const uint32_t r32 = fast_div((uint32_t)blk, d.kb_div);
+                    const uint32_t k32 = (uint32_t)blk - r32 * (uint32_t)d.kb;
+                    d.sf_swizzled[swizzle_offset32(r32, k32, (uint32_t)d.kpad4)] = (uint8_t)bestc;
+                } else {
+                    int64_t row, kbi;
+                    row_col(row, kbi);
+                    d.sf_swizzled[swizzle_offset(row, kbi, d.kpad4)] = (uint8_t)bestc;
+                }
             }
         }
     }
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>()
     Raw cur;
     if (cbase < total) {
         const int64_t g = cbase + tid - p.t[t].seg_begin;
-        if (g < p.t[t].nseg) load_raw<DT>(p.t[t].x, g, cur);
+        if (g < p.t[t].nseg) load_raw<DT>(p.t[t].x, g, METHOD != 1 && wide_input(p.t[t].x), cur);
     }
 
     while (cbase < total) {
@@ -407,17 +408,20 @@ __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>()
             Raw nxt;
             const int64_t nb = cbase + stride;
             if (nb < seg_end) {
-                if (g + stride < d.nseg) load_raw<DT>(d.x, g + stride, nxt);
+                if (g + stride < d.nseg) load_raw<DT>(d.x, g + stride, METHOD != 1 && wide_input(d.x), nxt);
             } else if (nb < total) {
                 const int tn = tensor_at(p, t, nb);
                 const int64_t gn = nb + tid - p.t[tn].seg_begin;
-                if (gn < p.t[tn].nseg) load_raw<DT>(p.t[tn].x, gn, nxt);
+                if (gn < p.t[tn].nseg) load_raw<DT>(p.t[tn].x, gn, METHOD != 1 && wide_input(p.t[tn].x), nxt);
             }
             sweep_segments<DT, METHOD, OBJ, BLOCK>(d, tab, cur, g, valid, E2, usable, w2, wkey, wok);
             cur = nxt;
         }
         t = tensor_at(p, t, cbase);
     }
+    if (BLOCK == 16)
+        for (int a = 0; a < count; a++)
+            zero_pads(p.t[a].sf_swizzled, p.t[a].rows, p.t[a].kb, p.t[a].kpad4, (int64_t)blockIdx.x * SW + tid, stride);
 }
 
 }  // namespace
@@ -586,22 +590,11 @@ cudaError_t launch_method(const GroupParams& p, int method, int obj, int block, 
 
 }  // namespace
 
-cudaError_t launch_quantize_group(const GroupParams& p, const int64_t* rows, int dtype, int method, int obj,
-                                  int block, int sms, cudaStream_t s) {
+cudaError_t launch_quantize_group(const GroupParams& p, int dtype, int method, int obj, int block, int sms,
+                                  cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     if (p.total_seg > 0 || p.dyn) {
         e = dtype == 0 ? launch_method<0>(p, method, obj, block, sms, s) : launch_method<1>(p, method, obj, block, sms, s);
-        if (e != cudaSuccess) return e;
-    }
-    for (int i = 0; i < p.count; i++) {
-        const GroupTensor& T = p.t[i];
-        if (!T.sf_swizzled) continue;
-        QuantParams q{};
-        q.sf_swizzled = T.sf_swizzled;
-        q.rows = rows[i];
-        q.kb = T.kb;
-        q.kpad4 = T.kpad4;
-        e = launch_swizzle_pad(q, sms, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

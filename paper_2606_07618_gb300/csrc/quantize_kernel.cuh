@@ -75,20 +75,23 @@ struct Raw {
     uint4 a, b, c, d;
 };
 
+// wide: x is 32-byte aligned (every segment then is too).
 template <int DT>
-__device__ __forceinline__ void load_raw(const void* x, int64_t g, Raw& r) {
-    if (DT == 0) {
-        const uint4* p = reinterpret_cast<const uint4*>(static_cast<const char*>(x) + g * 32);
-        r.a = ld_stream16(p);
-        r.b = ld_stream16(p + 1);
+__device__ __forceinline__ void load_raw(const void* x, int64_t g, bool wide, Raw& r) {
+    const char* p = static_cast<const char*>(x) + g * (DT == 0 ? 32 : 64);
+    if (wide) {
+        ld_stream32(p, r.a, r.b);
+        if (DT != 0) ld_stream32(p + 32, r.c, r.d);
     } else {
-        const uint4* p = reinterpret_cast<const uint4*>(static_cast<const char*>(x) + g * 64);
         r.a = ld_stream16(p);
-        r.b = ld_stream16(p + 1);
-        r.c = ld_stream16(p + 2);
-        r.d = ld_stream16(p + 3);
+        r.b = ld_stream16(p + 16);
+        if (DT != 0) {
+            r.c = ld_stream16(p + 32);
+            r.d = ld_stream16(p + 48);
+        }
     }
 }
+__device__ __forceinline__ bool wide_input(const void* x) { return (reinterpret_cast<uintptr_t>(x) & 31) == 0; }
 
 // NaN-propagating maxima: the block max is NaN if any element is NaN, so a
 // block holding a non-finite value is recognised from m alone (zero_block).
@@ -199,6 +202,30 @@ __device__ __forceinline__ float seg_loss(const u64 (&y2)[8], const u64 (&w2)[8]
     return __fadd_rn(a, b);
 }
 
+// Losses of codes c (r, nv) and c + 8 = twice the scale: fl(y fl(1/2v)) is half of
+// fl(y fl(1/v)), so the second code's multiply takes a constant operand.  The loop is
+// bound by register reads (two per cycle: a packed multiply-add with three operands
+// of its own takes 3 cycles, not 2), of which that saves two per element pair.
+template <int OBJ>
+__device__ __forceinline__ void seg_loss_octave(const u64 (&y2)[8], const u64 (&w2)[8], float r, uint16_t nv, float& L0,
+                                                float& L1) {
+    const u64 r2 = pack2(r, r), half2 = pack2(0.5f, 0.5f);
+    const uint16_t nv1 = (uint16_t)(nv + 0x0400u);               // -2 v: one f16 exponent up
+    u64 a0 = 0ull, a1 = 0ull;
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        const u64 t = mul2(y2[j], r2);
+        const u64 e = err2_of_t(t, y2[j], nv), f = err2_of_t(mul2(t, half2), y2[j], nv1);
+        a0 = fma2(OBJ == 1 ? mul2(w2[j], e) : e, e, a0);
+        a1 = fma2(OBJ == 1 ? mul2(w2[j], f) : f, f, a1);
+    }
+    float a, b;
+    unpack2(a0, a, b);
+    L0 = __fadd_rn(a, b);
+    unpack2(a1, a, b);
+    L1 = __fadd_rn(a, b);
+}
+
 template <int SEGS>
 __device__ __forceinline__ float group_sum(float v) {
     if (SEGS >= 2) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 1));
@@ -261,22 +288,64 @@ __host__ __device__ constexpr int bound_offsets() {
     return OBJ != 0 ? 4 : (BLOCK == 16 ? (GROUPED ? 2 : 1) : 6);
 }
 
+//
+// octave (WMSE, whose windows hold four pairs above the bounded offsets; MSE windows
+// hold one or two, and the second copy of the loop cost more than it gave): every
+// code above the bounded offsets is a normal E4M3 code
+// and the last one at most 126, so that code k + 8 is twice code k.  A warp all of
+// whose lanes say so scores those pairs together (seg_loss_octave): the same losses,
+// compared in ascending order within the lower, the middle and the upper codes
+// and then between them, so ties still go to the lowest code.
 template <int OBJ, int BLOCK, bool GROUPED>
 __device__ __forceinline__ int default_window_argmin(const u64 (&y2)[8], const u64 (&w2)[8], float ma, float mb,
-                                                     const Cand* tb, float& best, bool wok = true) {
+                                                     const Cand* tb, float& best, bool wok, bool octave) {
     constexpr int SEGS = BLOCK / 16;
     constexpr int FIX_LO = (OBJ == 0 && BLOCK == 16) ? -3 : -8;
     constexpr int FIX_K = 7 - FIX_LO + 1;
     constexpr int NB = bound_offsets<OBJ, BLOCK, GROUPED>();
     best = __int_as_float(0x7f800000);
     int bk = 0;
+    if (OBJ == 1 && __all_sync(0xffffffffu, octave)) {
+        float bu = __int_as_float(0x7f800000);
+        int ku = 0;
 #pragma unroll
-    for (int k = NB; k < FIX_K; k++) {
-        const Cand cd = tb[k];
-        const float L = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, cd.r, (uint16_t)cd.nv));
-        if (L < best) {
-            best = L;
-            bk = k;
+        for (int k = NB; k < FIX_K - 8; k++) {
+            const Cand cd = tb[k];
+            float L, Lu;
+            seg_loss_octave<OBJ>(y2, w2, cd.r, (uint16_t)cd.nv, L, Lu);
+            L = group_sum<SEGS>(L);
+            Lu = group_sum<SEGS>(Lu);
+            if (L < best) {
+                best = L;
+                bk = k;
+            }
+            if (Lu < bu) {
+                bu = Lu;
+                ku = k + 8;
+            }
+        }
+#pragma unroll
+        for (int k = FIX_K - 8; k < NB + 8; k++) {
+            const Cand cd = tb[k];
+            const float L = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, cd.r, (uint16_t)cd.nv));
+            if (L < best) {
+                best = L;
+                bk = k;
+            }
+        }
+        if (bu < best) {
+            best = bu;
+            bk = ku;
+        }
+    } else {
+#pragma unroll
+        for (int k = NB; k < FIX_K; k++) {
+            const Cand cd = tb[k];
+            const float L = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, cd.r, (uint16_t)cd.nv));
+            if (L < best) {
+                best = L;
+                bk = k;
+            }
         }
     }
     if (NB == 0) return bk;
@@ -316,6 +385,15 @@ __device__ __forceinline__ int default_window_argmin(const u64 (&y2)[8], const u
     return bk;
 }
 
+// The `octave` of default_window_argmin for a block's base code (a zero block's
+// losses are not read).
+template <int OBJ, int BLOCK, bool GROUPED>
+__device__ __forceinline__ bool octave_window(bool zero, int I0) {
+    constexpr int FIX_LO = (OBJ == 0 && BLOCK == 16) ? -3 : -8;
+    constexpr int LOW = 8 - FIX_LO - bound_offsets<OBJ, BLOCK, GROUPED>();     // I0 whose first code is 8
+    return zero || (unsigned)(I0 - LOW) <= (unsigned)(119 - LOW);
+}
+
 // Whether all 16 weights of a segment are non-negative (NaN counts as not).
 __device__ __forceinline__ bool weights_nonneg(const u64 (&w2)[8]) {
     float lo = __int_as_float(0x7f800000);
@@ -333,10 +411,6 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv& d) {
     const uint32_t t = __umulhi(n, d.mul);
     return (t + ((n - t) >> d.s1)) >> d.s2;
 }
-
-#ifndef NVFP4_QMINB
-#define NVFP4_QMINB 1
-#endif
 
 
 // Dynamic (per-call) global scale inside the sweep launch: every CTA folds the
@@ -459,7 +533,27 @@ __device__ __forceinline__ bool dynamic_scale(const QuantParams& p, float& S_out
     return true;
 }
 
-// FIX = 1: default window (fixed length, unrolled, poison-padded table).
+// Zero the padding bytes of a swizzled scale buffer (rows past `rows` up to a
+// multiple of 128, scale columns past `kb` up to a multiple of 4), thread `i` of
+// `n`: part of the sweep's own launch, since one of its own costs a small call as
+// much as the sweep does.
+__device__ __forceinline__ void zero_pads(uint8_t* sf, int64_t rows, int64_t kb, int64_t kpad4, int64_t i, int64_t n) {
+    if (!sf || ((rows & 127) == 0 && (kb & 3) == 0)) return;
+    const int64_t total = (((rows + 127) & ~(int64_t)127) - rows) * kpad4;      // groups of 4 bytes
+    const bool words = (reinterpret_cast<uintptr_t>(sf) & 3) == 0;
+    for (int64_t j = i; j < total; j += n) {
+        const int64_t q = total <= 0x7FFFFFFF ? (int64_t)((uint32_t)j / (uint32_t)kpad4) : j / kpad4;
+        uint8_t* d = sf + swizzle_offset(rows + q, (j - q * kpad4) * 4, kpad4);
+        if (words) *reinterpret_cast<uint32_t*>(d) = 0u;
+        else
+            for (int b = 0; b < 4; b++) d[b] = 0;
+    }
+    if (kb & 3)
+        for (int64_t r = i; r < rows; r += n)
+            for (int64_t k = kb; k < kpad4 * 4; k++) sf[swizzle_offset(r, k, kpad4)] = 0;
+}
+
+// quantize_kernel.  FIX = 1: default window (fixed length, unrolled, poison-padded table).
 // DYN = 1: the global scale is computed in this launch (see dynamic_scale).
 // On bf16 input, AbsMax is held to 64 registers (4 CTAs per SM) and 4/6 to 80
 // (3 CTAs per SM): both are issue- and latency-bound, not register-bound (AbsMax
@@ -467,13 +561,173 @@ __device__ __forceinline__ bool dynamic_scale(const QuantParams& p, float& S_out
 // fp32-input forms would spill, and the ScaleSweep sweeps run slower, at such bounds).
 template <int METHOD, int DT>
 constexpr int quantize_min_blocks() {
-    return DT != 0 ? NVFP4_QMINB : (METHOD == 1 ? 4 : (METHOD == 2 ? 3 : NVFP4_QMINB));
+    return METHOD == 0 ? 2 : DT != 0 ? 1 : (METHOD == 1 ? 4 : 3);
+}
+
+// One 16-element segment: its block's scale, nibbles, scale bytes and loss.  tab:
+// the candidate table; w2, wkey: the lane's weights and where they came from.
+template <int DT, int METHOD, int OBJ, int BLOCK, int FIX>
+__device__ __forceinline__ void quantize_segment(const QuantParams& p, const Cand* tab, const Raw& cur, int64_t g,
+                                                 bool valid, u64 E2, bool usable, u64 (&w2)[8], const float*& wkey) {
+    constexpr int SEGS = BLOCK / 16;
+    constexpr int FIX_LO = (OBJ == 0 && BLOCK == 16) ? -3 : -8;
+    u64 y2[8];
+    float m = 0.0f, ma = 0.0f, mb = 0.0f;         // ma, mb: largest |y| of each half (offset bound)
+    if (valid) {
+        m = METHOD == 0 ? raw_to_y_halves<DT>(cur, E2, y2, ma, mb) : raw_to_y<DT>(cur, E2, y2);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; j++) y2[j] = 0ull;
+    }
+    m = group_max<SEGS>(m);
+
+    const int64_t blk = g / SEGS;               // scale-block index
+    int64_t row = 0, kbi = 0;
+    uint32_t row32 = 0, kbi32 = 0;              // narrow: rows * kb < 2^32
+    if (p.need_rowcol) {
+        if (p.narrow) {
+            row32 = fast_div((uint32_t)blk, p.kb_div);
+            kbi32 = (uint32_t)blk - row32 * (uint32_t)p.kb;
+            row = row32;
+            kbi = kbi32;
+        } else {
+            row = blk / p.kb;
+            kbi = blk - row * p.kb;
+        }
+    }
+
+    if (OBJ == 1) {
+        const int64_t col = kbi * BLOCK + (int64_t)(g % SEGS) * 16;
+        const float* wp = p.w + row * p.w_row_stride + col;
+        if (valid && (METHOD == 0 || wp != wkey)) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const uint4 a = ld_ro16(wp + 4 * j);
+                w2[2 * j] = pack2(__uint_as_float(a.x), __uint_as_float(a.y));
+                w2[2 * j + 1] = pack2(__uint_as_float(a.z), __uint_as_float(a.w));
+            }
+            wkey = wp;
+        } else if (METHOD == 0) {
+#pragma unroll
+            for (int j = 0; j < 8; j++) w2[j] = 0ull;
+        }
+    }
+
+    const bool zero = zero_block(usable, m);
+    float best = __int_as_float(0x7f800000);
+    int bestc = 0;
+    if (METHOD == 0) {
+        const int I0 = e4m3_floor_code_of_sixth(m);
+        if (FIX) {
+            // the lane's weights are reloaded every segment, so their signs
+            // are checked every segment too
+            const Cand* tb = tab + (I0 + FIX_LO + kTabOff);
+            bestc = I0 + FIX_LO + default_window_argmin<OBJ, BLOCK, false>(
+                                        y2, w2, ma, mb, tb, best, OBJ == 0 || weights_nonneg(w2),
+                                        octave_window<OBJ, BLOCK, false>(zero, I0));
+        } else {
+            int lo_off = p.win_lo;
+            if ((p.tight & 2) && I0 >= 16 && I0 <= 120) {
+                const int b = I0 & 7;                       // Table 2: ceil(4/5 s) is 2 or 3 codes down
+                lo_off = (b == 0 || b == 7) ? -3 : -2;
+            }
+            const int clo = min(max(I0 + lo_off, 1), 126);
+            int chi = min(max(I0 + p.win_hi, 1), 126);
+            if (p.tight & 1) {     // Lemma 4.1: 3.5 v_c > m never beats v_c / 2 = code c - 8 (c >= 16)
+                while (chi > clo && chi >= 16 &&
+                       __fmul_rn(3.5f, f16bits_to_f32((uint16_t)(tab[chi + kTabOff].nv ^ 0x8000u))) > m)
+                    chi--;
+            }
+            const int n = zero ? 0 : chi - clo + 1;
+            const int nmax = __reduce_max_sync(0xffffffffu, (unsigned)n);
+            bestc = clo;
+            for (int k = 0; k < nmax; k++) {
+                const int c = min(clo + k, chi);    // repeats of chi never win the strict "<"
+                const Cand cd = tab[c + kTabOff];
+                const float L = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, cd.r, (uint16_t)cd.nv));
+                if (L < best) {
+                    best = L;
+                    bestc = c;
+                }
+            }
+        }
+    } else {
+        const int c6 = max((int)e4m3_rn_code(sixth(m)), 1);
+        bestc = c6;
+        if (METHOD == 2) {
+            const int c4 = max((int)e4m3_rn_code(__fmul_rn(m, 0.25f)), 1);
+            const Cand d6 = tab[c6 + kTabOff], d4 = tab[c4 + kTabOff];
+            const float L6 = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, d6.r, (uint16_t)d6.nv));
+            const float L4 = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, d4.r, (uint16_t)d4.nv));
+            best = L6;
+            if (L4 < L6) {
+                best = L4;
+                bestc = c4;
+            }
+        } else if (p.block_loss) {
+            const Cand d6 = tab[c6 + kTabOff];
+            best = group_sum<SEGS>(seg_loss<0>(y2, w2, d6.r, (uint16_t)d6.nv));
+        }
+    }
+
+    // Emit packed nibbles for this thread's 16 elements.
+    uint32_t packed[2];
+    if (zero) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            uint32_t acc = 0;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                float a, b;
+                unpack2(y2[4 * h + j], a, b);
+                const uint32_t byte = (signbit(a) ? 0x08u : 0u) | (signbit(b) ? 0x80u : 0u);
+                acc |= byte << (8 * j);
+            }
+            packed[h] = acc;
+        }
+        bestc = 0;
+        best = 0.0f;
+        if (p.block_loss) {
+            float s = 0.0f;
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                float a, b;
+                unpack2(y2[j], a, b);
+                if (OBJ == 1) {
+                    float wa, wb;
+                    unpack2(w2[j], wa, wb);
+                    s = __fmaf_rn(__fmul_rn(wa, a), a, s);
+                    s = __fmaf_rn(__fmul_rn(wb, b), b, s);
+                } else {
+                    s = __fmaf_rn(a, a, s);
+                    s = __fmaf_rn(b, b, s);
+                }
+            }
+            best = group_sum<SEGS>(s);
+        }
+    } else {
+        const float r = tab[bestc + kTabOff].r;
+        const u64 r2 = pack2(r, r);
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+            packed[h] = e2m1x8(mul2(y2[4 * h], r2), mul2(y2[4 * h + 1], r2), mul2(y2[4 * h + 2], r2),
+                               mul2(y2[4 * h + 3], r2));
+    }
+
+    if (valid) {
+        *reinterpret_cast<uint2*>(p.codes + g * 8) = make_uint2(packed[0], packed[1]);
+        if ((g % SEGS) == 0) {
+            if (p.sf_linear) p.sf_linear[blk] = (uint8_t)bestc;
+            if (p.sf_swizzled)
+                p.sf_swizzled[p.narrow ? swizzle_offset32(row32, kbi32, (uint32_t)p.kpad4)
+                                       : swizzle_offset(row, kbi, p.kpad4)] = (uint8_t)bestc;
+            if (p.block_loss) p.block_loss[blk] = best;
+        }
+    }
 }
 
 template <int DT, int METHOD, int OBJ, int BLOCK, int FIX, int DYN>
 __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quantize_kernel(QuantParams p) {
-    constexpr int SEGS = BLOCK / 16;
-    constexpr int FIX_LO = (OBJ == 0 && BLOCK == 16) ? -3 : -8;
     __shared__ Cand tab[kTabN];
     build_table(tab);
     __syncthreads();
@@ -493,176 +747,28 @@ __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quanti
     const int64_t nseg_pad = (p.nseg + 31) & ~(int64_t)31;
 
     int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+    const bool wide = METHOD != 1 && wide_input(p.x);      // AbsMax: 2% slower with 32-byte loads
     Raw cur;
-    if (base + lane < p.nseg) load_raw<DT>(p.x, base + lane, cur);
+    if (base + lane < p.nseg) load_raw<DT>(p.x, base + lane, wide, cur);
 
+    // 4/6 keeps a lane's weights while they come from the same address (the grid's
+    // stride is a multiple of a row's segments where it can be): four 16-byte loads 64
+    // bytes apart per lane were two thirds of its L1 traffic, and that bound it.  The
+    // sweep, bound elsewhere, is faster without 16 more loop-carried registers.
+    u64 w2[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) w2[j] = 0ull;
+    const float* wkey = nullptr;
     for (; base < nseg_pad; base += stride) {
         const int64_t g = base + lane;
         const bool valid = g < p.nseg;
         Raw nxt;
-        if (g + stride < p.nseg) load_raw<DT>(p.x, g + stride, nxt);
+        if (g + stride < p.nseg) load_raw<DT>(p.x, g + stride, wide, nxt);
 
-        u64 y2[8];
-        float m = 0.0f, ma = 0.0f, mb = 0.0f;         // ma, mb: largest |y| of each half (offset bound)
-        if (valid) {
-            m = METHOD == 0 ? raw_to_y_halves<DT>(cur, E2, y2, ma, mb) : raw_to_y<DT>(cur, E2, y2);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 8; j++) y2[j] = 0ull;
-        }
-        m = group_max<SEGS>(m);
+        quantize_segment<DT, METHOD, OBJ, BLOCK, FIX>(p, tab, cur, g, valid, E2, usable, w2, wkey);
         cur = nxt;
-
-        const int64_t blk = g / SEGS;               // scale-block index
-        int64_t row = 0, kbi = 0;
-        if (p.need_rowcol) {
-            if (p.narrow) {
-                const uint32_t b32 = (uint32_t)blk;
-                const uint32_t r32 = fast_div(b32, p.kb_div);
-                row = r32;
-                kbi = b32 - r32 * (uint32_t)p.kb;
-            } else {
-                row = blk / p.kb;
-                kbi = blk - row * p.kb;
-            }
-        }
-
-
-        u64 w2[8];
-        if (OBJ == 1) {
-            const int64_t col = kbi * BLOCK + (int64_t)(g % SEGS) * 16;
-            const float* wp = p.w + row * p.w_row_stride + col;
-            if (valid) {
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint4 a = ld_ro16(wp + 4 * j);
-                    w2[2 * j] = pack2(__uint_as_float(a.x), __uint_as_float(a.y));
-                    w2[2 * j + 1] = pack2(__uint_as_float(a.z), __uint_as_float(a.w));
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 8; j++) w2[j] = 0ull;
-            }
-        }
-
-        const bool zero = zero_block(usable, m);
-        float best = __int_as_float(0x7f800000);
-        int bestc = 0;
-        if (METHOD == 0) {
-            const float sbase = __fdiv_rn(m, 6.0f);
-            const int I0 = e4m3_floor_code(sbase);
-            if (FIX) {
-                // the lane's weights are reloaded every segment, so their signs
-                // are checked every segment too
-                const Cand* tb = tab + (I0 + FIX_LO + kTabOff);
-                bestc = I0 + FIX_LO + default_window_argmin<OBJ, BLOCK, false>(y2, w2, ma, mb, tb, best,
-                                                                               OBJ == 0 || weights_nonneg(w2));
-            } else {
-                int lo_off = p.win_lo;
-                if ((p.tight & 2) && I0 >= 16 && I0 <= 120) {
-                    const int b = I0 & 7;                       // Table 2: ceil(4/5 s) is 2 or 3 codes down
-                    lo_off = (b == 0 || b == 7) ? -3 : -2;
-                }
-                const int clo = min(max(I0 + lo_off, 1), 126);
-                int chi = min(max(I0 + p.win_hi, 1), 126);
-                if (p.tight & 1) {     // Lemma 4.1: 3.5 v_c > m never beats v_c / 2 = code c - 8 (c >= 16)
-                    while (chi > clo && chi >= 16 &&
-                           __fmul_rn(3.5f, f16bits_to_f32((uint16_t)(tab[chi + kTabOff].nv ^ 0x8000u))) > m)
-                        chi--;
-                }
-                const int n = zero ? 0 : chi - clo + 1;
-                const int nmax = __reduce_max_sync(0xffffffffu, (unsigned)n);
-                bestc = clo;
-                for (int k = 0; k < nmax; k++) {
-                    const int c = min(clo + k, chi);    // repeats of chi never win the strict "<"
-                    const Cand cd = tab[c + kTabOff];
-                    const float L = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, cd.r, (uint16_t)cd.nv));
-                    if (L < best) {
-                        best = L;
-                        bestc = c;
-                    }
-                }
-            }
-        } else {
-            const float sbase = __fdiv_rn(m, 6.0f);
-            const int c6 = max((int)e4m3_rn_code(sbase), 1);
-            bestc = c6;
-            if (METHOD == 2) {
-                const int c4 = max((int)e4m3_rn_code(__fdiv_rn(m, 4.0f)), 1);
-                const Cand d6 = tab[c6 + kTabOff], d4 = tab[c4 + kTabOff];
-                const float L6 = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, d6.r, (uint16_t)d6.nv));
-                const float L4 = group_sum<SEGS>(seg_loss<OBJ>(y2, w2, d4.r, (uint16_t)d4.nv));
-                best = L6;
-                if (L4 < L6) {
-                    best = L4;
-                    bestc = c4;
-                }
-            } else if (p.block_loss) {
-                const Cand d6 = tab[c6 + kTabOff];
-                best = group_sum<SEGS>(seg_loss<0>(y2, w2, d6.r, (uint16_t)d6.nv));
-            }
-        }
-
-        // Emit packed nibbles for this thread's 16 elements.
-        uint32_t packed[2];
-        if (zero) {
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                uint32_t acc = 0;
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    float a, b;
-                    unpack2(y2[4 * h + j], a, b);
-                    const uint32_t byte = (signbit(a) ? 0x08u : 0u) | (signbit(b) ? 0x80u : 0u);
-                    acc |= byte << (8 * j);
-                }
-                packed[h] = acc;
-            }
-            bestc = 0;
-            best = 0.0f;
-            if (p.block_loss) {
-                float s = 0.0f;
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    float a, b;
-                    unpack2(y2[j], a, b);
-                    if (OBJ == 1) {
-                        float wa, wb;
-                        unpack2(w2[j], wa, wb);
-                        s = __fmaf_rn(__fmul_rn(wa, a), a, s);
-                        s = __fmaf_rn(__fmul_rn(wb, b), b, s);
-                    } else {
-                        s = __fmaf_rn(a, a, s);
-                        s = __fmaf_rn(b, b, s);
-                    }
-                }
-                best = group_sum<SEGS>(s);
-            }
-        } else {
-            const float r = tab[bestc + kTabOff].r;
-            const u64 r2 = pack2(r, r);
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                uint32_t b[4];
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    float lo, hi;
-                    unpack2(mul2(y2[4 * h + j], r2), lo, hi);
-                    b[j] = e2m1x2(lo, hi);
-                }
-                packed[h] = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
-            }
-        }
-
-        if (valid) {
-            *reinterpret_cast<uint2*>(p.codes + g * 8) = make_uint2(packed[0], packed[1]);
-            if ((g % SEGS) == 0) {
-                if (p.sf_linear) p.sf_linear[blk] = (uint8_t)bestc;
-                if (p.sf_swizzled) p.sf_swizzled[swizzle_offset(row, kbi, p.kpad4)] = (uint8_t)bestc;
-                if (p.block_loss) p.block_loss[blk] = best;
-            }
-        }
     }
+    zero_pads(p.sf_swizzled, p.rows, p.kb, p.kpad4, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride);
 }
 
 
