@@ -408,14 +408,13 @@ nvfp4_status nvfp4_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
  * U_ik, What_k = Q(T_k), with Q the sweep's fp32 rounding at the fixed scale:
  * y = fl(T*E), q = RNE_E2M1(fl(y*fl(1/v))), What = fl(fl(q*v)*S); a zero scale
  * code or an unusable S quantizes to signed zeros, an exactly zero y to +0.
- *   The error-feedback updates run on the tensor cores (three TF32 products
- *   per term, as in nvfp4_ldlq_prepare; status bit 16 as there) when rows and
- *   cols are multiples of 4 and the buffers 16-byte aligned, else on the FP32
- *   pipe.
+ *   The error-feedback updates past a super-panel of 256 columns run on the
+ *   tensor cores (three TF32 products per term, as in nvfp4_ldlq_prepare; status
+ *   bit 16 as there, also for the bounded wait for U within a super-panel).
  *   perm, U from nvfp4_ldlq_prepare (cols = n); status_dev optional: |= 8 if
  *   perm holds an index outside [0, cols) (the entry is then read as 0).
  *   workspace   device bytes, at least nvfp4_ldlq_workspace(rows, cols):
- *           rows*cols*10 + rows*2048 + cols*4 plus alignment.
+ *           rows*cols*10 + rows*4096 + cols*4100 plus alignment.
  * Cost: rows*cols^2/2 fp32 multiply-adds; rows are independent.  The column
  * walk uses the high-priority stream described under nvfp4_ldlq_prepare (same
  * first-call and concurrency rules).

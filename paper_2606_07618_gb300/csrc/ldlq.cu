@@ -347,15 +347,16 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
     }
 }
 
-// The rows i >= k0 + 64 of one panel, 32 per CTA: the solved panel X = A Linv^T
-// (in place), then the next panel's block column, A[i][k0 + 64 ..] -= X Xtop^T, up
+// The rows i >= k0 + 64 of one panel, 32 per CTA: the solved panel X = A Linv^T (in
+// place, and split into TF32 halves Lh, Ll [n, 64] for the trailing update), then the next panel's block column, A[i][k0 + 64 ..] -= X Xtop^T, up
 // to column i.  Everything in fp32 from shared memory; a separate panel solve and a
 // tensor-core update of a 64-wide column spent 14 us here on launches, tile fills
 // and half-empty tiles.
 constexpr int kPanelRows = 32;
 constexpr int kPanelSmem = (2 * kP + 2 * kPanelRows) * kPad * 4;
 template <bool VEC>
-__global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t k0, const float* Linv, const float* Xtop) {
+__global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t k0, const float* Linv, const float* Xtop,
+                                                    float* Lh, float* Ll) {
     extern __shared__ __align__(16) float psm[];
     float* sl = psm;                                 // [64][kPad] Linv
     float* st = sl + kP * kPad;                      // [64][kPad] Xtop
@@ -410,7 +411,12 @@ __global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t
         if (r >= n) continue;
         float* a = A + r * n + k0 + 4 * tx;
         if (VEC) {
-            *reinterpret_cast<float4*>(a) = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+            const float4 x = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+            *reinterpret_cast<float4*>(a) = x;
+            float4 h, l;                              // the trailing update's operands
+            tc::split4(x, h, l);
+            *reinterpret_cast<float4*>(Lh + r * kP + 4 * tx) = h;
+            *reinterpret_cast<float4*>(Ll + r * kP + 4 * tx) = l;
             if (c0 + 3 <= r) vc[i] = *reinterpret_cast<const float4*>(A + r * n + c0);
         } else {
 #pragma unroll
@@ -434,9 +440,8 @@ __global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t
     }
 }
 
-// C[M, N] += alpha * op(A) * op(B).  op(A) = A [M, K] row-major, or (AT) A^T
-// with A stored [K, M] row-major; op(B) = B [K, N] row-major, or (BT) B^T with
-// B stored [N, K] row-major.  128 x 128 tiles, 256 threads, 8 x 8 outputs per
+// C[M, N] += alpha * A * op(B), A [M, K] row-major; op(B) = B [K, N] row-major, or
+// (BT) B^T with B stored [N, K] row-major.  128 x 128 tiles, 256 threads, 8 x 8 outputs per
 // thread, K in stages of 32 through two shared buffers filled by cp.async
 // (global to shared without registers) while the other stage is multiplied.
 // LOWER skips tiles entirely above the diagonal (n0 > m0 + 127).  VEC: C rows
@@ -449,7 +454,7 @@ __device__ __forceinline__ void cp_async4(float* dst, const float* src, bool val
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
 }
 
-template <bool AT, bool BT, bool LOWER, bool VEC>
+template <bool BT, bool LOWER, bool VEC>
 __global__ void __launch_bounds__(256, 2) gemm_kernel(float* C, int64_t ldc, const float* A, int64_t lda,
                                                       const float* B, int64_t ldb, int64_t M, int64_t N, int K,
                                                       float alpha) {
@@ -466,11 +471,7 @@ __global__ void __launch_bounds__(256, 2) gemm_kernel(float* C, int64_t ldc, con
 #pragma unroll
         for (int i = 0; i < 16; i++) {
             const int e = tid + 256 * i;
-            if (AT) {
-                const int k = e / 128, mm = e % 128;
-                const bool ok = k0 + k < K && m0 + mm < M;
-                cp_async4(as + k * kLd + mm, ok ? A + (int64_t)(k0 + k) * lda + m0 + mm : A, ok);
-            } else {
+            {
                 const int mm = e / kBK, k = e % kBK;
                 const bool ok = k0 + k < K && m0 + mm < M;
                 cp_async4(as + k * kLd + mm, ok ? A + (m0 + mm) * lda + k0 + k : A, ok);
@@ -553,7 +554,7 @@ __global__ void __launch_bounds__(256, 2) gemm_kernel(float* C, int64_t ldc, con
     }
 }
 
-template <bool AT, bool BT, bool LOWER, bool VEC>
+template <bool BT, bool LOWER, bool VEC>
 cudaError_t launch_gemm_t(float* C, int64_t ldc, const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M,
                           int64_t N, int K, float alpha, cudaStream_t s) {
     constexpr int kSmem = 4 * kBK * kLd * (int)sizeof(float);
@@ -562,34 +563,22 @@ cudaError_t launch_gemm_t(float* C, int64_t ldc, const float* A, int64_t lda, co
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(gemm_kernel<AT, BT, LOWER, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+        e = cudaFuncSetAttribute(gemm_kernel<BT, LOWER, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
     }
     const dim3 grid((unsigned)((N + 127) / 128), (unsigned)((M + 127) / 128));
-    gemm_kernel<AT, BT, LOWER, VEC><<<grid, 256, kSmem, s>>>(C, ldc, A, lda, B, ldb, M, N, K, alpha);
+    gemm_kernel<BT, LOWER, VEC><<<grid, 256, kSmem, s>>>(C, ldc, A, lda, B, ldb, M, N, K, alpha);
     return cudaGetLastError();
 }
 
-template <bool AT, bool BT, bool LOWER>
+template <bool BT, bool LOWER>
 cudaError_t launch_gemm(float* C, int64_t ldc, const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M,
                         int64_t N, int K, float alpha, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     const bool vec = (ldc % 4 == 0) && ((reinterpret_cast<uintptr_t>(C) & 15) == 0);
-    return vec ? launch_gemm_t<AT, BT, LOWER, true>(C, ldc, A, lda, B, ldb, M, N, K, alpha, s)
-               : launch_gemm_t<AT, BT, LOWER, false>(C, ldc, A, lda, B, ldb, M, N, K, alpha, s);
-}
-
-// C += alpha op(A) op(B) for the LDLQ updates: on the tensor cores (tcgen05,
-// 3xTF32, tc_gemm.cuh) wherever its TMA alignment rules hold (16-byte aligned
-// bases and row strides), else with the SIMT fp32 GEMM above.  AT: A stored
-// [K][M]; BT: B stored [N][K] (the tensor-core GEMM's B_MN is !BT).
-template <bool AT, bool BT, bool LOWER>
-cudaError_t update_gemm(float* C, int64_t ldc, const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M,
-                        int64_t N, int K, float alpha, int* status, cudaStream_t s) {
-    const cudaError_t e = tc::launch_gemm<AT, !BT, LOWER>(C, ldc, A, lda, B, ldb, M, N, K, alpha, status, s);
-    if (e != cudaErrorNotSupported) return e;
-    return launch_gemm<AT, BT, LOWER>(C, ldc, A, lda, B, ldb, M, N, K, alpha, s);
+    return vec ? launch_gemm_t<BT, LOWER, true>(C, ldc, A, lda, B, ldb, M, N, K, alpha, s)
+               : launch_gemm_t<BT, LOWER, false>(C, ldc, A, lda, B, ldb, M, N, K, alpha, s);
 }
 
 __global__ void diag_d_kernel(const float* A, int64_t n, float* D) {
@@ -730,7 +719,8 @@ __device__ __forceinline__ void mma_16n8k8_tf32(float (&c)[4], const uint32_t (&
 
 // UVEC: U is 16-byte aligned (its rows then are too: n is a multiple of 16).
 template <bool UVEC>
-__global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int64_t s0, int span, float* EpT) {
+__global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int64_t s0, int span, float* Eh,
+                                                               float* El) {
     extern __shared__ __align__(16) float dsm[];
     __shared__ __align__(8) uint64_t s_ubar;
     float* ut = dsm;                                              // U, see u_row
@@ -945,9 +935,14 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
                 }
                 step_barrier();                        // publish before the global stores
                 if (active) {
-                    float* eg = EpT + (int64_t)g * kGroupCols * p.rows + r;
+                    float4 h, l;                       // the trailing update's operands, [rows, kLdlqPanel] TF32 halves
+                    const int64_t at = r * kLdlqPanel + g * kGroupCols;
 #pragma unroll
-                    for (int j = 0; j < 8; j++) eg[(int64_t)j * p.rows] = ev[j];
+                    for (int j = 0; j < 8; j += 4) {
+                        tc::split4(make_float4(ev[j], ev[j + 1], ev[j + 2], ev[j + 3]), h, l);
+                        *reinterpret_cast<float4*>(Eh + at + j) = h;
+                        *reinterpret_cast<float4*>(El + at + j) = l;
+                    }
                     *reinterpret_cast<uint2*>(p.qb + rbase + g * kGroupCols) = make_uint2(packed[0], packed[1]);
                 }
                 fetch(q + 1);
@@ -984,6 +979,27 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
     }
 }
 
+// The TF32 halves of U's rows s0 .. s0 + 255, columns c0 .. n - 1, transposed: Bh, Bl
+// [n - c0, kLdlqPanel], the trailing update's second operand.  32 x 32 tiles.
+__global__ void __launch_bounds__(256) split_u_kernel(const float* U, int64_t n, int64_t s0, int64_t c0, float* Bh, float* Bl) {
+    __shared__ float t[32][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int64_t c = c0 + (int64_t)blockIdx.x * 32;
+    const int k = (int)blockIdx.y * 32;
+#pragma unroll
+    for (int i = 0; i < 32; i += 8) t[y + i][x] = c + x < n ? U[(s0 + k + y + i) * n + c + x] : 0.0f;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 32; i += 8)
+        if (c + y + i < n) {
+            float h, l;
+            tc::split_tf32(t[x][y + i], h, l);
+            const int64_t at = (c + y + i - c0) * kLdlqPanel + k + x;
+            Bh[at] = h;
+            Bl[at] = l;
+        }
+}
+
 // codes[r][c/2]: nibble of original column c from qb[r][inv[c]]
 __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* qb, const int32_t* inv, int64_t rows, int64_t n,
                                                    uint8_t* codes, int* status) {
@@ -999,7 +1015,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* qb, const int3
 }  // namespace
 
 size_t ldlq_prepare_workspace(int64_t n) {
-    return (size_t)((n * 4 + 255) / 256 * 256) + 256 + (size_t)2 * kP * kP * 4;
+    return (size_t)((n * 4 + 255) / 256 * 256) + 256 + (size_t)2 * kP * kP * 4 + (size_t)2 * n * kP * 4;
 }
 
 // Stream and events of the factorization's look-ahead, one set per device,
@@ -1011,7 +1027,7 @@ size_t ldlq_prepare_workspace(int64_t n) {
 // cannot interleave.
 struct LookAhead {
     cudaStream_t crit = nullptr;
-    cudaEvent_t fork = nullptr, panel_done = nullptr, rest_done = nullptr, crit_done = nullptr;
+    cudaEvent_t fork = nullptr, panel_done = nullptr, rest_done = nullptr, crit_done = nullptr, split_done = nullptr;
 };
 
 cudaError_t lookahead_for_current_device(LookAhead** out, std::unique_lock<std::mutex>* lock) {
@@ -1027,7 +1043,7 @@ cudaError_t lookahead_for_current_device(LookAhead** out, std::unique_lock<std::
         int least = 0, greatest = 0;
         if ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest)) != cudaSuccess) return e;
         if ((e = cudaStreamCreateWithPriority(&la.crit, cudaStreamNonBlocking, greatest)) != cudaSuccess) return e;
-        cudaEvent_t* evs[4] = {&la.fork, &la.panel_done, &la.rest_done, &la.crit_done};
+        cudaEvent_t* evs[5] = {&la.fork, &la.panel_done, &la.rest_done, &la.crit_done, &la.split_done};
         for (cudaEvent_t* ev : evs)
             if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return e;
     }
@@ -1043,6 +1059,8 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     float* lam = reinterpret_cast<float*>(w + (n * 4 + 255) / 256 * 256);
     float* Linv = lam + 64;
     float* Xtop = Linv + kP * kP;
+    float* Lh = Xtop + kP * kP;          // the solved panel's TF32 halves, [n, 64] each
+    float* Ll = Lh + n * kP;
     diag_kernel<<<1, 1024, 0, s>>>(H, n, damp, d, lam, status);
     rank_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(d, n, perm);
     const unsigned rg = (unsigned)imin64(n, (int64_t)sms * 8);
@@ -1074,13 +1092,16 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
             const int64_t nb2 = imin64(kP, rest);      // width of the next panel
             // the next block column also took the previous panel's rest update
             if (have_rest && (e = cudaStreamWaitEvent(c, la->rest_done, 0)) != cudaSuccess) return e;
-            panel<<<(unsigned)((rest + kPanelRows - 1) / kPanelRows), 128, kPanelSmem, c>>>(U, n, k0, Linv, Xtop);
+            panel<<<(unsigned)((rest + kPanelRows - 1) / kPanelRows), 128, kPanelSmem, c>>>(U, n, k0, Linv, Xtop, Lh, Ll);
             if (rest > nb2) {
-                float* P = U + (k0 + nb + nb2) * n + k0;      // the solved panel's rows past the next block column
-                float* C = P + nb + nb2;
+                const int64_t i0 = k0 + nb + nb2, m = rest - nb2;
+                float* P = U + i0 * n + k0;            // the solved panel's rows past the next block column
                 if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(s, la->panel_done, 0)) != cudaSuccess) return e;
-                e = update_gemm<false, true, true>(C, n, P, n, P, n, rest - nb2, rest - nb2, nb, -1.0f, status, s);
+                const tc::Split L{Lh + i0 * kP, Ll + i0 * kP, kP};
+                e = vec ? tc::launch_gemm<true>(U + i0 * n + i0, n, L, L, m, m, nb, -1.0f, status, s) : cudaErrorNotSupported;
+                if (e == cudaErrorNotSupported)
+                    e = launch_gemm<true, true>(U + i0 * n + i0, n, P, n, P, n, m, m, nb, -1.0f, s);
                 if (e != cudaSuccess) return e;
                 if ((e = cudaEventRecord(la->rest_done, s)) != cudaSuccess) return e;
                 have_rest = true;
@@ -1098,11 +1119,13 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     return cudaGetLastError();
 }
 
-// Workspace: T and Wp [rows, n] f32, qb and sfp [rows, n] bytes, two EpT
-// [kLdlqPanel, rows] f32 (alternating between super-panels), inv [n].
+// Workspace: T and Wp [rows, n] f32, qb and sfp [rows, n] bytes, inv [n], and, twice
+// (alternating between super-panels), the TF32 halves of a super-panel's errors
+// [rows, kLdlqPanel] and of its rows of U [n, kLdlqPanel].
 size_t ldlq_quantize_workspace(int64_t rows, int64_t n) {
     auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
-    return (size_t)(2 * up(rows * n * 4) + 2 * up(rows * n) + 2 * up((int64_t)kLdlqPanel * rows * 4) + up(n * 4));
+    return (size_t)(2 * up(rows * n * 4) + 2 * up(rows * n) + 4 * up((int64_t)kLdlqPanel * rows * 4) +
+                    4 * up((int64_t)kLdlqPanel * n * 4) + up(n * 4));
 }
 
 // Columns in super-panels of kLdlqPanel (256), each walked by walk_kernel; after
@@ -1110,7 +1133,8 @@ size_t ldlq_quantize_workspace(int64_t rows, int64_t n) {
 // are read and written once per 256 columns.  Look-ahead: that update
 // is split into the next super-panel's columns, which run with its panel walks
 // on the high-priority stream, and the rest, which runs on `s` concurrently
-// with them; the super-panels' errors alternate between two EpT buffers.
+// with them.  Before the rest of super-panel k, `s` also transposes and splits the rows
+// of U that super-panel k + 1 will need.
 cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* ws, int sms, cudaStream_t s) {
     if (p.rows <= 0 || p.n <= 0) return cudaSuccess;
     auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
@@ -1120,10 +1144,14 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     p.Wp = reinterpret_cast<float*>(w + mat4);
     p.qb = reinterpret_cast<uint8_t*>(w + 2 * mat4);
     p.sfp = reinterpret_cast<uint8_t*>(w + 2 * mat4 + mat1);
-    const int64_t ep = up((int64_t)kLdlqPanel * p.rows * 4);
-    float* EpTs[2] = {reinterpret_cast<float*>(w + 2 * mat4 + 2 * mat1),
-                      reinterpret_cast<float*>(w + 2 * mat4 + 2 * mat1 + ep)};
-    int32_t* inv = reinterpret_cast<int32_t*>(w + 2 * mat4 + 2 * mat1 + 2 * ep);
+    const int64_t ep = up((int64_t)kLdlqPanel * p.rows * 4), up4 = up((int64_t)kLdlqPanel * p.n * 4);
+    char* q = w + 2 * mat4 + 2 * mat1;
+    tc::Split Es[2], Us[2];                        // ld = kLdlqPanel
+    for (int i = 0; i < 2; i++, q += 2 * ep + 2 * up4) {
+        Es[i] = {reinterpret_cast<float*>(q), reinterpret_cast<float*>(q + ep), kLdlqPanel};
+        Us[i] = {reinterpret_cast<float*>(q + 2 * ep), reinterpret_cast<float*>(q + 2 * ep + up4), kLdlqPanel};
+    }
+    int32_t* inv = reinterpret_cast<int32_t*>(q);
     cudaError_t e = cudaMemsetAsync(inv, 0, (size_t)p.n * 4, s);
     if (e != cudaSuccess) return e;
     invperm_kernel<<<(unsigned)((p.n + 255) / 256), 256, 0, s>>>(p.perm, p.n, inv, p.status);
@@ -1156,29 +1184,47 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     if ((e = cudaEventRecord(la->fork, s)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(c, la->fork, 0)) != cudaSuccess) return e;
     bool have_rest = false;              // rest_done recorded by this call (waits stay inside a capture)
+    // the second operand of super-panel s0's trailing updates
+    auto split_u = [&](int64_t s0, int i) {
+        const int64_t c0 = s0 + kLdlqPanel;
+        if (c0 >= p.n) return cudaSuccess;
+        split_u_kernel<<<dim3((unsigned)((p.n - c0 + 31) / 32), kLdlqPanel / 32), 256, 0, s>>>(
+            p.U, p.n, s0, c0, const_cast<float*>(Us[i].hi), const_cast<float*>(Us[i].lo));
+        const cudaError_t r = cudaGetLastError();
+        return r != cudaSuccess ? r : cudaEventRecord(la->split_done, s);
+    };
+    // T[:, c0 + d ..] += the errors of super-panel s0 x U, `cols` columns from column d of its trailing ones
+    auto update = [&](int64_t s0, int i, int64_t d, int64_t cols, cudaStream_t st) {
+        float* C = p.T + s0 + kLdlqPanel + d;
+        const tc::Split B{Us[i].hi + d * kLdlqPanel, Us[i].lo + d * kLdlqPanel, kLdlqPanel};
+        cudaError_t r = tc::launch_gemm<false>(C, p.n, Es[i], B, p.rows, cols, kLdlqPanel, 1.0f, p.status, st);
+        if (r != cudaErrorNotSupported) return r;
+        const float* u = p.U + s0 * p.n + s0 + kLdlqPanel + d;         // no tensor maps: both halves on the FP32 pipe
+        r = launch_gemm<false, false>(C, p.n, Es[i].hi, kLdlqPanel, u, p.n, p.rows, cols, kLdlqPanel, 1.0f, st);
+        if (r != cudaSuccess) return r;
+        return launch_gemm<false, false>(C, p.n, Es[i].lo, kLdlqPanel, u, p.n, p.rows, cols, kLdlqPanel, 1.0f, st);
+    };
+    if ((e = split_u(0, 0)) != cudaSuccess) return e;
     int sp = 0;
-    for (int64_t s0 = 0; s0 < p.n; s0 += kLdlqPanel, sp++) {
+    for (int64_t s0 = 0; s0 < p.n; s0 += kLdlqPanel, sp ^= 1) {
         const int64_t span = imin64(kLdlqPanel, p.n - s0);
-        float* EpT = EpTs[sp & 1];
-        walk<<<wg, kWalkThreads, kWalkSmem, c>>>(p, s0, (int)span, EpT);
+        walk<<<wg, kWalkThreads, kWalkSmem, c>>>(p, s0, (int)span, const_cast<float*>(Es[sp].hi),
+                                                 const_cast<float*>(Es[sp].lo));
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const int64_t rest = p.n - (s0 + span);
         if (rest > 0) {
             const int64_t next = imin64(kLdlqPanel, rest);
             if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
-            // the next super-panel's columns also took the previous rest update, and
-            // that update read the EpT buffer the next super-panel overwrites
+            if ((e = cudaStreamWaitEvent(c, la->split_done, 0)) != cudaSuccess) return e;
+            // the next super-panel's columns also took the previous rest update, and that
+            // update read the buffers the next super-panel overwrites
             if (have_rest && (e = cudaStreamWaitEvent(c, la->rest_done, 0)) != cudaSuccess) return e;
-            e = update_gemm<true, false, false>(p.T + s0 + span, p.n, EpT, p.rows, p.U + s0 * p.n + s0 + span, p.n,
-                                                p.rows, next, (int)span, 1.0f, p.status, c);
-            if (e != cudaSuccess) return e;
+            if ((e = update(s0, sp, 0, next, c)) != cudaSuccess) return e;
+            if ((e = cudaStreamWaitEvent(s, la->panel_done, 0)) != cudaSuccess) return e;
+            if ((e = split_u(s0 + kLdlqPanel, sp ^ 1)) != cudaSuccess) return e;
             if (rest > next) {
-                if ((e = cudaStreamWaitEvent(s, la->panel_done, 0)) != cudaSuccess) return e;
-                e = update_gemm<true, false, false>(p.T + s0 + span + next, p.n, EpT, p.rows,
-                                                    p.U + s0 * p.n + s0 + span + next, p.n, p.rows, rest - next,
-                                                    (int)span, 1.0f, p.status, s);
-                if (e != cudaSuccess) return e;
+                if ((e = update(s0, sp, next, rest - next, s)) != cudaSuccess) return e;
                 if ((e = cudaEventRecord(la->rest_done, s)) != cudaSuccess) return e;
                 have_rest = true;
             }
