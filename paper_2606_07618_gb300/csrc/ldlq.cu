@@ -357,6 +357,7 @@ constexpr int kPanelSmem = (2 * kP + 2 * kPanelRows) * kPad * 4;
 template <bool VEC>
 __global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t k0, const float* Linv, const float* Xtop,
                                                     float* Lh, float* Ll) {
+    grid_launch_dependents();                        // the next diagonal factor waits for this grid's end
     extern __shared__ __align__(16) float psm[];
     float* sl = psm;                                 // [64][kPad] Linv
     float* st = sl + kP * kPad;                      // [64][kPad] Xtop
@@ -628,9 +629,10 @@ __device__ __forceinline__ float load_w(const void* W, int64_t idx) {
     return static_cast<const float*>(W)[idx];
 }
 
-// T[r][k] = Wp[r][k] = W[r][perm[k]] (fp32) and sfp[r][k] = sf[r][perm[k] / block].
+// T[r][k] = Wp[r][k] = W[r][perm[k]] (fp32) and sfp[r][k] = sf[r][perm[k] / block],
+// one row at a time straight from global memory: rows too long for gather_w_kernel.
 template <int DT>
-__global__ void __launch_bounds__(256) gather_w_kernel(LdlqParams p) {
+__global__ void __launch_bounds__(256) gather_w_long_kernel(LdlqParams p) {
     for (int64_t r = blockIdx.x; r < p.rows; r += gridDim.x)
         for (int64_t k = threadIdx.x; k < p.n; k += blockDim.x) {
             const int64_t c = checked_index(p.perm[k], p.n, p.status);
@@ -640,6 +642,61 @@ __global__ void __launch_bounds__(256) gather_w_kernel(LdlqParams p) {
             uint8_t code = p.sf[r * p.kb + c / p.block];
             p.sfp[r * p.n + k] = code > 126 ? 0 : code;      // 0x7F (NaN) and above: a zero scale
         }
+}
+
+// The same through shared memory, kGatherRows rows at a time: the rows come in
+// coalesced and the random reads are shared-memory ones.  Straight from global memory
+// every gathered word is a cache-line lookup of its own, which bound it (54 us at
+// 4096 x 4096 bf16, where writing the targets and weights takes 20).
+constexpr int kGatherRows = 4;
+template <int DT>
+__host__ __device__ inline int64_t gather_row_bytes(int64_t n) {        // a row's weights, 16 bytes apart
+    return n * (DT == 0 ? 2 : 4);
+}
+template <int DT>
+__global__ void __launch_bounds__(256) gather_w_kernel(LdlqParams p, int shift) {
+    extern __shared__ __align__(16) uint8_t gsm[];
+    const int64_t rb = gather_row_bytes<DT>(p.n);
+    uint8_t* ssf = gsm + kGatherRows * rb;                              // [kGatherRows][kb]
+    const bool wide = (reinterpret_cast<uintptr_t>(p.W) & 15) == 0;     // then every row is: n is a multiple of 16
+    for (int64_t r0 = (int64_t)blockIdx.x * kGatherRows; r0 < p.rows; r0 += (int64_t)gridDim.x * kGatherRows) {
+        const int nr = (int)(p.rows - r0 < kGatherRows ? p.rows - r0 : kGatherRows);
+        __syncthreads();                                                // the last rows are read
+        if (wide) {
+            const uint4* src = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(p.W) + r0 * rb);
+            for (int i = threadIdx.x; i < (int)(nr * rb / 16); i += 256) reinterpret_cast<uint4*>(gsm)[i] = src[i];
+        } else {
+            for (int i = threadIdx.x; i < (int)(nr * p.n); i += 256) {
+                if (DT == 0) reinterpret_cast<uint16_t*>(gsm)[i] = static_cast<const uint16_t*>(p.W)[r0 * p.n + i];
+                else reinterpret_cast<float*>(gsm)[i] = static_cast<const float*>(p.W)[r0 * p.n + i];
+            }
+        }
+        for (int i = threadIdx.x; i < (int)(nr * p.kb); i += 256) ssf[i] = p.sf[r0 * p.kb + i];
+        __syncthreads();
+        for (int64_t k = 4 * threadIdx.x; k < p.n; k += 4 * 256) {
+            int c[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) c[j] = (int)checked_index(p.perm[k + j], p.n, p.status);
+#pragma unroll
+            for (int i = 0; i < kGatherRows; i++) {
+                if (i >= nr) break;
+                float v[4];
+                uint32_t codes = 0;
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    if (DT == 0) v[j] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(gsm + i * rb)[c[j]] << 16);
+                    else v[j] = reinterpret_cast<const float*>(gsm + i * rb)[c[j]];
+                    const uint32_t code = ssf[i * p.kb + (c[j] >> shift)];
+                    codes |= (code > 126 ? 0u : code) << (8 * j);       // 0x7F (NaN) and above: a zero scale
+                }
+                const int64_t at = (r0 + i) * p.n + k;
+                const float4 q = make_float4(v[0], v[1], v[2], v[3]);
+                *reinterpret_cast<float4*>(p.T + at) = q;
+                *reinterpret_cast<float4*>(p.Wp + at) = q;
+                *reinterpret_cast<uint32_t*>(p.sfp + at) = codes;
+            }
+        }
+    }
 }
 
 // One super-panel of up to 256 columns (a multiple of 8): every column is
@@ -1000,9 +1057,9 @@ __global__ void __launch_bounds__(256) split_u_kernel(const float* U, int64_t n,
         }
 }
 
-// codes[r][c/2]: nibble of original column c from qb[r][inv[c]]
-__global__ void __launch_bounds__(256) pack_kernel(const uint8_t* qb, const int32_t* inv, int64_t rows, int64_t n,
-                                                   uint8_t* codes, int* status) {
+// codes[r][c/2]: nibble of original column c from qb[r][inv[c]]; rows too long for pack_kernel.
+__global__ void __launch_bounds__(256) pack_long_kernel(const uint8_t* qb, const int32_t* inv, int64_t rows, int64_t n,
+                                                        uint8_t* codes, int* status) {
     const int64_t half = n / 2;
     for (int64_t r = blockIdx.x; r < rows; r += gridDim.x)
         for (int64_t c2 = threadIdx.x; c2 < half; c2 += blockDim.x) {
@@ -1011,6 +1068,39 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint8_t* qb, const int3
             codes[r * half + c2] = (uint8_t)((lo & 0xF) | ((hi & 0xF) << 4));
         }
 }
+
+// The same through shared memory, kGatherRows rows at a time (23 us straight from
+// global memory at 4096 x 4096).
+__global__ void __launch_bounds__(256) pack_kernel(const uint8_t* qb, const int32_t* inv, int64_t rows, int64_t n,
+                                                   uint8_t* codes, int* status) {
+    extern __shared__ __align__(16) uint8_t gsm[];
+    const bool words = (reinterpret_cast<uintptr_t>(codes) & 3) == 0;   // then every row is: n / 2 is a multiple of 8
+    for (int64_t r0 = (int64_t)blockIdx.x * kGatherRows; r0 < rows; r0 += (int64_t)gridDim.x * kGatherRows) {
+        const int nr = (int)(rows - r0 < kGatherRows ? rows - r0 : kGatherRows);
+        __syncthreads();                                                // the last rows are read
+        for (int i = threadIdx.x; i < (int)(nr * n / 16); i += 256)
+            reinterpret_cast<uint4*>(gsm)[i] = reinterpret_cast<const uint4*>(qb + r0 * n)[i];
+        __syncthreads();
+        for (int64_t c = 8 * threadIdx.x; c < n; c += 8 * 256) {
+            int k[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) k[j] = (int)checked_index(inv[c + j], n, status);
+#pragma unroll
+            for (int i = 0; i < kGatherRows; i++) {
+                if (i >= nr) break;
+                uint32_t w = 0;
+#pragma unroll
+                for (int j = 0; j < 8; j++) w |= (uint32_t)(gsm[i * n + k[j]] & 0xFu) << (4 * j);
+                uint8_t* d = codes + ((r0 + i) * n + c) / 2;
+                if (words) *reinterpret_cast<uint32_t*>(d) = w;
+                else
+                    for (int b = 0; b < 4; b++) d[b] = (uint8_t)(w >> (8 * b));
+            }
+        }
+    }
+}
+
+constexpr int64_t kGatherSmemMax = 200 * 1024;     // dynamic shared memory of the two kernels above
 
 }  // namespace
 
@@ -1051,6 +1141,22 @@ cudaError_t lookahead_for_current_device(LookAhead** out, std::unique_lock<std::
     return cudaSuccess;
 }
 
+// Launch of `kernel` on `s` as a programmatic dependent of the kernel before it on the stream.
+template <typename... P, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned threads, int smem, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* perm, float* U, float* D,
                                 int* status, void* ws, int sms, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
@@ -1086,7 +1192,9 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     bool have_rest = false;              // rest_done recorded by this call (waits stay inside a capture)
     for (int64_t k0 = 0; k0 < n; k0 += kP) {
         const int nb = (int)imin64(kP, n - k0);
-        potrf_kernel<<<1, 256, kPotrfSmem, c>>>(U, n, k0, nb, Linv, Xtop, status);
+        // scheduled while the last panel kernel runs, ordered after its writes
+        if ((e = launch_dependent(potrf_kernel, 1, 256, kPotrfSmem, c, U, n, k0, nb, Linv, Xtop, status)) != cudaSuccess)
+            return e;
         const int64_t rest = n - k0 - nb;
         if (rest > 0) {
             const int64_t nb2 = imin64(kP, rest);      // width of the next panel
@@ -1156,10 +1264,19 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     if (e != cudaSuccess) return e;
     invperm_kernel<<<(unsigned)((p.n + 255) / 256), 256, 0, s>>>(p.perm, p.n, inv, p.status);
     const unsigned rg = (unsigned)imin64(p.rows, (int64_t)sms * 8);
-    if (dtype == 0)
-        gather_w_kernel<0><<<rg, 256, 0, s>>>(p);
-    else
-        gather_w_kernel<1><<<rg, 256, 0, s>>>(p);
+    const unsigned rg4 = (unsigned)imin64((p.rows + kGatherRows - 1) / kGatherRows, (int64_t)sms * 8);
+    const int64_t gsmem = kGatherRows * ((dtype == 0 ? gather_row_bytes<0>(p.n) : gather_row_bytes<1>(p.n)) + p.kb);
+    const int shift = p.block == 16 ? 4 : p.block == 32 ? 5 : 6;
+    if (gsmem > kGatherSmemMax) {
+        if (dtype == 0) gather_w_long_kernel<0><<<rg, 256, 0, s>>>(p);
+        else gather_w_long_kernel<1><<<rg, 256, 0, s>>>(p);
+    } else {
+        const auto gather = dtype == 0 ? gather_w_kernel<0> : gather_w_kernel<1>;
+        if (gsmem > 48 * 1024 &&
+            (e = cudaFuncSetAttribute(gather, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGatherSmemMax)) != cudaSuccess)
+            return e;
+        gather<<<rg4, 256, (size_t)gsmem, s>>>(p, shift);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const bool uvec = (reinterpret_cast<uintptr_t>(p.U) & 15) == 0;
@@ -1233,7 +1350,15 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     if ((e = cudaEventRecord(la->crit_done, c)) != cudaSuccess) return e;          // join
     if ((e = cudaStreamWaitEvent(s, la->crit_done, 0)) != cudaSuccess) return e;
     lock.unlock();
-    pack_kernel<<<rg, 256, 0, s>>>(p.qb, inv, p.rows, p.n, codes, p.status);
+    const int64_t psmem = kGatherRows * p.n;
+    if (psmem > kGatherSmemMax) {
+        pack_long_kernel<<<rg, 256, 0, s>>>(p.qb, inv, p.rows, p.n, codes, p.status);
+    } else {
+        if (psmem > 48 * 1024 && (e = cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)kGatherSmemMax)) != cudaSuccess)
+            return e;
+        pack_kernel<<<rg4, 256, (size_t)psmem, s>>>(p.qb, inv, p.rows, p.n, codes, p.status);
+    }
     return cudaGetLastError();
 }
 
