@@ -37,6 +37,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "nvfp4_device.cuh"
+
 namespace nvfp4 {
 namespace tc {
 
@@ -211,6 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ int s_abort, s_issued;
     __shared__ uint32_t s_tmem;
     const int m0 = (int)blockIdx.y * kTileM, n0 = (int)blockIdx.x * kTileN;
+    grid_launch_dependents();                                    // a dependent launch waits for this grid's end
     if (LOWER && n0 > m0 + kTileM - 1) return;
     const int nst = (K + kStageK - 1) / kStageK;
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
