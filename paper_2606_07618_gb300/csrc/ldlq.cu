@@ -113,27 +113,38 @@ __global__ void __launch_bounds__(256) gather_h_kernel(const float* H, int64_t n
 // c = c0 + CS j of a thread's 4 x 4 tile; x and y in shared memory, kPad words per
 // row, K a multiple of 4.  Even and odd k are summed apart (packed fp32).
 constexpr int kPad = kP + 4;          // rows 4 banks apart: eight lanes' 16-byte reads cover all banks
-template <int RS, int CS>
+// LOW (CS = 16): y is lower triangular, so column group j ends at k = 16 j + 15.
+template <int RS, int CS, bool LOW = false>
 __device__ __forceinline__ void tile_dot(const float* x, int r0, const float* y, int c0, int K, float (&out)[4][4]) {
     u64 acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; i++)
 #pragma unroll
         for (int j = 0; j < 4; j++) acc[i][j] = 0ull;
-#pragma unroll 2
-    for (int k = 0; k < K; k += 4) {
+    auto chunk = [&](int k, int j0) {
         float4 a[4], b[4];
 #pragma unroll
         for (int i = 0; i < 4; i++) a[i] = *reinterpret_cast<const float4*>(x + (r0 + RS * i) * kPad + k);
 #pragma unroll
-        for (int j = 0; j < 4; j++) b[j] = *reinterpret_cast<const float4*>(y + (c0 + CS * j) * kPad + k);
+        for (int j = 0; j < 4; j++)
+            if (j >= j0) b[j] = *reinterpret_cast<const float4*>(y + (c0 + CS * j) * kPad + k);
 #pragma unroll
         for (int i = 0; i < 4; i++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                acc[i][j] = fma2(pack2(a[i].x, a[i].y), pack2(b[j].x, b[j].y), acc[i][j]);
-                acc[i][j] = fma2(pack2(a[i].z, a[i].w), pack2(b[j].z, b[j].w), acc[i][j]);
-            }
+            for (int j = 0; j < 4; j++)
+                if (j >= j0) {
+                    acc[i][j] = fma2(pack2(a[i].x, a[i].y), pack2(b[j].x, b[j].y), acc[i][j]);
+                    acc[i][j] = fma2(pack2(a[i].z, a[i].w), pack2(b[j].z, b[j].w), acc[i][j]);
+                }
+    };
+    if (LOW) {
+#pragma unroll
+        for (int j0 = 0; j0 < 4; j0++)
+#pragma unroll 2
+            for (int k = 16 * j0; k < 16 * j0 + 16; k += 4) chunk(k, j0);
+    } else {
+#pragma unroll 2
+        for (int k = 0; k < K; k += 4) chunk(k, 0);
     }
 #pragma unroll
     for (int i = 0; i < 4; i++)
@@ -179,8 +190,12 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
     extern __shared__ __align__(16) float psm[];
     float* sl = psm;                                 // [64][kPad] Linv
     float* st = psm + kP * kPad;                     // [64][kPad] the next 64 rows of the panel
-    __shared__ __align__(16) float sw[kP][4], smul[kP][4], sx[kP][4];   // W, W / p, X_b^T
-    __shared__ float sm[6], sip[4], piv[kP];
+    // W, W / p, X_b^T: entry i of tile T at [i][T], so that a warp's tiles lie in distinct banks
+    // (one array, indexed: a pointer chosen between arrays would make the accesses generic)
+    constexpr int kW = 0, kMul = 4, kX = 8;
+    __shared__ __align__(16) float4 sb[12][16];
+    __shared__ __align__(16) float sm[8], sip[4];
+    __shared__ float piv[kP];
     const int I = threadIdx.x >> 4, J = threadIdx.x & 15;
     const bool low = J <= I, diag = I == J;
     const int R = low ? I : J, C = low ? J : I;      // the thread's tile: (R, C) of A (low) or of X
@@ -232,27 +247,11 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
 #pragma unroll
                     for (int l = j + 1; l <= i; l++) t[i][l] = __fmaf_rn(-m[i][j], t[l][j], t[i][l]);
             }
+            *reinterpret_cast<float4*>(sip) = make_float4(ip[0], ip[1], ip[2], ip[3]);
+            *reinterpret_cast<float4*>(sm) = make_float4(m[1][0], m[2][0], m[2][1], m[3][0]);
+            *reinterpret_cast<float2*>(sm + 4) = make_float2(m[3][1], m[3][2]);
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                sip[j] = ip[j];
-                piv[4 * b + j] = p[j];
-            }
-            sm[0] = m[1][0];
-            sm[1] = m[2][0];
-            sm[2] = m[2][1];
-            sm[3] = m[3][0];
-            sm[4] = m[3][1];
-            sm[5] = m[3][2];
-            // X's diagonal tile M_bb^-1 (unit lower), transposed for the update
-            xd[1][0] = -m[1][0];
-            xd[2][1] = -m[2][1];
-            xd[3][2] = -m[3][2];
-            xd[2][0] = __fmaf_rn(m[2][1], m[1][0], -m[2][0]);
-            xd[3][1] = __fmaf_rn(m[3][2], m[2][1], -m[3][1]);
-            xd[3][0] = __fmaf_rn(-m[3][2], xd[2][0], __fmaf_rn(-m[3][1], xd[1][0], -m[3][0]));
-#pragma unroll
-            for (int j = 0; j < 4; j++)
-                *reinterpret_cast<float4*>(sx[4 * b + j]) = make_float4(xd[0][j], xd[1][j], xd[2][j], xd[3][j]);
+            for (int j = 0; j < 4; j++) t[j][j] = p[j];
 #pragma unroll
             for (int i = 1; i < 4; i++)
 #pragma unroll
@@ -260,34 +259,48 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
         }
         __syncthreads();
         // W = A M_bb^-T below the block; X's row b, held transposed, takes the same steps
-        if (J == b && !diag) {
-            const float m10 = sm[0], m20 = sm[1], m21 = sm[2], m30 = sm[3], m31 = sm[4], m32 = sm[5];
-            float* dst = low ? &sw[4 * R][0] : &sx[4 * C][0];
+        if (J == b) {
+            if (!diag) {
+                const float4 ma = *reinterpret_cast<const float4*>(sm), ip = *reinterpret_cast<const float4*>(sip);
+                const float2 mb = *reinterpret_cast<const float2*>(sm + 4);
+                const int dst = low ? kW : kX, T = low ? R : C;
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
-                t[i][1] = __fmaf_rn(-t[i][0], m10, t[i][1]);
-                t[i][2] = __fmaf_rn(-t[i][0], m20, t[i][2]);
-                t[i][3] = __fmaf_rn(-t[i][0], m30, t[i][3]);
-                t[i][2] = __fmaf_rn(-t[i][1], m21, t[i][2]);
-                t[i][3] = __fmaf_rn(-t[i][1], m31, t[i][3]);
-                t[i][3] = __fmaf_rn(-t[i][2], m32, t[i][3]);
-                *reinterpret_cast<float4*>(dst + 4 * i) = make_float4(t[i][0], t[i][1], t[i][2], t[i][3]);
-                if (low)
-                    *reinterpret_cast<float4*>(smul[4 * R + i]) =
-                        make_float4(__fmul_rn(t[i][0], sip[0]), __fmul_rn(t[i][1], sip[1]), __fmul_rn(t[i][2], sip[2]),
-                                    __fmul_rn(t[i][3], sip[3]));
+                for (int i = 0; i < 4; i++) {
+                    t[i][1] = __fmaf_rn(-t[i][0], ma.x, t[i][1]);
+                    t[i][2] = __fmaf_rn(-t[i][0], ma.y, t[i][2]);
+                    t[i][3] = __fmaf_rn(-t[i][0], ma.w, t[i][3]);
+                    t[i][2] = __fmaf_rn(-t[i][1], ma.z, t[i][2]);
+                    t[i][3] = __fmaf_rn(-t[i][1], mb.x, t[i][3]);
+                    t[i][3] = __fmaf_rn(-t[i][2], mb.y, t[i][3]);
+                    sb[dst + i][T] = make_float4(t[i][0], t[i][1], t[i][2], t[i][3]);
+                    if (low)
+                        sb[kMul + i][T] = make_float4(__fmul_rn(t[i][0], ip.x), __fmul_rn(t[i][1], ip.y),
+                                                 __fmul_rn(t[i][2], ip.z), __fmul_rn(t[i][3], ip.w));
+                }
+            } else {
+                // X's diagonal tile M_bb^-1 (unit lower), transposed for the update
+                xd[1][0] = -t[1][0];
+                xd[2][1] = -t[2][1];
+                xd[3][2] = -t[3][2];
+                xd[2][0] = __fmaf_rn(t[2][1], t[1][0], -t[2][0]);
+                xd[3][1] = __fmaf_rn(t[3][2], t[2][1], -t[3][1]);
+                xd[3][0] = __fmaf_rn(-t[3][2], xd[2][0], __fmaf_rn(-t[3][1], xd[1][0], -t[3][0]));
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    sb[kX + j][b] = make_float4(xd[0][j], xd[1][j], xd[2][j], xd[3][j]);
+                    piv[4 * b + j] = t[j][j];
+                }
             }
         }
         __syncthreads();
         if (R > b && (low ? C > b : C <= b)) {
             // A: t[i][j] -= m_(R i) . W_(C j);  X^T: t[i][j] -= X_b^T_(C i) . m_(R j)
-            const float(*u)[4] = low ? &smul[4 * R] : &sx[4 * C];
-            const float(*y)[4] = low ? &sw[4 * C] : &smul[4 * R];
+            const int u = low ? kMul : kX, y = low ? kW : kMul, tu = low ? R : C, ty = low ? C : R;
             float4 mr[4], yc[4];
 #pragma unroll
             for (int i = 0; i < 4; i++) {
-                mr[i] = *reinterpret_cast<const float4*>(u[i]);
-                yc[i] = *reinterpret_cast<const float4*>(y[i]);
+                mr[i] = sb[u + i][tu];
+                yc[i] = sb[y + i][ty];
             }
 #pragma unroll
             for (int i = 0; i < 4; i++)
@@ -302,7 +315,7 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
     }
     // L into the block, Linv = diag(1 / sqrt p) X into shared and global memory
     __syncthreads();
-    float* sq = &sw[0][0];                           // sqrt p, then 1 / sqrt p
+    float* sq = &sb[0][0].x;                         // sqrt p, then 1 / sqrt p
     if (threadIdx.x < kP) {
         sq[threadIdx.x] = __fsqrt_rn(piv[threadIdx.x]);
         sq[kP + threadIdx.x] = __frsqrt_rn(piv[threadIdx.x]);
@@ -339,7 +352,7 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
     // Xtop: rows I + 16 i, columns J + 16 j of the solved panel
     if (nt > 0) {
         float o[4][4];
-        tile_dot<16, 16>(st, I, sl, J, kP, o);
+        tile_dot<16, 16, true>(st, I, sl, J, kP, o);
 #pragma unroll
         for (int i = 0; i < 4; i++)
 #pragma unroll
