@@ -1156,22 +1156,6 @@ cudaError_t lookahead_for_current_device(LookAhead** out, std::unique_lock<std::
     return cudaSuccess;
 }
 
-// Launch of `kernel` on `s` as a programmatic dependent of the kernel before it on the stream.
-template <typename... P, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned threads, int smem, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-}
-
 cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* perm, float* U, float* D,
                                 int* status, void* ws, int sms, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
@@ -1208,7 +1192,7 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     for (int64_t k0 = 0; k0 < n; k0 += kP) {
         const int nb = (int)imin64(kP, n - k0);
         // scheduled while the last panel kernel runs, ordered after its writes
-        if ((e = launch_dependent(potrf_kernel, 1, 256, kPotrfSmem, c, U, n, k0, nb, Linv, Xtop, status)) != cudaSuccess)
+        if ((e = launch_dependent_smem(potrf_kernel, 1, 256, kPotrfSmem, c, U, n, k0, nb, Linv, Xtop, status)) != cudaSuccess)
             return e;
         const int64_t rest = n - k0 - nb;
         if (rest > 0) {
@@ -1347,7 +1331,7 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
         const int64_t span = imin64(kLdlqPanel, p.n - s0);
         float *eh = const_cast<float*>(Es[sp].hi), *el = const_cast<float*>(Es[sp].lo);
         if (early) {
-            e = launch_dependent(walk, wg, kWalkThreads, kWalkSmem, c, p, s0, (int)span, eh, el);
+            e = launch_dependent_smem(walk, wg, kWalkThreads, kWalkSmem, c, p, s0, (int)span, eh, el);
         } else {
             walk<<<wg, kWalkThreads, kWalkSmem, c>>>(p, s0, (int)span, eh, el);
             e = cudaGetLastError();

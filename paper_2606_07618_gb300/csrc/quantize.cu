@@ -22,8 +22,7 @@ static cudaError_t launch_one(const QuantParams& p, int sms, cudaStream_t s) {
                     break;
                 }
     }
-    quantize_kernel<DT, METHOD, OBJ, BLOCK, FIX, 0><<<(int)grid, 256, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(quantize_kernel<DT, METHOD, OBJ, BLOCK, FIX, 0>, grid, 256, s, p);
 }
 
 template <int DT, int METHOD, int OBJ, int BLOCK>

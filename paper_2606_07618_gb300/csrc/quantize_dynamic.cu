@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kClusterThreads) quantize_cluster_kernel(Quant
     const int64_t g = (int64_t)blockIdx.x * kClusterThreads + tid;
     const bool valid = g < p.nseg;
     Raw cur = {};
-    if (valid) load_raw<DT>(p.x, g, wide_input(p.x), cur);
+    if (valid) load_raw<DT, true>(p.x, g, wide_input(p.x), cur);
     build_table(tab);
     // max |x| with NaN skipped, and whether anything is not finite (as dynamic_scale)
     float m = 0.0f;
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kClusterThreads) quantize_cluster_kernel(Quant
 #pragma unroll
     for (int j = 0; j < 8; j++) w2[j] = 0ull;
     const float* wkey = nullptr;
-    quantize_segment<DT, METHOD, OBJ, BLOCK, 1>(p, tab, cur, g, valid, pack2(E, E), usable, w2, wkey);
+    quantize_segment<DT, METHOD, OBJ, BLOCK, 1, true>(p, tab, cur, g, valid, pack2(E, E), usable, w2, wkey);
     zero_pads(p.sf_swizzled, p.rows, p.kb, p.kpad4, g, (int64_t)gridDim.x * kClusterThreads);
 }
 

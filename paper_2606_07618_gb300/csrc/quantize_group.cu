@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(THREADS, 2048 / THREADS)
 // another address (wkey): with a CTA stride that is a multiple of the
 // tensor's segments per row a lane keeps its columns, so per-channel weights
 // are loaded once per tensor.
-template <int DT, int METHOD, int OBJ, int BLOCK>
+template <int DT, int METHOD, int OBJ, int BLOCK, bool NC>
 __device__ __forceinline__ void sweep_segments(const GroupTensor& d, const Cand* tab, const Raw& cur, int64_t g,
                                                bool valid, u64 E2, bool usable, u64 (&w2)[8], const float*& wkey,
                                                bool& wok) {
@@ -267,7 +267,7 @@ __device__ __forceinline__ void sweep_segments(const GroupTensor& d, const Cand*
         if (valid && wp != wkey) {
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                const uint4 a = ld_ro16(wp + 4 * j);
+                const uint4 a = ld_ro16<NC>(wp + 4 * j);
                 w2[2 * j] = pack2(__uint_as_float(a.x), __uint_as_float(a.y));
                 w2[2 * j + 1] = pack2(__uint_as_float(a.z), __uint_as_float(a.w));
             }
@@ -362,8 +362,8 @@ __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>()
         if (blockIdx.x == 0 && (int)threadIdx.x < p.count)        // publish every tensor's S once
             p.S[p.t[threadIdx.x].s_index] =
                 __fdiv_rn(__uint_as_float(ld_relaxed_u32(p.amax_bits + threadIdx.x)), __fmul_rn(6.0f, p.fp8_div));
-    } else if (DYN == 2) {
-        // pipelined schedule: the scales come from the reduction grid launched
+    } else {
+        // pipelined schedule (DYN = 2): the scales come from the reduction grid launched
         // before this one; once every CTA is resident the next reduction grid
         // may be scheduled beside it
         grid_dependency_wait();
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>()
     Raw cur;
     if (cbase < total) {
         const int64_t g = cbase + tid - p.t[t].seg_begin;
-        if (g < p.t[t].nseg) load_raw<DT>(p.t[t].x, g, METHOD != 1 && wide_input(p.t[t].x), cur);
+        if (g < p.t[t].nseg) load_raw<DT, DYN != 0>(p.t[t].x, g, METHOD != 1 && wide_input(p.t[t].x), cur);
     }
 
     while (cbase < total) {
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>()
         const float S =
             DYN == 1 ? __fdiv_rn(__uint_as_float(ld_relaxed_u32(p.amax_bits + t)), __fmul_rn(6.0f, p.fp8_div))
             : DYN == 2 ? __uint_as_float(ld_relaxed_u32(reinterpret_cast<const unsigned*>(p.S + p.t[t].s_index)))
-                       : __ldg(p.S + p.t[t].s_index);
+                       : ld_f32(p.S + p.t[t].s_index);
         float E = __frcp_rn(S);
         const bool usable = (S > 0.0f) && isfinite(S) && isfinite(E);
         if (!usable) E = 1.0f;
@@ -408,13 +408,13 @@ __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>()
             Raw nxt;
             const int64_t nb = cbase + stride;
             if (nb < seg_end) {
-                if (g + stride < d.nseg) load_raw<DT>(d.x, g + stride, METHOD != 1 && wide_input(d.x), nxt);
+                if (g + stride < d.nseg) load_raw<DT, DYN != 0>(d.x, g + stride, METHOD != 1 && wide_input(d.x), nxt);
             } else if (nb < total) {
                 const int tn = tensor_at(p, t, nb);
                 const int64_t gn = nb + tid - p.t[tn].seg_begin;
-                if (gn < p.t[tn].nseg) load_raw<DT>(p.t[tn].x, gn, METHOD != 1 && wide_input(p.t[tn].x), nxt);
+                if (gn < p.t[tn].nseg) load_raw<DT, DYN != 0>(p.t[tn].x, gn, METHOD != 1 && wide_input(p.t[tn].x), nxt);
             }
-            sweep_segments<DT, METHOD, OBJ, BLOCK>(d, tab, cur, g, valid, E2, usable, w2, wkey, wok);
+            sweep_segments<DT, METHOD, OBJ, BLOCK, DYN != 0>(d, tab, cur, g, valid, E2, usable, w2, wkey, wok);
             cur = nxt;
         }
         t = tensor_at(p, t, cbase);
@@ -476,25 +476,7 @@ cudaError_t launch_group(const GroupParams& p, int sms, cudaStream_t s) {
         return cudaLaunchCooperativeKernel((const void*)quantize_group_kernel<DT, METHOD, OBJ, BLOCK, 1>,
                                            dim3((unsigned)grid), dim3(kSweepThreads), args, 0, s);
     }
-    quantize_group_kernel<DT, METHOD, OBJ, BLOCK, 0><<<(unsigned)grid, kSweepThreads, 0, s>>>(p);
-    return cudaGetLastError();
-}
-
-// Launch of `kernel` on `s` as a programmatic dependent of the kernel before
-// it on the stream.
-template <typename... Args>
-cudaError_t launch_dependent(void (*kernel)(Args...), int64_t grid, int threads, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    return launch_dependent(quantize_group_kernel<DT, METHOD, OBJ, BLOCK, 0>, grid, kSweepThreads, s, p);
 }
 
 // The tensors p.t[first..last) as a group of their own (segment space from 0,

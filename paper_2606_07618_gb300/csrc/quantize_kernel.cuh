@@ -76,18 +76,18 @@ struct Raw {
 };
 
 // wide: x is 32-byte aligned (every segment then is too).
-template <int DT>
+template <int DT, bool NC>
 __device__ __forceinline__ void load_raw(const void* x, int64_t g, bool wide, Raw& r) {
     const char* p = static_cast<const char*>(x) + g * (DT == 0 ? 32 : 64);
     if (wide) {
-        ld_stream32(p, r.a, r.b);
-        if (DT != 0) ld_stream32(p + 32, r.c, r.d);
+        ld_stream32<NC>(p, r.a, r.b);
+        if (DT != 0) ld_stream32<NC>(p + 32, r.c, r.d);
     } else {
-        r.a = ld_stream16(p);
-        r.b = ld_stream16(p + 16);
+        r.a = ld_stream16<NC>(p);
+        r.b = ld_stream16<NC>(p + 16);
         if (DT != 0) {
-            r.c = ld_stream16(p + 32);
-            r.d = ld_stream16(p + 48);
+            r.c = ld_stream16<NC>(p + 32);
+            r.d = ld_stream16<NC>(p + 48);
         }
     }
 }
@@ -566,7 +566,7 @@ constexpr int quantize_min_blocks() {
 
 // One 16-element segment: its block's scale, nibbles, scale bytes and loss.  tab:
 // the candidate table; w2, wkey: the lane's weights and where they came from.
-template <int DT, int METHOD, int OBJ, int BLOCK, int FIX>
+template <int DT, int METHOD, int OBJ, int BLOCK, int FIX, bool NC>
 __device__ __forceinline__ void quantize_segment(const QuantParams& p, const Cand* tab, const Raw& cur, int64_t g,
                                                  bool valid, u64 E2, bool usable, u64 (&w2)[8], const float*& wkey) {
     constexpr int SEGS = BLOCK / 16;
@@ -602,7 +602,7 @@ __device__ __forceinline__ void quantize_segment(const QuantParams& p, const Can
         if (valid && (METHOD == 0 || wp != wkey)) {
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                const uint4 a = ld_ro16(wp + 4 * j);
+                const uint4 a = ld_ro16<NC>(wp + 4 * j);
                 w2[2 * j] = pack2(__uint_as_float(a.x), __uint_as_float(a.y));
                 w2[2 * j + 1] = pack2(__uint_as_float(a.z), __uint_as_float(a.w));
             }
@@ -729,14 +729,16 @@ __device__ __forceinline__ void quantize_segment(const QuantParams& p, const Can
 template <int DT, int METHOD, int OBJ, int BLOCK, int FIX, int DYN>
 __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quantize_kernel(QuantParams p) {
     __shared__ Cand tab[kTabN];
+    grid_launch_dependents();
     build_table(tab);
     __syncthreads();
+    grid_dependency_wait();
 
     float S;
     if (DYN) {
         if (!dynamic_scale<DT>(p, S)) return;
     } else {
-        S = __ldg(p.S);
+        S = ld_f32(p.S);
     }
     float E = __frcp_rn(S);
     const bool usable = (S > 0.0f) && isfinite(S) && isfinite(E);
@@ -749,7 +751,7 @@ __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quanti
     int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
     const bool wide = METHOD != 1 && wide_input(p.x);      // AbsMax: 2% slower with 32-byte loads
     Raw cur;
-    if (base + lane < p.nseg) load_raw<DT>(p.x, base + lane, wide, cur);
+    if (base + lane < p.nseg) load_raw<DT, DYN != 0>(p.x, base + lane, wide, cur);
 
     // 4/6 keeps a lane's weights while they come from the same address (the grid's
     // stride is a multiple of a row's segments where it can be): four 16-byte loads 64
@@ -763,9 +765,9 @@ __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quanti
         const int64_t g = base + lane;
         const bool valid = g < p.nseg;
         Raw nxt;
-        if (g + stride < p.nseg) load_raw<DT>(p.x, g + stride, wide, nxt);
+        if (g + stride < p.nseg) load_raw<DT, DYN != 0>(p.x, g + stride, wide, nxt);
 
-        quantize_segment<DT, METHOD, OBJ, BLOCK, FIX>(p, tab, cur, g, valid, E2, usable, w2, wkey);
+        quantize_segment<DT, METHOD, OBJ, BLOCK, FIX, DYN != 0>(p, tab, cur, g, valid, E2, usable, w2, wkey);
         cur = nxt;
     }
     zero_pads(p.sf_swizzled, p.rows, p.kb, p.kpad4, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride);

@@ -25,6 +25,7 @@ template <int DT>
 __global__ void __launch_bounds__(512) amax_partial_kernel(const void* x, int64_t n, float* part_max,
                                                            int* part_bad) {
     constexpr int PER = DT == 0 ? 8 : 4;      // elements per 16-byte vector
+    grid_dependency_wait();
     const int64_t nvec = n / PER;
     float m = 0.0f;
     int bad = 0;
@@ -46,11 +47,11 @@ __global__ void __launch_bounds__(512) amax_partial_kernel(const void* x, int64_
     // two independent 16-byte loads in flight per thread; with 2048 threads
     // per SM that keeps ~10 MB in flight across the GPU
     for (; i + stride < nvec; i += 2 * stride) {
-        const uint4 u0 = ld_stream16(xv + i), u1 = ld_stream16(xv + i + stride);
+        const uint4 u0 = ld_stream16<false>(xv + i), u1 = ld_stream16<false>(xv + i + stride);
         fold(u0);
         fold(u1);
     }
-    if (i < nvec) fold(ld_stream16(xv + i));
+    if (i < nvec) fold(ld_stream16<false>(xv + i));
     // tail elements (n not a multiple of the vector width)
     if (blockIdx.x == 0 && threadIdx.x < (int)(n - nvec * PER)) {
         const int64_t i = nvec * PER + threadIdx.x;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(256) amax_final_kernel(const float* part_max, 
                                                          float fp8_div, float* S_out, int* status_dev) {
     // launched as a programmatic dependent of amax_partial_kernel: wait until
     // that grid has finished and its partials are visible (a no-op otherwise)
+    grid_launch_dependents();
     grid_dependency_wait();
     uint32_t v = 0u;
     int b = 0;
@@ -120,26 +122,13 @@ __global__ void __launch_bounds__(256) amax_final_kernel(const float* part_max, 
 // The folding CTA, allowed to start before amax_partial_kernel has drained.
 static cudaError_t launch_final(const float* part_max, const int* part_bad, int nparts, float fp8_div,
                                 float* S_out, int* status_dev, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, amax_final_kernel, part_max, part_bad, nparts, fp8_div, S_out, status_dev);
+    return launch_dependent(amax_final_kernel, 1, 256, s, part_max, part_bad, nparts, fp8_div, S_out, status_dev);
 }
 
 static cudaError_t launch_partial(const void* x, int dtype, int64_t n, float* part_max, int* part_bad, int grid,
                                   int threads, cudaStream_t s) {
-    if (dtype == 0)
-        amax_partial_kernel<0><<<grid, threads, 0, s>>>(x, n, part_max, part_bad);
-    else
-        amax_partial_kernel<1><<<grid, threads, 0, s>>>(x, n, part_max, part_bad);
-    return cudaGetLastError();
+    return launch_dependent(dtype == 0 ? amax_partial_kernel<0> : amax_partial_kernel<1>, grid, threads, s, x, n, part_max,
+                            part_bad);
 }
 
 cudaError_t launch_global_scale(const void* x, int dtype, int64_t n, float fp8_div, float* S_out,
@@ -188,7 +177,9 @@ constexpr int kDequantUnroll = 8;      // chunks per lane per tile: of 2, 4, 8, 
 template <int OUT_BF16>
 __global__ void __launch_bounds__(256) dequant_kernel(DequantParams p, FastDiv kbd, int bshift) {
     constexpr int EPT = OUT_BF16 ? 8 : 4;          // elements per thread
-    const float S = __ldg(p.S);
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const float S = ld_f32(p.S);
     const int64_t nchunk = p.nseg * (16 / EPT);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     auto scale_offset = [&](int64_t e0) -> int64_t {
@@ -207,8 +198,8 @@ __global__ void __launch_bounds__(256) dequant_kernel(DequantParams p, FastDiv k
         return swizzle_offset(row, kbi, p.kpad4);
     };
     auto load_codes = [&](int64_t c) -> uint32_t {
-        return EPT == 8 ? __ldg(reinterpret_cast<const uint32_t*>(p.codes) + c)
-                        : (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(p.codes) + c);
+        return EPT == 8 ? ld_u32(reinterpret_cast<const uint32_t*>(p.codes) + c)
+                        : ld_u16(reinterpret_cast<const uint16_t*>(p.codes) + c);
     };
     int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * kDequantUnroll + (threadIdx.x & 31);
     for (; c0 < nchunk; c0 += stride * kDequantUnroll) {
@@ -219,7 +210,7 @@ __global__ void __launch_bounds__(256) dequant_kernel(DequantParams p, FastDiv k
             const int64_t c = c0 + 32 * u;
             if (c < nchunk) {
                 cwv[u] = load_codes(c);
-                scv[u] = __ldg(p.sf + scale_offset(c * EPT));
+                scv[u] = (uint8_t)ld_u8(p.sf + scale_offset(c * EPT));
             }
         }
 #pragma unroll
@@ -262,11 +253,7 @@ cudaError_t launch_dequantize(const DequantParams& p, int out_dtype, int sms, cu
     const FastDiv kbd = (p.swizzled && p.narrow && p.kb > 0) ? make_fast_div((uint32_t)p.kb) : FastDiv{1, 0, 0};
     int bshift = 0;
     while ((1 << bshift) < p.block) bshift++;
-    if (out_dtype == 0)
-        dequant_kernel<1><<<(int)grid, 256, 0, s>>>(p, kbd, bshift);
-    else
-        dequant_kernel<0><<<(int)grid, 256, 0, s>>>(p, kbd, bshift);
-    return cudaGetLastError();
+    return launch_dependent(out_dtype == 0 ? dequant_kernel<1> : dequant_kernel<0>, grid, 256, s, p, kbd, bshift);
 }
 
 }  // namespace nvfp4
