@@ -391,6 +391,9 @@ nvfp4_status group_common(int method, const nvfp4_group_tensor* tensors, int cou
         seg += (g.nseg + unit - 1) / unit * unit;
     }
     p.count = count;
+    p.pads = 0;
+    for (int k = 0; k < count; k++)
+        if (p.t[k].sf_swizzled && (p.t[k].rows % 128 != 0 || p.t[k].kb % 4 != 0)) p.pads = 1;
     p.dyn = dyn ? 1 : 0;
     int64_t elements = 0;
     for (int i = 0; i < count; i++) elements += sh[i].n < kPipelineMinElements ? sh[i].n : kPipelineMinElements;

@@ -32,6 +32,7 @@ struct GroupParams {
     GroupTensor t[kGroupMax];  // in processing order
     int count;
     int dyn;                   // 1: S computed in the launch, 0: S read
+    int pads;                  // 1: a tensor's swizzled scales have padding to zero
     int pipelined;             // dyn only: 1 pipelined schedule, 0 two-phase cooperative launch
     int64_t total_seg;         // end of the concatenated segment space
     float fp8_div;

@@ -349,6 +349,11 @@ constexpr int group_min_blocks() {
     return METHOD == 1 ? 4 : (OBJ == 0 ? NVFP4_GROUP_MINB_MSE : NVFP4_GROUP_MINB);
 }
 
+// Every tensor's padding, out of line: inlined it cost the sweep's loop 0.7%.
+__device__ __noinline__ void zero_group_pads(const GroupParams& p, int64_t i, int64_t n) {
+    for (int a = 0; a < p.count; a++) zero_pads(p.t[a].sf_swizzled, p.t[a].rows, p.t[a].kb, p.t[a].kpad4, i, n);
+}
+
 template <int DT, int METHOD, int OBJ, int BLOCK, int DYN>
 __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>())
     quantize_group_kernel(const __grid_constant__ GroupParams p) {
@@ -419,9 +424,7 @@ __global__ void __launch_bounds__(kSweepThreads, group_min_blocks<METHOD, OBJ>()
         }
         t = tensor_at(p, t, cbase);
     }
-    if (BLOCK == 16)
-        for (int a = 0; a < count; a++)
-            zero_pads(p.t[a].sf_swizzled, p.t[a].rows, p.t[a].kb, p.t[a].kpad4, (int64_t)blockIdx.x * SW + tid, stride);
+    if (BLOCK == 16 && p.pads) zero_group_pads(p, (int64_t)blockIdx.x * SW + tid, stride);
 }
 
 }  // namespace
