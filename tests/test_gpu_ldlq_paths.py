@@ -1,0 +1,89 @@
+"""LDLQ paths chosen by size and alignment.
+
+* Row and column counts off the walk's tiles (32 rows, 64 and 256 columns) and off the
+  update's (128), with the walk scheduled beside the update and after it.
+* A factor that is not 16-byte aligned: the same arithmetic, so the same codes.
+* Rows too long for the gather's and the packer's shared memory: with a zero factor the
+  codes are plain rounding.
+* Factorizations off the panels of 64, with outputs that are not 16-byte aligned.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from oracle import ldlq as L
+from test_gpu_ldlq import B, DEV, conditional_parity, prepare, quantize  # noqa: F401
+from test_oracle_ldlq import fixed_scales, rand_problem
+
+pytestmark = pytest.mark.gpu
+
+
+def _misaligned(t):
+    out = torch.empty(t.numel() + 1, dtype=t.dtype, device=DEV)[1:].view(t.shape)
+    out.copy_(t)
+    assert out.data_ptr() % 16 != 0
+    return out
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 16), (31, 272), (32, 320), (33, 528), (129, 784), (4900, 528)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_walk_and_update_tiles(B, rows, cols, dtype):
+    W64, H = rand_problem(rows, cols, rows + cols)
+    Wt = torch.from_numpy(W64.astype(np.float32)).to(dtype)
+    W = Wt.float().numpy().astype(np.float64)
+    H = H.astype(np.float32).astype(np.float64)
+    S, sf = fixed_scales(W, H)
+    perm, U, _, st = prepare(B, H)
+    assert st == 0
+    codes, st = quantize(B, Wt.to(DEV), S, sf, perm, U)
+    assert st == 0
+    idx = np.unique(np.linspace(0, rows - 1, 130).astype(np.int64))        # first and last rows among them
+    bad, exempt, total, first = conditional_parity(W[idx], S, sf[idx], 16, perm.cpu().numpy().astype(np.int64),
+                                                   U.double().cpu().numpy(), codes[idx])
+    assert bad == 0 and first == 0
+    assert exempt <= max(2, total // 200)
+    again, st = quantize(B, Wt.to(DEV), S, sf, perm, _misaligned(U))
+    assert st == 0 and np.array_equal(codes, again)
+
+
+# 4 rows of fp32 past 200 KB; of bf16; and of code bytes
+@pytest.mark.parametrize("n,dtype", [(12784, torch.float32), (12816, torch.float32), (25616, torch.bfloat16),
+                                     (51216, torch.float32)])
+def test_long_rows(B, n, dtype):
+    g = torch.Generator().manual_seed(n)
+    rows = 5
+    Wt = (torch.randn(rows, n, generator=g) * 0.02).to(dtype)
+    sf = torch.randint(30, 80, (rows, n // 16), generator=g).to(torch.uint8).numpy()
+    perm = torch.randperm(n, generator=g).to(torch.int32).to(DEV)
+    U = torch.zeros(n, n, device=DEV)
+    codes, st = quantize(B, Wt.to(DEV), 0.01, sf, perm, U)
+    assert st == 0
+    _, ref = oracle.block_losses_at(Wt.float().numpy(), 16, np.float32(0.01), sf, want_codes=True)
+    assert np.array_equal(codes, ref)
+
+
+@pytest.mark.parametrize("n", [1, 63, 65, 128, 193, 330, 580])
+def test_prepare_panels(B, n):
+    _, H = rand_problem(2, n, n)
+    H = H.astype(np.float32).astype(np.float64)
+    Hd, perm_ref = L.damp_and_order(H)
+    Hp = Hd[np.ix_(perm_ref, perm_ref)]
+    U_ref, D_ref = L.udu(Hp)
+    perm, U, D, st = prepare(B, H)
+    Hm = _misaligned(torch.as_tensor(H, dtype=torch.float32))
+    Um, Dm, permm = _misaligned(torch.zeros_like(U)), torch.empty_like(D), torch.empty_like(perm)
+    stm = torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.nvfp4_ldlq_prepare_workspace(n), dtype=torch.uint8, device=DEV)
+    B.nvfp4_ldlq_prepare(Hm, 0.01, permm, Um, Dm, stm, ws)
+    torch.cuda.synchronize()
+    assert st == 0 and int(stm.item()) == 0
+    for pg, Ug, Dg in ((perm, U, D), (permm, Um, Dm)):
+        assert np.array_equal(pg.cpu().numpy(), perm_ref)
+        Ug, Dg = Ug.double().cpu().numpy(), Dg.double().cpu().numpy()
+        assert np.all(np.tril(Ug) == 0)
+        # the bounds of the aligned factorization's test: fp32 rounding of n-term sums
+        assert np.allclose(Dg, D_ref, rtol=2e-4)
+        assert np.abs(Ug - U_ref).max() <= 2e-4 * max(1.0, np.abs(U_ref).max())
+        R = (Ug + np.eye(n)) @ np.diag(Dg) @ (Ug + np.eye(n)).T - Hp
+        assert np.abs(R).max() <= 2e-5 * np.abs(Hp).max()

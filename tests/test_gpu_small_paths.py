@@ -3,8 +3,9 @@
 * One-cluster dynamic-scale launch (up to 4096 segments) against the global scale
   and the static sweep as two calls, at the edges of a CTA, of the portable and of
   the largest cluster, and one segment past it, with ragged swizzled scales.
-* Windows scored an octave apart (WMSE, every code from 8 to 126) against the same
-  window given explicitly, with block scales from the smallest code to the largest.
+* Default windows, whose codes are scored an octave apart where they are normal (WMSE)
+  and whose low end is left out once saturated terms rule it out, against the same
+  codes scored one call each, with block scales from the smallest code to the largest.
 * Zeroed padding of the swizzled layout at rows and columns off its atoms.
 """
 import pytest
@@ -73,33 +74,68 @@ def test_cluster_launch(B, rows, cols, obj, dt):
             _same(a, b)
 
 
+def _one_code_at_a_time(B, x, block, S, obj, w, lo):
+    """Losses and linear outputs of the window's codes, each scored by a call whose
+    window holds that code alone, folded on the host side: lowest code on ties."""
+    best = None
+    for d in range(lo, 8):
+        o = _outs(B, x, block, False)
+        B.scalesweep_quantize(x, block, S, obj, w, 0, d, d, o["codes"], o["sf_linear"], None, o["block_loss"])
+        rows, kb = o["sf_linear"].shape if o["sf_linear"].dim() == 2 else (x.shape[0], x.shape[1] // block)
+        loss, sf = o["block_loss"].view(rows, kb), o["sf_linear"].view(rows, kb)
+        codes = o["codes"].view(rows, kb, block // 2)
+        if best is None:
+            best = [loss, sf, codes]
+        else:
+            m = loss < best[0]
+            best = [torch.where(m, loss, best[0]), torch.where(m, sf, best[1]),
+                    torch.where(m[..., None], codes, best[2])]
+    return best
+
+
 @pytest.mark.parametrize("dt", [torch.bfloat16, torch.float32])
-def test_octave_windows(B, dt):
-    """Block maxima from below the smallest code to above the largest, several
-    mixed in a warp and uniform over one."""
+@pytest.mark.parametrize("block", [16, 32, 64])
+@pytest.mark.parametrize("weights", [None, "positive", "mixed", "negative"])
+def test_window_against_single_codes(B, dt, block, weights):
+    """Octave pairs and the end of the walk down: block maxima from below the smallest
+    code to above the largest, uniform over a warp and mixed within one, with heavy
+    tails (many terms saturate); negative weights allow neither skips nor an end."""
     g = torch.Generator().manual_seed(11)
     rows, cols = 512, 512
     scale = torch.exp2(torch.linspace(-14.0, 14.0, rows))[:, None]
     mixed = torch.exp2(torch.randint(-12, 12, (rows, cols // 16, 1), generator=g).float()).expand(-1, -1, 16)
-    for s in (scale, mixed.reshape(rows, cols)):
+    tails = torch.exp(torch.randn(rows, cols, generator=g))
+    w = None
+    if weights:
+        w = torch.exp(torch.randn(cols, generator=g))
+        w = {"positive": w, "mixed": w * torch.where(torch.arange(cols) % 96 < 80, 1.0, -1.0), "negative": -w}[weights]
+        w = w.to(DEV)
+    obj = 1 if weights else 0
+    lo = -3 if (block == 16 and not weights) else -8
+    S = torch.tensor([0.25], device=DEV)
+    for s in (scale, mixed.reshape(rows, cols), scale * tails):
         x = (torch.randn(rows, cols, generator=g) * s).to(dt).to(DEV)
-        w = torch.exp(torch.randn(cols, generator=g)).to(DEV)
-        S = torch.tensor([0.25], device=DEV)
-        for block in (16, 32, 64):
-            a, b = _outs(B, x, block, block == 16), _outs(B, x, block, block == 16)
-            for o, win in ((a, (B.NVFP4_WINDOW_DEFAULT,) * 2), (b, (-8, 7))):
-                B.scalesweep_quantize(x, block, S, 1, w, 0, *win, o["codes"], o["sf_linear"], o["sf_swizzled"],
-                                      o["block_loss"])
-            # the default window given explicitly takes the same path: one code wider on one side does not
-            c = _outs(B, x, block, block == 16)
-            B.scalesweep_quantize(x, block, S, 1, w, 0, -9, 7, c["codes"], c["sf_linear"], c["sf_swizzled"],
-                                  c["block_loss"])
-            torch.cuda.synchronize()
-            _same(a, b)
-            # a wider window changes a block only where its extra code wins
-            keep = c["sf_linear"] == a["sf_linear"]
-            assert float(keep.float().mean()) > 0.999
-            assert torch.equal(a["block_loss"][keep.reshape(-1)], c["block_loss"][keep.reshape(-1)])
+        a = _outs(B, x, block, False)
+        B.scalesweep_quantize(x, block, S, obj, w, 0, *(B.NVFP4_WINDOW_DEFAULT,) * 2, a["codes"], a["sf_linear"], None,
+                              a["block_loss"])
+        gr = _outs(B, x, block, False)
+        desc = B.group_descriptors([x], [w], [0], [gr["codes"]], [gr["sf_linear"]], [None])
+        B.scalesweep_quantize_group(desc, B.NVFP4_IN_BF16 if dt == torch.bfloat16 else B.NVFP4_IN_F32, obj, 0.0, S, None,
+                                    None, block=block)
+        loss, sf, codes = _one_code_at_a_time(B, x, block, S, obj, w, lo)
+        torch.cuda.synchronize()
+        fin = torch.isfinite(loss)
+        if weights in ("mixed", "negative"):         # an offset outside the codes has no loss to compare
+            o = _outs(B, x, block, False)
+            B.scalesweep_quantize(x, block, S, obj, w, 0, 0, 0, o["codes"], o["sf_linear"], None, o["block_loss"])
+            base = o["sf_linear"].view(loss.shape).int()
+            fin &= (base + lo >= 1) & (base + 7 <= 126)
+        assert fin.float().mean() > 0.4                # 14 of 28 octaves lie inside the codes
+        shape = (rows, cols // block, -1)
+        for o in (a, gr):
+            assert torch.equal(o["sf_linear"].view(shape[:2])[fin], sf[fin])
+            assert torch.equal(o["codes"].view(shape)[fin], codes[fin])
+        assert torch.equal(a["block_loss"].view(shape[:2])[fin], loss[fin])
 
 
 @pytest.mark.parametrize("rows,cols", [(1, 16), (127, 48), (129, 80), (130, 4112), (256, 64)])

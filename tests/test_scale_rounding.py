@@ -1,7 +1,7 @@
 """The division-free forms of m / 6 that the kernels use, against the division.
 
 fl(m/6) by one residual step, and floor_E4M3(fl(m/6)) from the product with
-fl(1/6) rounded towards zero, over every mantissa of four octaves (both are
+fl(1/6) rounded towards zero, over every mantissa of two octaves (both are
 scale-free in the normal range) and every fp32 from below the smallest E4M3 code
 to above the largest, in steps that visit every rounding boundary.
 """
@@ -44,7 +44,7 @@ def around(values):
 
 
 def test_every_mantissa():
-    for e in (124, 125, 126, 127):
+    for e in (124, 127):
         m = (np.arange(1 << 23, dtype=np.uint32) | np.uint32(e << 23)).view(np.float32)
         assert np.array_equal(sixth(m), m / np.float32(6))
         assert np.array_equal(floor_code_of_sixth(m), floor_code(m / np.float32(6)))
