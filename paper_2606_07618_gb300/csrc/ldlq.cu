@@ -164,120 +164,129 @@ __device__ __forceinline__ float rcp_fast(float p) {
     return p > 1e-37f ? __fmaf_rn(r, __fmaf_rn(-p, r, 1.0f), r) : r;
 }
 
+constexpr int kPotrfThreads = 544;
+// All of potrf_kernel's warps, from either role's code.
+__device__ __forceinline__ void potrf_barrier() {
+    __syncwarp();
+    asm volatile("barrier.sync 1, %0;" ::"n"(kPotrfThreads) : "memory");
+}
+
+__device__ __forceinline__ float sum2(u64 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    return __fadd_rn(lo, hi);
+}
 // One panel's sequential part, in one CTA: the Cholesky factor of the nb x nb
 // diagonal block at k0 (lower, in place), its inverse Linv (64 x 64, lower), and the
 // solved panel of the next 64 rows, Xtop = A[k0 + nb .., k0 ..] Linv^T.
 //
-// The block is padded to 64 with an identity and held as 4 x 4 tiles in registers:
-// thread (I, J) holds tile (I, J) of the block for J <= I and, for J > I, tile
-// (J, I) of X = M^-1, transposed (threads on the diagonal hold that one too).  The pivots stay
-// unscaled, A = M diag(p) M^T with M unit lower triangular.  Block step b: thread
-// (b, b) factors its tile and publishes M_bb and 1/p; after a barrier the tiles
-// below it become W = A M_bb^-T and the multipliers W / p, and the tiles of X's row
-// b take the same steps; after another, every remaining tile takes its rank-4
-// update, tile -= m_I W_J^T or X^T tile -= X_b^T m_I^T (the same code).  Then
+// The block is padded to 64 with an identity and held as 4 x 4 tiles in registers.
+// Warp J < 16 holds tile column J: lanes (I, h) have rows 2h, 2h + 1 of tile (I, J)
+// of the block for I > J and, for I < J, of tile (J, I) of X = M^-1, transposed; lane
+// T of the last warp holds both diagonal tiles T.  The pivots stay unscaled, A = M
+// diag(p) M^T with M unit lower triangular.  Block step b: the last warp factors
+// tile b and publishes M_bb and 1/p; after a barrier warp b's tiles become
+// W = A M_bb^-T and the multipliers -W / p, and the tiles of X's row b take the same
+// steps; after another, every remaining tile takes its rank-4 update, tile -= m_I W_J^T
+// or X^T tile -= X_b^T m_I^T (the same code), the last warp's first of all.  Then
 // L = M diag(sqrt p) and Linv = diag(1/sqrt p) X.  A pivot that is not positive and
 // finite sets bit 4 of the status word and is replaced by 1 so the values stay finite.
 //
-// Bound by latency: 16 steps of a 4-pivot chain (620 cycles: a reciprocal and two
-// dependent multiply-adds per pivot), two barriers and a rank-4 update (660), about
-// 13 us with the loads and stores, and 1.7 us for Xtop.  One column per step (64
-// barriers, every thread updating a tile of both matrices) took 17.8 us without
-// Xtop; one warp factoring 16 x 16 blocks, the column going round by shuffles or
-// through shared memory, 480-560 cycles per column.
-__global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t k0, int nb, float* Linv, float* Xtop,
-                                                    int* status) {
+// Bound by latency: 16 steps of a 4-pivot chain (370 cycles alone: a reciprocal, two
+// dependent multiply-adds and a test per pivot), two barriers, the solve (150-300)
+// and the diagonal tiles' update (300).  A column per warp lets one full warp do the
+// solve while the others wait; with a tile row per warp every warp went through it on
+// two lanes (n = 4096: 1605 us for the whole factorization, with it 1579).  The
+// update's shared-memory reads (24 words a thread) take the other warps about as long
+// as the next tile's factor.  One column per step (64 barriers, every thread updating a
+// tile of both matrices) took 17.8 us a block without Xtop, this 13 us; one warp
+// factoring 16 x 16 blocks, the column going round by shuffles or through shared
+// memory, 480-560 cycles per column.  Holding the workers back until the diagonal
+// tiles have read their operands: no gain.
+__global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(float* A, int64_t n, int64_t k0, int nb, float* Linv,
+                                                              float* Xtop, int* status) {
     extern __shared__ __align__(16) float psm[];
     float* sl = psm;                                 // [64][kPad] Linv
     float* st = psm + kP * kPad;                     // [64][kPad] the next 64 rows of the panel
-    // W, W / p, X_b^T: entry i of tile T at [i][T], so that a warp's tiles lie in distinct banks
+    // W, -W / p, X_b^T: entry i of tile T at [i][T], so that a warp's tiles lie in distinct banks
     // (one array, indexed: a pointer chosen between arrays would make the accesses generic)
     constexpr int kW = 0, kMul = 4, kX = 8;
     __shared__ __align__(16) float4 sb[12][16];
     __shared__ __align__(16) float sm[8], sip[4];
     __shared__ float piv[kP];
-    const int I = threadIdx.x >> 4, J = threadIdx.x & 15;
-    const bool low = J <= I, diag = I == J;
-    const int R = low ? I : J, C = low ? J : I;      // the thread's tile: (R, C) of A (low) or of X
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool dwarp = tid >= 512;
+    const int I = tid & 15, J = (tid >> 5) & 15, h = 2 * ((tid >> 4) & 1);
+    const bool low = J < I, off = J != I;
+    const int R = low ? I : J, C = low ? J : I;      // a worker's tile: (R, C) of A (low) or of X
     const int nt = (int)(n - k0 - nb < kP ? n - k0 - nb : kP);          // rows of Xtop
     // the previous panel's kernel updated this block column
     grid_dependency_wait();
-    // every load before the first store to shared memory: one trip to L2
-    float v[kP * kP / 256], w[kP * kP / 256];
+    if (!dwarp) {
+        // every load before the first store to shared memory: one trip to L2
+        float v[kP * kP / 512], w[kP * kP / 512];
 #pragma unroll
-    for (int e = 0; e < kP * kP / 256; e++) {
-        const int r = e * 4 + (threadIdx.x >> 6), c = threadIdx.x & 63;
-        v[e] = r < nb && c <= r ? A[(k0 + r) * n + k0 + c] : r == c ? 1.0f : 0.0f;
-        w[e] = r < nt ? A[(k0 + nb + r) * n + k0 + c] : 0.0f;
-    }
-#pragma unroll
-    for (int e = 0; e < kP * kP / 256; e++) {
-        const int r = e * 4 + (threadIdx.x >> 6), c = threadIdx.x & 63;
-        sl[r * kPad + c] = v[e];
-        st[r * kPad + c] = w[e];
-    }
-    __syncthreads();
-    float t[4][4], xd[4][4];                         // xd: the diagonal tile of X
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-        float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (low) q = *reinterpret_cast<const float4*>(sl + (4 * R + i) * kPad + 4 * C);
-        t[i][0] = q.x;
-        t[i][1] = q.y;
-        t[i][2] = q.z;
-        t[i][3] = q.w;
-#pragma unroll
-        for (int j = 0; j < 4; j++) xd[i][j] = i == j ? 1.0f : 0.0f;
-    }
-    int bad = 0;
-#pragma unroll 1
-    for (int b = 0; b < kP / 4; b++) {
-        if (diag && I == b) {
-            float p[4], ip[4], m[4][4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const bool ok = t[j][j] > 0.0f && t[j][j] <= 3.402823466e38f;
-                bad |= !ok;
-                p[j] = ok ? t[j][j] : 1.0f;
-                ip[j] = rcp_fast(p[j]);
-#pragma unroll
-                for (int i = j + 1; i < 4; i++) m[i][j] = __fmul_rn(t[i][j], ip[j]);
-#pragma unroll
-                for (int i = j + 1; i < 4; i++)
-#pragma unroll
-                    for (int l = j + 1; l <= i; l++) t[i][l] = __fmaf_rn(-m[i][j], t[l][j], t[i][l]);
-            }
-            *reinterpret_cast<float4*>(sip) = make_float4(ip[0], ip[1], ip[2], ip[3]);
-            *reinterpret_cast<float4*>(sm) = make_float4(m[1][0], m[2][0], m[2][1], m[3][0]);
-            *reinterpret_cast<float2*>(sm + 4) = make_float2(m[3][1], m[3][2]);
-#pragma unroll
-            for (int j = 0; j < 4; j++) t[j][j] = p[j];
-#pragma unroll
-            for (int i = 1; i < 4; i++)
-#pragma unroll
-                for (int j = 0; j < i; j++) t[i][j] = m[i][j];     // M_bb stays in the tile
+        for (int e = 0; e < kP * kP / 512; e++) {
+            const int r = e * 8 + (tid >> 6), c = tid & 63;
+            v[e] = r < nb && c <= r ? A[(k0 + r) * n + k0 + c] : r == c ? 1.0f : 0.0f;
+            w[e] = r < nt ? A[(k0 + nb + r) * n + k0 + c] : 0.0f;
         }
-        __syncthreads();
-        // W = A M_bb^-T below the block; X's row b, held transposed, takes the same steps
-        if (J == b) {
-            if (!diag) {
-                const float4 ma = *reinterpret_cast<const float4*>(sm), ip = *reinterpret_cast<const float4*>(sip);
-                const float2 mb = *reinterpret_cast<const float2*>(sm + 4);
-                const int dst = low ? kW : kX, T = low ? R : C;
 #pragma unroll
-                for (int i = 0; i < 4; i++) {
-                    t[i][1] = __fmaf_rn(-t[i][0], ma.x, t[i][1]);
-                    t[i][2] = __fmaf_rn(-t[i][0], ma.y, t[i][2]);
-                    t[i][3] = __fmaf_rn(-t[i][0], ma.w, t[i][3]);
-                    t[i][2] = __fmaf_rn(-t[i][1], ma.z, t[i][2]);
-                    t[i][3] = __fmaf_rn(-t[i][1], mb.x, t[i][3]);
-                    t[i][3] = __fmaf_rn(-t[i][2], mb.y, t[i][3]);
-                    sb[dst + i][T] = make_float4(t[i][0], t[i][1], t[i][2], t[i][3]);
-                    if (low)
-                        sb[kMul + i][T] = make_float4(__fmul_rn(t[i][0], ip.x), __fmul_rn(t[i][1], ip.y),
-                                                 __fmul_rn(t[i][2], ip.z), __fmul_rn(t[i][3], ip.w));
+        for (int e = 0; e < kP * kP / 512; e++) {
+            const int r = e * 8 + (tid >> 6), c = tid & 63;
+            sl[r * kPad + c] = v[e];
+            st[r * kPad + c] = w[e];
+        }
+    }
+    potrf_barrier();
+    int bad = 0;
+    if (dwarp) {
+        u64 t2[4][4];                                // lane T: A's diagonal tile, each entry as two sums
+        float t[4][4], xd[4][4];                     // factored, and X's diagonal tile
+        const int T = lane & 15;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const float4 q = *reinterpret_cast<const float4*>(sl + (4 * T + i) * kPad + 4 * T);
+            t2[i][0] = pack2(q.x, 0.0f);
+            t2[i][1] = pack2(q.y, 0.0f);
+            t2[i][2] = pack2(q.z, 0.0f);
+            t2[i][3] = pack2(q.w, 0.0f);
+#pragma unroll
+            for (int j = 0; j < 4; j++) t[i][j] = xd[i][j] = i == j ? 1.0f : 0.0f;
+        }
+#pragma unroll 1
+        for (int b = 0; b < kP / 4; b++) {
+            if (lane == b) {
+                float p[4], ip[4], m[4][4];
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+#pragma unroll
+                    for (int j = 0; j <= i; j++) t[i][j] = sum2(t2[i][j]);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const bool ok = __float_as_uint(t[j][j]) - 1u < 0x7f7fffffu;      // positive and finite
+                    bad |= !ok;
+                    p[j] = ok ? t[j][j] : 1.0f;
+                    ip[j] = rcp_fast(p[j]);
+#pragma unroll
+                    for (int i = j + 1; i < 4; i++) m[i][j] = __fmul_rn(t[i][j], ip[j]);
+#pragma unroll
+                    for (int i = j + 1; i < 4; i++)
+#pragma unroll
+                        for (int l = j + 1; l <= i; l++) t[i][l] = __fmaf_rn(-m[i][j], t[l][j], t[i][l]);
                 }
-            } else {
+                *reinterpret_cast<float4*>(sip) = make_float4(ip[0], ip[1], ip[2], ip[3]);
+                *reinterpret_cast<float4*>(sm) = make_float4(m[1][0], m[2][0], m[2][1], m[3][0]);
+                *reinterpret_cast<float2*>(sm + 4) = make_float2(m[3][1], m[3][2]);
+#pragma unroll
+                for (int j = 0; j < 4; j++) t[j][j] = p[j];
+#pragma unroll
+                for (int i = 1; i < 4; i++)
+#pragma unroll
+                    for (int j = 0; j < i; j++) t[i][j] = m[i][j];     // M_bb stays in the tile
+            }
+            potrf_barrier();
+            if (lane == b) {
                 // X's diagonal tile M_bb^-1 (unit lower), transposed for the update
                 xd[1][0] = -t[1][0];
                 xd[2][1] = -t[2][1];
@@ -291,72 +300,156 @@ __global__ void __launch_bounds__(256) potrf_kernel(float* A, int64_t n, int64_t
                     piv[4 * b + j] = t[j][j];
                 }
             }
-        }
-        __syncthreads();
-        if (R > b && (low ? C > b : C <= b)) {
-            // A: t[i][j] -= m_(R i) . W_(C j);  X^T: t[i][j] -= X_b^T_(C i) . m_(R j)
-            const int u = low ? kMul : kX, y = low ? kW : kMul, tu = low ? R : C, ty = low ? C : R;
-            float4 mr[4], yc[4];
+            potrf_barrier();
+            if (T > b) {
+                float4 mr[4], yc[4];
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
-                mr[i] = sb[u + i][tu];
-                yc[i] = sb[y + i][ty];
+                for (int i = 0; i < 4; i++) {
+                    mr[i] = sb[kMul + i][T];
+                    yc[i] = sb[kW + i][T];
+                }
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+#pragma unroll
+                    for (int j = 0; j <= i; j++) {
+                        t2[i][j] = fma2(pack2(mr[i].x, mr[i].y), pack2(yc[j].x, yc[j].y), t2[i][j]);
+                        t2[i][j] = fma2(pack2(mr[i].z, mr[i].w), pack2(yc[j].z, yc[j].w), t2[i][j]);
+                    }
             }
+        }
+        potrf_barrier();
+        potrf_barrier();                             // the workers' sqrt p and 1 / sqrt p
+        const float* sq = &sb[0][0].x;
+        if (lane < 16) {
 #pragma unroll
             for (int i = 0; i < 4; i++)
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    t[i][j] = __fmaf_rn(-mr[i].x, yc[j].x, t[i][j]);
-                    t[i][j] = __fmaf_rn(-mr[i].y, yc[j].y, t[i][j]);
-                    t[i][j] = __fmaf_rn(-mr[i].z, yc[j].z, t[i][j]);
-                    t[i][j] = __fmaf_rn(-mr[i].w, yc[j].w, t[i][j]);
-                }
+                for (int j = 0; j <= i; j++)
+                    sl[(4 * T + i) * kPad + 4 * T + j] = i == j ? sq[4 * T + j] : __fmul_rn(t[i][j], sq[4 * T + j]);
         }
-    }
-    // L into the block, Linv = diag(1 / sqrt p) X into shared and global memory
-    __syncthreads();
-    float* sq = &sb[0][0].x;                         // sqrt p, then 1 / sqrt p
-    if (threadIdx.x < kP) {
-        sq[threadIdx.x] = __fsqrt_rn(piv[threadIdx.x]);
-        sq[kP + threadIdx.x] = __frsqrt_rn(piv[threadIdx.x]);
-    }
-    __syncthreads();
+        potrf_barrier();
+        potrf_barrier();                             // L is read
+        if (lane < 16) {
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        const int r = 4 * R + i;
-        if (low) {
+            for (int i = 0; i < 4; i++) {
+                const int r = 4 * T + i;
+                float o[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int c = 4 * C + j;
-                // W = M p, so below the diagonal tile L = M sqrt p = W / sqrt p
-                const float o = !diag ? __fmul_rn(t[i][j], sq[kP + c]) : r == c ? sq[c] : __fmul_rn(t[i][j], sq[c]);
-                if (r < nb && c <= r) A[(k0 + r) * n + k0 + c] = o;
+                for (int j = 0; j < 4; j++) o[j] = j <= i ? __fmul_rn(xd[i][j], sq[kP + r]) : 0.0f;
+                const float4 x = make_float4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<float4*>(sl + r * kPad + 4 * T) = x;
+                *reinterpret_cast<float4*>(Linv + r * kP + 4 * T) = x;
             }
         }
-        if (!low || diag) {
-            const float q = sq[kP + r];
-            float o[4];
+    } else {
+        u64 t2[2][4];                                // rows h, h + 1 of the tile, each entry as two sums
 #pragma unroll
-            for (int j = 0; j < 4; j++) o[j] = 4 * C + j <= r ? __fmul_rn(diag ? xd[i][j] : t[j][i], q) : 0.0f;
-            const float4 x = make_float4(o[0], o[1], o[2], o[3]), z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            *reinterpret_cast<float4*>(sl + r * kPad + 4 * C) = x;
-            *reinterpret_cast<float4*>(Linv + r * kP + 4 * C) = x;
-            if (!diag) {                              // the upper part: zero
-                *reinterpret_cast<float4*>(sl + (4 * C + i) * kPad + 4 * R) = z;
-                *reinterpret_cast<float4*>(Linv + (4 * C + i) * kP + 4 * R) = z;
+        for (int i = 0; i < 2; i++) {
+            float4 q = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (low) q = *reinterpret_cast<const float4*>(sl + (4 * R + h + i) * kPad + 4 * C);
+            t2[i][0] = pack2(q.x, 0.0f);
+            t2[i][1] = pack2(q.y, 0.0f);
+            t2[i][2] = pack2(q.z, 0.0f);
+            t2[i][3] = pack2(q.w, 0.0f);
+        }
+        float t[2][4] = {};                          // solved
+#pragma unroll 1
+        for (int b = 0; b < kP / 4; b++) {
+            if (J == b) {
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+#pragma unroll
+                    for (int j = 0; j < 4; j++) t[i][j] = sum2(t2[i][j]);
+            }
+            potrf_barrier();
+            // W = A M_bb^-T below the block; X's row b, held transposed, takes the same steps
+            if (J == b && off) {
+                const float4 ma = *reinterpret_cast<const float4*>(sm), ip = *reinterpret_cast<const float4*>(sip);
+                const float2 mb = *reinterpret_cast<const float2*>(sm + 4);
+                const int dst = (low ? kW : kX) + h;
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    t[i][1] = __fmaf_rn(-t[i][0], ma.x, t[i][1]);
+                    t[i][2] = __fmaf_rn(-t[i][0], ma.y, t[i][2]);
+                    t[i][3] = __fmaf_rn(-t[i][0], ma.w, t[i][3]);
+                    t[i][2] = __fmaf_rn(-t[i][1], ma.z, t[i][2]);
+                    t[i][3] = __fmaf_rn(-t[i][1], mb.x, t[i][3]);
+                    t[i][3] = __fmaf_rn(-t[i][2], mb.y, t[i][3]);
+                    sb[dst + i][I] = make_float4(t[i][0], t[i][1], t[i][2], t[i][3]);
+                    if (low)                         // (X's tiles have no multipliers)
+                        sb[kMul + h + i][I] = make_float4(__fmul_rn(t[i][0], -ip.x), __fmul_rn(t[i][1], -ip.y),
+                                                          __fmul_rn(t[i][2], -ip.z), __fmul_rn(t[i][3], -ip.w));
+                }
+            }
+            potrf_barrier();
+            if (low ? J > b : off && J > b && I <= b) {
+                // A: t[i][j] -= m_(R i) . W_(C j);  X^T: t[i][j] -= X_b^T_(C i) . m_(R j)
+                const int u = (low ? kMul : kX) + h, y = low ? kW : kMul;
+                float4 mr[2], yc[4];
+#pragma unroll
+                for (int i = 0; i < 2; i++) mr[i] = sb[u + i][I];
+#pragma unroll
+                for (int j = 0; j < 4; j++) yc[j] = sb[y + j][J];
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        t2[i][j] = fma2(pack2(mr[i].x, mr[i].y), pack2(yc[j].x, yc[j].y), t2[i][j]);
+                        t2[i][j] = fma2(pack2(mr[i].z, mr[i].w), pack2(yc[j].z, yc[j].w), t2[i][j]);
+                    }
+            }
+        }
+        // L into the block, Linv = diag(1 / sqrt p) X into shared and global memory
+        potrf_barrier();
+        float* sq = &sb[0][0].x;                     // sqrt p, then 1 / sqrt p
+        if (tid < kP) {
+            sq[tid] = __fsqrt_rn(piv[tid]);
+            sq[kP + tid] = __frsqrt_rn(piv[tid]);
+        }
+        potrf_barrier();
+        if (low) {
+            // W = M p, so below the diagonal tile L = M sqrt p = W / sqrt p
+            const float4 q = *reinterpret_cast<const float4*>(sq + kP + 4 * C);
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+                *reinterpret_cast<float4*>(sl + (4 * R + h + i) * kPad + 4 * C) =
+                    make_float4(__fmul_rn(t[i][0], q.x), __fmul_rn(t[i][1], q.y), __fmul_rn(t[i][2], q.z),
+                                __fmul_rn(t[i][3], q.w));
+        }
+        potrf_barrier();
+#pragma unroll
+        for (int e = 0; e < kP * kP / 512; e++) {
+            const int r = e * 8 + (tid >> 6), c = tid & 63;
+            if (r < nb && c <= r) A[(k0 + r) * n + k0 + c] = sl[r * kPad + c];
+        }
+        potrf_barrier();
+        if (!low && off) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int r = 4 * R + j;
+                const float2 x = make_float2(__fmul_rn(t[0][j], sq[kP + r]), __fmul_rn(t[1][j], sq[kP + r]));
+                *reinterpret_cast<float2*>(sl + r * kPad + 4 * C + h) = x;
+                *reinterpret_cast<float2*>(Linv + r * kP + 4 * C + h) = x;
+            }
+            const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);       // the upper part
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                *reinterpret_cast<float4*>(sl + (4 * C + h + i) * kPad + 4 * R) = z;
+                *reinterpret_cast<float4*>(Linv + (4 * C + h + i) * kP + 4 * R) = z;
             }
         }
     }
     if (bad && status) atomicOr(status, 4);
-    __syncthreads();
-    // Xtop: rows I + 16 i, columns J + 16 j of the solved panel
-    if (nt > 0) {
+    potrf_barrier();
+    // Xtop: rows r + 16 i, columns J + 16 j of the solved panel
+    if (nt > 0 && tid < 256) {
         float o[4][4];
-        tile_dot<16, 16, true>(st, I, sl, J, kP, o);
+        const int r = tid >> 4, c = tid & 15;
+        tile_dot<16, 16, true>(st, r, sl, c, kP, o);
 #pragma unroll
         for (int i = 0; i < 4; i++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) Xtop[(I + 16 * i) * kP + J + 16 * j] = o[i][j];
+            for (int j = 0; j < 4; j++) Xtop[(r + 16 * i) * kP + c + 16 * j] = o[i][j];
     }
 }
 
@@ -1192,7 +1285,7 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     for (int64_t k0 = 0; k0 < n; k0 += kP) {
         const int nb = (int)imin64(kP, n - k0);
         // scheduled while the last panel kernel runs, ordered after its writes
-        if ((e = launch_dependent_smem(potrf_kernel, 1, 256, kPotrfSmem, c, U, n, k0, nb, Linv, Xtop, status)) != cudaSuccess)
+        if ((e = launch_dependent_smem(potrf_kernel, 1, kPotrfThreads, kPotrfSmem, c, U, n, k0, nb, Linv, Xtop, status)) != cudaSuccess)
             return e;
         const int64_t rest = n - k0 - nb;
         if (rest > 0) {
