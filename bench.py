@@ -276,8 +276,7 @@ def run_gpu(args, rank, world):
         if events is not None:
             events[1].record(stream)
 
-    # two reductions and two sweeps (the workspace reset is a memset; these
-    # shapes need no swizzle pad kernel)
+    # two reductions and two sweeps (the workspace reset is a memset)
     launches_per_step = 4 if st.pipelined else 1
 
     for _ in range(args.warmup):

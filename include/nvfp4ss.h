@@ -167,7 +167,8 @@ size_t nvfp4_dynamic_workspace(void);
  * reduction into the sweep for dynamic activation quantisation (the paper's
  * kernels leave fusion as future work, Sec. 5.2).  One cooperative launch (all
  * CTAs resident) with a grid barrier in between, preceded by a 4-byte
- * cudaMemsetAsync of the barrier counter in the workspace.
+ * cudaMemsetAsync of the barrier counter in the workspace; up to 65536 elements with a
+ * default window, one thread-block cluster, which uses no workspace.
  *   S_out       device float written with S (also returned implicitly by the codes).
  *   status_dev  optional device int: bit 0 OR-ed in for NaN/inf input, bit 1 if the
  *               grid barrier timed out (about a second; the outputs are then not
@@ -387,10 +388,10 @@ nvfp4_status nvfp4_dequantize(const uint8_t* codes, const uint8_t* sf, nvfp4_sf_
  *   workspace   device bytes, at least nvfp4_ldlq_prepare_workspace(n).
  * Cost: n^3/3 fp32 multiply-adds (blocked Cholesky, 64-wide panels).  The
  * trailing updates run on the tensor cores as three TF32 products per term
- * (products to ~2^-21 relative, accumulated in fp32) when n % 4 == 0 and H,
- * U are 16-byte aligned, else on the FP32 pipe.
+ * (products to ~2^-21 relative, accumulated in fp32) when n % 4 == 0 and U is
+ * 16-byte aligned, else on the FP32 pipe.
  * The factorization's critical chain runs on a high-priority stream the library
- * creates on the first call on a device and keeps (with four events) for the
+ * creates on the first call on a device and keeps (with five events) for the
  * process; it is forked from and joined back into `stream`, so the call stays
  * ordered on `stream` and can be captured in a CUDA graph -- make the first
  * call on each device outside a capture.  Concurrent calls on one device are

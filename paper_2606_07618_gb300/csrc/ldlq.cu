@@ -7,8 +7,9 @@
 //   lambda = damp * mean(diag H); perm = channels by (diag desc, index asc);
 //   A = J H_pi J + lambda I (J reverses the order), A = L L^T by a blocked
 //   right-looking Cholesky (64-wide panels: diagonal block factor and inverse
-//   in one CTA, panel solve by the inverse, trailing update by the K<=64 GEMM
-//   below on lower tiles only); then, in place,
+//   in one CTA, panel solve by the inverse and update of the next block column in
+//   one kernel, the rest of the trailing update by a K<=64 GEMM on lower tiles
+//   only); then, in place,
 //   H_pi = (U + I) D (U + I)^T with U_ik = L[n-1-i][n-1-k] / L[n-1-k][n-1-k]
 //   (J L J is upper triangular) and D_k = L[n-1-k][n-1-k]^2.
 // Quantize (rows independent):
@@ -176,6 +177,7 @@ __device__ __forceinline__ float sum2(u64 v) {
     unpack2(v, lo, hi);
     return __fadd_rn(lo, hi);
 }
+
 // One panel's sequential part, in one CTA: the Cholesky factor of the nb x nb
 // diagonal block at k0 (lower, in place), its inverse Linv (64 x 64, lower), and the
 // solved panel of the next 64 rows, Xtop = A[k0 + nb .., k0 ..] Linv^T.
