@@ -84,14 +84,13 @@ nvfp4_status check_shape(int64_t rows, int64_t cols, int block, Shape* sh) {
     return NVFP4_OK;
 }
 
-// Extra arguments of the dynamic-scale variants (global scale computed in the launch).
+// Extra arguments of the dynamic-scale variants (global scale computed by the call).
 struct DynArgs {
     float fp8_div;
     float* S_out;
     int* status_dev;
     void* workspace;
     size_t ws_bytes;
-    unsigned wait_extra;     // 0 except in nvfp4_selftest_wait_timeout
 };
 
 nvfp4_status quantize_common(int method, const void* x, nvfp4_dtype dt, int64_t rows, int64_t cols, int block,
@@ -188,8 +187,7 @@ nvfp4_status quantize_common(int method, const void* x, nvfp4_dtype dt, int64_t 
     p.status_dev = nullptr;
     p.part_max = nullptr;
     p.part_bad = nullptr;
-    p.barrier = nullptr;
-    p.wait_extra = 0;
+    p.nparts = 0;
     const int dti = dt == NVFP4_IN_BF16 ? 0 : 1, obji = obj == NVFP4_OBJ_WMSE ? 1 : 0;
     cudaError_t e;
     if (dyn) {
@@ -198,8 +196,6 @@ nvfp4_status quantize_common(int method, const void* x, nvfp4_dtype dt, int64_t 
         p.status_dev = dyn->status_dev;
         p.part_max = static_cast<float*>(dyn->workspace);
         p.part_bad = reinterpret_cast<int*>(p.part_max + kAmaxParts);
-        p.barrier = reinterpret_cast<unsigned*>(p.part_bad + kAmaxParts);
-        p.wait_extra = dyn->wait_extra;
         e = launch_quantize_dynamic(p, dti, method, obji, block, sms, static_cast<cudaStream_t>(stream));
     } else {
         e = launch_quantize(p, dti, method, obji, block, sms, static_cast<cudaStream_t>(stream));
@@ -268,7 +264,7 @@ nvfp4_status scalesweep_quantize_dynamic(const void* x, nvfp4_dtype dt, int64_t 
                                          int win_lo, int win_hi, float* S_out, int* status_dev, void* workspace,
                                          size_t ws_bytes, uint8_t* codes, uint8_t* sf_linear, uint8_t* sf_swizzled,
                                          float* block_loss, void* stream) {
-    const DynArgs d{fp8_div, S_out, status_dev, workspace, ws_bytes, 0};
+    const DynArgs d{fp8_div, S_out, status_dev, workspace, ws_bytes};
     return quantize_common(0, x, dt, rows, cols, block, nullptr, obj, w, w_row_stride, win_lo, win_hi, codes,
                            sf_linear, sf_swizzled, block_loss, stream, &d);
 }
@@ -438,12 +434,8 @@ nvfp4_status nvfp4_selftest_wait_timeout(int which, const void* x, int64_t rows,
                                          int* status_dev, void* workspace, size_t ws_bytes, uint8_t* codes,
                                          uint8_t* sf_linear, void* stream) {
     if ((which != 0 && which != 1) || !status_dev || rows <= 0 || cols <= 0) return NVFP4_ERR_INVALID_ARG;
-    if (which == 0) {
-        const DynArgs d{256.0f, S, status_dev, workspace, ws_bytes, 1};
-        return quantize_common(0, x, NVFP4_IN_BF16, rows, cols, 16, nullptr, NVFP4_OBJ_MSE, nullptr, 0,
-                               NVFP4_WINDOW_DEFAULT, NVFP4_WINDOW_DEFAULT, codes, sf_linear, nullptr, nullptr, stream,
-                               &d);
-    }
+    if (which == 0 && (!workspace || ws_bytes < kDynWorkspace)) return NVFP4_ERR_INVALID_ARG;
+    // the grouped launch is the one sweep with a wait in device code: both settings run it
     const nvfp4_group_tensor t{x, rows, cols, nullptr, 0, codes, sf_linear, nullptr};
     return group_common(0, &t, 1, NVFP4_IN_BF16, 16, NVFP4_OBJ_MSE, 256.0f, S, status_dev, workspace, ws_bytes,
                         stream, 1, NVFP4_GROUP_SCHEDULE_TWO_PHASE);
@@ -453,7 +445,7 @@ nvfp4_status absmax_quantize_dynamic(const void* x, nvfp4_dtype dt, int64_t rows
                                      float fp8_div, float* S_out, int* status_dev, void* workspace, size_t ws_bytes,
                                      uint8_t* codes, uint8_t* sf_linear, uint8_t* sf_swizzled, float* block_loss,
                                      void* stream) {
-    const DynArgs d{fp8_div, S_out, status_dev, workspace, ws_bytes, 0};
+    const DynArgs d{fp8_div, S_out, status_dev, workspace, ws_bytes};
     return quantize_common(1, x, dt, rows, cols, block, nullptr, NVFP4_OBJ_MSE, nullptr, 0, 0, 0, codes, sf_linear,
                            sf_swizzled, block_loss, stream, &d);
 }

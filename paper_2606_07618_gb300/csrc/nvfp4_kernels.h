@@ -27,22 +27,21 @@ struct QuantParams {
     uint8_t* sf_linear;
     uint8_t* sf_swizzled;
     float* block_loss;
-    // dynamic (per-call) global scale, computed inside the sweep launch
+    // dynamic (per-call) global scale, folded by the sweep from the reduction's partials
     float fp8_div;
     float* S_out;
     int* status_dev;
     float* part_max;
     int* part_bad;
-    unsigned* barrier;
-    unsigned wait_extra;     // added to the barrier's arrival target; 0 except in the wait self-test
+    int nparts;
 };
 
 // dtype 0 bf16 / 1 f32; method 0 ScaleSweep / 1 AbsMax / 2 four-over-six;
 // obj 0 MSE / 1 WMSE; block 16/32/64; sms = multiprocessor count.
 cudaError_t launch_quantize(const QuantParams& p, int dtype, int method, int obj, int block, int sms,
                             cudaStream_t s);
-// Same with the global scale computed in the launch (method 0 or 1; p.S unused,
-// p.S_out/part_max/part_bad/barrier in the caller's workspace).
+// Same with the global scale computed by the call (method 0 or 1; p.S unused,
+// p.part_max/part_bad in the caller's workspace, p.nparts set here).
 cudaError_t launch_quantize_dynamic(const QuantParams& p, int dtype, int method, int obj, int block, int sms,
                                     cudaStream_t s);
 // Fill the derived fields of p (window mode, row/column need, fast divider).
@@ -52,7 +51,11 @@ void prepare_quant_params(QuantParams& p, int method, int obj, int block, bool* 
 cudaError_t launch_global_scale(const void* x, int dtype, int64_t n, float fp8_div, float* S_out,
                                 int* status_dev, void* ws, int sms, cudaStream_t s);
 constexpr int kAmaxParts = 1024;   // partial slots in the workspace
-// Dynamic-scale workspace: partial maxima, partial flags, barrier counter.
+// The partial maxima and flags of n elements (n a multiple of 16 bytes' worth or with a
+// tail): at most kAmaxParts of them, *nparts written.
+cudaError_t launch_amax_partials(const void* x, int dtype, int64_t n, float* part_max, int* part_bad, int* nparts,
+                                 int sms, cudaStream_t s);
+// Dynamic-scale workspace: partial maxima and flags (and 256 bytes nothing uses).
 constexpr size_t kDynWorkspace = (size_t)kAmaxParts * 8 + 256;
 
 // Same two kernels with caller-chosen partial slots and grid (grid <= slots).

@@ -1,9 +1,9 @@
-// Sweep launches that compute the per-call global scale themselves (one
-// cooperative launch instead of amax reduction + final + sweep): the fused
-// dynamic-activation path.  The grid barrier counter lives in the caller's
-// workspace and is zeroed with an asynchronous memset right before the launch.
-// Tensors of at most 4096 segments (a decode batch) take one thread-block cluster
-// instead, whose barrier is the hardware's.
+// Sweeps with a per-call global scale (the dynamic-activation path).  Tensors of at
+// most 4096 segments (a decode batch) with a default window: one launch of one
+// thread-block cluster.  Larger ones, and explicit windows: the global scale's
+// reduction, then the sweep as its programmatic dependent, whose CTAs fold the
+// partial maxima themselves: two ordinary launches, no counter to reset, no wait in
+// device code.
 #include "quantize_kernel.cuh"
 
 namespace nvfp4 {
@@ -124,9 +124,8 @@ static cudaError_t launch_cluster(const QuantParams& p, cudaStream_t s) {
 
 template <int DT, int METHOD, int OBJ, int BLOCK, int FIX>
 static cudaError_t launch_dyn(const QuantParams& p_in, int sms, cudaStream_t s) {
-    // the wait self-test needs the barrier in global memory
     if constexpr (FIX == 1) {
-        if (p_in.nseg <= (int64_t)kClusterCtas * kClusterThreads && p_in.wait_extra == 0) {
+        if (p_in.nseg <= (int64_t)kClusterCtas * kClusterThreads) {
             const cudaError_t e = launch_cluster<DT, METHOD, OBJ, BLOCK>(p_in, s);
             if (e != cudaErrorNotSupported) return e;
         }
@@ -134,15 +133,11 @@ static cudaError_t launch_dyn(const QuantParams& p_in, int sms, cudaStream_t s) 
     static std::atomic<int> occ_cache[kOccDevices];
     const int occ = occupancy_per_sm(occ_cache, quantize_kernel<DT, METHOD, OBJ, BLOCK, FIX, 1>, 256);
     QuantParams p = p_in;
-    int64_t grid = (p.nseg + 255) / 256;
-    if (grid > (int64_t)sms * occ) grid = (int64_t)sms * occ;   // every CTA resident: the barrier can complete
-    if (grid > kAmaxParts) grid = kAmaxParts;
-    if (grid < 1) grid = 1;
-    cudaError_t e = cudaMemsetAsync(p.barrier, 0, sizeof(unsigned), s);
+    const cudaError_t e = launch_amax_partials(p.x, DT, p.nseg * 16, p.part_max, p.part_bad, &p.nparts, sms, s);
     if (e != cudaSuccess) return e;
-    void* args[] = {(void*)&p};
-    return cudaLaunchCooperativeKernel((const void*)quantize_kernel<DT, METHOD, OBJ, BLOCK, FIX, 1>, dim3((unsigned)grid),
-                                       dim3(256), args, 0, s);
+    int64_t grid = (p.nseg + 255) / 256;
+    if (grid > (int64_t)sms * occ) grid = (int64_t)sms * occ;
+    return launch_dependent(quantize_kernel<DT, METHOD, OBJ, BLOCK, FIX, 1>, grid, 256, s, p);
 }
 
 template <int DT, int METHOD, int OBJ>

@@ -434,16 +434,6 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv& d) {
 }
 
 
-// Dynamic (per-call) global scale inside the sweep launch: every CTA folds the
-// max |x| of its grid-stride share into one partial, all CTAs meet at a grid
-// barrier (cooperative launch, so all are resident; the counter is zeroed by
-// the host before the launch), then each CTA folds all partials into the same
-// S = fl(amax / fl(6 D)).  The barrier wait is bounded by the global timer
-// (1 s): on timeout the kernel sets bit 1 of the status word and returns
-// without writing outputs.  p.wait_extra raises the arrival target (0 in every
-// real call; the wait self-test uses it to make the wait run out).
-constexpr unsigned long long kBarrierWaitNs = 1000000000ull;
-
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -456,85 +446,21 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     return v;
 }
 
-template <int DT>
-__device__ __forceinline__ bool dynamic_scale(const QuantParams& p, float& S_out) {
-    __shared__ uint32_t sm[32];
-    __shared__ int sb[32];
-    __shared__ int s_timeout;
-    constexpr int PER = DT == 0 ? 8 : 4;
-    const int64_t nvec = (p.nseg * 16) / PER;
-    const uint4* xv = static_cast<const uint4*>(p.x);
-    float m = 0.0f;
-    int bad = 0;
-    auto fold = [&](const uint4& u) {
-        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            if (DT == 0) {
-                const float a = bf16lo(w[j]), b = bf16hi(w[j]);
-                bad |= (!isfinite(a)) | (!isfinite(b));
-                m = fmaxf(m, fmaxf(fabsf(a), fabsf(b)));
-            } else {
-                const float a = __uint_as_float(w[j]);
-                bad |= !isfinite(a);
-                m = fmaxf(m, fabsf(a));
-            }
-        }
-    };
-    const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + 7 * gstride < nvec; i += 8 * gstride) {      // eight 16-byte loads in flight per thread
-        uint4 u[8];
-#pragma unroll
-        for (int j = 0; j < 8; j++) u[j] = ld_stream16(xv + i + j * gstride);
-#pragma unroll
-        for (int j = 0; j < 8; j++) fold(u[j]);
-    }
-    for (; i < nvec; i += gstride) fold(ld_stream16(xv + i));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    uint32_t mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-    int wb = __reduce_or_sync(0xffffffffu, (unsigned)bad);
-    if (lane == 0) {
-        sm[warp] = mb;
-        sb[warp] = wb;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t v = 0;
-        int b = 0;
-        for (int i = 0; i < nw; i++) {
-            v = max(v, sm[i]);
-            b |= sb[i];
-        }
-        p.part_max[blockIdx.x] = __uint_as_float(v);
-        p.part_bad[blockIdx.x] = b;
-        __threadfence();
-        atomicAdd(p.barrier, 1u);
-        const unsigned long long t0 = globaltimer_ns();
-        int timeout = 0;
-        while (ld_acquire_u32(p.barrier) < gridDim.x + p.wait_extra) {
-            if (globaltimer_ns() - t0 > kBarrierWaitNs) {
-                timeout = 1;
-                break;
-            }
-            __nanosleep(128);
-        }
-        s_timeout = timeout;
-    }
-    __syncthreads();
-    if (s_timeout) {
-        if (threadIdx.x == 0 && p.status_dev) atomicOr(p.status_dev, 2);
-        return false;
-    }
+// Dynamic (per-call) global scale: every CTA folds the partial maxima that the
+// reduction before this grid wrote into the same S = fl(amax / fl(6 D)), and the
+// first one writes it and the status out.
+__device__ __forceinline__ float dynamic_scale(const QuantParams& p) {
+    __shared__ uint32_t sm[8];
+    __shared__ int sb[8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t v = 0;
     int b = 0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-        v = max(v, __float_as_uint(__ldcg(p.part_max + i)));
-        b |= __ldcg(p.part_bad + i);
+    for (int i = threadIdx.x; i < p.nparts; i += blockDim.x) {
+        v = max(v, ld_u32(p.part_max + i));          // non-negative floats order like their bit patterns
+        b |= (int)ld_u32(p.part_bad + i);
     }
     v = __reduce_max_sync(0xffffffffu, v);
     b = __reduce_or_sync(0xffffffffu, (unsigned)b);
-    __syncthreads();
     if (lane == 0) {
         sm[warp] = v;
         sb[warp] = b;
@@ -542,16 +468,17 @@ __device__ __forceinline__ bool dynamic_scale(const QuantParams& p, float& S_out
     __syncthreads();
     uint32_t amaxb = 0;
     int anyb = 0;
-    for (int i = 0; i < nw; i++) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
         amaxb = max(amaxb, sm[i]);
         anyb |= sb[i];
     }
-    S_out = __fdiv_rn(__uint_as_float(amaxb), __fmul_rn(6.0f, p.fp8_div));
+    const float S = __fdiv_rn(__uint_as_float(amaxb), __fmul_rn(6.0f, p.fp8_div));
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        p.S_out[0] = S_out;
+        p.S_out[0] = S;
         if (anyb && p.status_dev) atomicOr(p.status_dev, 1);
     }
-    return true;
+    return S;
 }
 
 // Zero the padding bytes of a swizzled scale buffer (rows past `rows` up to a
@@ -575,7 +502,7 @@ __device__ __forceinline__ void zero_pads(uint8_t* sf, int64_t rows, int64_t kb,
 }
 
 // quantize_kernel.  FIX = 1: default window (fixed length, unrolled, poison-padded table).
-// DYN = 1: the global scale is computed in this launch (see dynamic_scale).
+// DYN = 1: the global scale comes from the reduction launched before (dynamic_scale).
 // On bf16 input, AbsMax is held to 64 registers (4 CTAs per SM) and 4/6 to 80
 // (3 CTAs per SM): both are issue- and latency-bound, not register-bound (AbsMax
 // 0.0677 -> 0.0636 ms, 4/6 WMSE 0.120 -> 0.115 ms at 16384 x 8192; the
@@ -755,12 +682,7 @@ __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quanti
     __syncthreads();
     grid_dependency_wait();
 
-    float S;
-    if (DYN) {
-        if (!dynamic_scale<DT>(p, S)) return;
-    } else {
-        S = ld_f32(p.S);
-    }
+    const float S = DYN ? dynamic_scale(p) : ld_f32(p.S);
     float E = __frcp_rn(S);
     const bool usable = (S > 0.0f) && isfinite(S) && isfinite(E);
     if (!usable) E = 1.0f;                          // y = x: only signs (and sum w x^2) are emitted
@@ -772,7 +694,7 @@ __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quanti
     int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
     const bool wide = METHOD != 1 && wide_input(p.x);      // AbsMax: 2% slower with 32-byte loads
     Raw cur;
-    if (base + lane < p.nseg) load_raw<DT, DYN != 0>(p.x, base + lane, wide, cur);
+    if (base + lane < p.nseg) load_raw<DT, false>(p.x, base + lane, wide, cur);
 
     // 4/6 keeps a lane's weights while they come from the same address (the grid's
     // stride is a multiple of a row's segments where it can be): four 16-byte loads 64
@@ -786,9 +708,9 @@ __global__ void __launch_bounds__(256, quantize_min_blocks<METHOD, DT>()) quanti
         const int64_t g = base + lane;
         const bool valid = g < p.nseg;
         Raw nxt;
-        if (g + stride < p.nseg) load_raw<DT, DYN != 0>(p.x, g + stride, wide, nxt);
+        if (g + stride < p.nseg) load_raw<DT, false>(p.x, g + stride, wide, nxt);
 
-        quantize_segment<DT, METHOD, OBJ, BLOCK, FIX, DYN != 0>(p, tab, cur, g, valid, E2, usable, w2, wkey);
+        quantize_segment<DT, METHOD, OBJ, BLOCK, FIX, false>(p, tab, cur, g, valid, E2, usable, w2, wkey);
         cur = nxt;
     }
     zero_pads(p.sf_swizzled, p.rows, p.kb, p.kpad4, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride);

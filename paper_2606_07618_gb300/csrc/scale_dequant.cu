@@ -131,10 +131,8 @@ static cudaError_t launch_partial(const void* x, int dtype, int64_t n, float* pa
                             part_bad);
 }
 
-cudaError_t launch_global_scale(const void* x, int dtype, int64_t n, float fp8_div, float* S_out,
-                                int* status_dev, void* ws, int sms, cudaStream_t s) {
-    float* part_max = static_cast<float*>(ws);
-    int* part_bad = reinterpret_cast<int*>(part_max + kAmaxParts);
+cudaError_t launch_amax_partials(const void* x, int dtype, int64_t n, float* part_max, int* part_bad, int* nparts,
+                                 int sms, cudaStream_t s) {
     // 512-thread CTAs, 4 per SM, two loads in flight each: measured fastest of
     // 128/256/512 threads x 1/2/4/8 loads and of 32-byte loads on GB300
     constexpr int kThreads = 512;
@@ -144,9 +142,18 @@ cudaError_t launch_global_scale(const void* x, int dtype, int64_t n, float fp8_d
     if (grid > (int64_t)sms * 4) grid = (int64_t)sms * 4;
     if (grid > kAmaxParts) grid = kAmaxParts;
     if (grid < 1) grid = 1;
-    cudaError_t e = launch_partial(x, dtype, n, part_max, part_bad, (int)grid, kThreads, s);
+    *nparts = (int)grid;
+    return launch_partial(x, dtype, n, part_max, part_bad, (int)grid, kThreads, s);
+}
+
+cudaError_t launch_global_scale(const void* x, int dtype, int64_t n, float fp8_div, float* S_out,
+                                int* status_dev, void* ws, int sms, cudaStream_t s) {
+    float* part_max = static_cast<float*>(ws);
+    int* part_bad = reinterpret_cast<int*>(part_max + kAmaxParts);
+    int nparts = 0;
+    const cudaError_t e = launch_amax_partials(x, dtype, n, part_max, part_bad, &nparts, sms, s);
     if (e != cudaSuccess) return e;
-    return launch_final(part_max, part_bad, (int)grid, fp8_div, S_out, status_dev, s);
+    return launch_final(part_max, part_bad, nparts, fp8_div, S_out, status_dev, s);
 }
 
 cudaError_t launch_global_scale_parts(const void* x, int dtype, int64_t n, float fp8_div, float* S_out,
