@@ -161,18 +161,16 @@ nvfp4_status scalesweep_quantize(const void* x, nvfp4_dtype dt, int64_t rows, in
 size_t nvfp4_dynamic_workspace(void);
 
 /*
- * ScaleSweep quantisation with a per-call (dynamic) global scale computed in
- * the same launch: S = fl32(amax / fl32(6*fp8_div)) (Sec. 4.2.1) over the whole
+ * ScaleSweep quantisation with a per-call (dynamic) global scale computed by
+ * the same call: S = fl32(amax / fl32(6*fp8_div)) (Sec. 4.2.1) over the whole
  * tensor, then the sweep of scalesweep_quantize with that S.  This fuses the
  * reduction into the sweep for dynamic activation quantisation (the paper's
- * kernels leave fusion as future work, Sec. 5.2).  One cooperative launch (all
- * CTAs resident) with a grid barrier in between, preceded by a 4-byte
- * cudaMemsetAsync of the barrier counter in the workspace; up to 65536 elements with a
- * default window, one thread-block cluster, which uses no workspace.
+ * kernels leave fusion as future work, Sec. 5.2).  Two launches: the reduction,
+ * and the sweep as its programmatic dependent, which folds the partial maxima;
+ * up to 65536 elements with a default window, one launch of one thread-block cluster,
+ * which uses no workspace.
  *   S_out       device float written with S (also returned implicitly by the codes).
- *   status_dev  optional device int: bit 0 OR-ed in for NaN/inf input, bit 1 if the
- *               grid barrier timed out (about a second; the outputs are then not
- *               written -- a resident grid makes this unreachable in practice).
+ *   status_dev  optional device int: bit 0 OR-ed in for NaN/inf input.
  *   workspace   nvfp4_dynamic_workspace() bytes, 16-byte aligned, no initialisation.
  * Other arguments as scalesweep_quantize.  rows*cols == 0 launches nothing.
  * Concurrent calls must use distinct workspaces.
@@ -291,10 +289,10 @@ nvfp4_status absmax_quantize_group(const nvfp4_group_tensor* tensors, int count,
 
 /*
  * Self-test of the bounded device waits (failure detection; the paper has no
- * counterpart).  Runs scalesweep_quantize_dynamic (which = 0: bf16 x, block
- * 16, MSE, default window) or scalesweep_quantize_group with a dynamic scale
- * (which = 1: x as its one tensor, MSE) with the wait's arrival target raised
- * past what the launch can reach, so every device wait gives up after its
+ * counterpart).  Runs scalesweep_quantize_group with a dynamic scale (x as its
+ * one tensor: bf16, block 16, MSE; which = 0 or 1: the dynamic per-tensor call has
+ * no wait in device code, so both run this one) with the wait's arrival target
+ * raised past what the launch can reach, so every device wait gives up after its
  * limit (about a second): bit 1 is OR-ed into *status_dev (required here), the
  * waiting warps return without writing codes or scales, and the CUDA context
  * stays usable.  Arguments and buffers as in those calls; workspace of

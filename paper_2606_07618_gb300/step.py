@@ -8,7 +8,7 @@ every block (Sec. 4.2.2), writing packed E2M1 codes and E4M3 scales.
   * several tensors, or a single weight: ``scalesweep_quantize_group`` with
     in-launch scales (a layer's weights, the KV-cache/query tensors, ...);
   * a single activation tensor (``activation=True``): the fused
-    ``scalesweep_quantize_dynamic`` (amax and sweep in one cooperative launch).
+    ``scalesweep_quantize_dynamic`` (amax, then the sweep as its dependent launch).
 
 ``absmax`` runs the AbsMax baseline (Sec. 3.2) over the same tensors in the
 same launch shape, so the two can be compared call for call.  Every step runs
