@@ -6,6 +6,7 @@
 * Default windows, whose codes are scored an octave apart where they are normal (WMSE)
   and whose low end is left out once saturated terms rule it out, against the same
   codes scored one call each, with block scales from the smallest code to the largest.
+* The screened optimal scale against every segment scored.
 * Zeroed padding of the swizzled layout at rows and columns off its atoms.
 """
 import pytest
@@ -152,3 +153,34 @@ def test_swizzle_padding(B, rows, cols):
     off = ((r // 128) * kpad4 + k // 4) * 512 + (r % 32) * 16 + (r // 32 % 4) * 4 + k % 4
     want[off.reshape(-1)] = lin.reshape(-1)
     assert torch.equal(o["sf_swizzled"].cpu(), want)
+
+
+@pytest.mark.parametrize("block", [16, 32, 64])
+@pytest.mark.parametrize("kind", ["normal", "tails", "equal", "few", "zero_weights"])
+def test_optimal_screen(B, block, kind):
+    """The screened optimum against every segment scored: weights times 2^100 are past
+    the screen's range, and a power of two changes no rounding of the scored form."""
+    g = torch.Generator().manual_seed(block)
+    rows, cols = 64, 512
+    x = torch.randn(rows, cols, generator=g)
+    if kind == "tails":
+        x = x * torch.exp(torch.randn(rows, cols, generator=g))
+    elif kind == "equal":                              # every segment coincides: past the list
+        x = torch.sign(x) * torch.arange(1, rows + 1)[:, None] / 16
+    elif kind == "few":
+        x = torch.sign(x) * torch.randint(0, 4, (rows, cols), generator=g)
+    w = torch.exp(torch.randn(cols, generator=g))
+    if kind == "zero_weights":
+        w[torch.rand(cols, generator=g) < 0.6] = 0.0
+    x, S = x.to(torch.bfloat16).to(DEV), torch.ones(1, device=DEV)
+    nb = rows * cols // block
+    res = []
+    for f in (1.0, 2.0 ** 100):
+        o = (torch.empty(nb, device=DEV), torch.empty(nb, device=DEV), torch.empty(nb, dtype=torch.uint8, device=DEV),
+             torch.empty(nb, device=DEV))
+        B.nvfp4_optimal_scale(x, block, S, 1, (w * f).to(DEV), 0, *o)
+        res.append(o)
+    torch.cuda.synchronize()
+    (s1, l1, c1, f1), (s2, l2, c2, f2) = res
+    assert torch.equal(s1, s2) and torch.equal(c1, c2)
+    assert torch.equal(l1 * 2.0 ** 100, l2) and torch.equal(f1 * 2.0 ** 100, f2)
