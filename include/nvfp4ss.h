@@ -382,7 +382,7 @@ nvfp4_status nvfp4_dequantize(const uint8_t* codes, const uint8_t* sf, nvfp4_sf_
  *           replaced by 1 so the outputs stay finite, but they are not a
  *           factorization then).
  *           |= 16 if a tensor-core update's bounded wait ran out (about a
- *           second; that update is then not applied).
+ *           second; that update is then incomplete).
  *   workspace   device bytes, at least nvfp4_ldlq_prepare_workspace(n).
  * Cost: n^3/3 fp32 multiply-adds (blocked Cholesky, 64-wide panels).  The
  * trailing updates run on the tensor cores as three TF32 products per term

@@ -1301,7 +1301,7 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
                 if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(s, la->panel_done, 0)) != cudaSuccess) return e;
                 const tc::Split L{Lh + i0 * kP, Ll + i0 * kP, kP};
-                e = vec ? tc::launch_gemm<true>(U + i0 * n + i0, n, L, L, m, m, nb, -1.0f, status, s) : cudaErrorNotSupported;
+                e = vec ? tc::launch_gemm<true>(U + i0 * n + i0, n, L, L, m, m, nb, -1.0f, status, sms, s) : cudaErrorNotSupported;
                 if (e == cudaErrorNotSupported)
                     e = launch_gemm<true, true>(U + i0 * n + i0, n, P, n, P, n, m, m, nb, -1.0f, s);
                 if (e != cudaSuccess) return e;
@@ -1408,7 +1408,7 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     auto update = [&](int64_t s0, int i, int64_t d, int64_t cols, cudaStream_t st) {
         float* C = p.T + s0 + kLdlqPanel + d;
         const tc::Split B{Us[i].hi + d * kLdlqPanel, Us[i].lo + d * kLdlqPanel, kLdlqPanel};
-        cudaError_t r = tc::launch_gemm<false>(C, p.n, Es[i], B, p.rows, cols, kLdlqPanel, 1.0f, p.status, st);
+        cudaError_t r = tc::launch_gemm<false>(C, p.n, Es[i], B, p.rows, cols, kLdlqPanel, 1.0f, p.status, sms, st);
         if (r != cudaErrorNotSupported) return r;
         const float* u = p.U + s0 * p.n + s0 + kLdlqPanel + d;         // no tensor maps: both halves on the FP32 pipe
         r = launch_gemm<false, false>(C, p.n, Es[i].hi, kLdlqPanel, u, p.n, p.rows, cols, kLdlqPanel, 1.0f, st);

@@ -28,10 +28,13 @@
 //     lanes 32(w%4).. = rows, 64 columns each), forms C = fma(alpha, acc, C) in
 //     shared memory and TMA stores the tile.
 //
+// Updates of several tiles per SM take gemm_strip_kernel: up to four tiles to a CTA,
+// loads, MMAs and epilogue in warps of their own.
+//
 // Every mbarrier wait is bounded by the global timer (1 s).  On a timeout the
 // CTA sets bit 4 (16) of the status word, stops issuing, waits (bounded again)
 // for the copies and MMAs it has in flight, frees its tensor memory and
-// returns without writing C.
+// returns without writing (the rest of) C.
 #pragma once
 #include <cstdint>
 #include <cuda.h>
@@ -45,11 +48,14 @@ namespace tc {
 constexpr int kTileM = 128;
 constexpr int kTileN = 128;
 constexpr int kStageK = 32;                               // fp32 per swizzle row (128 bytes)
-constexpr int kThreads = 256;                             // warps w, w + 4 read TMEM lanes 32(w % 4)..
+constexpr int kEpiThreads = 256;                          // warps w, w + 4 read TMEM lanes 32(w % 4)..
+constexpr int kThreads = 256;
+constexpr int kStripThreads = kEpiThreads + 64;           // a warp for the loads and one for the MMAs
 constexpr int kOpBytes = kTileM * kStageK * 4;            // one operand tile: 16 KB
 constexpr int kStages = 3;
 constexpr int kStageBytes = 4 * kOpBytes;                 // A hi, A lo, B hi, B lo
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 128;   // + alignment, barriers
+constexpr int kStripSmem = kSmemBytes + 2 * kOpBytes;     // + boxes of C
 constexpr int kTmemCols = kTileN;                         // fp32 accumulator columns
 constexpr unsigned long long kWaitNs = 1000000000ull;
 constexpr int kStatusTimeout = 16;
@@ -66,6 +72,9 @@ __device__ __forceinline__ unsigned long long now_ns() {
 // ---- mbarriers
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -103,10 +112,10 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int c0, int
                  ::"l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(src)
                  : "memory");
 }
-__device__ __forceinline__ void tma_store_commit_and_wait() {
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// The committed stores have read shared memory / have completed.
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // ---- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t holder, uint32_t ncols) {
@@ -157,6 +166,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// 16 consecutive fp32 accumulator columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
 // Shared-memory matrix descriptor of a K-major 128-byte-swizzled operand tile:
@@ -328,7 +352,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int j = 0; j < kTileN / 32; j++)
                 tma_store_2d(&tmC, n0 + 32 * j, m0, smem_u32(cbase + j * kOpBytes));
-            tma_store_commit_and_wait();
+            tma_store_commit();
+            tma_store_wait();
         }
     } else if (tid == 0 && status) {
         atomicOr(status, kStatusTimeout);
@@ -336,6 +361,174 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+}
+
+// The warps that add accumulators to C.
+__device__ __forceinline__ void epi_barrier() {
+    __syncwarp();
+    asm volatile("barrier.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+}
+
+// The same with a CTA for up to `tiles` tiles of C side by side, for updates of several
+// tiles per SM: loads, MMAs and the update of C run beside each other.  Stages run on through them: warp
+// 8's first thread loads stage s into slot s % 3 once the MMAs of stage s - 3 have
+// read it, warp 9's issues the MMAs of s once it has landed, alternating between two
+// accumulators, and the other eight warps add a finished accumulator to C, 32 columns
+// at a time through two boxes that thread 0 loads and stores, beside the next tile's
+// MMAs.
+template <bool LOWER>
+__global__ void __launch_bounds__(kStripThreads, 1)
+    gemm_strip_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
+                const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl,
+                const __grid_constant__ CUtensorMap tmC, int N, int K, int tiles, float alpha, int* status) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ int s_abort, s_lost;                              // a wait ran out: of the other two warps, of these eight
+    __shared__ uint32_t s_tmem;
+    const int m0 = (int)blockIdx.y * kTileM, nb = (int)blockIdx.x * tiles * kTileN;
+    grid_launch_dependents();                                    // a dependent launch waits for this grid's end
+    if (LOWER && nb > m0 + kTileM - 1) return;
+    const int last = LOWER ? min(N - 1, m0 + kTileM - 1) : N - 1;                // last column of this CTA's rows
+    const int nt = min(tiles, (last - nb) / kTileN + 1);
+    const int nst = (K + kStageK - 1) / kStageK;
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* cbox = base + kStages * kStageBytes;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(cbox + 2 * kOpBytes);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kStages, cfull0 = empty0 + 8 * kStages;
+    const uint32_t accf0 = cfull0 + 16, acce0 = accf0 + 16, dbar = acce0 + 16;
+
+    if (warp == 0) tmem_alloc(smem_u32(&s_tmem), 2 * kTmemCols);
+    if (tid == 0) {
+        for (int b = 0; b < kStages; b++) {
+            mbar_init(full0 + 8 * b, 1);
+            mbar_init(empty0 + 8 * b, 1);
+        }
+        for (int b = 0; b < 2; b++) {
+            mbar_init(cfull0 + 8 * b, 1);
+            mbar_init(accf0 + 8 * b, 1);
+            mbar_init(acce0 + 8 * b, kEpiThreads / 32);
+        }
+        mbar_init(dbar, 1);
+        s_abort = s_lost = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+
+    if (tid == kEpiThreads) {
+        int s = 0;
+        for (; s < nt * nst; s++) {
+            const int r = s % kStages;
+            if (s >= kStages && !mbar_wait(empty0 + 8 * r, (s / kStages - 1) & 1)) {
+                atomicOr(&s_abort, 1);
+                break;
+            }
+            const uint32_t bar = full0 + 8 * r, st = smem_u32(base + r * kStageBytes);
+            const int k = s % nst * kStageK, n0 = nb + s / nst * kTileN;
+            mbar_expect_tx(bar, kStageBytes);
+            tma_load_2d(st, &tmAh, k, m0, bar);
+            tma_load_2d(st + kOpBytes, &tmAl, k, m0, bar);
+            tma_load_2d(st + 2 * kOpBytes, &tmBh, k, n0, bar);
+            tma_load_2d(st + 3 * kOpBytes, &tmBl, k, n0, bar);
+        }
+        for (int i = s < kStages ? 0 : s - kStages; i < s; i++)  // none in flight at the end (bounded)
+            if (!mbar_wait(full0 + 8 * (i % kStages), (i / kStages) & 1)) atomicOr(&s_abort, 1);
+    } else if (tid == kEpiThreads + 32) {
+        constexpr uint32_t idesc = idesc_tf32();
+        bool ok = true;
+        for (int t = 0; ok && t < nt; t++) {
+            const uint32_t acc = tmem + (uint32_t)((t & 1) * kTileN);
+            if (t >= 2 && !mbar_wait(acce0 + 8 * (t & 1), (t / 2 - 1) & 1)) ok = false;
+            tc_fence_after();
+            for (int i = 0; ok && i < nst; i++) {
+                const int s = t * nst + i, r = s % kStages;
+                if (!mbar_wait(full0 + 8 * r, (s / kStages) & 1)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t st = smem_u32(base + r * kStageBytes);
+#pragma unroll
+                for (int kk = 0; kk < kStageK / 8; kk++) {       // the k-step's 32 bytes of each 128-byte row
+                    const uint64_t ahi = smem_desc(st + kk * 32, 16, 1024);
+                    const uint64_t alo = smem_desc(st + kOpBytes + kk * 32, 16, 1024);
+                    const uint64_t bhi = smem_desc(st + 2 * kOpBytes + kk * 32, 16, 1024);
+                    const uint64_t blo = smem_desc(st + 3 * kOpBytes + kk * 32, 16, 1024);
+                    mma_tf32(acc, ahi, bhi, idesc, (i | kk) != 0);
+                    mma_tf32(acc, ahi, blo, idesc, 1);
+                    mma_tf32(acc, alo, bhi, idesc, 1);
+                }
+                mma_commit(empty0 + 8 * r);
+            }
+            if (ok) mma_commit(accf0 + 8 * (t & 1));
+        }
+        mma_commit(dbar);                                        // after every MMA issued, also on a timeout
+        if (!ok) atomicOr(&s_abort, 1);
+        if (!mbar_wait(dbar, 0)) atomicOr(&s_abort, 1);
+    } else if (tid < kEpiThreads) {
+        // C += alpha * acc in shared memory (thread = row and half of the box's columns;
+        // the box rows are 128-byte swizzled, so the eight lanes of a quarter warp touch
+        // eight distinct 16-byte chunks), then TMA stores the box (out-of-range rows and
+        // columns are not written)
+        const int q = warp & 3, h = warp >> 2, r = 32 * q + lane;    // TMEM lane quarter q = rows 32q..32q+31
+        constexpr int kBoxes = kTileN / 32;
+        auto load_c = [&](int c) {
+            mbar_expect_tx(cfull0 + 8 * (c & 1), kOpBytes);
+            tma_load_2d(smem_u32(cbox + (c & 1) * kOpBytes), &tmC, nb + 32 * c, m0, cfull0 + 8 * (c & 1));
+        };
+        int issued = 0;                                          // thread 0: boxes loaded
+        if (tid == 0)
+            for (; issued < 2; issued++) load_c(issued);
+        int c = 0;
+        for (; c < nt * kBoxes; c++) {
+            const int t = c / kBoxes, j = c % kBoxes;
+            bool ok = mbar_wait(cfull0 + 8 * (c & 1), (c >> 1) & 1);
+            if (j == 0) ok = ok && mbar_wait(accf0 + 8 * (t & 1), (t >> 1) & 1);
+            if (!ok) atomicOr(&s_lost, 1);
+            epi_barrier();                                       // one decision for all eight warps: s_lost is
+            if (*reinterpret_cast<volatile int*>(&s_lost)) break;    // written before this barrier, read before the next
+            tc_fence_after();
+            __syncwarp();
+            float v[16];
+            tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((t & 1) * kTileN + 32 * j + 16 * h), v);
+            uint8_t* box = cbox + (c & 1) * kOpBytes + r * 128;
+#pragma unroll
+            for (int g = 0; g < 4; g++) {
+                float4* o4 = reinterpret_cast<float4*>(box + (((4 * h + g) ^ r) & 7) * 16);
+                float4 o = *o4;
+                o.x = __fmaf_rn(alpha, v[4 * g], o.x);
+                o.y = __fmaf_rn(alpha, v[4 * g + 1], o.y);
+                o.z = __fmaf_rn(alpha, v[4 * g + 2], o.z);
+                o.w = __fmaf_rn(alpha, v[4 * g + 3], o.w);
+                *o4 = o;
+            }
+            if (j == kBoxes - 1) {                               // the accumulator is read
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acce0 + 8 * (t & 1));
+            }
+            fence_proxy_async();
+            epi_barrier();
+            if (tid == 0) {
+                tma_store_2d(&tmC, nb + 32 * c, m0, smem_u32(cbox + (c & 1) * kOpBytes));
+                tma_store_commit();
+                if (issued < nt * kBoxes) {
+                    tma_store_wait_read();
+                    load_c(issued++);
+                }
+            }
+        }
+        if (tid == 0) {
+            for (; c < issued; c++) (void)mbar_wait(cfull0 + 8 * (c & 1), (c >> 1) & 1);   // after a timeout: bounded
+            tma_store_wait();
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (tid == 0 && (s_abort | s_lost) && status) atomicOr(status, kStatusTimeout);
+    if (warp == 0) tmem_dealloc(tmem, 2 * kTmemCols);
 }
 
 }  // namespace tc
@@ -394,7 +587,7 @@ struct Split {
 // 16-byte aligned, a size is beyond the tensor maps' limits, or the driver has none.
 template <bool LOWER>
 cudaError_t launch_gemm(float* C, int64_t ldc, const Split& A, const Split& B, int64_t M, int64_t N, int K, float alpha,
-                        int* status, cudaStream_t s) {
+                        int* status, int sms, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     auto al = [](const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 4 == 0 && ld < (1ll << 35); };
     if (!al(A.hi, A.ld) || !al(A.lo, A.ld) || !al(B.hi, B.ld) || !al(B.lo, B.ld) || !al(C, ldc) || M >= (1ll << 30) ||
@@ -411,11 +604,28 @@ cudaError_t launch_gemm(float* C, int64_t ldc, const Split& A, const Split& B, i
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
         e = cudaFuncSetAttribute(gemm_kernel<LOWER>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(gemm_strip_kernel<LOWER>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripSmem);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
     }
-    const dim3 grid((unsigned)((N + kTileN - 1) / kTileN), (unsigned)((M + kTileM - 1) / kTileM));
-    gemm_kernel<LOWER><<<grid, kThreads, kSmemBytes, s>>>(mah, mal, mbh, mbl, mc, K, alpha, status);
+    const int64_t tm = (M + kTileM - 1) / kTileM, tn = (N + kTileN - 1) / kTileN;
+    // Tiles per SM.  One tile to a CTA spends almost half its time filling the ring and
+    // adding to C (9 us at K = 256, 5 of them loads and MMAs); two or four overlap that,
+    // but leave the SMs less evenly filled and later for a waiting walk or factor.
+    // Passes with one / from 2 / from 3 / from 4 tiles per SM on: 4096 x 4096 929 / 916 /
+    // 917 / 918 us, 14336 x 4096 2.84 / 2.66 / 2.65 / 2.66 ms, 4096 x 14336 7.23 / 6.44 /
+    // 6.43 / 6.44; the factor at n = 4096 1.579 / 1.613 / 1.581 / 1.581 and n = 14336 21.8 /
+    // 20.7 / 20.7 / 20.7.  Four tiles from 4 per SM on: 4096 x 4096 931; never: 4096 x 14336 6.76.
+    const int64_t waves = (LOWER ? tm * tn / 2 : tm * tn) / sms;
+    if (waves < 3) {
+        gemm_kernel<LOWER><<<dim3((unsigned)tn, (unsigned)tm), kThreads, kSmemBytes, s>>>(mah, mal, mbh, mbl, mc, K, alpha,
+                                                                                          status);
+    } else {
+        const int tiles = waves < 8 ? 2 : 4;
+        gemm_strip_kernel<LOWER><<<dim3((unsigned)((tn + tiles - 1) / tiles), (unsigned)tm), kStripThreads, kStripSmem, s>>>(
+            mah, mal, mbh, mbl, mc, (int)N, K, tiles, alpha, status);
+    }
     return cudaGetLastError();
 }
 

@@ -1,7 +1,8 @@
 """LDLQ paths chosen by size and alignment.
 
 * Row and column counts off the walk's tiles (32 rows, 64 and 256 columns) and off the
-  update's (128), with the walk scheduled beside the update and after it.
+  update's (128, alone and in strips of two and four), with the walk scheduled beside
+  the update and after it.
 * A factor that is not 16-byte aligned: the same arithmetic, so the same codes.
 * Rows too long for the gather's and the packer's shared memory: with a zero factor the
   codes are plain rounding.
@@ -26,7 +27,7 @@ def _misaligned(t):
     return out
 
 
-@pytest.mark.parametrize("rows,cols", [(1, 16), (31, 272), (32, 320), (33, 528), (129, 784), (4900, 528)])
+@pytest.mark.parametrize("rows,cols", [(1, 16), (31, 272), (32, 320), (33, 528), (129, 784), (4900, 528), (24000, 1296)])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_walk_and_update_tiles(B, rows, cols, dtype):
     W64, H = rand_problem(rows, cols, rows + cols)
