@@ -300,7 +300,6 @@ __host__ __device__ constexpr int bound_offsets() {
     return OBJ != 0 ? 4 : (BLOCK == 16 ? (GROUPED ? 2 : 1) : 6);
 }
 
-//
 // octave (WMSE, whose windows hold four pairs above the bounded offsets; MSE windows
 // hold one or two, and the second copy of the loop cost more than it gave): every
 // code above the bounded offsets is a normal E4M3 code
@@ -433,12 +432,6 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv& d) {
     return (t + ((n - t) >> d.s1)) >> d.s2;
 }
 
-
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     unsigned v;
