@@ -956,7 +956,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
     if (tid < 128)
         rtab[tid] = (usable && tid >= 1 && tid <= 126) ? __frcp_rn(f16bits_to_f32(e4m3_to_f16bits((uint32_t)tid))) : 0.0f;
 
-    // all of the above is older than the update of these columns, which the targets come from
+    // all of the above is older than the update of these columns, which the targets come
+    // from and the only grid this one may start before the end of
     grid_dependency_wait();
     if (wc < span) set_rows(p.T + rbase + wc);
     // targets of this warp's groups in sub-panels 1.. as accumulator fragments: rows
@@ -1420,12 +1421,14 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     // then the walk is scheduled beside the update and stages U, the weights and the
     // scales meanwhile (1024 x 4096: 0.601 -> 0.538 ms).  Otherwise its waiting CTAs
     // would only keep SMs from the rest of the update (4096 x 4096: 0.925 -> 0.941 ms).
+    // The first walk has no update before it: it goes out the ordinary way, ordered after
+    // the gather that writes the weights and scales it reads before its wait.
     const bool early = wg + ((p.rows + 127) / 128) * (kLdlqPanel / 128) <= sms;
     int sp = 0;
     for (int64_t s0 = 0; s0 < p.n; s0 += kLdlqPanel, sp ^= 1) {
         const int64_t span = imin64(kLdlqPanel, p.n - s0);
         float *eh = const_cast<float*>(Es[sp].hi), *el = const_cast<float*>(Es[sp].lo);
-        if (early) {
+        if (early && s0 > 0) {
             e = launch_dependent_smem(walk, wg, kWalkThreads, kWalkSmem, c, p, s0, (int)span, eh, el);
         } else {
             walk<<<wg, kWalkThreads, kWalkSmem, c>>>(p, s0, (int)span, eh, el);

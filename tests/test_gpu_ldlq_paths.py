@@ -7,7 +7,10 @@
 * Rows too long for the gather's and the packer's shared memory: with a zero factor the
   codes are plain rounding.
 * Factorizations off the panels of 64, with outputs that are not 16-byte aligned.
+* Dependencies of a captured pass: only a walk behind an update may start before it ends.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -88,3 +91,44 @@ def test_prepare_panels(B, n):
         assert np.abs(Ug - U_ref).max() <= 2e-4 * max(1.0, np.abs(U_ref).max())
         R = (Ug + np.eye(n)) @ np.diag(Dg) @ (Ug + np.eye(n)).T - Hp
         assert np.abs(R).max() <= 2e-5 * np.abs(Hp).max()
+
+
+def programmatic_edges(graph):
+    """How many of a captured graph's edges let a node start before the one ahead of it ends."""
+    class Edge(ctypes.Structure):
+        _fields_ = [("from_port", ctypes.c_ubyte), ("to_port", ctypes.c_ubyte), ("type", ctypes.c_ubyte),
+                    ("reserved", ctypes.c_ubyte * 5)]
+
+    get = ctypes.CDLL("libcuda.so.1").cuGraphGetEdges_v2
+    h, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert get(h, None, None, None, ctypes.byref(n)) == 0 and n.value > 0
+    src, dst, data = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)(), (Edge * n.value)()
+    assert get(h, src, dst, data, ctypes.byref(n)) == 0
+    return sum(e.type != 0 for e in data)
+
+
+# super-panels of 256 columns; 64 rows: every walk but the first is scheduled beside an update
+@pytest.mark.parametrize("cols,behind_update", [(256, 0), (528, 2)])
+def test_first_walk_waits_for_the_gather(B, cols, behind_update):
+    """The walk reads the gathered weights and scales before it waits for the grid ahead
+    of it: the gather must have ended by then, so its edge is a full dependency."""
+    rows = 64
+    W64, H = rand_problem(rows, cols, cols)
+    S, sf = fixed_scales(W64, H)
+    Wt = torch.from_numpy(W64.astype(np.float32)).to(DEV)
+    perm, U, _, _ = prepare(B, H)                             # also the first call on the device
+    eager, _ = quantize(B, Wt, S, sf, perm, U)
+    codes = torch.empty(rows, cols // 2, dtype=torch.uint8, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.nvfp4_ldlq_workspace(rows, cols), dtype=torch.uint8, device=DEV)
+    Sd = torch.tensor([S], dtype=torch.float32, device=DEV)
+    sfd = torch.as_tensor(np.ascontiguousarray(sf), dtype=torch.uint8).to(DEV)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, stream=s):
+        B.ldlq_quantize(Wt, 16, Sd, sfd, perm, U, codes, st, ws, stream=s)
+    assert programmatic_edges(g) == behind_update
+    g.replay()
+    torch.cuda.synchronize()
+    assert st.item() == 0 and np.array_equal(codes.cpu().numpy(), eager)
