@@ -289,14 +289,20 @@ nvfp4_status absmax_quantize_group(const nvfp4_group_tensor* tensors, int count,
 
 /*
  * Self-test of the bounded device waits (failure detection; the paper has no
- * counterpart).  Runs scalesweep_quantize_group with a dynamic scale (x as its
- * one tensor: bf16, block 16, MSE; which = 0 or 1: the dynamic per-tensor call has
- * no wait in device code, so both run this one) with the wait's arrival target
- * raised past what the launch can reach, so every device wait gives up after its
- * limit (about a second): bit 1 is OR-ed into *status_dev (required here), the
- * waiting warps return without writing codes or scales, and the CUDA context
- * stays usable.  Arguments and buffers as in those calls; workspace of
- * max(nvfp4_dynamic_workspace(), scalesweep_quantize_group_workspace()) bytes.
+ * counterpart): a call whose device waits are made to give up after their limit
+ * (about a second) by a barrier that expects one arrival too many.  The status word
+ * (required here) reports it and the CUDA context stays usable.
+ *   which = 0, 1  scalesweep_quantize_group with a dynamic scale, x as its one tensor
+ *             (bf16, block 16, MSE; the dynamic per-tensor call has no wait in device
+ *             code, so both run this one): status bit 1, no codes or scales written.
+ *             workspace of max(nvfp4_dynamic_workspace(),
+ *             scalesweep_quantize_group_workspace()) bytes.
+ *   which = 2, 3  ldlq_quantize of x (bf16, block 16; S and sf_linear are read): status
+ *             bit 16.  2: the walk's wait for U, in every super-panel: all codes are
+ *             zero.  3: the trailing updates' wait for their operands: none is
+ *             applied.  workspace, 256-byte aligned: perm [cols] int32 and U [cols,
+ *             cols] float as the caller filled them, each padded to a multiple of 256
+ *             bytes, then nvfp4_ldlq_workspace(rows, cols) bytes.
  */
 nvfp4_status nvfp4_selftest_wait_timeout(int which, const void* x, int64_t rows, int64_t cols, float* S,
                                          int* status_dev, void* workspace, size_t ws_bytes, uint8_t* codes,
@@ -409,7 +415,8 @@ nvfp4_status nvfp4_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
  * code or an unusable S quantizes to signed zeros, an exactly zero y to +0.
  *   The error-feedback updates past a super-panel of 256 columns run on the
  *   tensor cores (three TF32 products per term, as in nvfp4_ldlq_prepare; status
- *   bit 16 as there, also for the bounded wait for U within a super-panel).
+ *   bit 16 as there, also for the bounded wait for U within a super-panel, whose
+ *   codes are then zeros: with bit 16 the result is not the LDLQ pass's).
  *   perm, U from nvfp4_ldlq_prepare (cols = n); status_dev optional: |= 8 if
  *   perm holds an index outside [0, cols) (the entry is then read as 0).
  *   workspace   device bytes, at least nvfp4_ldlq_workspace(rows, cols):

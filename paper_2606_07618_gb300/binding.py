@@ -259,8 +259,9 @@ def absmax_quantize_group(desc, dtype: int, fp8_div: float, S, status=None, work
 
 
 def nvfp4_selftest_wait_timeout(which: int, x, S, status, workspace, codes, sf_linear, stream=None):
-    """Makes the device wait of the grouped launch with a dynamic scale (which = 0
-    or 1) run out; status bit 1 reports it."""
+    """Makes a bounded device wait run out: the grouped launch's with a dynamic scale
+    (which = 0 or 1; status bit 1), LDLQ's walk's (2) or trailing updates' (3; status
+    bit 16; workspace: perm, U, then LDLQ's own).  See nvfp4ss.h."""
     rows, cols = x.shape
     ws_bytes = workspace.numel() * workspace.element_size()
     rc = lib().nvfp4_selftest_wait_timeout(int(which), _ptr(x), rows, cols, _ptr(S), _ptr(status), _ptr(workspace),

@@ -430,10 +430,23 @@ nvfp4_status absmax_quantize_group(const nvfp4_group_tensor* tensors, int count,
                         stream, 0);
 }
 
+static nvfp4_status ldlq_common(const void* W, nvfp4_dtype dt, int64_t rows, int64_t cols, int block, const float* S,
+                                const uint8_t* sf_linear, const int32_t* perm, const float* U, uint8_t* codes,
+                                int* status_dev, void* workspace, size_t ws_bytes, int starve, void* stream);
+
 nvfp4_status nvfp4_selftest_wait_timeout(int which, const void* x, int64_t rows, int64_t cols, float* S,
                                          int* status_dev, void* workspace, size_t ws_bytes, uint8_t* codes,
                                          uint8_t* sf_linear, void* stream) {
-    if ((which != 0 && which != 1) || !status_dev || rows <= 0 || cols <= 0) return NVFP4_ERR_INVALID_ARG;
+    if (which < 0 || which > 3 || !status_dev || rows <= 0 || cols <= 0) return NVFP4_ERR_INVALID_ARG;
+    if (which >= 2) {                       // LDLQ: perm, U and its workspace, one after the other
+        if (cols > (int64_t)1 << 20) return NVFP4_ERR_RANGE;
+        const size_t pb = (size_t)(cols * 4 + 255) / 256 * 256, ub = (size_t)(cols * cols * 4 + 255) / 256 * 256;
+        if (!workspace || ws_bytes < pb + ub) return NVFP4_ERR_INVALID_ARG;
+        char* w = static_cast<char*>(workspace);
+        return ldlq_common(x, NVFP4_IN_BF16, rows, cols, 16, S, sf_linear, reinterpret_cast<int32_t*>(w),
+                           reinterpret_cast<float*>(w + pb), codes, status_dev, w + pb + ub, ws_bytes - pb - ub,
+                           which == 2 ? kStarveWalk : kStarveUpdate, stream);
+    }
     if (which == 0 && (!workspace || ws_bytes < kDynWorkspace)) return NVFP4_ERR_INVALID_ARG;
     // the grouped launch is the one sweep with a wait in device code: both settings run it
     const nvfp4_group_tensor t{x, rows, cols, nullptr, 0, codes, sf_linear, nullptr};
@@ -583,9 +596,9 @@ size_t nvfp4_ldlq_workspace(int64_t rows, int64_t cols) {
     return ldlq_quantize_workspace(rows, cols);
 }
 
-nvfp4_status ldlq_quantize(const void* W, nvfp4_dtype dt, int64_t rows, int64_t cols, int block, const float* S,
-                           const uint8_t* sf_linear, const int32_t* perm, const float* U, uint8_t* codes,
-                           int* status_dev, void* workspace, size_t ws_bytes, void* stream) {
+static nvfp4_status ldlq_common(const void* W, nvfp4_dtype dt, int64_t rows, int64_t cols, int block, const float* S,
+                                const uint8_t* sf_linear, const int32_t* perm, const float* U, uint8_t* codes,
+                                int* status_dev, void* workspace, size_t ws_bytes, int starve, void* stream) {
     if (dt != NVFP4_IN_BF16 && dt != NVFP4_IN_F32) return NVFP4_ERR_INVALID_ARG;
     Shape sh;
     nvfp4_status st = check_shape(rows, cols, block, &sh);
@@ -625,9 +638,17 @@ nvfp4_status ldlq_quantize(const void* W, nvfp4_dtype dt, int64_t rows, int64_t 
     p.Wp = nullptr;
     p.qb = nullptr;
     p.sfp = nullptr;
+    p.starve = starve;
     cudaError_t e = launch_ldlq_quantize(p, dt == NVFP4_IN_BF16 ? 0 : 1, codes, workspace, sms,
                                          static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? NVFP4_OK : NVFP4_ERR_CUDA;
+}
+
+nvfp4_status ldlq_quantize(const void* W, nvfp4_dtype dt, int64_t rows, int64_t cols, int block, const float* S,
+                           const uint8_t* sf_linear, const int32_t* perm, const float* U, uint8_t* codes,
+                           int* status_dev, void* workspace, size_t ws_bytes, void* stream) {
+    return ldlq_common(W, dt, rows, cols, block, S, sf_linear, perm, U, codes, status_dev, workspace, ws_bytes, 0,
+                       stream);
 }
 
 nvfp4_status nvfp4_row_shard_layout(int64_t rows, int64_t cols, int block, int world, int rank,

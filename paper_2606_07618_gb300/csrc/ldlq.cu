@@ -928,7 +928,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
     const uint32_t ubar = tc::smem_u32(&s_ubar);
     if (UVEC) {
         if (tid == 0) {
-            tc::mbar_init(ubar, 1);
+            tc::mbar_init(ubar, 1 + (p.starve & kStarveWalk));
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             tc::mbar_expect_tx(ubar, (uint32_t)(32 * kGroupCols * ng * (ng + 1) / 2));   // 8 rows of 32 (ng - g) bytes per group
         }
@@ -1020,8 +1020,19 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
     bool staged = true;
     if (UVEC) staged = tc::mbar_wait(ubar, 0);
     else asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (__syncthreads_or(!staged)) {                   // U never arrived: report it and leave the outputs alone
+    if (__syncthreads_or(!staged)) {
+        // U never arrived: report it, give the copies a second bounded wait (they must not
+        // land in a later CTA's shared memory) and leave zero errors and zero codes, so
+        // that nothing stale from the workspace reaches the updates or the result
         if (tid == 0 && p.status) atomicOr(p.status, tc::kStatusTimeout);
+        if (UVEC) (void)tc::mbar_wait(ubar, 0);
+        const int nr = (int)min((int64_t)kWalkRows, p.rows - row0);
+        for (int i = tid; i < nr * span; i += kWalkThreads) {
+            const int64_t rr = row0 + i / span;
+            const int c = i % span;
+            Eh[rr * kLdlqPanel + c] = El[rr * kLdlqPanel + c] = 0.0f;
+            p.qb[rr * p.n + s0 + c] = 0;
+        }
         return;
     }
     scales();
@@ -1302,7 +1313,7 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
                 if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(s, la->panel_done, 0)) != cudaSuccess) return e;
                 const tc::Split L{Lh + i0 * kP, Ll + i0 * kP, kP};
-                e = vec ? tc::launch_gemm<true>(U + i0 * n + i0, n, L, L, m, m, nb, -1.0f, status, sms, s) : cudaErrorNotSupported;
+                e = vec ? tc::launch_gemm<true>(U + i0 * n + i0, n, L, L, m, m, nb, -1.0f, status, 0, sms, s) : cudaErrorNotSupported;
                 if (e == cudaErrorNotSupported)
                     e = launch_gemm<true, true>(U + i0 * n + i0, n, P, n, P, n, m, m, nb, -1.0f, s);
                 if (e != cudaSuccess) return e;
@@ -1409,7 +1420,8 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     auto update = [&](int64_t s0, int i, int64_t d, int64_t cols, cudaStream_t st) {
         float* C = p.T + s0 + kLdlqPanel + d;
         const tc::Split B{Us[i].hi + d * kLdlqPanel, Us[i].lo + d * kLdlqPanel, kLdlqPanel};
-        cudaError_t r = tc::launch_gemm<false>(C, p.n, Es[i], B, p.rows, cols, kLdlqPanel, 1.0f, p.status, sms, st);
+        cudaError_t r = tc::launch_gemm<false>(C, p.n, Es[i], B, p.rows, cols, kLdlqPanel, 1.0f, p.status,
+                                               (p.starve & kStarveUpdate) != 0, sms, st);
         if (r != cudaErrorNotSupported) return r;
         const float* u = p.U + s0 * p.n + s0 + kLdlqPanel + d;         // no tensor maps: both halves on the FP32 pipe
         r = launch_gemm<false, false>(C, p.n, Es[i].hi, kLdlqPanel, u, p.n, p.rows, cols, kLdlqPanel, 1.0f, st);

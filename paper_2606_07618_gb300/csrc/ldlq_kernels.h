@@ -9,6 +9,9 @@ namespace nvfp4 {
 
 // LDLQ (GPTQ) with fixed block scales, static reordering (ldlq.cu).
 constexpr int kLdlqPanel = 256;       // columns per trailing update of the error feedback
+// Barriers initialised with one arrival too many, so that the wait on them runs out:
+// the walk's for U, the trailing updates' for their operands.
+constexpr int kStarveWalk = 1, kStarveUpdate = 2;
 struct LdlqParams {
     const void* W;            // [rows, n] bf16 or f32, original column order
     int64_t rows, n;
@@ -23,6 +26,7 @@ struct LdlqParams {
     float* Wp;                // workspace: W in processing order, f32
     uint8_t* qb;              // workspace: nibbles [rows, n], processing order
     uint8_t* sfp;             // workspace: each element's scale code, processing order
+    int starve;               // kStarve* bits: waits that never end (self-test), else 0
 };
 size_t ldlq_prepare_workspace(int64_t n);
 cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* perm, float* U, float* D,

@@ -232,7 +232,7 @@ template <bool LOWER>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
                 const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl,
-                const __grid_constant__ CUtensorMap tmC, int K, float alpha, int* status) {
+                const __grid_constant__ CUtensorMap tmC, int K, float alpha, int* status, int starve) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ int s_abort, s_issued;
     __shared__ uint32_t s_tmem;
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
     if (tid == 0) {
         for (int b = 0; b < kStages; b++) {
-            mbar_init(full0 + 8 * b, 1);
+            mbar_init(full0 + 8 * b, 1 + starve);
             mbar_init(empty0 + 8 * b, 1);
         }
         mbar_init(cbar, 1);
@@ -380,7 +380,7 @@ template <bool LOWER>
 __global__ void __launch_bounds__(kStripThreads, 1)
     gemm_strip_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
                 const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl,
-                const __grid_constant__ CUtensorMap tmC, int N, int K, int tiles, float alpha, int* status) {
+                const __grid_constant__ CUtensorMap tmC, int N, int K, int tiles, float alpha, int* status, int starve) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ int s_abort, s_lost;                              // a wait ran out: of the other two warps, of these eight
     __shared__ uint32_t s_tmem;
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kStripThreads, 1)
     if (warp == 0) tmem_alloc(smem_u32(&s_tmem), 2 * kTmemCols);
     if (tid == 0) {
         for (int b = 0; b < kStages; b++) {
-            mbar_init(full0 + 8 * b, 1);
+            mbar_init(full0 + 8 * b, 1 + starve);
             mbar_init(empty0 + 8 * b, 1);
         }
         for (int b = 0; b < 2; b++) {
@@ -583,11 +583,12 @@ struct Split {
 };
 
 // C[M, N] += alpha * A B^T on the tensor cores (3xTF32), A [M, K] and B [N, K] split.
-// Returns cudaErrorNotSupported (nothing launched) where a base or row stride is not
+// starve: 1 makes the wait for the operands run out (self-test).  Returns
+// cudaErrorNotSupported (nothing launched) where a base or row stride is not
 // 16-byte aligned, a size is beyond the tensor maps' limits, or the driver has none.
 template <bool LOWER>
 cudaError_t launch_gemm(float* C, int64_t ldc, const Split& A, const Split& B, int64_t M, int64_t N, int K, float alpha,
-                        int* status, int sms, cudaStream_t s) {
+                        int* status, int starve, int sms, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     auto al = [](const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ld % 4 == 0 && ld < (1ll << 35); };
     if (!al(A.hi, A.ld) || !al(A.lo, A.ld) || !al(B.hi, B.ld) || !al(B.lo, B.ld) || !al(C, ldc) || M >= (1ll << 30) ||
@@ -620,11 +621,11 @@ cudaError_t launch_gemm(float* C, int64_t ldc, const Split& A, const Split& B, i
     const int64_t waves = (LOWER ? tm * tn / 2 : tm * tn) / sms;
     if (waves < 3) {
         gemm_kernel<LOWER><<<dim3((unsigned)tn, (unsigned)tm), kThreads, kSmemBytes, s>>>(mah, mal, mbh, mbl, mc, K, alpha,
-                                                                                          status);
+                                                                                          status, starve);
     } else {
         const int tiles = waves < 8 ? 2 : 4;
         gemm_strip_kernel<LOWER><<<dim3((unsigned)((tn + tiles - 1) / tiles), (unsigned)tm), kStripThreads, kStripSmem, s>>>(
-            mah, mal, mbh, mbl, mc, (int)N, K, tiles, alpha, status);
+            mah, mal, mbh, mbl, mc, (int)N, K, tiles, alpha, status, starve);
     }
     return cudaGetLastError();
 }

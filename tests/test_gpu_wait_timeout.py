@@ -1,11 +1,13 @@
 """Failure detection on the GPU without a fault: every device wait is bounded.
 
-nvfp4_selftest_wait_timeout raises the arrival target of the dynamic-scale
-sweep's grid barrier (which = 0) and of the grouped launch's scale wait
-(which = 1) past what the launch can reach.  Each wait must give up after its
-limit (about a second), report it in bit 1 of the status word, leave the
-outputs unwritten, and leave the context usable: the same call without the
-raised target right after gives the normal result.
+nvfp4_selftest_wait_timeout makes a barrier expect one arrival more than it can get:
+the grouped launch's scale wait (which = 0 and 1), the LDLQ walk's wait for its copies
+of U (2), and the waits of LDLQ's trailing updates for their operands (3; one tile to a
+CTA, and strips of tiles).  Each wait must give up after its limit (about a second),
+report it in the status word (bit 1; LDLQ: bit 16), leave the outputs as documented --
+unwritten; zero codes and no errors fed on; an update not applied -- and leave the
+context usable: the same call without the raised target right after gives the normal
+result.
 """
 import time
 
@@ -61,3 +63,53 @@ def test_wait_runs_out_and_is_reported(B, which):
     torch.cuda.synchronize()
     assert st.item() == 0 and S2.item() == S3.item()
     assert torch.equal(codes, ref["codes"]) and torch.equal(sfl, ref["sf_linear"])
+
+
+def ldlq_buffers(B, rows, cols, seed):
+    g = torch.Generator().manual_seed(seed)
+    x = (torch.randn(rows, cols, generator=g) * 0.02).to(torch.bfloat16).to(DEV)
+    sf = torch.randint(40, 80, (rows, cols // 16), generator=g).to(torch.uint8).to(DEV)
+    perm = torch.randperm(cols, generator=g).to(torch.int32).to(DEV)
+    U = torch.triu(torch.randn(cols, cols, generator=g) * 0.05, 1).to(DEV)
+    pad = lambda n: -(-n // 256) * 256
+    head = pad(4 * cols) + pad(4 * cols * cols)
+    # stale bytes everywhere the call writes: none of them may come back
+    ws = torch.full((head + B.nvfp4_ldlq_workspace(rows, cols),), 0xEE, dtype=torch.uint8, device=DEV)
+    ws[:4 * cols].view(torch.int32).copy_(perm)
+    ws[pad(4 * cols):pad(4 * cols) + 4 * cols * cols].view(torch.float32).copy_(U.reshape(-1))
+    return x, sf, perm, U, ws, torch.full((rows, cols // 2), 0xEE, dtype=torch.uint8, device=DEV)
+
+
+def ldlq_pass(B, x, S, sf, perm, U):
+    rows, cols = x.shape
+    codes = torch.empty(rows, cols // 2, dtype=torch.uint8, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.nvfp4_ldlq_workspace(rows, cols), dtype=torch.uint8, device=DEV)
+    B.ldlq_quantize(x, 16, S, sf, perm, U, codes, st, ws)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    return codes
+
+
+# 2: three super-panels, the last of 16 columns.  3: one update of 256 columns, as two
+# tiles alone, and as 229 x 2 on 152 SMs, which go in strips.
+@pytest.mark.parametrize("which,rows,cols", [(2, 45, 528), (3, 45, 512), (3, 29300, 512)])
+def test_ldlq_wait_runs_out_and_is_reported(B, which, rows, cols):
+    x, sf, perm, U, ws, codes = ldlq_buffers(B, rows, cols, rows + cols)
+    S = torch.full((1,), 0.01, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    want = torch.zeros_like(codes) if which == 2 else None
+    if which == 3:                                  # the update of columns 256.. left out
+        cut = U.clone()
+        cut[:256, 256:] = 0.0
+        want = ldlq_pass(B, x, S, sf, perm, cut)
+    torch.cuda.synchronize()
+    t0 = time.time()
+    B.nvfp4_selftest_wait_timeout(which, x, S, st, ws, codes, sf)
+    torch.cuda.synchronize()
+    assert 0.5 < time.time() - t0 < 60
+    assert st.item() == 16
+    assert torch.equal(codes, want)
+    ref = ldlq_pass(B, x, S, sf, perm, U)           # the context is still usable
+    assert not torch.equal(ref, want)
+    assert torch.equal(ref, ldlq_pass(B, x, S, sf, perm, U))
