@@ -819,11 +819,16 @@ __global__ void __launch_bounds__(256) gather_w_kernel(LdlqParams p, int shift) 
 // the barrier), so the next walk starts after 32 packed operations.  Beside the
 // walk every other warp applies published errors to its groups of the later
 // sub-panels with mma.sync (K = 8, three TF32 products per term as the trailing
-// GEMM), a group's 32 x 8 targets being two accumulator fragments: the last
+// GEMM), a group's 32 x 8 sums being two accumulator fragments: the last
 // published errors to the next sub-panel, those of the sub-panel before to the
 // ones after it.  A walking warp makes up the one step it missed when the
 // sub-panel is done, and turns its next group's fragments into rows (through
 // shared memory, 12-word rows).
+//
+// The error sums start from zero, those of 8 errors in the MMA and their running sum
+// in fp32, and meet the target, which is many times larger, in one addition when its
+// group is walked.  (An MMA does not round its sum to nearest: accumulating on the
+// targets themselves put them 1.14e-6 from 64 bits at 4096 x 4096 bf16.)
 //
 // Bound by the chain: 35 cycles of dependent arithmetic per column (52 with the
 // rest of a column's instructions), and a barrier and the last group's update per
@@ -901,8 +906,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
     const bool active = r <= last;
     const int64_t rbase = (active ? r : last) * p.n + s0;         // lanes past the last row repeat it and store nothing
     float* tw = turn + warp * kWalkRows * kTurnStride;
-    // the row's targets in the group being walked, packed pairs
-    u64 t[4];
+    // the sums of errors on the row's targets in the group to be walked, packed pairs
+    u64 t[4] = {0ull, 0ull, 0ull, 0ull};
     auto set_rows = [&](const float* src) {
         const float4 a = *reinterpret_cast<const float4*>(src);
         const float4 b = *reinterpret_cast<const float4*>(src + 4);
@@ -911,8 +916,9 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
         t[2] = pack2(b.x, b.y);
         t[3] = pack2(b.z, b.w);
     };
-    // operands of the warp's next walk: original weights and scale codes
-    float4 wa, wb;
+    // operands of the warp's next walk: original weights, scale codes and, written by the
+    // update before this grid, the targets without the super-panel's own errors
+    float4 wa, wb, ta, tb;
     uint2 cd;
     auto fetch = [&](int q) {
         const int c = q * kSubCols + wc;
@@ -920,6 +926,13 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
             wa = *reinterpret_cast<const float4*>(p.Wp + rbase + c);
             wb = *reinterpret_cast<const float4*>(p.Wp + rbase + c + 4);
             cd = *reinterpret_cast<const uint2*>(p.sfp + rbase + c);
+        }
+    };
+    auto fetch_targets = [&](int q) {
+        const int c = q * kSubCols + wc;
+        if (c < span) {
+            ta = *reinterpret_cast<const float4*>(p.T + rbase + c);
+            tb = *reinterpret_cast<const float4*>(p.T + rbase + c + 4);
         }
     };
     fetch(0);
@@ -959,26 +972,10 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
     // all of the above is older than the update of these columns, which the targets come
     // from and the only grid this one may start before the end of
     grid_dependency_wait();
-    if (wc < span) set_rows(p.T + rbase + wc);
-    // targets of this warp's groups in sub-panels 1.. as accumulator fragments: rows
-    // 16 m + lane / 4 (+ 8), columns 2 (lane % 4), + 1
-    float acc[kSubs][2][4];
-#pragma unroll
-    for (int q = 1; q < kSubs; q++) {
-        const int c = q * kSubCols + wc;
-        if (c < span) {
-#pragma unroll
-            for (int m = 0; m < 2; m++)
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    int64_t rr = row0 + 16 * m + 8 * h + (lane >> 2);
-                    rr = rr <= last ? rr : last;
-                    const float2 v = *reinterpret_cast<const float2*>(p.T + rr * p.n + s0 + c + 2 * (lane & 3));
-                    acc[q][m][2 * h] = v.x;
-                    acc[q][m][2 * h + 1] = v.y;
-                }
-        }
-    }
+    fetch_targets(0);
+    // the errors' sums for this warp's groups in sub-panels 1.. as accumulator fragments:
+    // rows 16 m + lane / 4 (+ 8), columns 2 (lane % 4), + 1
+    float acc[kSubs][2][4] = {};
     float rs[kGroupCols];
     uint16_t vh[kGroupCols];
     auto scales = [&]() {
@@ -1009,12 +1006,17 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
     };
     auto products = [&](float (&c)[2][4], const uint32_t (&ah)[2][4], const uint32_t (&al)[2][4], const uint32_t (&bh)[2],
                         const uint32_t (&bl)[2]) {
+        float d[2][4] = {};
 #pragma unroll
-        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(c[m], ah[m], bh);
+        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(d[m], al[m], bh);
 #pragma unroll
-        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(c[m], ah[m], bl);
+        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(d[m], ah[m], bl);
 #pragma unroll
-        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(c[m], al[m], bh);
+        for (int m = 0; m < 2; m++) mma_16n8k8_tf32(d[m], ah[m], bh);
+#pragma unroll
+        for (int m = 0; m < 2; m++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) c[m][i] = __fadd_rn(c[m][i], d[m][i]);
     };
 
     bool staged = true;
@@ -1080,8 +1082,13 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
             }
             if (warp == o) {
                 float tt[8], ev[8];
+                const float tw8[8] = {ta.x, ta.y, ta.z, ta.w, tb.x, tb.y, tb.z, tb.w};
 #pragma unroll
-                for (int h = 0; h < 4; h++) unpack2(t[h], tt[2 * h], tt[2 * h + 1]);
+                for (int h = 0; h < 4; h++) {
+                    unpack2(t[h], tt[2 * h], tt[2 * h + 1]);
+                    tt[2 * h] = __fadd_rn(tw8[2 * h], tt[2 * h]);
+                    tt[2 * h + 1] = __fadd_rn(tw8[2 * h + 1], tt[2 * h + 1]);
+                }
                 const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
                 float* e = es + (g & (2 * kWalkWarps - 1)) * kErrSlot + lane;
                 const float* ud = ut + u_row(g);
@@ -1125,6 +1132,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
                     *reinterpret_cast<uint2*>(p.qb + rbase + g * kGroupCols) = make_uint2(packed[0], packed[1]);
                 }
                 fetch(q + 1);
+                fetch_targets(q + 1);
                 continue;
             }
             if (warp > o && warp < nq) {

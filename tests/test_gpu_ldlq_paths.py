@@ -7,6 +7,7 @@
 * Rows too long for the gather's and the packer's shared memory: with a zero factor the
   codes are plain rounding.
 * Factorizations off the panels of 64, with outputs that are not 16-byte aligned.
+* Sums of errors: kept where each is below the target's last place.
 * Dependencies of a captured pass: only a walk behind an update may start before it ends.
 """
 import ctypes
@@ -132,3 +133,29 @@ def test_first_walk_waits_for_the_gather(B, cols, behind_update):
     g.replay()
     torch.cuda.synchronize()
     assert st.item() == 0 and np.array_equal(codes.cpu().numpy(), eager)
+
+
+# rows not a multiple of 4; a factor off 16 bytes
+@pytest.mark.parametrize("rows,aligned", [(64, True), (33, True), (64, False)])
+def test_small_errors_add_up(B, rows, aligned):
+    """Every column's error is 2^-12 and reaches the columns k = 64, 128, 192 and 256
+    with factor 2^-16: 2^-28 each, 1/32 of those targets' last place.  Column k lies
+    k / 64 places below the boundary 1.25, which rounds down to 1; its errors, 2 k / 64
+    places less 1/32 for each earlier k, take it above.  Every product and every sum of
+    errors is exact."""
+    cols, at = 272, [64, 128, 192, 256]
+    W = torch.full((rows, cols), 1 + 2.0 ** -12)
+    U = torch.zeros(cols, cols)
+    for k in at:
+        W[:, k] = 1.25 - k / 64 * 2.0 ** -23
+        U[:k, k] = 2.0 ** -16
+    U[at] = 0                                                 # their own errors go nowhere
+    sf = np.full((rows, cols // 16), 56, dtype=np.uint8)      # E4M3 1.0
+    perm = torch.arange(cols, dtype=torch.int32, device=DEV)
+    Ud = U.to(DEV) if aligned else _misaligned(U)
+    codes, st = quantize(B, W.to(DEV), 1.0, sf, perm, Ud)
+    assert st == 0
+    nib = np.stack([codes & 15, codes >> 4], axis=-1).reshape(rows, cols)
+    want = np.full((rows, cols), 2)                           # E2M1 1.0
+    want[:, at] = 3                                           # 1.5
+    assert np.array_equal(nib, want)
