@@ -392,8 +392,8 @@ nvfp4_status nvfp4_dequantize(const uint8_t* codes, const uint8_t* sf, nvfp4_sf_
  *   workspace   device bytes, at least nvfp4_ldlq_prepare_workspace(n).
  * Cost: n^3/3 fp32 multiply-adds (blocked Cholesky, 64-wide panels).  The
  * trailing updates run on the tensor cores as three TF32 products per term
- * (products to ~2^-21 relative, accumulated in fp32) when n % 4 == 0 and U is
- * 16-byte aligned, else on the FP32 pipe.
+ * (products to ~2^-21 relative, the large and the small ones summed apart) when
+ * n % 4 == 0 and U is 16-byte aligned, else on the FP32 pipe.
  * The factorization's critical chain runs on a high-priority stream the library
  * creates on the first call on a device and keeps (with five events) for the
  * process; it is forked from and joined back into `stream`, so the call stays
@@ -413,10 +413,12 @@ nvfp4_status nvfp4_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
  * U_ik, What_k = Q(T_k), with Q the sweep's fp32 rounding at the fixed scale:
  * y = fl(T*E), q = RNE_E2M1(fl(y*fl(1/v))), What = fl(fl(q*v)*S); a zero scale
  * code or an unusable S quantizes to signed zeros, an exactly zero y to +0.
- *   The error-feedback updates past a super-panel of 256 columns run on the
- *   tensor cores (three TF32 products per term, as in nvfp4_ldlq_prepare; status
- *   bit 16 as there, also for the bounded wait for U within a super-panel, whose
- *   codes are then zeros: with bit 16 the result is not the LDLQ pass's).
+ *   Errors reach the columns of their own 64 (in processing order) by fp32
+ *   multiply-adds and all later columns through the tensor cores (three TF32
+ *   products per term, as in nvfp4_ldlq_prepare), whatever the sizes and alignments;
+ *   sums of errors start from zero and are added to a target in fp32.  Status bit 16
+ *   as there, also for the bounded wait for U within a super-panel of 256 columns,
+ *   whose codes are then zeros: with bit 16 the result is not the LDLQ pass's.
  *   perm, U from nvfp4_ldlq_prepare (cols = n); status_dev optional: |= 8 if
  *   perm holds an index outside [0, cols) (the entry is then read as 0).
  *   workspace   device bytes, at least nvfp4_ldlq_workspace(rows, cols):

@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(256) gather_w_kernel(LdlqParams p, int shift) 
 // The error sums start from zero, those of 8 errors in the MMA and their running sum
 // in fp32, and meet the target, which is many times larger, in one addition when its
 // group is walked.  (An MMA does not round its sum to nearest: accumulating on the
-// targets themselves put them 1.14e-6 from 64 bits at 4096 x 4096 bf16.)
+// targets themselves put them 1.14e-6 from 64 bits at 4096 x 4096 bf16, this 1.3e-7.)
 //
 // Bound by the chain: 35 cycles of dependent arithmetic per column (52 with the
 // rest of a column's instructions), and a barrier and the last group's update per
@@ -875,10 +875,10 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 // Every warp arrives once per step, the walking one from its own branch.
 __device__ __forceinline__ void step_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
 
-// x = hi + lo, hi a TF32 value (13 mantissa bits cleared), lo exact in fp32 (the MMA reads its top 11 bits).
+// tc::split_tf32 as bit patterns, lo not masked (the MMA reads its top 11 bits).
 __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
     hi = __float_as_uint(x) & 0xFFFFE000u;
-    lo = __float_as_uint(__fsub_rn(x, __uint_as_float(hi)));
+    lo = __float_as_uint(__fsub_rn(x, __uint_as_float(hi))) + 0x1000u;
 }
 __device__ __forceinline__ void mma_16n8k8_tf32(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "

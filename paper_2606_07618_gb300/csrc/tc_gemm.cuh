@@ -3,11 +3,20 @@
 // A[M, K] B[N, K]^T with fp32 accumulation, three TF32 products per term
 // ("3xTF32"):
 //
-//   a = a_hi + a_lo with a_hi = a with its low 13 mantissa bits cleared (a TF32
-//   value) and a_lo = a - a_hi (exact in fp32); the tensor core reads TF32, so
-//   a_lo contributes its top 11 bits.  a*b ~ a_hi*b_hi + a_hi*b_lo + a_lo*b_hi,
-//   dropping a_lo*b_lo (~2^-22 relative): products to ~2^-21 relative, against
-//   2^-24 for one fp32 FMA.
+//   a ~ a_hi + a_lo, both TF32 values (split_tf32), a*b ~ a_hi*b_hi + a_hi*b_lo +
+//   a_lo*b_hi, dropping a_lo*b_lo (~2^-22 relative): products to ~2^-21 relative,
+//   against 2^-24 for one fp32 FMA.
+//
+// The sums decide the error, not the products: each MMA adds its 8-term sum to an
+// accumulator without rounding to nearest, and that error follows the accumulator's
+// size.  So the two small products go to an accumulator of their own, K goes in two parts
+// with a pair of accumulators each, and the epilogue adds them in fp32 (both kernels the
+// same).  LDLQ's targets against 64 bits, over 24 shapes of 535 to 3820 rows and 256 to
+// 3760 columns: 0.28 to 0.36 of the error with all products in one accumulator, 0.47 to
+// 0.87 of that of FP32 multiply-adds (one part: up to 1.09).  The factor's D at n = 4096:
+// 1.5e-5 in one accumulator, 3.5e-6.  Time, with one accumulator and now: weights of 4096
+// x 4096 0.924 / 0.964 ms, 14336 x 4096 2.66 / 2.75, 4096 x 14336 6.45 / 6.75; factors of
+// n = 4096 1.591 / 1.603 ms, n = 14336 20.7 / 20.7.
 //
 // The operands arrive already split, K-major (K contiguous): the kernels that
 // produce them (the panel walk, the panel solve, a transpose of U) write the hi and lo
@@ -21,10 +30,10 @@
 //     by TMA (cp.async.bulk.tensor) into a three-stage ring of 128-byte-swizzled
 //     shared memory: A hi, A lo, B hi, B lo, 64 KB per stage;
 //   * one thread issues 4 k-steps x 3 tcgen05.mma.kind::tf32 (M = 128, N = 128,
-//     K = 8) per stage into a 128-column fp32 accumulator in tensor memory, and
+//     K = 8) per stage into 128-column fp32 accumulators in tensor memory, and
 //     tcgen05.commit frees the stage's slot;
 //   * the C tile arrives by TMA in the first slot that no stage needs any more; the
-//     epilogue reads the accumulator with tcgen05.ld (warps w and w + 4 read TMEM
+//     epilogue reads the accumulators with tcgen05.ld (warps w and w + 4 read TMEM
 //     lanes 32(w%4).. = rows, 64 columns each), forms C = fma(alpha, acc, C) in
 //     shared memory and TMA stores the tile.
 //
@@ -56,7 +65,12 @@ constexpr int kStages = 3;
 constexpr int kStageBytes = 4 * kOpBytes;                 // A hi, A lo, B hi, B lo
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 128;   // + alignment, barriers
 constexpr int kStripSmem = kSmemBytes + 2 * kOpBytes;     // + boxes of C
-constexpr int kTmemCols = kTileN;                         // fp32 accumulator columns
+constexpr int kPairCols = 2 * kTileN;                     // fp32 accumulators: the large products, the small ones
+constexpr int kTmemCols = 2 * kPairCols;                  // a pair for each part of K
+// Stages of the first part of K: all but a quarter, or all of a short K.  Even parts are
+// a fifth more exact, but the strips' second pair then waits for the epilogue (4096 x
+// 14336 6.91 ms, 6.75 so, 6.50 with one part; 7 of 8 stages 6.71).
+__host__ __device__ constexpr int first_stages(int nst) { return nst >= 4 ? nst - nst / 4 : nst; }
 constexpr unsigned long long kWaitNs = 1000000000ull;
 constexpr int kStatusTimeout = 16;
 
@@ -150,37 +164,33 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
 }
-// 32 consecutive fp32 accumulator columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
-}
-
-// 16 consecutive fp32 accumulator columns of this thread's TMEM lane.
+// 16 consecutive fp32 accumulator columns of this thread's TMEM lane; the values are
+// there after tmem_wait_ld, which names them so that no use moves above it.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
         "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+          "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
         : "r"(taddr)
         : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld(float (&a)[16], float (&b)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
+                   "+f"(a[8]), "+f"(a[9]), "+f"(a[10]), "+f"(a[11]), "+f"(a[12]), "+f"(a[13]), "+f"(a[14]), "+f"(a[15])
+                 :: "memory");
+    asm volatile("" : "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7]),
+                      "+f"(b[8]), "+f"(b[9]), "+f"(b[10]), "+f"(b[11]), "+f"(b[12]), "+f"(b[13]), "+f"(b[14]), "+f"(b[15]));
+}
+// The two accumulators at taddr and taddr + gap, added.
+__device__ __forceinline__ void tmem_sum16(uint32_t taddr, uint32_t gap, float (&v)[16]) {
+    float l[16];
+    tmem_ld16(taddr, v);
+    tmem_ld16(taddr + gap, l);
+    tmem_wait_ld(v, l);
 #pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 16; i++) v[i] = __fadd_rn(v[i], l[i]);
 }
 
 // Shared-memory matrix descriptor of a K-major 128-byte-swizzled operand tile:
@@ -210,10 +220,12 @@ __host__ __device__ constexpr uint32_t idesc_tf32() {
 namespace nvfp4 {
 namespace tc {
 
-// x = hi + lo, hi a TF32 value (13 mantissa bits cleared), lo exact in fp32.
+// x ~ hi + lo, both TF32 values: hi is x with its low 13 mantissa bits cleared, lo the
+// rest rounded to nearest (half of the last place away from zero).  Left to the MMA,
+// which drops the bits past its eleven, lo would be too small by 2^-23 of x on average.
 __device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
     hi = __uint_as_float(__float_as_uint(x) & 0xFFFFE000u);
-    lo = __fsub_rn(x, hi);
+    lo = __uint_as_float((__float_as_uint(__fsub_rn(x, hi)) + 0x1000u) & 0xFFFFE000u);
 }
 __device__ __forceinline__ void split4(const float4& x, float4& h, float4& l) {
     split_tf32(x.x, h.x, l.x);
@@ -240,6 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     grid_launch_dependents();                                    // a dependent launch waits for this grid's end
     if (LOWER && n0 > m0 + kTileM - 1) return;
     const int nst = (K + kStageK - 1) / kStageK;
+    const int first = first_stages(nst);
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* bars = reinterpret_cast<uint64_t*>(base + kStages * kStageBytes);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -300,15 +313,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             tc_fence_after();
             const uint32_t st = smem_u32(base + r * kStageBytes);
+            const uint32_t acc = tmem + (s < first ? 0 : kPairCols);
+            const int i = s < first ? s : s - first;             // the stage within its part
 #pragma unroll
             for (int kk = 0; kk < kStageK / 8; kk++) {           // the k-step's 32 bytes of each 128-byte row
                 const uint64_t ahi = smem_desc(st + kk * 32, 16, 1024);
                 const uint64_t alo = smem_desc(st + kOpBytes + kk * 32, 16, 1024);
                 const uint64_t bhi = smem_desc(st + 2 * kOpBytes + kk * 32, 16, 1024);
                 const uint64_t blo = smem_desc(st + 3 * kOpBytes + kk * 32, 16, 1024);
-                mma_tf32(tmem, ahi, bhi, idesc, (s | kk) != 0);
-                mma_tf32(tmem, ahi, blo, idesc, 1);
-                mma_tf32(tmem, alo, bhi, idesc, 1);
+                mma_tf32(acc, ahi, bhi, idesc, i | kk);
+                mma_tf32(acc + kTileN, ahi, blo, idesc, i | kk);
+                mma_tf32(acc + kTileN, alo, bhi, idesc, 1);
             }
             mma_commit(empty0 + 8 * r);
         }
@@ -333,7 +348,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
         for (int j = 2 * (warp >> 2); j < 2 * (warp >> 2) + 2; j++) {   // warps 0-3: boxes 0-1, 4-7: 2-3
             float v[32];
-            tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * j), v);   // .sync.aligned
+            const uint32_t at = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * j);
+#pragma unroll
+            for (int e = 0; e < 32; e += 16) {
+                float a[16];
+                tmem_sum16(at + e, kTileN, a);                   // .sync.aligned
+                if (nst > first) {
+                    float b[16];
+                    tmem_sum16(at + kPairCols + e, kTileN, b);
+#pragma unroll
+                    for (int i = 0; i < 16; i++) a[i] = __fadd_rn(a[i], b[i]);
+                }
+#pragma unroll
+                for (int i = 0; i < 16; i++) v[e + i] = a[i];
+            }
             uint8_t* box = cbase + j * kOpBytes + r * 128;
 #pragma unroll
             for (int g = 0; g < 8; g++) {
@@ -373,7 +401,8 @@ __device__ __forceinline__ void epi_barrier() {
 // tiles per SM: loads, MMAs and the update of C run beside each other.  Stages run on through them: warp
 // 8's first thread loads stage s into slot s % 3 once the MMAs of stage s - 3 have
 // read it, warp 9's issues the MMAs of s once it has landed, alternating between two
-// accumulators, and the other eight warps add a finished accumulator to C, 32 columns
+// pairs of accumulators, one for each part of K; the other eight warps take the first
+// part into registers beside the second one's MMAs and add both to C, 32 columns
 // at a time through two boxes that thread 0 loads and stores, beside the next tile's
 // MMAs.
 template <bool LOWER>
@@ -390,6 +419,7 @@ __global__ void __launch_bounds__(kStripThreads, 1)
     const int last = LOWER ? min(N - 1, m0 + kTileM - 1) : N - 1;                // last column of this CTA's rows
     const int nt = min(tiles, (last - nb) / kTileN + 1);
     const int nst = (K + kStageK - 1) / kStageK;
+    const int first = first_stages(nst), parts = first < nst ? 2 : 1;
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* cbox = base + kStages * kStageBytes;
     uint64_t* bars = reinterpret_cast<uint64_t*>(cbox + 2 * kOpBytes);
@@ -397,7 +427,7 @@ __global__ void __launch_bounds__(kStripThreads, 1)
     const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kStages, cfull0 = empty0 + 8 * kStages;
     const uint32_t accf0 = cfull0 + 16, acce0 = accf0 + 16, dbar = acce0 + 16;
 
-    if (warp == 0) tmem_alloc(smem_u32(&s_tmem), 2 * kTmemCols);
+    if (warp == 0) tmem_alloc(smem_u32(&s_tmem), kTmemCols);
     if (tid == 0) {
         for (int b = 0; b < kStages; b++) {
             mbar_init(full0 + 8 * b, 1 + starve);
@@ -438,11 +468,12 @@ __global__ void __launch_bounds__(kStripThreads, 1)
     } else if (tid == kEpiThreads + 32) {
         constexpr uint32_t idesc = idesc_tf32();
         bool ok = true;
-        for (int t = 0; ok && t < nt; t++) {
-            const uint32_t acc = tmem + (uint32_t)((t & 1) * kTileN);
-            if (t >= 2 && !mbar_wait(acce0 + 8 * (t & 1), (t / 2 - 1) & 1)) ok = false;
+        for (int u = 0; ok && u < nt * parts; u++) {
+            const int t = u / parts, from = u % parts ? first : 0, to = u % parts ? nst : first;
+            const uint32_t acc = tmem + (uint32_t)((u & 1) * kPairCols);
+            if (u >= 2 && !mbar_wait(acce0 + 8 * (u & 1), (u / 2 - 1) & 1)) ok = false;
             tc_fence_after();
-            for (int i = 0; ok && i < nst; i++) {
+            for (int i = from; ok && i < to; i++) {
                 const int s = t * nst + i, r = s % kStages;
                 if (!mbar_wait(full0 + 8 * r, (s / kStages) & 1)) {
                     ok = false;
@@ -456,13 +487,13 @@ __global__ void __launch_bounds__(kStripThreads, 1)
                     const uint64_t alo = smem_desc(st + kOpBytes + kk * 32, 16, 1024);
                     const uint64_t bhi = smem_desc(st + 2 * kOpBytes + kk * 32, 16, 1024);
                     const uint64_t blo = smem_desc(st + 3 * kOpBytes + kk * 32, 16, 1024);
-                    mma_tf32(acc, ahi, bhi, idesc, (i | kk) != 0);
-                    mma_tf32(acc, ahi, blo, idesc, 1);
-                    mma_tf32(acc, alo, bhi, idesc, 1);
+                    mma_tf32(acc, ahi, bhi, idesc, (i - from) | kk);
+                    mma_tf32(acc + kTileN, ahi, blo, idesc, (i - from) | kk);
+                    mma_tf32(acc + kTileN, alo, bhi, idesc, 1);
                 }
                 mma_commit(empty0 + 8 * r);
             }
-            if (ok) mma_commit(accf0 + 8 * (t & 1));
+            if (ok) mma_commit(accf0 + 8 * (u & 1));
         }
         mma_commit(dbar);                                        // after every MMA issued, also on a timeout
         if (!ok) atomicOr(&s_abort, 1);
@@ -481,43 +512,69 @@ __global__ void __launch_bounds__(kStripThreads, 1)
         int issued = 0;                                          // thread 0: boxes loaded
         if (tid == 0)
             for (; issued < 2; issued++) load_c(issued);
-        int c = 0;
-        for (; c < nt * kBoxes; c++) {
-            const int t = c / kBoxes, j = c % kBoxes;
-            bool ok = mbar_wait(cfull0 + 8 * (c & 1), (c >> 1) & 1);
-            if (j == 0) ok = ok && mbar_wait(accf0 + 8 * (t & 1), (t >> 1) & 1);
-            if (!ok) atomicOr(&s_lost, 1);
-            epi_barrier();                                       // one decision for all eight warps: s_lost is
-            if (*reinterpret_cast<volatile int*>(&s_lost)) break;    // written before this barrier, read before the next
-            tc_fence_after();
+        // the pair of accumulators of one part, columns 32 j + 16 h .., added
+        auto pair_sum = [&](int u, int j, float (&v)[16]) {
+            tmem_sum16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((u & 1) * kPairCols + 32 * j + 16 * h), kTileN, v);
+        };
+        auto pair_read = [&](int u) {
+            tc_fence_before();
             __syncwarp();
-            float v[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((t & 1) * kTileN + 32 * j + 16 * h), v);
-            uint8_t* box = cbox + (c & 1) * kOpBytes + r * 128;
-#pragma unroll
-            for (int g = 0; g < 4; g++) {
-                float4* o4 = reinterpret_cast<float4*>(box + (((4 * h + g) ^ r) & 7) * 16);
-                float4 o = *o4;
-                o.x = __fmaf_rn(alpha, v[4 * g], o.x);
-                o.y = __fmaf_rn(alpha, v[4 * g + 1], o.y);
-                o.z = __fmaf_rn(alpha, v[4 * g + 2], o.z);
-                o.w = __fmaf_rn(alpha, v[4 * g + 3], o.w);
-                *o4 = o;
-            }
-            if (j == kBoxes - 1) {                               // the accumulator is read
-                tc_fence_before();
+            if (lane == 0) mbar_arrive(acce0 + 8 * (u & 1));
+        };
+        int c = 0;
+        bool lost = false;
+        for (int t = 0; !lost && t < nt; t++) {
+            const int ul = t * parts + parts - 1;                // the tile's last part
+            bool ok = true;
+            float v[kBoxes][16];
+            if (parts == 2) {                                    // the first one, beside the second one's MMAs
+                ok = mbar_wait(accf0 + 8 * ((ul - 1) & 1), ((ul - 1) >> 1) & 1);
+                tc_fence_after();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(acce0 + 8 * (t & 1));
+#pragma unroll
+                for (int j = 0; j < kBoxes; j++) pair_sum(ul - 1, j, v[j]);
+                pair_read(ul - 1);
             }
-            fence_proxy_async();
-            epi_barrier();
-            if (tid == 0) {
-                tma_store_2d(&tmC, nb + 32 * c, m0, smem_u32(cbox + (c & 1) * kOpBytes));
-                tma_store_commit();
-                if (issued < nt * kBoxes) {
-                    tma_store_wait_read();
-                    load_c(issued++);
+            ok = ok && mbar_wait(accf0 + 8 * (ul & 1), (ul >> 1) & 1);
+#pragma unroll
+            for (int j = 0; j < kBoxes; j++) {
+                ok = ok && mbar_wait(cfull0 + 8 * (c & 1), (c >> 1) & 1);
+                if (!ok) atomicOr(&s_lost, 1);
+                epi_barrier();                                   // one decision for all eight warps: s_lost is
+                if (*reinterpret_cast<volatile int*>(&s_lost)) {     // written before this barrier, read before the next
+                    lost = true;
+                    break;
                 }
+                tc_fence_after();
+                __syncwarp();
+                float w[16];
+                pair_sum(ul, j, w);
+                if (parts == 2)
+#pragma unroll
+                    for (int i = 0; i < 16; i++) w[i] = __fadd_rn(v[j][i], w[i]);
+                uint8_t* box = cbox + (c & 1) * kOpBytes + r * 128;
+#pragma unroll
+                for (int g = 0; g < 4; g++) {
+                    float4* o4 = reinterpret_cast<float4*>(box + (((4 * h + g) ^ r) & 7) * 16);
+                    float4 o = *o4;
+                    o.x = __fmaf_rn(alpha, w[4 * g], o.x);
+                    o.y = __fmaf_rn(alpha, w[4 * g + 1], o.y);
+                    o.z = __fmaf_rn(alpha, w[4 * g + 2], o.z);
+                    o.w = __fmaf_rn(alpha, w[4 * g + 3], o.w);
+                    *o4 = o;
+                }
+                if (j == kBoxes - 1) pair_read(ul);
+                fence_proxy_async();
+                epi_barrier();
+                if (tid == 0) {
+                    tma_store_2d(&tmC, nb + 32 * c, m0, smem_u32(cbox + (c & 1) * kOpBytes));
+                    tma_store_commit();
+                    if (issued < nt * kBoxes) {
+                        tma_store_wait_read();
+                        load_c(issued++);
+                    }
+                }
+                c++;
             }
         }
         if (tid == 0) {
@@ -528,7 +585,7 @@ __global__ void __launch_bounds__(kStripThreads, 1)
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && (s_abort | s_lost) && status) atomicOr(status, kStatusTimeout);
-    if (warp == 0) tmem_dealloc(tmem, 2 * kTmemCols);
+    if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
 }  // namespace tc
@@ -618,6 +675,7 @@ cudaError_t launch_gemm(float* C, int64_t ldc, const Split& A, const Split& B, i
     // 917 / 918 us, 14336 x 4096 2.84 / 2.66 / 2.65 / 2.66 ms, 4096 x 14336 7.23 / 6.44 /
     // 6.43 / 6.44; the factor at n = 4096 1.579 / 1.613 / 1.581 / 1.581 and n = 14336 21.8 /
     // 20.7 / 20.7 / 20.7.  Four tiles from 4 per SM on: 4096 x 4096 931; never: 4096 x 14336 6.76.
+    // (Taken with one accumulator to a tile.)
     const int64_t waves = (LOWER ? tm * tn / 2 : tm * tn) / sms;
     if (waves < 3) {
         gemm_kernel<LOWER><<<dim3((unsigned)tn, (unsigned)tm), kThreads, kSmemBytes, s>>>(mah, mal, mbh, mbl, mc, K, alpha,

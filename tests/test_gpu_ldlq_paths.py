@@ -7,7 +7,8 @@
 * Rows too long for the gather's and the packer's shared memory: with a zero factor the
   codes are plain rounding.
 * Factorizations off the panels of 64, with outputs that are not 16-byte aligned.
-* Sums of errors: kept where each is below the target's last place.
+* Sums of errors: kept where each is below the target's last place, and as close to 64
+  bits as sums on the FP32 pipe.
 * Dependencies of a captured pass: only a walk behind an update may start before it ends.
 """
 import ctypes
@@ -159,3 +160,53 @@ def test_small_errors_add_up(B, rows, aligned):
     want = np.full((rows, cols), 2)                           # E2M1 1.0
     want[:, at] = 3                                           # 1.5
     assert np.array_equal(nib, want)
+
+
+def _factor64(H):
+    perm = torch.argsort(torch.diagonal(H), descending=True, stable=True)
+    Hp = H.double()[perm][:, perm]
+    Hp.diagonal().add_(0.01 * float(torch.diagonal(H).double().mean()))
+    R = torch.linalg.cholesky(Hp.flip(0, 1)).flip(0, 1)
+    return perm, torch.triu(R / torch.diagonal(R)[None, :], 1).float()
+
+
+@pytest.mark.parametrize("rows,cols", [(4096, 4096), (4095, 4096), (16384, 1040)])
+def test_decisions_follow_64_bits(B, rows, cols):
+    """How many codes differ from those of 64-bit targets formed from the same earlier
+    codes.  A target with error d crosses a rounding boundary with probability rho d, rho
+    the density of targets around the boundaries, so errors of 2^-22 of the rows' rms
+    (2.4e-7; all sums on the FP32 pipe give 2.0e-7 at 4096 columns) flip about
+    rho E|d| of them.  (Adding the 8-column sums to the targets one by one: 3 to 5
+    times as many as that pipe's.)"""
+    g = torch.Generator(device=DEV).manual_seed(rows + cols)
+    scale = torch.exp(0.8 * torch.randn(cols, device=DEV, generator=g))
+    A = torch.randn(cols, 256, device=DEV, generator=g) * scale[:, None]
+    H = (A.double() @ A.double().T / 256 + torch.diag(scale.double() ** 2 * 0.05)).float()
+    perm, U = _factor64(H)
+    W = torch.randn(rows, cols, device=DEV, generator=g) * 0.02
+    S = (W.abs().max() / 1536).reshape(1)
+    win = (B.NVFP4_WINDOW_DEFAULT, B.NVFP4_WINDOW_DEFAULT)
+    sf = torch.empty(rows, cols // 16, dtype=torch.uint8, device=DEV)
+    codes = torch.empty(rows, cols // 2, dtype=torch.uint8, device=DEV)
+    B.scalesweep_quantize(W, 16, S, B.NVFP4_OBJ_WMSE, torch.diagonal(H).contiguous(), 0, *win, codes, sf)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    ws = torch.empty(B.nvfp4_ldlq_workspace(rows, cols), dtype=torch.uint8, device=DEV)
+    B.ldlq_quantize(W, 16, S, sf, perm.to(torch.int32), U, codes, st, ws)
+    assert st.item() == 0
+    grid = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6], device=DEV)
+    mids = torch.tensor([.25, .75, 1.25, 1.75, 2.5, 3.5, 5.], dtype=torch.float64, device=DEV)
+    e4m3 = torch.tensor([(8 + (c & 7)) * 2.0 ** ((c >> 3) - 10) if c >= 8 else c * 2.0 ** -9 for c in range(127)],
+                        device=DEV)
+    nib = torch.stack([codes & 15, codes >> 4], -1).reshape(rows, cols)[:, perm].long()
+    v = e4m3[sf.long()][:, perm // 16]
+    q = torch.where(nib > 7, -grid[nib & 7], grid[nib & 7])
+    Wp = W[:, perm]
+    T = Wp.double() + (Wp - (q * v) * S).double() @ U.double()
+    unit = v.double() * S.double()
+    t = T.abs() / unit.clamp_min(1e-300)
+    flips = int((((torch.bucketize(t, mids)) != (nib & 7)) & (v > 0)).sum())
+    gap = (t[..., None] - mids).abs().amin(-1) * unit / T.square().mean().sqrt()      # in units of the rms
+    rho = int((gap < 1e-4).sum()) / 2e-4
+    mean = rho * (2 / np.pi) ** 0.5 * 2.0 ** -22                                      # E|d| of a normal error
+    print(f"[ldlq] {rows} x {cols}: {flips} codes off their 64-bit targets' (FP32 sums: about {mean:.1f})")
+    assert flips <= mean + 4 * mean ** 0.5
