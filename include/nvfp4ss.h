@@ -389,7 +389,8 @@ nvfp4_status nvfp4_dequantize(const uint8_t* codes, const uint8_t* sf, nvfp4_sf_
  *           factorization then).
  *           |= 16 if a tensor-core update's bounded wait ran out (about a
  *           second; that update is then incomplete).
- *   workspace   device bytes, at least nvfp4_ldlq_prepare_workspace(n).
+ *   workspace   nvfp4_ldlq_prepare_workspace(n) device bytes; with fewer, but at
+ *           least 4 n (to a multiple of 256) + 16640, the updates take the FP32 pipe.
  * Cost: n^3/3 fp32 multiply-adds (blocked Cholesky, 64-wide panels).  The
  * trailing updates run on the tensor cores as three TF32 products per term
  * (products to ~2^-21 relative, the large and the small ones summed apart) when
@@ -421,8 +422,10 @@ nvfp4_status nvfp4_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
  *   whose codes are then zeros: with bit 16 the result is not the LDLQ pass's.
  *   perm, U from nvfp4_ldlq_prepare (cols = n); status_dev optional: |= 8 if
  *   perm holds an index outside [0, cols) (the entry is then read as 0).
- *   workspace   device bytes, at least nvfp4_ldlq_workspace(rows, cols):
- *           rows*cols*10 + rows*4096 + cols*4100 plus alignment.
+ *   workspace   nvfp4_ldlq_workspace(rows, cols) device bytes: rows*cols*10 +
+ *           rows*4096 + cols*4100 plus alignment.  With fewer, but at least rows*cols*10
+ *           + rows*2048 + cols*4 (each of its seven parts to a multiple of 256), the
+ *           updates past a super-panel of 256 columns take the FP32 pipe.
  * Cost: rows*cols^2/2 fp32 multiply-adds; rows are independent.  The column
  * walk uses the high-priority stream described under nvfp4_ldlq_prepare (same
  * first-call and concurrency rules).

@@ -180,7 +180,8 @@ __device__ __forceinline__ float sum2(u64 v) {
 
 // One panel's sequential part, in one CTA: the Cholesky factor of the nb x nb
 // diagonal block at k0 (lower, in place), its inverse Linv (64 x 64, lower), and the
-// solved panel of the next 64 rows, Xtop = A[k0 + nb .., k0 ..] Linv^T.
+// solved panel of the next 64 rows, Xtop = A[k0 + nb .., k0 ..] Linv^T, element (r, c) at
+// r xr + c xc.
 //
 // The block is padded to 64 with an identity and held as 4 x 4 tiles in registers.
 // Warp J < 16 holds tile column J: lanes (I, h) have rows 2h, 2h + 1 of tile (I, J)
@@ -206,7 +207,7 @@ __device__ __forceinline__ float sum2(u64 v) {
 // memory, 480-560 cycles per column.  Holding the workers back until the diagonal
 // tiles have read their operands: no gain.
 __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(float* A, int64_t n, int64_t k0, int nb, float* Linv,
-                                                              float* Xtop, int* status) {
+                                                              float* Xtop, int64_t xr, int64_t xc, int* status) {
     extern __shared__ __align__(16) float psm[];
     float* sl = psm;                                 // [64][kPad] Linv
     float* st = psm + kP * kPad;                     // [64][kPad] the next 64 rows of the panel
@@ -451,20 +452,21 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(float* A, int64_t 
 #pragma unroll
         for (int i = 0; i < 4; i++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) Xtop[(r + 16 * i) * kP + c + 16 * j] = o[i][j];
+            for (int j = 0; j < 4; j++)
+                if (r + 16 * i < nt) Xtop[(r + 16 * i) * xr + (c + 16 * j) * xc] = o[i][j];
     }
 }
 
 // The rows i >= k0 + 64 of one panel, 32 per CTA: the solved panel X = A Linv^T (in
-// place, and split into TF32 halves Lh, Ll [n, 64] for the trailing update), then the next panel's block column, A[i][k0 + 64 ..] -= X Xtop^T, up
-// to column i.  Everything in fp32 from shared memory; a separate panel solve and a
+// place, and, unless Lh is null, split into TF32 halves Lh, Ll [n, 64] for the trailing
+// update), then the next panel's block column, A[i][k0 + 64 ..] -= X Xtop^T, up to column i.  Everything in fp32 from shared memory; a separate panel solve and a
 // tensor-core update of a 64-wide column spent 14 us here on launches, tile fills
 // and half-empty tiles.
 constexpr int kPanelRows = 32;
 constexpr int kPanelSmem = (2 * kP + 2 * kPanelRows) * kPad * 4;
 template <bool VEC>
 __global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t k0, const float* Linv, const float* Xtop,
-                                                    float* Lh, float* Ll) {
+                                                    int64_t xr, int64_t xc, float* Lh, float* Ll) {
     grid_launch_dependents();                        // the next diagonal factor waits for this grid's end
     extern __shared__ __align__(16) float psm[];
     float* sl = psm;                                 // [64][kPad] Linv
@@ -489,7 +491,13 @@ __global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t
 #pragma unroll
     for (int u = 0; u < kP * kQ / 128; u++) {
         vl[u] = reinterpret_cast<const float4*>(Linv)[threadIdx.x + 128 * u];
-        vt[u] = reinterpret_cast<const float4*>(Xtop)[threadIdx.x + 128 * u];
+        const int e = threadIdx.x + 128 * u, r = e / kQ, c = 4 * (e % kQ);
+        vt[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (k0 + kP + r < n) {
+            const float* x = Xtop + r * xr + c * xc;
+            if (xc == 1) vt[u] = *reinterpret_cast<const float4*>(x);
+            else vt[u] = make_float4(x[0], x[xc], x[2 * xc], x[3 * xc]);
+        }
     }
 #pragma unroll
     for (int u = 0; u < kPanelRows * kQ / 128; u++) {
@@ -522,10 +530,12 @@ __global__ void __launch_bounds__(128) panel_kernel(float* A, int64_t n, int64_t
         if (VEC) {
             const float4 x = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
             *reinterpret_cast<float4*>(a) = x;
-            float4 h, l;                              // the trailing update's operands
-            tc::split4(x, h, l);
-            *reinterpret_cast<float4*>(Lh + r * kP + 4 * tx) = h;
-            *reinterpret_cast<float4*>(Ll + r * kP + 4 * tx) = l;
+            if (Lh) {                                 // the trailing update's operands
+                float4 h, l;
+                tc::split4(x, h, l);
+                *reinterpret_cast<float4*>(Lh + r * kP + 4 * tx) = h;
+                *reinterpret_cast<float4*>(Ll + r * kP + 4 * tx) = l;
+            }
             if (c0 + 3 <= r) vc[i] = *reinterpret_cast<const float4*>(A + r * n + c0);
         } else {
 #pragma unroll
@@ -1032,7 +1042,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
         for (int i = tid; i < nr * span; i += kWalkThreads) {
             const int64_t rr = row0 + i / span;
             const int c = i % span;
-            Eh[rr * kLdlqPanel + c] = El[rr * kLdlqPanel + c] = 0.0f;
+            Eh[rr * kLdlqPanel + c] = 0.0f;
+            if (El) El[rr * kLdlqPanel + c] = 0.0f;
             p.qb[rr * p.n + s0 + c] = 0;
         }
         return;
@@ -1121,13 +1132,16 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(LdlqParams p, int
                 }
                 step_barrier();                        // publish before the global stores
                 if (active) {
-                    float4 h, l;                       // the trailing update's operands, [rows, kLdlqPanel] TF32 halves
+                    // the trailing update's operands, [rows, kLdlqPanel]: TF32 halves, or the error itself
                     const int64_t at = r * kLdlqPanel + g * kGroupCols;
 #pragma unroll
                     for (int j = 0; j < 8; j += 4) {
-                        tc::split4(make_float4(ev[j], ev[j + 1], ev[j + 2], ev[j + 3]), h, l);
+                        float4 h = make_float4(ev[j], ev[j + 1], ev[j + 2], ev[j + 3]), l;
+                        if (El) {
+                            tc::split4(h, h, l);
+                            *reinterpret_cast<float4*>(El + at + j) = l;
+                        }
                         *reinterpret_cast<float4*>(Eh + at + j) = h;
-                        *reinterpret_cast<float4*>(El + at + j) = l;
                     }
                     *reinterpret_cast<uint2*>(p.qb + rbase + g * kGroupCols) = make_uint2(packed[0], packed[1]);
                 }
@@ -1234,8 +1248,10 @@ constexpr int64_t kGatherSmemMax = 200 * 1024;     // dynamic shared memory of t
 
 }  // namespace
 
-size_t ldlq_prepare_workspace(int64_t n) {
-    return (size_t)((n * 4 + 255) / 256 * 256) + 256 + (size_t)2 * kP * kP * 4 + (size_t)2 * n * kP * 4;
+// diag(H), lambda, Linv; with split, Xtop and the solved panel's TF32 halves.
+size_t ldlq_prepare_workspace(int64_t n, bool split) {
+    const size_t least = (size_t)((n * 4 + 255) / 256 * 256) + 256 + (size_t)kP * kP * 4;
+    return split ? least + (size_t)kP * kP * 4 + (size_t)2 * n * kP * 4 : least;
 }
 
 // Stream and events of the factorization's look-ahead, one set per device,
@@ -1272,15 +1288,16 @@ cudaError_t lookahead_for_current_device(LookAhead** out, std::unique_lock<std::
 }
 
 cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* perm, float* U, float* D,
-                                int* status, void* ws, int sms, cudaStream_t s) {
+                                int* status, void* ws, bool split, int sms, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     char* w = static_cast<char*>(ws);
     float* d = reinterpret_cast<float*>(w);
     float* lam = reinterpret_cast<float*>(w + (n * 4 + 255) / 256 * 256);
     float* Linv = lam + 64;
-    float* Xtop = Linv + kP * kP;
-    float* Lh = Xtop + kP * kP;          // the solved panel's TF32 halves, [n, 64] each
-    float* Ll = Lh + n * kP;
+    const bool vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
+    float* Xw = split ? Linv + kP * kP : nullptr;
+    float* Lh = split && vec ? Xw + kP * kP : nullptr;          // the solved panel's TF32 halves, [n, 64] each
+    float* Ll = Lh ? Lh + n * kP : nullptr;
     diag_kernel<<<1, 1024, 0, s>>>(H, n, damp, d, lam, status);
     rank_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(d, n, perm);
     const unsigned rg = (unsigned)imin64(n, (int64_t)sms * 8);
@@ -1300,28 +1317,36 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
     if ((e = cudaStreamWaitEvent(c, la->fork, 0)) != cudaSuccess) return e;
     constexpr int kPotrfSmem = 2 * kP * kPad * 4;
     static_assert(kPotrfSmem <= 48 * 1024, "no shared-memory opt-in");
-    const bool vec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
     const auto panel = vec ? panel_kernel<true> : panel_kernel<false>;
     if ((e = cudaFuncSetAttribute(panel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPanelSmem)) != cudaSuccess) return e;
     bool have_rest = false;              // rest_done recorded by this call (waits stay inside a capture)
     for (int64_t k0 = 0; k0 < n; k0 += kP) {
         const int nb = (int)imin64(kP, n - k0);
+        // without room of its own Xtop lies transposed above the diagonal, right of the
+        // diagonal block, where nothing else is kept until the factor is turned over
+        float* Xtop = Xw ? Xw : U + k0 * n + k0 + nb;
+        const int64_t xr = Xw ? kP : 1, xc = Xw ? 1 : n;
         // scheduled while the last panel kernel runs, ordered after its writes
-        if ((e = launch_dependent_smem(potrf_kernel, 1, kPotrfThreads, kPotrfSmem, c, U, n, k0, nb, Linv, Xtop, status)) != cudaSuccess)
+        if ((e = launch_dependent_smem(potrf_kernel, 1, kPotrfThreads, kPotrfSmem, c, U, n, k0, nb, Linv, Xtop, xr,
+                                       xc, status)) != cudaSuccess)
             return e;
         const int64_t rest = n - k0 - nb;
         if (rest > 0) {
             const int64_t nb2 = imin64(kP, rest);      // width of the next panel
             // the next block column also took the previous panel's rest update
             if (have_rest && (e = cudaStreamWaitEvent(c, la->rest_done, 0)) != cudaSuccess) return e;
-            panel<<<(unsigned)((rest + kPanelRows - 1) / kPanelRows), 128, kPanelSmem, c>>>(U, n, k0, Linv, Xtop, Lh, Ll);
+            panel<<<(unsigned)((rest + kPanelRows - 1) / kPanelRows), 128, kPanelSmem, c>>>(U, n, k0, Linv, Xtop, xr, xc, Lh,
+                                                                                                Ll);
             if (rest > nb2) {
                 const int64_t i0 = k0 + nb + nb2, m = rest - nb2;
                 float* P = U + i0 * n + k0;            // the solved panel's rows past the next block column
                 if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(s, la->panel_done, 0)) != cudaSuccess) return e;
-                const tc::Split L{Lh + i0 * kP, Ll + i0 * kP, kP};
-                e = vec ? tc::launch_gemm<true>(U + i0 * n + i0, n, L, L, m, m, nb, -1.0f, status, 0, sms, s) : cudaErrorNotSupported;
+                e = cudaErrorNotSupported;
+                if (Lh) {
+                    const tc::Split L{Lh + i0 * kP, Ll + i0 * kP, kP};
+                    e = tc::launch_gemm<true>(U + i0 * n + i0, n, L, L, m, m, nb, -1.0f, status, 0, sms, s);
+                }
                 if (e == cudaErrorNotSupported)
                     e = launch_gemm<true, true>(U + i0 * n + i0, n, P, n, P, n, m, m, nb, -1.0f, s);
                 if (e != cudaSuccess) return e;
@@ -1342,12 +1367,12 @@ cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* 
 }
 
 // Workspace: T and Wp [rows, n] f32, qb and sfp [rows, n] bytes, inv [n], and, twice
-// (alternating between super-panels), the TF32 halves of a super-panel's errors
-// [rows, kLdlqPanel] and of its rows of U [n, kLdlqPanel].
-size_t ldlq_quantize_workspace(int64_t rows, int64_t n) {
+// (alternating between super-panels), a super-panel's errors [rows, kLdlqPanel], or with
+// split the TF32 halves of them and of its rows of U [n, kLdlqPanel].
+size_t ldlq_quantize_workspace(int64_t rows, int64_t n, bool split) {
     auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
-    return (size_t)(2 * up(rows * n * 4) + 2 * up(rows * n) + 4 * up((int64_t)kLdlqPanel * rows * 4) +
-                    4 * up((int64_t)kLdlqPanel * n * 4) + up(n * 4));
+    const int64_t ep = up((int64_t)kLdlqPanel * rows * 4), up4 = up((int64_t)kLdlqPanel * n * 4);
+    return (size_t)(2 * up(rows * n * 4) + 2 * up(rows * n) + (split ? 4 * ep + 4 * up4 : 2 * ep) + up(n * 4));
 }
 
 // Columns in super-panels of kLdlqPanel (256), each walked by walk_kernel; after
@@ -1356,9 +1381,12 @@ size_t ldlq_quantize_workspace(int64_t rows, int64_t n) {
 // is split into the next super-panel's columns, which run with its panel walks
 // on the high-priority stream, and the rest, which runs on `s` concurrently
 // with them.  Before the rest of super-panel k, `s` also transposes and splits the rows
-// of U that super-panel k + 1 will need.
-cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* ws, int sms, cudaStream_t s) {
+// of U that super-panel k + 1 will need.  Without the workspace for that (split false)
+// or a driver with tensor maps, the updates run on the FP32 pipe.
+cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* ws, bool split, int sms,
+                                 cudaStream_t s) {
     if (p.rows <= 0 || p.n <= 0) return cudaSuccess;
+    if (tc::encode_fn() == nullptr) split = false;
     auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
     char* w = static_cast<char*>(ws);
     const int64_t mat4 = up(p.rows * p.n * 4), mat1 = up(p.rows * p.n);
@@ -1368,10 +1396,14 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     p.sfp = reinterpret_cast<uint8_t*>(w + 2 * mat4 + mat1);
     const int64_t ep = up((int64_t)kLdlqPanel * p.rows * 4), up4 = up((int64_t)kLdlqPanel * p.n * 4);
     char* q = w + 2 * mat4 + 2 * mat1;
-    tc::Split Es[2], Us[2];                        // ld = kLdlqPanel
-    for (int i = 0; i < 2; i++, q += 2 * ep + 2 * up4) {
-        Es[i] = {reinterpret_cast<float*>(q), reinterpret_cast<float*>(q + ep), kLdlqPanel};
-        Us[i] = {reinterpret_cast<float*>(q + 2 * ep), reinterpret_cast<float*>(q + 2 * ep + up4), kLdlqPanel};
+    tc::Split Es[2], Us[2];                        // ld = kLdlqPanel; without split hi is the whole error
+    for (int i = 0; i < 2; i++) {
+        Es[i] = {reinterpret_cast<float*>(q), split ? reinterpret_cast<float*>(q + ep) : nullptr, kLdlqPanel};
+        q += split ? 2 * ep : ep;
+        if (split) {
+            Us[i] = {reinterpret_cast<float*>(q), reinterpret_cast<float*>(q + up4), kLdlqPanel};
+            q += 2 * up4;
+        }
     }
     int32_t* inv = reinterpret_cast<int32_t*>(q);
     cudaError_t e = cudaMemsetAsync(inv, 0, (size_t)p.n * 4, s);
@@ -1418,7 +1450,7 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     // the second operand of super-panel s0's trailing updates
     auto split_u = [&](int64_t s0, int i) {
         const int64_t c0 = s0 + kLdlqPanel;
-        if (c0 >= p.n) return cudaSuccess;
+        if (!split || c0 >= p.n) return cudaSuccess;
         split_u_kernel<<<dim3((unsigned)((p.n - c0 + 31) / 32), kLdlqPanel / 32), 256, 0, s>>>(
             p.U, p.n, s0, c0, const_cast<float*>(Us[i].hi), const_cast<float*>(Us[i].lo));
         const cudaError_t r = cudaGetLastError();
@@ -1427,14 +1459,12 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
     // T[:, c0 + d ..] += the errors of super-panel s0 x U, `cols` columns from column d of its trailing ones
     auto update = [&](int64_t s0, int i, int64_t d, int64_t cols, cudaStream_t st) {
         float* C = p.T + s0 + kLdlqPanel + d;
+        if (!split)
+            return launch_gemm<false, false>(C, p.n, Es[i].hi, kLdlqPanel, p.U + s0 * p.n + s0 + kLdlqPanel + d, p.n,
+                                             p.rows, cols, kLdlqPanel, 1.0f, st);
         const tc::Split B{Us[i].hi + d * kLdlqPanel, Us[i].lo + d * kLdlqPanel, kLdlqPanel};
-        cudaError_t r = tc::launch_gemm<false>(C, p.n, Es[i], B, p.rows, cols, kLdlqPanel, 1.0f, p.status,
-                                               (p.starve & kStarveUpdate) != 0, sms, st);
-        if (r != cudaErrorNotSupported) return r;
-        const float* u = p.U + s0 * p.n + s0 + kLdlqPanel + d;         // no tensor maps: both halves on the FP32 pipe
-        r = launch_gemm<false, false>(C, p.n, Es[i].hi, kLdlqPanel, u, p.n, p.rows, cols, kLdlqPanel, 1.0f, st);
-        if (r != cudaSuccess) return r;
-        return launch_gemm<false, false>(C, p.n, Es[i].lo, kLdlqPanel, u, p.n, p.rows, cols, kLdlqPanel, 1.0f, st);
+        return tc::launch_gemm<false>(C, p.n, Es[i], B, p.rows, cols, kLdlqPanel, 1.0f, p.status,
+                                      (p.starve & kStarveUpdate) != 0, sms, st);
     };
     if ((e = split_u(0, 0)) != cudaSuccess) return e;
     // The walk and the update of its columns (one CTA per SM both) fit the GPU together:
@@ -1459,7 +1489,7 @@ cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* 
         if (rest > 0) {
             const int64_t next = imin64(kLdlqPanel, rest);
             if ((e = cudaEventRecord(la->panel_done, c)) != cudaSuccess) return e;
-            if ((e = cudaStreamWaitEvent(c, la->split_done, 0)) != cudaSuccess) return e;
+            if (split && (e = cudaStreamWaitEvent(c, la->split_done, 0)) != cudaSuccess) return e;
             // the next super-panel's columns also took the previous rest update, and that
             // update read the buffers the next super-panel overwrites
             if (have_rest && (e = cudaStreamWaitEvent(c, la->rest_done, 0)) != cudaSuccess) return e;

@@ -28,10 +28,13 @@ struct LdlqParams {
     uint8_t* sfp;             // workspace: each element's scale code, processing order
     int starve;               // kStarve* bits: waits that never end (self-test), else 0
 };
-size_t ldlq_prepare_workspace(int64_t n);
+// Workspaces: with split operands for the tensor cores, or (split false) the least a call
+// takes, with the updates on the FP32 pipe.
+size_t ldlq_prepare_workspace(int64_t n, bool split);
 cudaError_t launch_ldlq_prepare(const float* H, int64_t n, float damp, int32_t* perm, float* U, float* D,
-                                int* status, void* ws, int sms, cudaStream_t s);
-size_t ldlq_quantize_workspace(int64_t rows, int64_t n);
-cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* ws, int sms, cudaStream_t s);
+                                int* status, void* ws, bool split, int sms, cudaStream_t s);
+size_t ldlq_quantize_workspace(int64_t rows, int64_t n, bool split);
+cudaError_t launch_ldlq_quantize(LdlqParams p, int dtype, uint8_t* codes, void* ws, bool split, int sms,
+                                 cudaStream_t s);
 
 }  // namespace nvfp4

@@ -299,3 +299,23 @@ def test_build_covers_every_source_for_sm_103a():
     inputs = set(os.path.basename(f) for f in Bd._inputs())
     headers = {f for f in os.listdir(Bd.CSRC) if f.endswith((".h", ".cuh"))} | {"nvfp4ss.h"}
     assert headers | set(cu) <= inputs
+
+
+def test_ldlq_takes_the_least_workspace(L):
+    """The sizes that the header documents pass the size check (the misaligned input
+    behind it is then refused), one byte less does not."""
+    f = ctypes.c_float
+    up = lambda b: -(-b // 256) * 256
+    for n in (64, 1040):
+        least = up(4 * n) + 256 + 4 * 64 * 64
+        prep = lambda b: L.nvfp4_ldlq_prepare(FAKE + 2, n, f(0.01), FAKE + 0x10000000, FAKE + 0x20000000,
+                                              FAKE + 0x30000000, None, FAKE + 0x40000000, b, None)
+        assert (prep(least - 1), prep(least)) == (1, 3)
+        assert least < L.nvfp4_ldlq_prepare_workspace(n)
+        rows, rc = 100, 100 * n
+        least = 2 * up(4 * rc) + 2 * up(rc) + 2 * up(1024 * rows) + up(4 * n)
+        q = lambda b: L.ldlq_quantize(FAKE + 1, 0, rows, n, 16, FAKE + 0x10000000, FAKE + 0x20000000,
+                                      FAKE + 0x30000000, FAKE + 0x40000000, FAKE + 0x50000000, None,
+                                      FAKE + 0x60000000, b, None)
+        assert (q(least - 1), q(least)) == (1, 3)
+        assert least < L.nvfp4_ldlq_workspace(rows, n)

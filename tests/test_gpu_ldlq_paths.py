@@ -7,6 +7,7 @@
 * Rows too long for the gather's and the packer's shared memory: with a zero factor the
   codes are plain rounding.
 * Factorizations off the panels of 64, with outputs that are not 16-byte aligned.
+* The least workspaces, without the split operands: updates on the FP32 pipe.
 * Sums of errors: kept where each is below the target's last place, and as close to 64
   bits as sums on the FP32 pipe.
 * Dependencies of a captured pass: only a walk behind an update may start before it ends.
@@ -69,6 +70,21 @@ def test_long_rows(B, n, dtype):
     assert np.array_equal(codes, ref)
 
 
+@pytest.mark.parametrize("n", [1, 63, 65, 129, 193, 330, 580])
+def test_least_factor_workspace(B, n):
+    _, H = rand_problem(2, n, n)
+    perm, U, D, _ = prepare(B, H)
+    pb = _least(1, n)[0]
+    w = _guarded(pb)
+    perm2, U2, D2 = torch.empty_like(perm), torch.empty_like(U), torch.empty_like(D)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    B.nvfp4_ldlq_prepare(torch.as_tensor(H, dtype=torch.float32, device=DEV), 0.01, perm2, U2, D2, st, w[:pb])
+    torch.cuda.synchronize()
+    assert st.item() == 0 and torch.all(w[pb:] == 0xA5)
+    assert torch.equal(perm, perm2) and torch.all(torch.tril(U2) == 0)
+    assert torch.allclose(D2, D, rtol=2e-4) and (U2 - U).abs().max() <= 2e-4 * max(1.0, float(U.abs().max()))
+
+
 @pytest.mark.parametrize("n", [1, 63, 65, 128, 193, 330, 580])
 def test_prepare_panels(B, n):
     _, H = rand_problem(2, n, n)
@@ -93,6 +109,44 @@ def test_prepare_panels(B, n):
         assert np.abs(Ug - U_ref).max() <= 2e-4 * max(1.0, np.abs(U_ref).max())
         R = (Ug + np.eye(n)) @ np.diag(Dg) @ (Ug + np.eye(n)).T - Hp
         assert np.abs(R).max() <= 2e-5 * np.abs(Hp).max()
+
+
+def _guarded(nbytes):
+    return torch.full((nbytes + 4096,), 0xA5, dtype=torch.uint8, device=DEV)
+
+
+def _least(rows, n):
+    up = lambda b: -(-b // 256) * 256
+    return (up(4 * n) + 256 + 4 * 64 * 64,
+            2 * up(4 * rows * n) + 2 * up(rows * n) + 2 * up(1024 * rows) + up(4 * n))
+
+
+# one panel; a ragged second one; several, off and on multiples of 4; several super-panels
+@pytest.mark.parametrize("rows,n", [(5, 64), (33, 80), (40, 304), (129, 784), (600, 1040)])
+def test_least_workspaces(B, rows, n):
+    W64, H = rand_problem(rows, n, rows * n)
+    W = W64.astype(np.float32)
+    S, sf = fixed_scales(W64, H)
+    pb, qb = _least(rows, n)
+    wp, wq = _guarded(pb), _guarded(qb)
+    Hd = torch.as_tensor(H, dtype=torch.float32, device=DEV)
+    perm, U, D, _ = prepare(B, Hd.double().cpu().numpy())     # with its full workspace
+    perm2, U2, D2 = torch.empty_like(perm), torch.empty_like(U), torch.empty_like(D)
+    codes = torch.empty(rows, n // 2, dtype=torch.uint8, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    B.nvfp4_ldlq_prepare(Hd, 0.01, perm2, U2, D2, st, wp[:pb])
+    sfd = torch.as_tensor(np.ascontiguousarray(sf), dtype=torch.uint8).to(DEV)
+    B.ldlq_quantize(torch.from_numpy(W).to(DEV), 16, torch.tensor([S], dtype=torch.float32, device=DEV), sfd, perm2, U2,
+                    codes, st, wq[:qb])
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    assert torch.all(wp[pb:] == 0xA5) and torch.all(wq[qb:] == 0xA5)
+    assert torch.equal(perm, perm2) and torch.all(torch.tril(U2) == 0)
+    # two fp32 factorizations of one matrix: the bounds of the tests against 64 bits
+    assert torch.allclose(D2, D, rtol=2e-4) and (U2 - U).abs().max() <= 2e-4 * max(1.0, float(U.abs().max()))
+    bad, exempt, total, first = conditional_parity(W.astype(np.float64), S, sf, 16, perm2.cpu().numpy().astype(np.int64),
+                                                   U2.double().cpu().numpy(), codes.cpu().numpy())
+    assert bad == 0 and first == 0 and exempt <= max(2, total // 200)
 
 
 def programmatic_edges(graph):
