@@ -128,6 +128,69 @@ __device__ __noinline__ void score_segment(Column<OBJ> col, int i, int k, float&
     }
 }
 
+// The seven segments of element i one after the other, with the operations of
+// score_segment, two segments to a packed one and four pairs to a pass: what blocks
+// without a screen take for all of their elements.  One segment at a time those were
+// slower than before there was a screen (512 x 8192 bf16 WMSE: one weight in ten
+// negative 540 -> 674 us, all magnitudes equal 530 -> 623; so 446 and 432).
+template <int BLOCK, int OBJ>
+__device__ __noinline__ void score_element(Column<OBJ> col, int i, float& best, float& best_s) {
+    const float ai = col.mag(i);
+    if (!(ai > 0.0f)) return;
+    const float ra = __frcp_rn(ai);
+    u64 r2[4], B2[4], C2[4], L2[4], ns2[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        r2[q] = pack2(segment_rcp(kMid[2 * q], ra), segment_rcp(kMid[2 * q + 1], ra));
+        B2[q] = C2[q] = L2[q] = 0ull;
+    }
+    auto grid2 = [&](int j, u64 a2, int q) -> u64 {
+        float tl, th, gl, gh;
+        unpack2(mul2(a2, r2[q]), tl, th);
+        rn_grid2(tl, th, gl, gh);
+        return j == i ? pack2(kGrid[2 * q], kGrid[2 * q + 1]) : pack2(gl, gh);
+    };
+#pragma unroll 4
+    for (int j = 0; j < BLOCK; j++) {
+        const float a = col.mag(j), w = col.wt(j);
+        const float wa = OBJ ? __fmul_rn(w, a) : a;
+        const u64 a2 = pack2(a, a), wa2 = pack2(wa, wa), w2 = pack2(w, w);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const u64 g2 = grid2(j, a2, q);
+            B2[q] = fma2(wa2, g2, B2[q]);
+            C2[q] = fma2(OBJ ? mul2(w2, g2) : g2, g2, C2[q]);
+        }
+    }
+    float b[8], c[8], L[8];                          // [7]: no segment
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        unpack2(B2[q], b[2 * q], b[2 * q + 1]);
+        unpack2(C2[q], c[2 * q], c[2 * q + 1]);
+#pragma unroll
+        for (int h = 2 * q; h < 2 * q + 2; h++) b[h] = __fdiv_rn(b[h], c[h]);        // the scale
+        ns2[q] = pack2(-b[2 * q], -b[2 * q + 1]);
+    }
+#pragma unroll 4
+    for (int j = 0; j < BLOCK; j++) {
+        const float a = col.mag(j), w = col.wt(j);
+        const u64 a2 = pack2(a, a), w2 = pack2(w, w);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const u64 e2 = fma2(ns2[q], grid2(j, a2, q), a2);
+            L2[q] = fma2(OBJ ? mul2(w2, e2) : e2, e2, L2[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) unpack2(L2[q], L[2 * q], L[2 * q + 1]);
+#pragma unroll
+    for (int h = 0; h < 7; h++)
+        if (c[h] > 0.0f && (L[h] < best * (1.0f - 1e-6f) || (L[h] <= best * (1.0f + 1e-6f) && b[h] < best_s))) {
+            best = fminf(best, L[h]);
+            best_s = b[h];
+        }
+}
+
 // How far the screen's A - B^2/C can lie from the scored loss, relative to A:
 // B and C carry at most n + 1 roundings each and B^2/C <= A (Cauchy-Schwarz), so
 // 3(n + 1) + 4 roundings of A, and the list entry drops 2^-14 of its own value
@@ -236,8 +299,7 @@ __global__ void __launch_bounds__(kOptThreads) optimal_scale_kernel(OptParams p)
             }
         }
         if (!screen_ok || noted > kOptList) {
-            for (int i = 0; i < BLOCK; i++)
-                for (int k = 0; k < 7; k++) score_segment<BLOCK, OBJ>(col, i, k, best, best_s);
+            for (int i = 0; i < BLOCK; i++) score_element<BLOCK, OBJ>(col, i, best, best_s);
         } else {
             const float limit = screen_limit<BLOCK>(least, A);
             for (int n = 0; n < noted; n++) {

@@ -184,3 +184,34 @@ def test_optimal_screen(B, block, kind):
     (s1, l1, c1, f1), (s2, l2, c2, f2) = res
     assert torch.equal(s1, s2) and torch.equal(c1, c2)
     assert torch.equal(l1 * 2.0 ** 100, l2) and torch.equal(f1 * 2.0 ** 100, f2)
+
+
+@pytest.mark.parametrize("block", [16, 32, 64])
+@pytest.mark.parametrize("kind", ["normal", "tails", "few", "negative"])
+def test_optimal_screen_unweighted(B, block, kind):
+    """The MSE form's screen against equal weights of 2^100, which are past it; and
+    (negative) blocks with a negative weight, which have no screen: their scale is that
+    of the same weights times 2^100."""
+    g = torch.Generator().manual_seed(block + 1)
+    rows, cols = 64, 512
+    x = torch.randn(rows, cols, generator=g)
+    if kind == "tails":
+        x = x * torch.exp(torch.randn(rows, cols, generator=g))
+    elif kind == "few":
+        x = torch.sign(x) * torch.randint(0, 4, (rows, cols), generator=g)
+    x, S = x.to(torch.bfloat16).to(DEV), torch.ones(1, device=DEV)
+    w = torch.ones(cols, device=DEV)
+    if kind == "negative":
+        w = torch.exp(torch.randn(cols, generator=g)).to(DEV)
+        w[::block] *= -0.1
+    nb = rows * cols // block
+    res = []
+    for obj, f in ((int(kind == "negative"), 1.0), (1, 2.0 ** 100)):
+        o = (torch.empty(nb, device=DEV), torch.empty(nb, device=DEV), torch.empty(nb, dtype=torch.uint8, device=DEV),
+             torch.empty(nb, device=DEV))
+        B.nvfp4_optimal_scale(x, block, S, obj, w * f if obj else None, 0, *o)
+        res.append(o)
+    torch.cuda.synchronize()
+    (s1, l1, c1, f1), (s2, l2, c2, f2) = res
+    assert torch.equal(s1, s2) and torch.equal(c1, c2)
+    assert torch.equal(l1 * 2.0 ** 100, l2) and torch.equal(f1 * 2.0 ** 100, f2)
