@@ -127,8 +127,8 @@ __device__ __forceinline__ float sixth(float m) {
 
 // e4m3_floor_code(fl(m / 6)) for m >= 0 (NaN and inf give 126): m >= 6 v_c exactly
 // when the product of m and fl(1/6), which is a third of an ulp above 1/6, rounded
-// towards zero reaches v_c -- compared with the division for every fp32 m that
-// reaches a code below the largest.  Normal codes are the top bits of that
+// towards zero reaches v_c -- compared with the division for every fp32 m from the
+// octave of the smallest 6 v_c to that of the largest.  Normal codes are the top bits of that
 // product, those below 2^-5 its integer part in units of 2^-9.
 __device__ __forceinline__ int e4m3_floor_code_of_sixth(float m) {
     const float s = __fmul_rz(m, 0.16666667163372039794921875f);

@@ -1,14 +1,15 @@
 """The default-window sweep skips low window offsets that a warp rules out with
 a lower bound on their loss (the block's largest element's own error term).
-That must not change anything: codes, both scale layouts and per-block losses
-are compared bit for bit against the same window given explicitly, a call
-that evaluates every candidate of the window with no skipping, on inputs that
+That must not change anything: codes, scales and per-block losses are compared
+bit for bit against the window given in two calls, [lo, 6] and [7, 7], which
+evaluate every candidate with no skipping (and the same window given in one,
+which takes the default's path, also in the swizzled layout), on inputs that
 stress the bound: heavy-tailed blocks (where the bound skips), blocks whose
 largest value repeats, all-zero and NaN/inf blocks in the same warp, negative
 and NaN weights (for which skipping must switch itself off), per-row weights,
 global scales near the ends of the E4M3 range, and blocks of 16, 32 and 64 in
-both input types.  The per-tensor sweep skips for MSE; the grouped launch,
-which must give the same bytes, skips for MSE and for WMSE with blocks of 16.
+both input types.  The per-tensor and the grouped sweep skip for both objectives and every block
+size, and must give the same bytes.
 """
 import numpy as np
 import pytest
@@ -86,6 +87,22 @@ def run_group(B, x, block, S, obj, w, stride):
     return out
 
 
+def two_windows(B, x, block, S, obj, w, stride, lo):
+    """The window [lo, 7] as [lo, 6] and [7, 7], the lower code on ties; and the blocks
+    all of whose codes exist (with negative weights a code that does not wins or not
+    by the path)."""
+    rows, cols = x.shape
+    a = run(B, x, block, S, obj, w, stride, (lo, 6))
+    b = run(B, x, block, S, obj, w, stride, (7, 7))
+    base = run(B, x, block, S, obj, w, stride, (0, 0))["sf_linear"].int()
+    hi = (b["block_loss"] < a["block_loss"]).view(rows, -1)
+    out = {"sf_linear": torch.where(hi, b["sf_linear"], a["sf_linear"]),
+           "block_loss": torch.where(hi, b["block_loss"].view(rows, -1), a["block_loss"].view(rows, -1)),
+           "codes": torch.where(hi[..., None], b["codes"].view(rows, cols // block, -1),
+                                a["codes"].view(rows, cols // block, -1))}
+    return out, (base + lo >= 1) & (base + 7 <= 126)
+
+
 def same(a, b):
     for k in ("codes", "sf_linear", "sf_swizzled", "block_loss"):
         if a[k] is None:
@@ -113,7 +130,12 @@ def test_skipping_sweep_equals_full_window(B, dtype, block, obj, wkind, xkind):
         fast = run(B, xd, block, S, obj, wd, stride, (B.NVFP4_WINDOW_DEFAULT, B.NVFP4_WINDOW_DEFAULT))
         full = run(B, xd, block, S, obj, wd, stride, (lo, 7))
         same(fast, full)
-        grouped = run_group(B, xd, block, S, obj, wd, stride)      # the grouped sweep skips for WMSE too
+        every, inside = two_windows(B, xd, block, S, obj, wd, stride, lo)
+        at = inside if wkind in ("negative", "nan") else torch.ones_like(inside)
+        assert torch.equal(fast["sf_linear"][at], every["sf_linear"][at])
+        assert torch.equal(fast["codes"].view(rows, cols // block, -1)[at], every["codes"][at])
+        assert torch.equal(fast["block_loss"].view(rows, -1)[at].view(torch.int32), every["block_loss"][at].view(torch.int32))
+        grouped = run_group(B, xd, block, S, obj, wd, stride) 
         for k in ("codes", "sf_linear", "sf_swizzled"):
             if grouped[k] is not None:
                 assert torch.equal(grouped[k], full[k]), k
