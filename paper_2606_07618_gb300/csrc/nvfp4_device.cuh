@@ -35,17 +35,6 @@ __device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
     return d;
 }
 
-// Two fp32 -> one byte of two E2M1 codes (RNE, saturating at 6): `hi` goes to
-// the upper nibble, `lo` to the lower nibble.
-__device__ __forceinline__ uint32_t e2m1x2(float lo, float hi) {
-    uint32_t r;
-    asm("{\n\t.reg .b8 q;\n\t"
-        "cvt.rn.satfinite.e2m1x2.f32 q, %1, %2;\n\t"
-        "cvt.u32.u8 %0, q;\n\t}"
-        : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-
 // Eight fp32 (four packed pairs) -> a word of eight E2M1 codes, the first in the
 // lowest nibble: the converts' bytes are assembled by the conversions themselves.
 __device__ __forceinline__ uint32_t e2m1x8(u64 t0, u64 t1, u64 t2, u64 t3) {

@@ -41,10 +41,8 @@
 // CTAs on the registers they leave free: the largest tensor is reduced, then
 // swept while the other tensors are reduced beside it, then the others are
 // swept.  Only the first reduction is exposed.  On the two Qwen2.5-72B-shaped
-// matrices (WMSE, full-window sweep) 1.506-1.512 ms per call against
-// 1.568-1.573 ms two-phase and 1.406-1.411 ms with static scales; on the
-// Llama-3-8B layer 0.681 against 0.735 (static 0.643).  (With the sweep's octave pairs
-// and its early end of the low codes the pipelined calls take 1.300 and 0.587 ms.)
+// matrices (WMSE) 1.307 ms per call against 1.350 ms two-phase and 1.194 ms with
+// static scales.
 #include <atomic>
 
 #include "group_kernels.h"

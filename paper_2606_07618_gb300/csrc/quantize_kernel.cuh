@@ -359,7 +359,6 @@ __device__ __forceinline__ int default_window_argmin(const u64 (&y2)[8], const u
             }
         }
     }
-    if (NB == 0) return bk;
     const u64 m2 = pack2(ma, mb);
     u64 wab = 0ull;
     float none = 0.0f;

@@ -671,11 +671,10 @@ cudaError_t launch_gemm(float* C, int64_t ldc, const Split& A, const Split& B, i
     // Tiles per SM.  One tile to a CTA spends almost half its time filling the ring and
     // adding to C (9 us at K = 256, 5 of them loads and MMAs); two or four overlap that,
     // but leave the SMs less evenly filled and later for a waiting walk or factor.
-    // Passes with one / from 2 / from 3 / from 4 tiles per SM on: 4096 x 4096 929 / 916 /
-    // 917 / 918 us, 14336 x 4096 2.84 / 2.66 / 2.65 / 2.66 ms, 4096 x 14336 7.23 / 6.44 /
-    // 6.43 / 6.44; the factor at n = 4096 1.579 / 1.613 / 1.581 / 1.581 and n = 14336 21.8 /
-    // 20.7 / 20.7 / 20.7.  Four tiles from 4 per SM on: 4096 x 4096 931; never: 4096 x 14336 6.76.
-    // (Taken with one accumulator to a tile.)
+    // Passes with one / from 2 / from 3 / from 4 tiles per SM on: 4096 x 4096 966 / 954 /
+    // 949 / 953 us, 14336 x 4096 2.92 / 2.72 / 2.72 / 2.72 ms, 4096 x 14336 7.54 / 6.68 /
+    // 6.68 / 6.68; the factor at n = 4096 1.607 / 1.628 / 1.605 / 1.606 and n = 14336 22.3 /
+    // 20.8 / 20.8 / 20.8.  Four tiles from 4 per SM on: 4096 x 4096 966; never: 4096 x 14336 7.01.
     const int64_t waves = (LOWER ? tm * tn / 2 : tm * tn) / sms;
     if (waves < 3) {
         gemm_kernel<LOWER><<<dim3((unsigned)tn, (unsigned)tm), kThreads, kSmemBytes, s>>>(mah, mal, mbh, mbl, mc, K, alpha,
