@@ -150,17 +150,6 @@ __device__ __forceinline__ uint32_t ld_u32(const void* p) {
     asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint32_t ld_u16(const void* p) {
-    uint16_t v;
-    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ uint32_t ld_u8(const void* p) {
-    uint32_t v;
-    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-
 // Streaming 16-byte load that bypasses L1 allocation (each byte is read once).  NC:
 // the non-coherent form, for data that nothing writes while the kernel is scheduled
 // (any launch but a programmatic dependent of the data's producer; 0.5% on the sweeps).

@@ -181,10 +181,16 @@ constexpr int kDequantUnroll = 8;      // chunks per lane per tile: of 2, 4, 8, 
 // 0.214 ms against two integer divisions).  Linear layout: e0 / block as
 // written measured faster than the shift (0.210 against 0.226 ms on the Qwen
 // shapes): the slower index spaces the scale-byte loads behind the code loads.
+//
+// A programmatic dependent itself, it lets no later grid in before its CTAs end: waiting
+// CTAs beside it cost up to a tenth (16384 x 8192 bf16, linear scales 58.3 us a call, 67.9
+// with an early trigger and volatile loads; swizzled 59.3 / 60.9; fp32 107.8 / 112.8 and
+// 106.8 / 119.5; launched the ordinary way 61.2 / 62.6 and 109.7 / 110.3).  The code and
+// scale loads are ordinary ones, which the compiler schedules as it likes below the wait
+// (it cannot make them non-coherent: the output may alias them).
 template <int OUT_BF16>
 __global__ void __launch_bounds__(256) dequant_kernel(DequantParams p, FastDiv kbd, int bshift) {
     constexpr int EPT = OUT_BF16 ? 8 : 4;          // elements per thread
-    grid_launch_dependents();
     grid_dependency_wait();
     const float S = ld_f32(p.S);
     const int64_t nchunk = p.nseg * (16 / EPT);
@@ -205,8 +211,8 @@ __global__ void __launch_bounds__(256) dequant_kernel(DequantParams p, FastDiv k
         return swizzle_offset(row, kbi, p.kpad4);
     };
     auto load_codes = [&](int64_t c) -> uint32_t {
-        return EPT == 8 ? ld_u32(reinterpret_cast<const uint32_t*>(p.codes) + c)
-                        : ld_u16(reinterpret_cast<const uint16_t*>(p.codes) + c);
+        return EPT == 8 ? reinterpret_cast<const uint32_t*>(p.codes)[c]
+                        : (uint32_t)reinterpret_cast<const uint16_t*>(p.codes)[c];
     };
     int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * kDequantUnroll + (threadIdx.x & 31);
     for (; c0 < nchunk; c0 += stride * kDequantUnroll) {
@@ -217,7 +223,7 @@ __global__ void __launch_bounds__(256) dequant_kernel(DequantParams p, FastDiv k
             const int64_t c = c0 + 32 * u;
             if (c < nchunk) {
                 cwv[u] = load_codes(c);
-                scv[u] = (uint8_t)ld_u8(p.sf + scale_offset(c * EPT));
+                scv[u] = p.sf[scale_offset(c * EPT)];
             }
         }
 #pragma unroll
